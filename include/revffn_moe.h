@@ -459,16 +459,14 @@ int revffn_moe_step_host(const revffn_moe_desc* desc, const revffn_moe_weights* 
  * Limits and sharing
  *   - (E + 1) * h <= REVFFN_ROUTE_NOALLOC_MAX_ELEMS (512 KB of scratch, held by
  *     every device that loads the library until the process exits); otherwise
- *     REVFFN_ERR_NOALLOC_LIMIT and nothing is launched.  The router kernel keeps
- *     a 32-token tile of logits in shared memory, 8 * 32 * (E + 1) bytes plus
- *     27.3 KB of operand staging: above 48 KB in total (E >= 83) the first call on
- *     a device raises the kernel's dynamic shared-memory limit, which is a
- *     function attribute, not an allocation; E = 256 needs 92 KB.
+ *     REVFFN_ERR_NOALLOC_LIMIT and nothing is launched.  The router kernel needs
+ *     more dynamic shared memory than a kernel may use by default (59 KB at E = 60, 200 KB at E = 256): the first
+ *     call on a device raises its limit, which is a function attribute, not an allocation.
  *   - REVFFN_FLAG_GATE_SOFTMAX_ALL is not supported here (its gates need the
  *     softmax over all E logits, which this entry point does not form):
  *     REVFFN_ERR_UNSUPPORTED, nothing is launched.  Other flags are ignored.
- *   - The first call on a device looks up the array's device address (and may
- *     raise the shared-memory limit, above); make that first call outside any
+ *   - The first call on a device looks up the array's device address and
+ *     raises the shared-memory limit (above); make that first call outside any
  *     stream capture.
  *   - All calls on a device share the one array.  Each call rewrites the part
  *     it uses before reading it, so nothing has to be cleared, but two calls

@@ -16,8 +16,6 @@ typedef __nv_bfloat16 bf16;
 // multiple of ROW_PAD rows, so that a 128-row GEMM tile never spans two experts
 // and the per-expert K range of a weight-gradient GEMM is a whole number of tiles.
 constexpr int ROW_PAD = 128;
-// Tokens per block in the counting sort that builds the permutation.
-constexpr int MAP_CHUNK = 128;
 
 __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 __host__ __device__ inline int64_t round_up(int64_t a, int64_t b) { return ceil_div(a, b) * b; }

@@ -90,7 +90,7 @@ constexpr int GUARD_BYTES = 256;
 
 struct WsLayout {
   // forward / inverse
-  Buf status, rows_total, w_rc, w_rc_part, n, r, idx, gates, sgate, prob, local_rank, chunk_cnt, chunk_base, expert_cnt,
+  Buf status, rows_total, w_rc, w_rc_part, n, r, idx, gates, sgate, prob, local_rank, chunk_cnt, expert_cnt,
       expert_off, tile_group, tok_chunks, tok_row, row_tok, row_gate, u, up, hmid, o, hs, s, z, upq, up_scale, hq, h_scale;
   int max_chunks = 0;
   size_t fwd_bytes = 0;
@@ -115,7 +115,7 @@ static WsLayout plan_workspace(const revffn_moe_desc& D) {
   const int64_t T = D.tokens, d = D.d_model, h = d / 2, E = D.n_experts, k = D.top_k, I = D.d_expert,
                 Is = D.d_shared;
   L.rows_pad = max_padded_rows(T, (int)k, (int)E);
-  L.n_chunks = (int)ceil_div(T > 0 ? T : 1, MAP_CHUNK);
+  L.n_chunks = (int)ceil_div(T > 0 ? T : 1, map_chunk_tokens(T));
   L.max_tiles = (int)(L.rows_pad / ROW_PAD);
   L.dg_ld = (int)ceil_div(I, SIMT_BN);
   L.strips = (int)ceil_div(T > 0 ? T : 1, STRIP);
@@ -142,7 +142,6 @@ static WsLayout plan_workspace(const revffn_moe_desc& D) {
   take(L.prob, (D.flags & REVFFN_FLAG_GATE_SOFTMAX_ALL) ? (size_t)T * E * 4 : 0);
   take(L.local_rank, (size_t)T * k * 4);
   take(L.chunk_cnt, (size_t)L.n_chunks * E * 4);
-  take(L.chunk_base, (size_t)L.n_chunks * E * 4);
   take(L.expert_cnt, (size_t)E * 4);
   take(L.expert_off, (size_t)(E + 1) * 4);
   take(L.tile_group, (size_t)L.max_tiles * 4);
@@ -409,13 +408,29 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
   }
   CK(cudaGetLastError());
 
+  // P_up: U = N W_up^T
+  auto p_up = [&]() -> int {
+    GemmProblem p = blank_problem();
+    p.M = Tn; p.N = d; p.K = h;
+    p.A = c.template p<T>(L.n); p.lda = h;
+    p.B0 = w_up; p.ldb = h;
+    p.epilogue = EPI_STORE; p.C = c.template p<T>(L.u); p.ldc = d;
+    return run_gemm(c, p, TG_PUP);
+  };
+  // The logits and P_up can run at the same time, but once the logits' blocks fill the GPU they only get in each
+  // other's way: a product CTA needs a whole SM and its tiles are dealt out in advance, so SMs that the router
+  // gives up late hold up the whole product.  At 8192 tokens, in the inverse pass: beside each other 104-148 us for
+  // P_up, maps ready after 150 us; one after the other 42 us and after 128 us.  The line is two router blocks per SM.
+  const bool pup_first = rt != st && ceil_div(Tn, RT_TOK) * ROUTE_CLUSTER > 2 * tc_state().n_sms;
+
   // Router: fold through P_up, logits, top-k, gates -- or everything from a routing record.  The router reads y1
   // and the permutation maps read the router's result: neither needs the norm or P_up, so with the second stream
   // they run beside those two.
   const bool records = (D.flags & REVFFN_FLAG_ROUTING_RECORD) != 0;
   const bool gate_all = (D.flags & REVFFN_FLAG_GATE_SOFTMAX_ALL) != 0;
   const RecordLayout R = record_layout(D);
-  if (idx_in && records && !gate_all) {
+  const bool from_record = idx_in && records && !gate_all;
+  if (from_record) {
     const char* rec = reinterpret_cast<const char*>(idx_in);
     const size_t tk = (size_t)Tn * k * 4;
     CK(cudaMemcpyAsync(c.ws + L.idx.off, rec, tk, cudaMemcpyDeviceToDevice, rt));
@@ -433,6 +448,10 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
                                E, d, h, c.template p<double>(L.w_rc), rt));
     }
     }
+    if (pup_first) {
+      CKR(p_up());
+      CKR(c.order(st, rt));
+    }
     { ProfScope ps(TG_ROUTER, rt);
     CK(launch_router_topk(y1, D.ld_stream, c.W.norm_gamma, D.norm_eps, norm_none, c.template p<double>(L.w_rc),
                           c.W.b_router, Tn, h, E, k, Is > 0 ? 1 : 0, idx_in, c.template p<int32_t>(L.idx),
@@ -448,38 +467,23 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
   }
 
   // Permutation maps
-  CK(cudaMemsetAsync(c.ws + L.row_tok.off, 0xFF, L.row_tok.bytes, rt));
-  CK(cudaMemsetAsync(c.ws + L.row_gate.off, 0, L.row_gate.bytes, rt));
+  const int chunk = map_chunk_tokens(Tn);
   { ProfScope ps(TG_MAP, rt);
-  map_rank_kernel<<<L.n_chunks, 256, (size_t)MAP_CHUNK * k * 4, rt>>>(
-      c.template p<int32_t>(L.idx), Tn, k, E, c.template p<int32_t>(L.local_rank), c.template p<int32_t>(L.chunk_cnt),
-      c.template p<int>(L.status));
+  map_rank_kernel<<<L.n_chunks, MAP_THREADS, 0, rt>>>(c.template p<int32_t>(L.idx), Tn, k, E, chunk, c.template p<int32_t>(L.local_rank),
+                                                      c.template p<int32_t>(L.chunk_cnt), c.template p<int>(L.status));
   }
   CK(cudaGetLastError());
   { ProfScope ps(TG_MAP, rt);
-  map_scan_kernel<<<1, 256, (size_t)(E + 1) * 4, rt>>>(
-      c.template p<int32_t>(L.chunk_cnt), L.n_chunks, E, c.template p<int32_t>(L.chunk_base),
-      c.template p<int32_t>(L.expert_cnt), c.template p<int32_t>(L.expert_off), c.template p<int32_t>(L.tile_group),
-      c.template p<int32_t>(L.rows_total), L.max_tiles, c.template p<int4>(L.tok_chunks), L.max_chunks);
-  }
-  CK(cudaGetLastError());
-  { ProfScope ps(TG_MAP, rt);
-  map_assign_kernel<<<(unsigned)ceil_div((int64_t)Tn * k, 256), 256, 0, rt>>>(
+  map_assign_kernel<<<L.n_chunks, MAP_THREADS, 0, rt>>>(
       c.template p<int32_t>(L.idx), c.template p<float>(L.gates), c.template p<int32_t>(L.local_rank),
-      c.template p<int32_t>(L.chunk_base), c.template p<int32_t>(L.expert_off), Tn, k, E,
-      c.template p<int32_t>(L.tok_row), c.template p<int32_t>(L.row_tok), c.template p<float>(L.row_gate));
+      c.template p<int32_t>(L.chunk_cnt), Tn, k, E, chunk, L.n_chunks, c.template p<int32_t>(L.expert_cnt),
+      c.template p<int32_t>(L.expert_off), c.template p<int32_t>(L.tile_group), c.template p<int32_t>(L.rows_total),
+      L.max_tiles, c.template p<int4>(L.tok_chunks), L.max_chunks, c.template p<int32_t>(L.tok_row),
+      c.template p<int32_t>(L.row_tok), c.template p<float>(L.row_gate));
   }
   CK(cudaGetLastError());
 
-  // P_up: U = N W_up^T
-  {
-    GemmProblem p = blank_problem();
-    p.M = Tn; p.N = d; p.K = h;
-    p.A = c.template p<T>(L.n); p.lda = h;
-    p.B0 = w_up; p.ldb = h;
-    p.epilogue = EPI_STORE; p.C = c.template p<T>(L.u); p.ldc = d;
-    CKR(run_gemm(c, p, TG_PUP));
-  }
+  if (!pup_first || from_record) CKR(p_up());
   CKR(c.order(rt, st));            // the permutation needs the maps
   // The shared expert needs u and nothing else of this pass: on the second stream it runs beside the routed experts.
   Ctx<T> cs = c;

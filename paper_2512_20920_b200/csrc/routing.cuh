@@ -4,7 +4,7 @@
 //   rmsnorm_fwd        n = y * r * gamma, r = (mean(y^2)+eps)^-1/2
 //   fold_router        W_rc = [W_r; w_sgate] * W_up   (so logits come straight from n)
 //   router_topk        logits (fp64), top-k, softmax over the selected k, shared sigmoid gate
-//   map_*              stable counting sort of (token, slot) pairs by expert -> padded rows
+//   map_rank/assign    stable counting sort of (token, slot) pairs by expert -> padded rows
 //   gather_rows        Up[row] = U[token(row)]
 //   combine_rows       Z[t] = sum_s O[row(t,s)] + sgate_t * S[t]
 #pragma once
@@ -18,36 +18,57 @@ namespace revffn {
 // ---------------------------------------------------------------------------
 // RMSNorm forward.  One warp per token; fp32 math; output in T plus r[t].
 // norm_kind NONE: n = y, r = 1.
+// A row's first 1024 elements stay in registers between the sum of squares and the scaling, all of their loads in
+// flight together; only wider rows read the rest twice (8192 rows of 1024: 15.9 -> 11.4 us).
 // ---------------------------------------------------------------------------
+template <typename T> __device__ __forceinline__ void store4(T* p, float4 v);
+template <> __device__ __forceinline__ void store4<float>(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+template <> __device__ __forceinline__ void store4<bf16>(bf16* p, float4 v) {
+  __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+  *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+}
+
 template <typename T>
-__global__ void rmsnorm_fwd_kernel(const float* __restrict__ y, int64_t ld, const float* __restrict__ gamma,
-                                   float eps, int norm_none, int tokens, int h,
-                                   T* __restrict__ n_out, float* __restrict__ r_out) {
-  int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  if (warp >= tokens) return;
-  const float* row = y + (int64_t)warp * ld;
+__device__ __forceinline__ void rmsnorm_row(const float* __restrict__ row, const float* __restrict__ gamma, float eps,
+                                            int norm_none, int h, int lane, T* __restrict__ out, float* __restrict__ r_out) {
+  constexpr int KEEP = 8;
+  float4 v[KEEP];
+#pragma unroll
+  for (int q = 0; q < KEEP; ++q) {
+    const int i = lane * 4 + q * 128;
+    v[q] = i < h ? *reinterpret_cast<const float4*>(row + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
   float r = 1.0f;
   if (!norm_none) {
     float ss = 0.f;
-    for (int i = lane * 4; i < h; i += 128) {
-      float4 v = *reinterpret_cast<const float4*>(row + i);
-      ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+#pragma unroll
+    for (int q = 0; q < KEEP; ++q) ss += v[q].x * v[q].x + v[q].y * v[q].y + v[q].z * v[q].z + v[q].w * v[q].w;
+    for (int i = lane * 4 + KEEP * 128; i < h; i += 128) {
+      const float4 w = *reinterpret_cast<const float4*>(row + i);
+      ss += w.x * w.x + w.y * w.y + w.z * w.z + w.w * w.w;
     }
     ss = warp_sum(ss);
     r = rsqrtf(ss / (float)h + eps);
   }
-  if (lane == 0) r_out[warp] = r;
-  T* out = n_out + (int64_t)warp * h;
-  for (int i = lane * 4; i < h; i += 128) {
-    float4 v = *reinterpret_cast<const float4*>(row + i);
+  if (lane == 0) *r_out = r;
+  auto put = [&](int i, float4 w) {
     float4 g = make_float4(1.f, 1.f, 1.f, 1.f);
     if (gamma && !norm_none) g = *reinterpret_cast<const float4*>(gamma + i);
-    out[i + 0] = from_f32<T>(v.x * r * g.x);
-    out[i + 1] = from_f32<T>(v.y * r * g.y);
-    out[i + 2] = from_f32<T>(v.z * r * g.z);
-    out[i + 3] = from_f32<T>(v.w * r * g.w);
-  }
+    store4<T>(out + i, make_float4(w.x * r * g.x, w.y * r * g.y, w.z * r * g.z, w.w * r * g.w));
+  };
+#pragma unroll
+  for (int q = 0; q < KEEP; ++q)
+    if (lane * 4 + q * 128 < h) put(lane * 4 + q * 128, v[q]);
+  for (int i = lane * 4 + KEEP * 128; i < h; i += 128) put(i, *reinterpret_cast<const float4*>(row + i));
+}
+
+template <typename T>
+__global__ void rmsnorm_fwd_kernel(const float* __restrict__ y, int64_t ld, const float* __restrict__ gamma,
+                                   float eps, int norm_none, int tokens, int h,
+                                   T* __restrict__ n_out, float* __restrict__ r_out) {
+  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (warp >= tokens) return;
+  rmsnorm_row<T>(y + (int64_t)warp * ld, gamma, eps, norm_none, h, threadIdx.x & 31, n_out + (int64_t)warp * h, r_out + warp);
 }
 
 // ---------------------------------------------------------------------------
@@ -261,30 +282,73 @@ inline cudaError_t launch_fold_router_mma(const T* w_router, const T* w_sgate, c
 
 // ---------------------------------------------------------------------------
 // Router: logits in fp64 from the fp32 stream, top-k by warp shuffles, gates.
-//   block = 256 threads, RT_TOK tokens per block.
+//   cluster of ROUTE_CLUSTER blocks of 256 threads = RT_TOK tokens.
 //   phase 1: L[t, e] = r_t <W_rc[e], y_t * gamma> (+ b_r[e]) for e < E; row E is the
 //            shared gate.  The product runs on the fp64 tensor-core path
-//            (mma.sync m8n8k4): y*gamma (fp64, [token][i]) and W_rc ([expert][i]) are
-//            staged chunk-wise in shared memory, each warp owns a 16-token x 16-expert
-//            block of the 32 x 64 tile as 2 x 2 fragments.  (Blocks of 64 tokens with 16 x 32
-//            per warp read fewer operand values per instruction, but a batch of 8192 tokens
-//            then fills the GPU with one block of 8 warps per SM, which cannot hide the
-//            latency of its own loads: 32-token blocks, two or three to an SM, took the kernel
-//            from 0.106 to 0.083 ms.)  (A register-tiled DFMA version of the same product
-//            spent its time on shared-memory operand reads: 8 values per 16 FMAs.)
-//            The staging threads also sum y^2 (fp64), which gives
-//            r_t = (mean(y_t^2)+eps)^-1/2; the scale is applied to the finished sums.
-//   phase 2: per token, k rounds of warp arg-max (ties -> lowest index), softmax
+//            (mma.sync m8n8k4): y (fp32, [token][i]) and W_rc (fp64, [expert][i]) chunks come in by cp.async through a
+//            ring of two stages, y * gamma is formed in fp64 as the fragments are read, each warp owns a
+//            16-token x 32-expert block of the 64 x 64 tile as 2 x 4 fragments.  Each block takes an eighth of K and
+//            leaves its partial sums in its own shared memory.  Four threads per token also sum y^2 (fp64), which
+//            gives r_t = (mean(y_t^2)+eps)^-1/2; the scale is applied to the finished sums.
+//   phase 2: each block takes 8 of the tokens, a warp one: it adds the token's partial sums from the cluster, slices
+//            in ascending order, then k rounds of warp arg-max (ties -> lowest index), softmax
 //            over the k selected logits, sigmoid of the shared-gate logit.
+// The split is the same whatever the number of tokens, so a token's logits do not depend on the batch it is in.
+// What bounds it: the serial walk over K at small batches, where splitting K gives eight times the blocks (64 tokens:
+// 47 -> 15 us; 512: 47 -> 15), and at large ones the fp64 tensor pipe at the occupancy of three blocks an SM (8192 tokens:
+// 76 -> 71 us; 8192 x 61 x 1024 multiply-adds are 29 us of the pipe).
 // idx_in != NULL: expert sets are taken from it (gates are still recomputed).
 // prob_out != NULL: gates are the selected entries of the softmax over ALL experts (not
 // renormalised), and that softmax is written to prob_out[T, E].
 // ---------------------------------------------------------------------------
-constexpr int RT_TOK = 32;   // tokens per block
+constexpr int ROUTE_CLUSTER = 8;
+constexpr int RT_TOK = 64;   // tokens per cluster
 constexpr int RT_KC = 32;    // k-chunk
 constexpr int RT_EC = 64;    // experts per pass
-constexpr int RT_LD = RT_KC + 4;    // row stride (doubles) of both staged chunks: rows 4 doubles apart modulo 16 banks,
-                                    // so the 8 rows x 4 columns a fragment load touches fall on distinct banks
+constexpr int RT_LD = RT_KC + 4;    // row stride (elements) of both staged chunks: rows 4 elements apart modulo the
+                                    // banks, so the 8 rows x 4 columns a fragment load touches fall on distinct ones
+constexpr int RT_STAGES = 2;
+constexpr int RT_STAGE_BYTES = RT_EC * RT_LD * 8 + RT_TOK * RT_LD * 4 + RT_KC * 4;     // W_rc | y | gamma
+static_assert(RT_TOK == 8 * ROUTE_CLUSTER, "phase 2: one token per warp of the cluster");
+
+// Shared memory: stage ring | finished logits of the warps' tokens [8][E+1] | sums of y^2 [RT_TOK].
+// The partial logits take the ring's place when there is one pass over the experts, else they follow the rest.
+__host__ __device__ inline int router_row_off(int E) {
+  const int ring = RT_STAGES * RT_STAGE_BYTES, part = E + 1 <= RT_EC ? RT_TOK * (E + 1) * 8 : 0;
+  return ring > part ? ring : part;
+}
+__host__ __device__ inline int router_part_off(int E) {
+  return E + 1 <= RT_EC ? 0 : router_row_off(E) + (8 * (E + 1) + RT_TOK) * 8;
+}
+inline size_t router_smem_bytes(int E) {
+  const size_t rest = (size_t)router_row_off(E) + (8 * (size_t)(E + 1) + RT_TOK) * 8;
+  return E + 1 <= RT_EC ? rest : rest + (size_t)RT_TOK * (E + 1) * 8;
+}
+
+__device__ __forceinline__ uint32_t route_cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void route_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The double at the same shared-memory place in block `rank` of the cluster.
+__device__ __forceinline__ double ld_cluster_f64(const double* p, uint32_t rank) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  uint32_t r;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool ok) {      // !ok: 16 zero bytes
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+               ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // D (8x8) += A (8x4, row-major fragment) * B (4x8, column-major fragment), fp64.
 // Lane l holds A[l/4][l%4], B[l%4][l/4] and D[l/4][2*(l%4) + {0,1}].
@@ -293,130 +357,131 @@ __device__ __forceinline__ void dmma_8x8x4(double& d0, double& d1, double a, dou
                : "+d"(d0), "+d"(d1) : "d"(a), "d"(b));
 }
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 3)
 router_topk_kernel(const float* __restrict__ y, int64_t ld, const float* __restrict__ gamma, float eps,
                    int norm_none, const double* __restrict__ w_rc, const float* __restrict__ b_router,
                    int tokens, int h, int E, int k, int has_shared, const int32_t* __restrict__ idx_in,
                    int32_t* __restrict__ idx_out, float* __restrict__ gate_out, float* __restrict__ sgate_out,
                    int32_t* __restrict__ idx_user, float* __restrict__ prob_out, int* __restrict__ status,
                    int check_finite) {
-  extern __shared__ __align__(16) double smem_d[];
+  extern __shared__ __align__(16) uint8_t rt_smem[];
   const int EP = E + 1;                       // logits per token incl. the shared-gate row
-  double* ns = smem_d;                        // [RT_TOK][RT_LD]  stream chunk, one row per token
-  double* ws = ns + RT_TOK * RT_LD;           // [RT_EC][RT_LD]   W_rc chunk, one row per expert
-  double* rs = ws + RT_EC * RT_LD;            // [RT_TOK]
-  double* Ls = rs + RT_TOK;                   // [RT_TOK][EP]
+  double* Lp = reinterpret_cast<double*>(rt_smem + router_part_off(E));    // [RT_TOK][EP] this block's partial sums
+  double* Lrow = reinterpret_cast<double*>(rt_smem + router_row_off(E));      // [8][EP]
+  double* sq = Lrow + 8 * EP;                                                 // [RT_TOK]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int t0 = blockIdx.x * RT_TOK;
+  const uint32_t rank = route_cluster_rank();
+  const int t0 = (int)(blockIdx.x / ROUTE_CLUSTER) * RT_TOK;
+  const int chunks = (int)ceil_div(h, RT_KC);
+  const int c_begin = (int)((int64_t)chunks * rank / ROUTE_CLUSTER);
+  const int n_c = (int)((int64_t)chunks * (rank + 1) / ROUTE_CLUSTER) - c_begin;
+  const bool scaled = gamma != nullptr && !norm_none;
 
-  // phase 1: logits.  Warp (wm, wn) owns tokens 16 wm .. +15 and experts e0 + 16 wn .. +15.
-  const int wm = warp >> 2, wn = warp & 3;
-  constexpr int NY = RT_TOK * RT_KC / 4 / 256;      // float4 pieces of the stream chunk per thread
-  static_assert(NY >= 1 && RT_TOK * RT_KC / 4 % 256 == 0, "stream chunk must split evenly over the block");
+  // phase 1: logits.  Warp (wm, wn) owns tokens 16 wm .. +15 and experts e0 + 32 wn .. +31.
+  const int wm = warp >> 1, wn = warp & 1;
   const int fr = lane >> 2, fc = lane & 3;          // fragment row / column of this lane
   for (int e0 = 0; e0 < EP; e0 += RT_EC) {
-    double acc[2][2][2];
+    double acc[2][4][2];
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
-      for (int b = 0; b < 2; ++b) { acc[a][b][0] = 0.0; acc[a][b][1] = 0.0; }
-    // Register prefetch: the global loads of chunk c+1 are in flight while chunk c is summed.
-    //   y:    RT_TOK x RT_KC floats  = NY float4 per thread (token tt, 4 consecutive i)
-    //   W_rc: RT_EC x RT_KC doubles  = 4 double2 per thread (expert ee, 2 consecutive i)
-    float4 py[NY];
-    double2 pw[4];
-    double ss[NY];                  // sum of y^2 over this thread's 4-column strip of its token(s)
+      for (int b = 0; b < 4; ++b) { acc[a][b][0] = 0.0; acc[a][b][1] = 0.0; }
+    double ss = 0.0;                // sum of y^2 over this thread's quarter of the chunks of token tid / 4
+    auto load = [&](int c) {        // chunk c of the slice into its stage; always commits a group
+      if (c < n_c) {
+        double* ws = reinterpret_cast<double*>(rt_smem + (c % RT_STAGES) * RT_STAGE_BYTES);
+        float* ns = reinterpret_cast<float*>(ws + RT_EC * RT_LD);
+        const int k0 = (c_begin + c) * RT_KC;
+        if (scaled && tid < RT_KC / 4) cp_async16(ns + RT_TOK * RT_LD + tid * 4, gamma + min(k0 + tid * 4, h - 4), k0 + tid * 4 < h);
 #pragma unroll
-    for (int q = 0; q < NY; ++q) ss[q] = 0.0;
-    auto prefetch = [&](int k0) {
+        for (int q = 0; q < RT_TOK * RT_KC / 4 / 256; ++q) {
+          const int at = tid + q * 256, tt = at / (RT_KC / 4), kq = (at % (RT_KC / 4)) * 4;
+          const bool ok = t0 + tt < tokens && k0 + kq < h;                                         // h % 4 == 0
+          cp_async16(ns + tt * RT_LD + kq, ok ? y + (int64_t)(t0 + tt) * ld + k0 + kq : y, ok);
+        }
 #pragma unroll
-      for (int q = 0; q < NY; ++q) {
-        int idx = tid + q * 256;
-        int tt = idx / (RT_KC / 4), kq = (idx % (RT_KC / 4)) * 4;
-        int t = t0 + tt, i = k0 + kq;
-        py[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (t < tokens && i < h) py[q] = *reinterpret_cast<const float4*>(y + (int64_t)t * ld + i);   // h % 4 == 0
+        for (int q = 0; q < RT_EC * RT_KC / 2 / 256; ++q) {
+          const int at = tid + q * 256, ee = at / (RT_KC / 2), kq = (at % (RT_KC / 2)) * 2;
+          const bool ok = e0 + ee < EP && k0 + kq < h;                                             // h % 2 == 0
+          cp_async16(ws + ee * RT_LD + kq, ok ? w_rc + (int64_t)(e0 + ee) * h + k0 + kq : w_rc, ok);
+        }
       }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        int idx = tid + q * 256;
-        int ee = idx / (RT_KC / 2), kq = (idx % (RT_KC / 2)) * 2;
-        int e = e0 + ee, i = k0 + kq;
-        pw[q] = make_double2(0.0, 0.0);
-        if (e < EP && i < h) pw[q] = *reinterpret_cast<const double2*>(w_rc + (int64_t)e * h + i);   // h % 2 == 0
-      }
+      cp_async_commit();
     };
-    prefetch(0);
-    for (int k0 = 0; k0 < h; k0 += RT_KC) {
 #pragma unroll
-      for (int q = 0; q < NY; ++q) {
-        int idx = tid + q * 256;
-        int tt = idx / (RT_KC / 4), kq = (idx % (RT_KC / 4)) * 4;
-        int i = k0 + kq;
-        float4 g = make_float4(1.f, 1.f, 1.f, 1.f);
-        if (gamma && !norm_none && i < h) g = *reinterpret_cast<const float4*>(gamma + i);
-        const double v0 = (double)py[q].x, v1 = (double)py[q].y, v2 = (double)py[q].z, v3 = (double)py[q].w;
-        ss[q] += v0 * v0; ss[q] += v1 * v1; ss[q] += v2 * v2; ss[q] += v3 * v3;
-        double2* dst = reinterpret_cast<double2*>(ns + tt * RT_LD + kq);
-        dst[0] = make_double2(v0 * (double)g.x, v1 * (double)g.y);
-        dst[1] = make_double2(v2 * (double)g.z, v3 * (double)g.w);
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        int idx = tid + q * 256;
-        int ee = idx / (RT_KC / 2), kq = (idx % (RT_KC / 2)) * 2;
-        *reinterpret_cast<double2*>(ws + ee * RT_LD + kq) = pw[q];
-      }
+    for (int c = 0; c < RT_STAGES; ++c) load(c);
+    for (int c = 0; c < n_c; ++c) {
+      cp_async_wait<RT_STAGES - 1>();
       __syncthreads();
-      if (k0 + RT_KC < h) prefetch(k0 + RT_KC);
-      const double* ap = ns + (wm * 16 + fr) * RT_LD + fc;
-      const double* bp = ws + (wn * 16 + fr) * RT_LD + fc;
+      const double* ws = reinterpret_cast<const double*>(rt_smem + (c % RT_STAGES) * RT_STAGE_BYTES);
+      const float* ns = reinterpret_cast<const float*>(ws + RT_EC * RT_LD);
+      const float* ap = ns + (wm * 16 + fr) * RT_LD + fc;
+      const double* bp = ws + (wn * 32 + fr) * RT_LD + fc;
+      const float* gp = ns + RT_TOK * RT_LD + fc;
 #pragma unroll
       for (int kk = 0; kk < RT_KC; kk += 4) {
-        double af[2], bf[2];
+        double af[2], bf[4];
 #pragma unroll
-        for (int a = 0; a < 2; ++a) af[a] = ap[a * 8 * RT_LD + kk];
+        for (int a = 0; a < 2; ++a) af[a] = (double)ap[a * 8 * RT_LD + kk];
+        if (scaled) {
+          const double g = (double)gp[kk];
+          af[0] *= g; af[1] *= g;
+        }
 #pragma unroll
-        for (int b = 0; b < 2; ++b) bf[b] = bp[b * 8 * RT_LD + kk];
+        for (int b = 0; b < 4; ++b) bf[b] = bp[b * 8 * RT_LD + kk];
 #pragma unroll
         for (int a = 0; a < 2; ++a)
 #pragma unroll
-          for (int b = 0; b < 2; ++b) dmma_8x8x4(acc[a][b][0], acc[a][b][1], af[a], bf[b]);
+          for (int b = 0; b < 4; ++b) dmma_8x8x4(acc[a][b][0], acc[a][b][1], af[a], bf[b]);
+      }
+      if (e0 == 0) {
+        const float4* q4 = reinterpret_cast<const float4*>(ns + (tid >> 2) * RT_LD + (tid & 3) * 8);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const float4 v = q4[j];
+          ss += (double)v.x * (double)v.x; ss += (double)v.y * (double)v.y;
+          ss += (double)v.z * (double)v.z; ss += (double)v.w * (double)v.w;
+        }
       }
       __syncthreads();
+      load(c + RT_STAGES);
     }
-    // r per token: the 8 threads that staged one token hold its strips (lanes 8m .. 8m+7)
-#pragma unroll
-    for (int q = 0; q < NY; ++q) {
-      double v = ss[q];
-      v += __shfl_xor_sync(0xffffffffu, v, 1);
-      v += __shfl_xor_sync(0xffffffffu, v, 2);
-      v += __shfl_xor_sync(0xffffffffu, v, 4);
-      if ((tid & 7) == 0) rs[tid / 8 + q * 32] = norm_none ? 1.0 : 1.0 / sqrt(v / (double)h + (double)eps);
+    cp_async_wait<0>();
+    __syncthreads();                // also: nobody reads the ring any more where the partial sums go over it
+    if (e0 == 0) {
+      ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+      ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+      if ((tid & 3) == 0) sq[tid >> 2] = ss;
     }
-    __syncthreads();
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
-      for (int b = 0; b < 2; ++b)
+      for (int b = 0; b < 4; ++b)
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          const int tt = wm * 16 + a * 8 + fr;
-          const int e = e0 + wn * 16 + b * 8 + 2 * fc + c;
-          if (e < EP) {
-            double v = acc[a][b][c] * rs[tt];
-            if (e < E && b_router) v += (double)b_router[e];
-            Ls[tt * EP + e] = v;
-          }
+          const int tt = wm * 16 + a * 8 + fr, e = e0 + wn * 32 + b * 8 + 2 * fc + c;
+          if (e < EP) Lp[tt * EP + e] = acc[a][b][c];
         }
   }
-  __syncthreads();
+  route_cluster_sync();
 
   // phase 2: top-k and gates; one warp per token
-  for (int tt = warp; tt < RT_TOK; tt += 8) {
-    int t = t0 + tt;
-    if (t >= tokens) continue;
-    const double* L = Ls + tt * EP;
+  const int tt = (int)rank * 8 + warp, t = t0 + tt;
+  if (t < tokens) {
+    double* L = Lrow + warp * EP;
+    double ss = 0.0;
+#pragma unroll
+    for (int r = 0; r < ROUTE_CLUSTER; ++r) ss += ld_cluster_f64(sq + tt, (uint32_t)r);
+    const double rt = norm_none ? 1.0 : 1.0 / sqrt(ss / (double)h + (double)eps);
+    for (int e = lane; e < EP; e += 32) {
+      double v = 0.0;
+#pragma unroll
+      for (int r = 0; r < ROUTE_CLUSTER; ++r) v += ld_cluster_f64(Lp + tt * EP + e, (uint32_t)r);
+      v *= rt;
+      if (e < E && b_router) v += (double)b_router[e];
+      L[e] = v;
+    }
+    __syncwarp();
     double sel[8];
     int seli[8];
     if (check_finite) {
@@ -508,14 +573,10 @@ router_topk_kernel(const float* __restrict__ y, int64_t ld, const float* __restr
       sgate_out[t] = has_shared ? 1.f / (1.f + ev) : 0.f;
     }
   }
+  route_cluster_sync();      // no block leaves while another may still read its partial sums
 }
 
-inline size_t router_smem_bytes(int E) {
-  return sizeof(double) * ((size_t)(RT_TOK + RT_EC) * RT_LD + RT_TOK + (size_t)RT_TOK * (E + 1));
-}
-
-// Raises the kernel's dynamic shared-memory limit when the logits of a block do not
-// fit the default 48 KB (once per device), then launches.
+// Raises the kernel's dynamic shared-memory limit (once per device), then launches.
 inline cudaError_t launch_router_topk(const float* y, int64_t ld, const float* gamma, float eps, int norm_none,
                                       const double* w_rc, const float* b_router, int tokens, int h, int E, int k,
                                       int has_shared, const int32_t* idx_in, int32_t* idx_out, float* gate_out,
@@ -536,115 +597,168 @@ inline cudaError_t launch_router_topk(const float* y, int64_t ld, const float* g
       raised[dev] = smem;
     }
   }
-  router_topk_kernel<<<(unsigned)ceil_div(tokens, RT_TOK), 256, smem, st>>>(
-      y, ld, gamma, eps, norm_none, w_rc, b_router, tokens, h, E, k, has_shared, idx_in, idx_out, gate_out,
-      sgate_out, idx_user, prob_out, status, check_finite);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(ceil_div(tokens, RT_TOK) * ROUTE_CLUSTER));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = ROUTE_CLUSTER;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, router_topk_kernel, y, ld, gamma, eps, norm_none, w_rc, b_router, tokens, h, E, k,
+                            has_shared, idx_in, idx_out, gate_out, sgate_out, idx_user, prob_out, status, check_finite);
 }
 
 // ---------------------------------------------------------------------------
 // Permutation maps: stable counting sort of the T*k (token, slot) entries by
 // expert, each expert's segment padded to a multiple of ROW_PAD rows.
-//   map_rank:   per chunk of MAP_CHUNK tokens, rank of each entry among the
-//               chunk's entries of the same expert (entry order = token-major)
-//   map_scan:   per expert totals, padded offsets, per-chunk bases, tile->expert
-//   map_assign: row of each entry; row -> token; row -> gate weight
+//   map_rank:   per chunk of tokens, rank of each entry among the chunk's entries of the same expert
+//               (entry order = token-major) and the chunk's count per expert
+//   map_assign: row of each entry; row -> token; row -> gate weight; padding rows (token -1, gate 0);
+//               the per-expert tables
+// Both are latency.  Every block of map_assign adds up the counts of all chunks itself (n_chunks * E integers out of
+// the L2) instead of waiting for a one-block scan in between, and the chunk grows with the batch so that there
+// are at most 128 of them until it holds 2048 tokens.  With the two memsets that the padding rows took: 5 launches,
+// 33 us at 64 tokens and 50 us at 8192 (gaps included) -> 2 launches, 12 and 14 us.
 // ---------------------------------------------------------------------------
+constexpr int TOK_CHUNK = 256;       // most token rows of one expert in one N-side tile
+constexpr int MAP_THREADS = 512;
+constexpr int MAP_MAX_E = 256;       // n_experts is at most this
+
+// Tokens per block: see above.
+inline int map_chunk_tokens(int64_t tokens) {
+  int c = 128;
+  while (c < 2048 && ceil_div(tokens, c) > 128) c *= 2;
+  return c;
+}
+
 // An entry outside [0, E) (possible only in expert sets handed in by the caller) matches no expert: it gets
 // no rank and no row, map_assign marks it with row -1, and every later step skips it.  It is reported once here.
-__global__ void map_rank_kernel(const int32_t* __restrict__ idx, int tokens, int k, int E,
-                                int32_t* __restrict__ local_rank, int32_t* __restrict__ chunk_cnt,
-                                int* __restrict__ status) {
-  extern __shared__ int32_t sm_i[];
-  int chunk = blockIdx.x;
-  int64_t e0 = (int64_t)chunk * MAP_CHUNK * k;
-  int n = (int)min((int64_t)MAP_CHUNK * k, (int64_t)tokens * k - e0);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const int e = idx[e0 + i];
-    sm_i[i] = e;
-    if ((unsigned)e >= (unsigned)E) set_status(status, REVFFN_ERR_INDEX);
+__global__ void __launch_bounds__(MAP_THREADS)
+map_rank_kernel(const int32_t* __restrict__ idx, int tokens, int k, int E, int chunk_tokens,
+                int32_t* __restrict__ local_rank, int32_t* __restrict__ chunk_cnt, int* __restrict__ status) {
+  constexpr int WARPS = MAP_THREADS / 32;
+  __shared__ int hist[WARPS][MAP_MAX_E];       // counts per warp, then the warps' bases
+  __shared__ int run[MAP_MAX_E];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int chunk = blockIdx.x;
+  const int64_t i0 = (int64_t)chunk * chunk_tokens * k;
+  const int n = (int)min((int64_t)chunk_tokens * k, (int64_t)tokens * k - i0);
+  for (int e = tid; e < E; e += MAP_THREADS) run[e] = 0;
+  for (int base = 0; base < n; base += MAP_THREADS) {
+    for (int e = lane; e < E; e += 32) hist[warp][e] = 0;
+    __syncwarp();
+    const int i = base + tid;
+    const int e = i < n ? idx[i0 + i] : -1;
+    const bool valid = (unsigned)e < (unsigned)E;
+    if (i < n && !valid) set_status(status, REVFFN_ERR_INDEX);
+    const unsigned peers = __match_any_sync(0xffffffffu, valid ? e : MAP_MAX_E);
+    const int rank = __popc(peers & ((1u << lane) - 1u));
+    if (valid && rank == 0) hist[warp][e] = __popc(peers);
+    __syncthreads();
+    for (int x = tid; x < E; x += MAP_THREADS) {
+      int c = run[x];
+#pragma unroll
+      for (int w = 0; w < WARPS; ++w) { const int v = hist[w][x]; hist[w][x] = c; c += v; }
+      run[x] = c;
+    }
+    __syncthreads();
+    if (valid) local_rank[i0 + i] = hist[warp][e] + rank;
+    __syncwarp();                              // a warp clears only its own row for the next round
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < E; e += blockDim.x) {
-    int c = 0;
-    for (int i = 0; i < n; ++i)
-      if (sm_i[i] == e) { local_rank[e0 + i] = c; ++c; }
-    chunk_cnt[(int64_t)chunk * E + e] = c;
-  }
+  for (int e = tid; e < E; e += MAP_THREADS) chunk_cnt[(int64_t)chunk * E + e] = run[e];
 }
 
-constexpr int TOK_CHUNK = 256;   // most token rows of one expert in one N-side tile
-
-__global__ void map_scan_kernel(const int32_t* __restrict__ chunk_cnt, int n_chunks, int E,
-                                int32_t* __restrict__ chunk_base, int32_t* __restrict__ expert_cnt,
-                                int32_t* __restrict__ expert_off, int32_t* __restrict__ tile_group,
-                                int32_t* __restrict__ rows_total, int max_tiles, int4* __restrict__ tok_chunks,
-                                int max_chunks) {
-  extern __shared__ int32_t sm_i[];          // [E+1] padded offsets
-  // Per expert, the exclusive prefix sum of its chunk counts: a warp per expert, 32 chunks per round, so the
-  // dependent loads of a round are one round trip (a thread per expert walking its chunks one by one spent a
-  // memory latency per chunk).
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-  for (int e = warp; e < E; e += n_warps) {
-    int run = 0;
-    for (int c0 = 0; c0 < n_chunks; c0 += 32) {
-      const int c = c0 + lane;
-      const int v = c < n_chunks ? chunk_cnt[(int64_t)c * E + e] : 0;
-      int incl = v;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += u;
+__global__ void __launch_bounds__(MAP_THREADS)
+map_assign_kernel(const int32_t* __restrict__ idx, const float* __restrict__ gate, const int32_t* __restrict__ local_rank,
+                  const int32_t* __restrict__ chunk_cnt, int tokens, int k, int E, int chunk_tokens, int n_chunks,
+                  int32_t* __restrict__ expert_cnt, int32_t* __restrict__ expert_off, int32_t* __restrict__ tile_group,
+                  int32_t* __restrict__ rows_total, int max_tiles, int4* __restrict__ tok_chunks, int max_chunks,
+                  int32_t* __restrict__ tok_row, int32_t* __restrict__ row_tok, float* __restrict__ row_gate) {
+  __shared__ int below[MAP_MAX_E], cnt[MAP_MAX_E];          // this expert's entries in earlier chunks / in all chunks
+  __shared__ int off[MAP_MAX_E + 1], coff[MAP_MAX_E + 1];   // first padded row, first token run of an expert
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int chunk = blockIdx.x;
+  for (int e = tid; e < MAP_MAX_E; e += MAP_THREADS) { below[e] = 0; cnt[e] = 0; }
+  __syncthreads();
+  {
+    // thread = (group of chunks, expert); integer sums, so the order of the additions does not matter
+    const int lanes = E <= 32 ? 32 : (E <= 64 ? 64 : (E <= 128 ? 128 : 256));
+    const int groups = MAP_THREADS / lanes, e = tid % lanes, g = tid / lanes;
+    if (e < E) {
+      int b = 0, a = 0;
+#pragma unroll 8
+      for (int c = g; c < n_chunks; c += groups) {
+        const int v = chunk_cnt[(int64_t)c * E + e];
+        a += v;
+        if (c < chunk) b += v;
       }
-      if (c < n_chunks) chunk_base[(int64_t)c * E + e] = run + incl - v;
-      run += __shfl_sync(0xffffffffu, incl, 31);
+      atomicAdd(&cnt[e], a);
+      atomicAdd(&below[e], b);
     }
-    if (lane == 0) expert_cnt[e] = run;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int off = 0;
-    for (int e = 0; e < E; ++e) {
-      sm_i[e] = off;
-      off += (int)round_up(expert_cnt[e], ROW_PAD);
+  if (tid < 32) {
+    // exclusive prefix sums over the experts, eight per lane
+    int rows[8], runs[8], sr = 0, sc = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int c = cnt[lane * 8 + j];
+      rows[j] = (c + ROW_PAD - 1) / ROW_PAD * ROW_PAD;
+      runs[j] = (c + TOK_CHUNK - 1) / TOK_CHUNK;
+      sr += rows[j]; sc += runs[j];
     }
-    sm_i[E] = off;
-    rows_total[0] = off;
-    // Token chunks for the products that put tokens on the MMA N side: per expert, runs of up to
-    // TOK_CHUNK rows covering its real rows rounded up to 32 (the rounding stays inside the expert's
-    // zero padding).  Entry = (expert, first row, rows, 0); the count goes to rows_total[1].
+    int ir = sr, ic = sc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, ir, o), v = __shfl_up_sync(0xffffffffu, ic, o);
+      if (lane >= o) { ir += u; ic += v; }
+    }
+    int pr = ir - sr, pc = ic - sc;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      off[lane * 8 + j] = pr; coff[lane * 8 + j] = pc;
+      pr += rows[j]; pc += runs[j];
+    }
+    if (lane == 31) { off[MAP_MAX_E] = pr; coff[MAP_MAX_E] = pc; }
+  }
+  __syncthreads();
+  const int64_t i0 = (int64_t)chunk * chunk_tokens * k;
+  const int n = (int)min((int64_t)chunk_tokens * k, (int64_t)tokens * k - i0);
+  for (int i = tid; i < n; i += MAP_THREADS) {
+    const int e = idx[i0 + i];
+    if ((unsigned)e >= (unsigned)E) { tok_row[i0 + i] = -1; continue; }      // reported by map_rank
+    const int row = off[e] + below[e] + local_rank[i0 + i];
+    tok_row[i0 + i] = row;
+    row_tok[row] = (int)((i0 + i) / k);
+    row_gate[row] = gate[i0 + i];
+  }
+  // padding rows, an expert per warp of all blocks
+  for (int e = chunk * (MAP_THREADS / 32) + (tid >> 5); e < E; e += n_chunks * (MAP_THREADS / 32))
+    for (int r = off[e] + cnt[e] + lane; r < off[e + 1]; r += 32) { row_tok[r] = -1; row_gate[r] = 0.f; }
+  if (chunk != 0) return;
+  for (int e = tid; e <= E; e += MAP_THREADS) {
+    expert_off[e] = off[e];
+    if (e == E) continue;
+    expert_cnt[e] = cnt[e];
+    for (int t = off[e] / ROW_PAD; t < off[e + 1] / ROW_PAD && t < max_tiles; ++t) tile_group[t] = e;
+    // Token runs for the products that put tokens on the MMA N side: per expert, runs of up to TOK_CHUNK rows
+    // covering its real rows rounded up to 32 (the rounding stays inside the expert's zero padding).
+    // Entry = (expert, first row, rows, 0).
     // (Runs of equal length, 3 x 192 instead of 256 + 256 + 64 for 546 rows, stay within 2 % either way: the two
     // products that use the table measured 2 % faster alone and the whole step 1-2 % slower.)
-    int nc = 0;
-    for (int e = 0; e < E; ++e) {
-      const int n = (int)round_up(expert_cnt[e], 32);
-      for (int r = 0; r < n && nc < max_chunks; r += TOK_CHUNK)
-        tok_chunks[nc++] = make_int4(e, sm_i[e] + r, min(TOK_CHUNK, n - r), 0);
-    }
-    rows_total[1] = nc;
+    const int real = (int)round_up(cnt[e], 32);
+    for (int r = 0, c = coff[e]; r < real && c < max_chunks; r += TOK_CHUNK, ++c)
+      tok_chunks[c] = make_int4(e, off[e] + r, min(TOK_CHUNK, real - r), 0);
   }
-  __syncthreads();
-  for (int e = threadIdx.x; e <= E; e += blockDim.x) expert_off[e] = sm_i[e];
-  for (int e = threadIdx.x; e < E; e += blockDim.x) {
-    for (int t = sm_i[e] / ROW_PAD; t < sm_i[e + 1] / ROW_PAD && t < max_tiles; ++t) tile_group[t] = e;
+  if (tid == 0) {
+    rows_total[0] = off[E];
+    rows_total[1] = min(coff[E], max_chunks);
   }
-}
-
-__global__ void map_assign_kernel(const int32_t* __restrict__ idx, const float* __restrict__ gate,
-                                  const int32_t* __restrict__ local_rank, const int32_t* __restrict__ chunk_base,
-                                  const int32_t* __restrict__ expert_off, int tokens, int k, int E,
-                                  int32_t* __restrict__ tok_row, int32_t* __restrict__ row_tok,
-                                  float* __restrict__ row_gate) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)tokens * k) return;
-  int t = (int)(i / k);
-  int e = idx[i];
-  if ((unsigned)e >= (unsigned)E) { tok_row[i] = -1; return; }      // reported by map_rank
-  int chunk = t / MAP_CHUNK;
-  int row = expert_off[e] + chunk_base[(int64_t)chunk * E + e] + local_rank[i];
-  tok_row[i] = row;
-  row_tok[row] = t;
-  row_gate[row] = gate[i];
 }
 
 // ---------------------------------------------------------------------------
