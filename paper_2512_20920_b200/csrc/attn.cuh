@@ -16,6 +16,7 @@
 namespace revffn {
 
 __global__ void rope_table_kernel(int S, int hd, double theta, float2* __restrict__ cs) {
+  pdl_sync();
   const int half = hd / 2;
   int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= S * half) return;
@@ -32,6 +33,7 @@ template <typename T>
 __global__ void rmsnorm2_fwd_kernel(const float* __restrict__ x1, const float* __restrict__ x2, int64_t ld,
                                     const float* __restrict__ gamma, float eps, int tokens, int h, T* __restrict__ n_out,
                                     float* __restrict__ r_out) {
+  pdl_sync();
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (warp >= 2 * tokens) return;
@@ -60,6 +62,7 @@ __global__ void rmsnorm2_fwd_kernel(const float* __restrict__ x1, const float* _
 template <typename TIn, typename T>
 __global__ void to_heads_kernel(const TIn* __restrict__ in, int64_t ld_in, const float* __restrict__ bias,
                                 const float2* __restrict__ cs, int S, int Sp, int n, int hd, T* __restrict__ out) {
+  pdl_sync();
   const int t = blockIdx.x, b = t / S, s = t % S, half = hd / 2;
   const TIn* row = in + (int64_t)t * ld_in;
   for (int p = threadIdx.x; p < n * half; p += blockDim.x) {
@@ -84,6 +87,7 @@ __global__ void to_heads_kernel(const TIn* __restrict__ in, int64_t ld_in, const
 template <typename TIn, typename T>
 __global__ void from_heads_kernel(const TIn* __restrict__ in, const float2* __restrict__ cs, float sign, int S, int Sp,
                                   int n, int hd, T* __restrict__ out, int64_t ld_out, int col0) {
+  pdl_sync();
   const int t = blockIdx.x, b = t / S, s = t % S, half = hd / 2;
   T* row = out + (int64_t)t * ld_out + col0;
   for (int p = threadIdx.x; p < n * half; p += blockDim.x) {
@@ -108,6 +112,7 @@ __global__ void from_heads_kernel(const TIn* __restrict__ in, const float2* __re
 template <typename TIn, typename T>
 __global__ void to_heads_vec_kernel(const TIn* __restrict__ in, int64_t ld_in, const float* __restrict__ bias,
                                     const float2* __restrict__ cs, int tokens, int S, int Sp, int n, int hd, T* __restrict__ out) {
+  pdl_sync();
   const int half = hd / 2, units = n * half / 8;
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int t = (int)(gid / units), u = (int)(gid % units);
@@ -138,6 +143,7 @@ __global__ void to_heads_vec_kernel(const TIn* __restrict__ in, int64_t ld_in, c
 template <typename TIn, typename T>
 __global__ void from_heads_vec_kernel(const TIn* __restrict__ in, const float2* __restrict__ cs, float sign, int tokens, int S,
                                       int Sp, int n, int hd, T* __restrict__ out, int64_t ld_out, int col0) {
+  pdl_sync();
   const int half = hd / 2, units = n * half / 8;
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int t = (int)(gid / units), u = (int)(gid % units);
@@ -171,9 +177,9 @@ inline cudaError_t launch_to_heads(const TIn* in, int64_t ld_in, const float* bi
   if (tokens <= 0) return cudaSuccess;
   if ((hd / 2) % 8 == 0 && ld_in % 8 == 0) {
     const int64_t threads = (int64_t)tokens * (n * (hd / 2) / 8);
-    to_heads_vec_kernel<TIn, T><<<(unsigned)ceil_div(threads, 256), 256, 0, st>>>(in, ld_in, bias, cs, tokens, S, Sp, n, hd, out);
+    launch_k(to_heads_vec_kernel<TIn, T>, (unsigned)ceil_div(threads, 256), 256, 0, st, in, ld_in, bias, cs, tokens, S, Sp, n, hd, out);
   } else {
-    to_heads_kernel<TIn, T><<<tokens, 256, 0, st>>>(in, ld_in, bias, cs, S, Sp, n, hd, out);
+    launch_k(to_heads_kernel<TIn, T>, tokens, 256, 0, st, in, ld_in, bias, cs, S, Sp, n, hd, out);
   }
   return cudaGetLastError();
 }
@@ -184,10 +190,10 @@ inline cudaError_t launch_from_heads(const TIn* in, const float2* cs, float sign
   if (tokens <= 0) return cudaSuccess;
   if ((hd / 2) % 8 == 0 && ld_out % 8 == 0 && col0 % 8 == 0) {
     const int64_t threads = (int64_t)tokens * (n * (hd / 2) / 8);
-    from_heads_vec_kernel<TIn, T><<<(unsigned)ceil_div(threads, 256), 256, 0, st>>>(in, cs, sign, tokens, S, Sp, n, hd, out,
+    launch_k(from_heads_vec_kernel<TIn, T>, (unsigned)ceil_div(threads, 256), 256, 0, st, in, cs, sign, tokens, S, Sp, n, hd, out,
                                                                                     ld_out, col0);
   } else {
-    from_heads_kernel<TIn, T><<<tokens, 256, 0, st>>>(in, cs, sign, S, Sp, n, hd, out, ld_out, col0);
+    launch_k(from_heads_kernel<TIn, T>, tokens, 256, 0, st, in, cs, sign, S, Sp, n, hd, out, ld_out, col0);
   }
   return cudaGetLastError();
 }
@@ -197,6 +203,7 @@ inline cudaError_t launch_from_heads(const TIn* in, const float2* cs, float sign
 template <typename T>
 __global__ void softmax_causal_kernel(const float* __restrict__ sc, int S, int Sp, float scale_log2e, int64_t rows,
                                       T* __restrict__ P) {
+  pdl_sync();
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
@@ -223,6 +230,7 @@ __global__ void softmax_causal_kernel(const float* __restrict__ sc, int S, int S
 template <typename T>
 __global__ void dsoftmax_causal_kernel(const T* __restrict__ P, const float* __restrict__ dP, int S, int Sp, float scale,
                                        int64_t rows, T* __restrict__ dS) {
+  pdl_sync();
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
@@ -246,6 +254,7 @@ __global__ void dsoftmax_causal_kernel(const T* __restrict__ P, const float* __r
 __global__ void attn_tables_kernel(int n_tiles, int tiles_per_head, int rep, int n_groups, int rows_per_group,
                                    int32_t* __restrict__ tile_group, int32_t* __restrict__ group_off,
                                    int32_t* __restrict__ rows_total) {
+  pdl_sync();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n_tiles) tile_group[i] = (i / tiles_per_head) / rep;
   if (i <= n_groups) group_off[i] = i * rows_per_group;
@@ -255,6 +264,7 @@ __global__ void attn_tables_kernel(int n_tiles, int tiles_per_head, int rep, int
 // out[t, :] = in[t, :] for fp32 streams with row strides (dx1 starts as dy1).
 __global__ void copy_stream_kernel(const float* __restrict__ in, int64_t ld_in, int tokens, int h, float* __restrict__ out,
                                    int64_t ld_out) {
+  pdl_sync();
   int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (i >= (int64_t)tokens * h) return;
   int t = (int)(i / h), c = (int)(i % h);

@@ -10,6 +10,7 @@ namespace revffn {
 // Gb = T(G): the upstream gradient as a GEMM operand.
 template <typename T>
 __global__ void cast_stream_kernel(const float* __restrict__ g, int64_t ld, int tokens, int h, T* __restrict__ out) {
+  pdl_sync();
   int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (i >= (int64_t)tokens * h) return;
   int t = (int)(i / h), c = (int)(i % h);
@@ -25,6 +26,7 @@ template <typename T>
 __global__ void shared_gate_bwd_kernel(const T* __restrict__ dZ, const T* __restrict__ S,
                                        const float* __restrict__ sgate, int width, T* __restrict__ dS,
                                        float* __restrict__ dl) {
+  pdl_sync();
   __shared__ float red[32];
   int t = blockIdx.x;
   float sg = sgate[t];
@@ -50,6 +52,7 @@ __global__ void shared_gate_bwd_kernel(const T* __restrict__ dZ, const T* __rest
 __global__ void router_bwd_kernel(const float* __restrict__ dg_part, int dg_ld, int n_part,
                                   const float* __restrict__ gate, const int32_t* __restrict__ tok_row,
                                   int tokens, int k, float* __restrict__ tok_dl, float* __restrict__ row_dl) {
+  pdl_sync();
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= tokens) return;
   float dg[8], g[8], mix = 0.f;
@@ -78,6 +81,7 @@ __global__ void router_bwd_dense_kernel(const float* __restrict__ dg_part, int d
                                         const float* __restrict__ prob, const int32_t* __restrict__ idx,
                                         const int32_t* __restrict__ tok_row, int tokens, int k, int E, int ld_dl,
                                         T* __restrict__ dl_out) {
+  pdl_sync();
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= tokens) return;
   float dg[8];
@@ -113,6 +117,7 @@ template <typename T>
 __global__ void router_wgrad_kernel(const T* __restrict__ Up, const float* __restrict__ row_dl,
                                     const int32_t* __restrict__ expert_off, const int32_t* __restrict__ expert_cnt,
                                     int d, int accumulate, float* __restrict__ dWr, float* __restrict__ dbr) {
+  pdl_sync();
   int e = blockIdx.y;
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   int r0 = expert_off[e], n = expert_cnt[e];
@@ -138,6 +143,7 @@ __global__ void router_wgrad_kernel(const T* __restrict__ Up, const float* __res
 template <typename T, int V>
 __global__ void colsum_partial_kernel(const T* __restrict__ X, int64_t ldx, const float* __restrict__ w,
                                       int rows, int cols, int strip, float* __restrict__ part) {
+  pdl_sync();
   int c = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   int b = blockIdx.y;
   if (c >= cols) return;
@@ -170,10 +176,10 @@ inline cudaError_t launch_colsum_partial(const T* X, int64_t ldx, const float* w
                                          float* part, cudaStream_t st) {
   if (cols % 4 == 0 && ldx % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0) {
     dim3 grid((unsigned)ceil_div(cols, 4 * 128), (unsigned)n_strips);
-    colsum_partial_kernel<T, 4><<<grid, 128, 0, st>>>(X, ldx, w, rows, cols, strip, part);
+    launch_k(colsum_partial_kernel<T, 4>, grid, 128, 0, st, X, ldx, w, rows, cols, strip, part);
   } else {
     dim3 grid((unsigned)ceil_div(cols, 256), (unsigned)n_strips);
-    colsum_partial_kernel<T, 1><<<grid, 256, 0, st>>>(X, ldx, w, rows, cols, strip, part);
+    launch_k(colsum_partial_kernel<T, 1>, grid, 256, 0, st, X, ldx, w, rows, cols, strip, part);
   }
   return cudaGetLastError();
 }
@@ -183,6 +189,7 @@ inline cudaError_t launch_colsum_partial(const T* X, int64_t ldx, const float* w
 constexpr int COLSUM_FINAL_COLS = 32;
 __global__ void __launch_bounds__(256)
 colsum_final_kernel(const float* __restrict__ part, int n_strips, int cols, int accumulate, float* __restrict__ out) {
+  pdl_sync();
   __shared__ float red[8][COLSUM_FINAL_COLS];
   const int cl = threadIdx.x % COLSUM_FINAL_COLS, g = threadIdx.x / COLSUM_FINAL_COLS;
   const int c = blockIdx.x * COLSUM_FINAL_COLS + cl;
@@ -219,6 +226,7 @@ du_reduce_kernel(const T* __restrict__ dUp, const int32_t* __restrict__ tok_row,
                  const T* __restrict__ dUsh, const T* __restrict__ w_router, int n_experts, int slab,
                  const float* __restrict__ dl, const T* __restrict__ w_sgate,
                  const T* __restrict__ dUr, int width, int tokens, T* __restrict__ dU) {
+  pdl_sync();
   extern __shared__ __align__(16) uint8_t du_smem[];
   T* wsl = reinterpret_cast<T*>(du_smem);                  // [n_experts][DU_COLS] when slab != 0
   constexpr int KS = K ? K : 8;
@@ -309,7 +317,7 @@ inline cudaError_t launch_du_reduce(const T* dUp, const int32_t* tok_row, const 
     if (e != cudaSuccess) return e;                                                                                  \
     const int groups = (tokens + 7) / 8;                                                                             \
     const dim3 grid(std::max(1, std::min(groups, wave / col_slabs)), col_slabs);                                     \
-    du_reduce_kernel<T, KK><<<grid, 256, smem, st>>>(dUp, tok_row, idx, tok_dl, k, dUsh, w_router, n_experts, slab,  \
+    launch_k(du_reduce_kernel<T, KK>, grid, 256, smem, st, dUp, tok_row, idx, tok_dl, k, dUsh, w_router, n_experts, slab,  \
                                                      dl, w_sgate, dUr, width, tokens, dU);                           \
   }
   switch (k) {
@@ -327,6 +335,7 @@ inline cudaError_t launch_du_reduce(const T* dUp, const int32_t* tok_row, const 
 __global__ void rmsnorm_bwd_rows_kernel(const float* __restrict__ dn, const float* __restrict__ y, int64_t ld,
                                         const float* __restrict__ gamma, const float* __restrict__ r,
                                         int norm_none, int tokens, int h, float* __restrict__ dy1, int64_t ld_dy) {
+  pdl_sync();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
   if (warp >= tokens) return;
@@ -353,6 +362,7 @@ __global__ void rmsnorm_bwd_rows_kernel(const float* __restrict__ dn, const floa
 __global__ void dgamma_partial_kernel(const float* __restrict__ dn, const float* __restrict__ y, int64_t ld,
                                       const float* __restrict__ r, int tokens, int h, int strip,
                                       float* __restrict__ part) {
+  pdl_sync();
   int c = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
   int b = blockIdx.y;
   if (c >= h) return;
@@ -370,7 +380,7 @@ __global__ void dgamma_partial_kernel(const float* __restrict__ dn, const float*
 inline cudaError_t launch_dgamma_partial(const float* dn, const float* y, int64_t ld, const float* r, int tokens, int h, int strip,
                                          int n_strips, float* part, cudaStream_t st) {
   dim3 grid((unsigned)ceil_div(h, 4 * 128), (unsigned)n_strips);
-  dgamma_partial_kernel<<<grid, 128, 0, st>>>(dn, y, ld, r, tokens, h, strip, part);
+  launch_k(dgamma_partial_kernel, grid, 128, 0, st, dn, y, ld, r, tokens, h, strip, part);
   return cudaGetLastError();
 }
 

@@ -65,6 +65,44 @@ __device__ __forceinline__ void set_status(int* status, int code) {
   if (status) atomicCAS(status, 0, code);
 }
 
+// Programmatic dependent launch.  Every kernel of the library is launched with launch_k / launch_cluster: it may then be
+// set up, and its blocks may become resident, while the kernel before it on the stream still runs its last blocks.
+//   pdl_wait     blocks until everything the launch depends on has completed and its writes are visible.  EVERY
+//                kernel calls it, in every thread, before its first access to global memory and before any early return:
+//                that also makes "the kernel before me has completed" imply "so have all before that one".
+//   pdl_trigger  lets the next launch on the stream be set up (once every block has called it or has exited).
+// What it saves is the 1.5-4 us between two dependent launches; a small stack of blocks is 530 of them (four d = 512 blocks, 384 tokens:
+// 3788 -> 2908 us a training step; attention branch, 7 x 613 positions: 1337 -> 1252).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Short kernels release the next launch at once; the matrix products and attention kernels do it when a block's last
+// operand loads are on their way, so that a waiting block does not hold an SM that another stream could use.
+__device__ __forceinline__ void pdl_sync() { pdl_wait(); pdl_trigger(); }
+
+template <typename... Params, typename... Args>
+inline cudaError_t launch_cluster(void (*kernel)(Params...), dim3 grid, dim3 cluster, dim3 block, size_t smem, cudaStream_t st,
+                                  Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2] = {};
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster.x;
+  attr[1].val.clusterDim.y = cluster.y;
+  attr[1].val.clusterDim.z = cluster.z;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster.x * cluster.y * cluster.z > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+template <typename... Params, typename... Args>
+inline cudaError_t launch_k(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+  return launch_cluster(kernel, grid, dim3(1, 1, 1), block, smem, st, args...);
+}
+
 // 8 elements of T as one vector: loads/stores of 16 bytes for bf16, 2x16 for float.
 // Blocks of `kernel` that are resident on the current device at once (one wave) for this block size and dynamic
 // shared memory: the grid size of the grid-stride kernels.

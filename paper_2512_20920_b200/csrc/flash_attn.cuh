@@ -155,6 +155,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
                  ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -185,6 +186,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
             tma_load_2d(base + FA_V_OFF + (2 * s + kb) * FA_TILE + nj * 8192, &map_v, 64 * nj,
                         kv_row0 + j * FA_BLK + 64 * kb, bar(B_VFULL + s));
       }
+      pdl_trigger();
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
@@ -390,7 +392,7 @@ inline int launch_flash_fwd(const bf16* q, const bf16* k, const bf16* v, int bat
   P.scale_log2e = P.scale * 1.4426950408889634f;
   P.status = status;
   const int grid = batch * n_heads * (Sp / FA_BLK);
-  flash_fwd_kernel<<<grid, FA_THREADS, FA_SMEM_BYTES, st>>>(P, mq, mk, mv);
+  launch_k(flash_fwd_kernel, grid, FA_THREADS, FA_SMEM_BYTES, st, P, mq, mk, mv);
   return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 
@@ -528,6 +530,7 @@ flash_bwd_dkv_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap
                  ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -560,6 +563,7 @@ flash_bwd_dkv_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap
           tma_load_2d(ys + FA_TILE + kb * 8192, &map_y1, 64 * kb, yr, bar(B_YFULL + st));
         }
       }
+      pdl_trigger();
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
@@ -768,6 +772,7 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
                  ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -792,6 +797,7 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
           tma_load_2d(ys + (2 + kb) * FA_TILE, &map_v, 64 * kb, yr, bar(B_YFULL + st));
         }
       }
+      pdl_trigger();
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
@@ -951,6 +957,7 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
 // bf16: D stands for sum_j P_j dP_j, and with a peaked row dP - D cancels, so an error in D would show in dS.
 __global__ void attn_rowdot_kernel(const float* __restrict__ o32, const bf16* __restrict__ d_o, const float* __restrict__ lse,
                                    int S, int Sp, int64_t rows, float scale, float2* __restrict__ lse_d) {
+  pdl_sync();
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (row >= rows || (int)(row % Sp) >= S) return;
@@ -1003,13 +1010,13 @@ inline int launch_flash_bwd(const bf16* q, const bf16* k, const bf16* v, const b
   P.out1 = dkv; P.ld_out1 = ld_dkv; P.col1 = 0;
   P.heads_own = n_kv_heads;
   P.x0 = nullptr; P.x1 = nullptr;
-  flash_bwd_dkv_kernel<<<batch * n_kv_heads * (Sp / FA_BLK), FA_THREADS, FB_SMEM_BYTES, st>>>(P, k128, v128, q64, do64);
+  launch_k(flash_bwd_dkv_kernel, batch * n_kv_heads * (Sp / FA_BLK), FA_THREADS, FB_SMEM_BYTES, st, P, k128, v128, q64, do64);
   if (cudaGetLastError() != cudaSuccess) return REVFFN_ERR_CUDA;
   P.out0 = nullptr; P.ld_out0 = 0; P.col0 = 0;
   P.out1 = dq; P.ld_out1 = ld_dq; P.col1 = 0;
   P.heads_own = n_heads;
   P.x0 = q; P.x1 = d_o;
-  flash_bwd_dq_kernel<<<batch * n_heads * (Sp / FA_BLK), FA_THREADS, FQ_SMEM_BYTES, st>>>(P, k128, v128);
+  launch_k(flash_bwd_dq_kernel, batch * n_heads * (Sp / FA_BLK), FA_THREADS, FQ_SMEM_BYTES, st, P, k128, v128);
   return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 

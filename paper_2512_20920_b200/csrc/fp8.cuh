@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(256)
 quantize_rows_e4m3_kernel(const bf16* __restrict__ in, int64_t ld_in, const int32_t* __restrict__ row_map,
                           const int32_t* __restrict__ rows_total, int64_t rows, int width, uint8_t* __restrict__ out,
                           float* __restrict__ scale) {
+  pdl_sync();
   const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows || (rows_total && row >= *rows_total)) return;
@@ -80,7 +81,7 @@ inline cudaError_t launch_quantize_rows(const bf16* in, int64_t ld_in, const int
                                         int64_t rows, int width, uint8_t* out, float* scale, cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
   if (width % 8 != 0 || width > 2048) return cudaErrorInvalidValue;
-  quantize_rows_e4m3_kernel<<<(unsigned)ceil_div(rows, 8), 256, 0, st>>>(in, ld_in, row_map, rows_total, rows, width, out, scale);
+  launch_k(quantize_rows_e4m3_kernel, (unsigned)ceil_div(rows, 8), 256, 0, st, in, ld_in, row_map, rows_total, rows, width, out, scale);
   return cudaGetLastError();
 }
 

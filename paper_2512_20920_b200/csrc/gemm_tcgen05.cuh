@@ -499,6 +499,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
   }
+  pdl_wait();      // barriers and tensor memory are set up beside the last blocks of the kernel before this one
   tc_fence_before();
   __syncthreads();
   if constexpr (PAIR) cluster_sync_all();      // the partner's barriers exist before anything signals them
@@ -669,6 +670,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           if (++stage == Cfg::STAGES) { stage = 0; phase ^= 1u; }
         }
       }
+      if (la) pdl_trigger();
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
@@ -1335,25 +1337,12 @@ inline int tc_dg_parts(int N) { return 2 * (int)ceil_div(N, 256); }   // two epi
 template <int MMA_N, int EPI>
 inline int tc_launch(const TcParams& P, const CUtensorMap& ma, const CUtensorMap& mb0, const CUtensorMap& mb1,
                      const CUtensorMap& mc, const CUtensorMap& mc1, int grid, bool pair, cudaStream_t st) {
-  if (!pair) {
-    gemm_tc_kernel<MMA_N, EPI, false><<<grid, TC_THREADS, TcCfg<MMA_N, EPI, false>::SMEM_BYTES, st>>>(P, ma, mb0, mb1, mc, mc1);
-    return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
-  }
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(TC_THREADS);
-  cfg.dynamicSmemBytes = TcCfg<MMA_N, EPI, true>::SMEM_BYTES;
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = 2;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<MMA_N, EPI, true>, P, ma, mb0, mb1, mc, mc1) == cudaSuccess
-             ? REVFFN_OK : REVFFN_ERR_CUDA;
+  const cudaError_t e =
+      pair ? launch_cluster(gemm_tc_kernel<MMA_N, EPI, true>, dim3((unsigned)grid), dim3(2), dim3(TC_THREADS),
+                            TcCfg<MMA_N, EPI, true>::SMEM_BYTES, st, P, ma, mb0, mb1, mc, mc1)
+           : launch_k(gemm_tc_kernel<MMA_N, EPI, false>, dim3((unsigned)grid), dim3(TC_THREADS),
+                      TcCfg<MMA_N, EPI, false>::SMEM_BYTES, st, P, ma, mb0, mb1, mc, mc1);
+  return e == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 
 inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {

@@ -136,13 +136,13 @@ static int a_setup(const ACtx<T>& c, bool backward) {
   cudaStream_t st = c.st;
   const int n_tab = L.n_tiles > L.groups + 1 ? L.n_tiles : L.groups + 1;
   { ProfScope ps(TG_A_TABLES, st);
-  attn_tables_kernel<<<(unsigned)ceil_div(n_tab, 256), 256, 0, st>>>(
+  launch_k(attn_tables_kernel, (unsigned)ceil_div(n_tab, 256), 256, 0, st, 
       L.n_tiles, L.Sp / ROW_PAD, D.n_heads / D.n_kv_heads, L.groups, (D.n_heads / D.n_kv_heads) * L.Sp,
       c.template p<int32_t>(L.tile_group), c.template p<int32_t>(L.group_off), c.template p<int32_t>(L.rows_total));
   }
   CK(cudaGetLastError());
   { ProfScope ps(TG_A_TABLES, st);
-  rope_table_kernel<<<(unsigned)ceil_div((int64_t)D.seq_len * (L.hd / 2), 256), 256, 0, st>>>(
+  launch_k(rope_table_kernel, (unsigned)ceil_div((int64_t)D.seq_len * (L.hd / 2), 256), 256, 0, st, 
       D.seq_len, L.hd, (double)D.rope_theta, c.template p<float2>(L.cs));
   }
   CK(cudaGetLastError());
@@ -163,7 +163,7 @@ static int a_norm_up(const ACtx<T>& c, const float* x, int side) {
   const int Tn = L.T, d = D.d_model, h = L.h;
   T* n = c.template p<T>(L.n12) + (int64_t)side * Tn * h;
   { ProfScope ps(TG_NORM, c.st);
-  rmsnorm_fwd_kernel<T><<<(unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, c.st>>>(
+  launch_k(rmsnorm_fwd_kernel<T>, (unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, c.st, 
       x, D.ld_stream, c.W.norm_gamma, D.norm_eps, 0, Tn, h, n, c.template p<float>(L.r12) + (int64_t)side * Tn);
   }
   CK(cudaGetLastError());
@@ -237,7 +237,7 @@ static int a_core(const ACtx<T>& c, bool need_p, bool keep_o32 = false) {
     CKR(a_gemm(c, p, TG_A_SCORES));
   }
   { ProfScope ps(TG_A_SOFTMAX, c.st);
-  softmax_causal_kernel<T><<<(unsigned)ceil_div(L.rows * 32, 256), 256, 0, c.st>>>(
+  launch_k(softmax_causal_kernel<T>, (unsigned)ceil_div(L.rows * 32, 256), 256, 0, c.st, 
       c.template p<float>(L.sc), D.seq_len, L.Sp, 1.4426950408889634f / sqrtf((float)L.hd), L.rows, c.template p<T>(L.p));
   }
   CK(cudaGetLastError());
@@ -303,7 +303,7 @@ static int a_forward(const ACtx<T>& c, const float* x1, const float* x2, float* 
   const AttnLayout& L = c.L;
   CKR(a_setup(c, false));
   { ProfScope ps(TG_NORM, c.st);
-  rmsnorm2_fwd_kernel<T><<<(unsigned)ceil_div((int64_t)2 * L.T * 32, 128), 128, 0, c.st>>>(
+  launch_k(rmsnorm2_fwd_kernel<T>, (unsigned)ceil_div((int64_t)2 * L.T * 32, 128), 128, 0, c.st, 
       x1, x2, D.ld_stream, c.W.norm_gamma, D.norm_eps, L.T, L.h, c.template p<T>(L.n12), c.template p<float>(L.r12));
   }
   CK(cudaGetLastError());
@@ -328,7 +328,7 @@ static int a_inverse(const ACtx<T>& c, const float* y1, const float* x2, float* 
   const AttnLayout& L = c.L;
   if (n_iter == 0) {
     if (x1 != y1) {
-      copy_stream_kernel<<<(unsigned)ceil_div((int64_t)L.T * L.h, 4 * 256), 256, 0, c.st>>>(y1, c.D.ld_stream, L.T, L.h, x1,
+      launch_k(copy_stream_kernel, (unsigned)ceil_div((int64_t)L.T * L.h, 4 * 256), 256, 0, c.st, y1, c.D.ld_stream, L.T, L.h, x1,
                                                                                             c.D.ld_stream);
       ++g_prof.launches;
       CK(cudaGetLastError());
@@ -395,7 +395,7 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
     CK(launch_colsum_partial<T>(X, ldx, nullptr, Tn, cols, strip, strips, c.template p<float>(L.part), st));
     }
     { ProfScope ps(TG_A_BIAS, st);
-    colsum_final_kernel<<<(unsigned)ceil_div(cols, COLSUM_FINAL_COLS), 256, 0, st>>>(c.template p<float>(L.part), strips, cols, acc, out);
+    launch_k(colsum_final_kernel, (unsigned)ceil_div(cols, COLSUM_FINAL_COLS), 256, 0, st, c.template p<float>(L.part), strips, cols, acc, out);
     }
     CK(cudaGetLastError());
     return REVFFN_OK;
@@ -403,7 +403,7 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
 
   // P_down and W_o backward
   { ProfScope ps(TG_CAST, st);
-  cast_stream_kernel<T><<<(unsigned)ceil_div((int64_t)Tn * h, 4 * 256), 256, 0, st>>>(dy1, D.ld_stream, Tn, h,
+  launch_k(cast_stream_kernel<T>, (unsigned)ceil_div((int64_t)Tn * h, 4 * 256), 256, 0, st, dy1, D.ld_stream, Tn, h,
                                                                                       c.template p<T>(L.dyb));
   }
   CK(cudaGetLastError());
@@ -429,7 +429,7 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
   if (fused) {
     if constexpr (std::is_same<T, bf16>::value) {
       { ProfScope ps(TG_A_SOFTMAX, st);
-      attn_rowdot_kernel<<<(unsigned)ceil_div(L.rows * 32, 256), 256, 0, st>>>(
+      launch_k(attn_rowdot_kernel, (unsigned)ceil_div(L.rows * 32, 256), 256, 0, st, 
           c.template p<float>(L.sc), c.template p<bf16>(L.doh), c.template p<float>(L.lse), D.seq_len, Sp, L.rows,
           1.f / sqrtf((float)hd), c.template p<float2>(L.lse_d));
       }
@@ -453,7 +453,7 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
       CKR(a_gemm(c, p, TG_A_DP));
     }
     { ProfScope ps(TG_A_SOFTMAX, st);
-    dsoftmax_causal_kernel<T><<<(unsigned)ceil_div(L.rows * 32, 256), 256, 0, st>>>(
+    launch_k(dsoftmax_causal_kernel<T>, (unsigned)ceil_div(L.rows * 32, 256), 256, 0, st, 
         c.template p<T>(L.p), c.template p<float>(L.sc), D.seq_len, Sp, 1.f / sqrtf((float)hd), L.rows, c.template p<T>(L.ds));
     }
     CK(cudaGetLastError());
@@ -520,7 +520,7 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
   if (G.w_up) CKR(wgrad(G.w_up, d, h, du1, d, 0, c.template p<T>(L.n12), h, 2 * Tn, acc));
   CKR(dgrad(TG_DN, 2 * Tn, h, d, du1, d, c.W.w_up, h, c.template p<float>(L.dn12), true));
   if (dx1 != dy1) {
-    copy_stream_kernel<<<(unsigned)ceil_div((int64_t)Tn * h, 4 * 256), 256, 0, st>>>(dy1, D.ld_stream, Tn, h, dx1,
+    launch_k(copy_stream_kernel, (unsigned)ceil_div((int64_t)Tn * h, 4 * 256), 256, 0, st, dy1, D.ld_stream, Tn, h, dx1,
                                                                                      D.ld_stream);
     ++g_prof.launches;
     CK(cudaGetLastError());
@@ -530,12 +530,12 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
   const float* r1 = c.template p<float>(L.r12);
   const float* r2 = r1 + Tn;
   { ProfScope ps(TG_NORM_BWD, st);
-  rmsnorm_bwd_rows_kernel<<<(unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, st>>>(dn1, x1, D.ld_stream, c.W.norm_gamma, r1,
+  launch_k(rmsnorm_bwd_rows_kernel, (unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, st, dn1, x1, D.ld_stream, c.W.norm_gamma, r1,
                                                                                      0, Tn, h, dx1, D.ld_stream);
   }
   CK(cudaGetLastError());
   { ProfScope ps(TG_NORM_BWD, st);
-  rmsnorm_bwd_rows_kernel<<<(unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, st>>>(dn2, x2, D.ld_stream, c.W.norm_gamma, r2,
+  launch_k(rmsnorm_bwd_rows_kernel, (unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, st, dn2, x2, D.ld_stream, c.W.norm_gamma, r2,
                                                                                      0, Tn, h, dx2, D.ld_stream);
   }
   CK(cudaGetLastError());
@@ -547,7 +547,7 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
                                c.template p<float>(L.part), st));
       }
       { ProfScope ps(TG_DGAMMA, st);
-      colsum_final_kernel<<<(unsigned)ceil_div(h, COLSUM_FINAL_COLS), 256, 0, st>>>(c.template p<float>(L.part), strips, h,
+      launch_k(colsum_final_kernel, (unsigned)ceil_div(h, COLSUM_FINAL_COLS), 256, 0, st, c.template p<float>(L.part), strips, h,
                                                                       side ? 1 : acc, G.norm_gamma);
       }
       CK(cudaGetLastError());

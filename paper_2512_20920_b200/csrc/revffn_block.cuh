@@ -32,6 +32,7 @@ static int plan_block(const revffn_block_desc* D, BlockLayout* L) {
 
 // first error wins: keeps the status word of a branch call that a later branch call will clear
 __global__ void status_merge_kernel(int* __restrict__ accum, const int* __restrict__ word) {
+  pdl_sync();
   if (*accum == 0 && *word != 0) *accum = *word;
 }
 
@@ -49,7 +50,7 @@ static BlockWs block_ws(void* ws, const BlockLayout& L, size_t ws_bytes) {
   return b;
 }
 static int block_merge(const BlockWs& b, cudaStream_t st) {
-  status_merge_kernel<<<1, 1, 0, st>>>(b.accum, reinterpret_cast<const int*>(b.ws));
+  launch_k(status_merge_kernel, 1, 1, 0, st, b.accum, reinterpret_cast<const int*>(b.ws));
   return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 

@@ -273,10 +273,12 @@ struct GuardTable { int n; unsigned long long off[MAX_GUARDS]; };
 __device__ __forceinline__ uint32_t guard_word(int zone, int i) { return 0xC0DE0000u ^ (uint32_t)(zone * 64 + i) * 2654435761u; }
 
 __global__ void guard_fill_kernel(char* __restrict__ ws, const GuardTable g) {
+  pdl_sync();
   const int z = blockIdx.x, i = threadIdx.x;
   reinterpret_cast<uint32_t*>(ws + g.off[z])[i] = guard_word(z, i);
 }
 __global__ void guard_check_kernel(const char* __restrict__ ws, const GuardTable g, int* __restrict__ status) {
+  pdl_sync();
   const int z = blockIdx.x, i = threadIdx.x;
   if (reinterpret_cast<const uint32_t*>(ws + g.off[z])[i] != guard_word(z, i)) set_status(status, REVFFN_ERR_CANARY);
 }
@@ -292,13 +294,13 @@ static GuardTable guard_table(const WsLayout& L, size_t limit) {
 static int guards_fill(const WsLayout& L, size_t limit, char* ws, cudaStream_t st) {
   const GuardTable g = guard_table(L, limit);
   if (g.n == 0) return REVFFN_OK;
-  guard_fill_kernel<<<g.n, GUARD_BYTES / 4, 0, st>>>(ws, g);
+  launch_k(guard_fill_kernel, g.n, GUARD_BYTES / 4, 0, st, ws, g);
   return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 static int guards_check(const WsLayout& L, size_t limit, char* ws, cudaStream_t st) {
   const GuardTable g = guard_table(L, limit);
   if (g.n == 0) return REVFFN_OK;
-  guard_check_kernel<<<g.n, GUARD_BYTES / 4, 0, st>>>(ws, g, reinterpret_cast<int*>(ws + L.status.off));
+  launch_k(guard_check_kernel, g.n, GUARD_BYTES / 4, 0, st, ws, g, reinterpret_cast<int*>(ws + L.status.off));
   return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 
@@ -403,7 +405,7 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
 
   // Norm
   { ProfScope ps(TG_NORM, st);
-  rmsnorm_fwd_kernel<T><<<(unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, st>>>(
+  launch_k(rmsnorm_fwd_kernel<T>, (unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, st, 
       y1, D.ld_stream, c.W.norm_gamma, D.norm_eps, norm_none, Tn, h, c.template p<T>(L.n), c.template p<float>(L.r));
   }
   CK(cudaGetLastError());
@@ -469,12 +471,12 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
   // Permutation maps
   const int chunk = map_chunk_tokens(Tn);
   { ProfScope ps(TG_MAP, rt);
-  map_rank_kernel<<<L.n_chunks, MAP_THREADS, 0, rt>>>(c.template p<int32_t>(L.idx), Tn, k, E, chunk, c.template p<int32_t>(L.local_rank),
+  launch_k(map_rank_kernel, L.n_chunks, MAP_THREADS, 0, rt, c.template p<int32_t>(L.idx), Tn, k, E, chunk, c.template p<int32_t>(L.local_rank),
                                                       c.template p<int32_t>(L.chunk_cnt), c.template p<int>(L.status));
   }
   CK(cudaGetLastError());
   { ProfScope ps(TG_MAP, rt);
-  map_assign_kernel<<<L.n_chunks, MAP_THREADS, 0, rt>>>(
+  launch_k(map_assign_kernel, L.n_chunks, MAP_THREADS, 0, rt, 
       c.template p<int32_t>(L.idx), c.template p<float>(L.gates), c.template p<int32_t>(L.local_rank),
       c.template p<int32_t>(L.chunk_cnt), Tn, k, E, chunk, L.n_chunks, c.template p<int32_t>(L.expert_cnt),
       c.template p<int32_t>(L.expert_off), c.template p<int32_t>(L.tile_group), c.template p<int32_t>(L.rows_total),
@@ -535,7 +537,7 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
   if (!fp8) {
     // Permute: Up[row] = U[token(row)]
     { ProfScope ps(TG_GATHER, st);
-    gather_rows_kernel<T><<<(unsigned)L.rows_pad, 256, 0, st>>>(c.template p<T>(L.u), d, c.template p<int32_t>(L.row_tok),
+    launch_k(gather_rows_kernel<T>, (unsigned)L.rows_pad, 256, 0, st, c.template p<T>(L.u), d, c.template p<int32_t>(L.row_tok),
                                                                 c.template p<int32_t>(L.rows_total), d,
                                                                 c.template p<T>(L.up));
     }
@@ -720,7 +722,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
     {
       ProfScope ps(tag, cw.st);
       const int64_t count = (int64_t)M * N;
-      splitk_reduce_kernel<T><<<(unsigned)ceil_div(count, 4 * 256), 256, 0, cw.st>>>(
+      launch_k(splitk_reduce_kernel<T>, (unsigned)ceil_div(count, 4 * 256), 256, 0, cw.st, 
           c.template p<float>(L.ksplit), n_split, count, out, acc, upd ? reinterpret_cast<T*>(const_cast<void*>(W)) : nullptr,
           upd ? master : nullptr, upd ? sgd->rule : UpdRule{}, upd ? sgd->mom[wi] : nullptr, upd ? sgd->var[wi] : nullptr);
     }
@@ -734,7 +736,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
 
   // P_down backward: dZ = G W_down;  dW_down = G^T Z
   { ProfScope ps(TG_CAST, st);
-  cast_stream_kernel<T><<<(unsigned)ceil_div((int64_t)Tn * h, 4 * 256), 256, 0, st>>>(dy2, D.ld_stream, Tn, h,
+  launch_k(cast_stream_kernel<T>, (unsigned)ceil_div((int64_t)Tn * h, 4 * 256), 256, 0, st, dy2, D.ld_stream, Tn, h,
                                                                                       c.template p<T>(L.gb));
   }
   CK(cudaGetLastError());
@@ -752,7 +754,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
   // Shared expert backward
   if (Is > 0) {
     { ProfScope ps(TG_SHGATE_BWD, st);
-    shared_gate_bwd_kernel<T><<<Tn, 256, 0, st>>>(c.template p<T>(L.dz), c.template p<T>(L.s),
+    launch_k(shared_gate_bwd_kernel<T>, Tn, 256, 0, st, c.template p<T>(L.dz), c.template p<T>(L.s),
                                                   c.template p<float>(L.sgate), d, c.template p<T>(L.ds),
                                                   c.template p<float>(L.dl));
     }
@@ -799,7 +801,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
                                   c.template p<float>(L.part), cw.st));
       }
       { ProfScope ps(TG_WG_SGATE, cw.st);
-      colsum_final_kernel<<<(unsigned)ceil_div(d, COLSUM_FINAL_COLS), 256, 0, cw.st>>>(c.template p<float>(L.part), L.strips, d, acc,
+      launch_k(colsum_final_kernel, (unsigned)ceil_div(d, COLSUM_FINAL_COLS), 256, 0, cw.st, c.template p<float>(L.part), L.strips, d, acc,
                                                                       G.ws_sgate);
       }
       CK(cudaGetLastError());
@@ -808,7 +810,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
 
   // Routed experts backward
   { ProfScope ps(TG_GATHER_DZ, st);
-  gather_rows_kernel<T><<<(unsigned)Rp, 256, 0, st>>>(c.template p<T>(L.dz), d, c.template p<int32_t>(L.row_tok),
+  launch_k(gather_rows_kernel<T>, (unsigned)Rp, 256, 0, st, c.template p<T>(L.dz), d, c.template p<int32_t>(L.row_tok),
                                                       c.template p<int32_t>(L.rows_total), d, c.template p<T>(L.dop));
   }
   CK(cudaGetLastError());
@@ -859,7 +861,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
   const bool dense_gate = (D.flags & REVFFN_FLAG_GATE_SOFTMAX_ALL) != 0;
   if (!dense_gate) {
     { ProfScope ps(TG_ROUTER_BWD, st);
-    router_bwd_kernel<<<(unsigned)ceil_div(Tn, 128), 128, 0, st>>>(
+    launch_k(router_bwd_kernel, (unsigned)ceil_div(Tn, 128), 128, 0, st, 
         c.template p<float>(L.dg_part), L.dg_ld, n_part, c.template p<float>(L.gates), c.template p<int32_t>(L.tok_row),
         Tn, k, c.template p<float>(L.tok_dl), c.template p<float>(L.row_dl));
     }
@@ -868,7 +870,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
       dim3 grid((unsigned)ceil_div(d, 256), (unsigned)E);
       CKR(c.order(st, cw.st));
       { ProfScope ps(TG_WG_ROUTER, cw.st);
-      router_wgrad_kernel<T><<<grid, 256, 0, cw.st>>>(c.template p<T>(L.up), c.template p<float>(L.row_dl),
+      launch_k(router_wgrad_kernel<T>, grid, 256, 0, cw.st, c.template p<T>(L.up), c.template p<float>(L.row_dl),
                                                    c.template p<int32_t>(L.expert_off), c.template p<int32_t>(L.expert_cnt),
                                                    d, acc, G.w_router, G.b_router);
       }
@@ -877,7 +879,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
   } else {
     // every logit carries a gradient: dL is a dense [T, E] matrix and its products are matrix products
     { ProfScope ps(TG_ROUTER_BWD, st);
-    router_bwd_dense_kernel<T><<<(unsigned)ceil_div(Tn, 128), 128, 0, st>>>(
+    launch_k(router_bwd_dense_kernel<T>, (unsigned)ceil_div(Tn, 128), 128, 0, st, 
         c.template p<float>(L.dg_part), L.dg_ld, n_part, c.template p<float>(L.prob), c.template p<int32_t>(L.idx),
         c.template p<int32_t>(L.tok_row), Tn, k, E, L.ld_dlf, c.template p<T>(L.dlf));
     }
@@ -900,7 +902,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
                                   c.template p<float>(L.part), cw.st));
       }
       { ProfScope ps(TG_WG_ROUTER, cw.st);
-      colsum_final_kernel<<<(unsigned)ceil_div(E, COLSUM_FINAL_COLS), 256, 0, cw.st>>>(c.template p<float>(L.part), L.strips, E, acc,
+      launch_k(colsum_final_kernel, (unsigned)ceil_div(E, COLSUM_FINAL_COLS), 256, 0, cw.st, c.template p<float>(L.part), L.strips, E, acc,
                                                                       G.b_router);
       }
       CK(cudaGetLastError());
@@ -927,7 +929,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
   CKR(wgrad(TG_WG_PUP, REVFFN_UPD_W_UP, G.w_up, c.W.w_up, S.m_w_up, d, h, c.template p<T>(L.du), d, 0, c.template p<T>(L.n), h,
             false, 0));
   { ProfScope ps(TG_NORM_BWD, st);
-  rmsnorm_bwd_rows_kernel<<<(unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, st>>>(
+  launch_k(rmsnorm_bwd_rows_kernel, (unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, st, 
       c.template p<float>(L.dn), y1, D.ld_stream, c.W.norm_gamma, c.template p<float>(L.r), norm_none, Tn, h, dy1,
       D.ld_stream);
   }
@@ -942,7 +944,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
                                c.template p<float>(L.part), cw.st));
       }
       { ProfScope ps(TG_DGAMMA, cw.st);
-      colsum_final_kernel<<<(unsigned)ceil_div(h, COLSUM_FINAL_COLS), 256, 0, cw.st>>>(c.template p<float>(L.part), L.strips, h, acc,
+      launch_k(colsum_final_kernel, (unsigned)ceil_div(h, COLSUM_FINAL_COLS), 256, 0, cw.st, c.template p<float>(L.part), L.strips, h, acc,
                                                                       G.norm_gamma);
       }
       CK(cudaGetLastError());

@@ -66,6 +66,7 @@ template <typename T>
 __global__ void rmsnorm_fwd_kernel(const float* __restrict__ y, int64_t ld, const float* __restrict__ gamma,
                                    float eps, int norm_none, int tokens, int h,
                                    T* __restrict__ n_out, float* __restrict__ r_out) {
+  pdl_sync();
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (warp >= tokens) return;
   rmsnorm_row<T>(y + (int64_t)warp * ld, gamma, eps, norm_none, h, threadIdx.x & 31, n_out + (int64_t)warp * h, r_out + warp);
@@ -93,6 +94,7 @@ template <typename T>
 __global__ void __launch_bounds__(FD_THREADS)
 fold_router_kernel(const T* __restrict__ w_router, const T* __restrict__ w_sgate,
                    const T* __restrict__ w_up, int E, int d, int h, double* __restrict__ w_rc) {
+  pdl_sync();
   constexpr int PER16 = 16 / (int)sizeof(T);                  // elements per 16-byte piece
   constexpr int ROW_PIECES = FD_I / PER16;                    // pieces per staged row
   constexpr int N_PIECES = FD_J * ROW_PIECES / FD_THREADS;    // pieces per thread and chunk
@@ -171,7 +173,7 @@ template <typename T>
 inline cudaError_t launch_fold_router(const T* w_router, const T* w_sgate, const T* w_up, int E, int d, int h,
                                       double* w_rc, cudaStream_t st) {
   dim3 grid((unsigned)ceil_div(h, FD_I), (unsigned)ceil_div(E + 1, FD_E));
-  fold_router_kernel<T><<<grid, FD_THREADS, 0, st>>>(w_router, w_sgate, w_up, E, d, h, w_rc);
+  launch_k(fold_router_kernel<T>, grid, FD_THREADS, 0, st, w_router, w_sgate, w_up, E, d, h, w_rc);
   return cudaGetLastError();
 }
 
@@ -201,6 +203,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 fold_router_mma_kernel(const T* __restrict__ w_router, const T* __restrict__ w_sgate, const T* __restrict__ w_up,
                        int E, int d, int h, double* __restrict__ part) {
+  pdl_sync();
   constexpr int PER16 = 16 / (int)sizeof(T);
   constexpr int FM_J = fold_slice_rows<T>();
   constexpr int LDA = FM_J + FM_PAD, LDB = 64 + FM_PAD;
@@ -258,6 +261,7 @@ fold_router_mma_kernel(const T* __restrict__ w_router, const T* __restrict__ w_s
 
 __global__ void fold_router_reduce_kernel(const double* __restrict__ part, int n_slices, int64_t n,
                                           double* __restrict__ w_rc) {
+  pdl_sync();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double v = part[i];
@@ -272,11 +276,11 @@ inline cudaError_t launch_fold_router_mma(const T* w_router, const T* w_sgate, c
   const int n_slices = (int)ceil_div(d, fold_slice_rows<T>());
   if (n_slices > FOLD_SLICES) return cudaErrorInvalidValue;
   dim3 grid((unsigned)ceil_div(h, 64), (unsigned)ceil_div(E + 1, 64), (unsigned)n_slices);
-  fold_router_mma_kernel<T><<<grid, 256, 0, st>>>(w_router, w_sgate, w_up, E, d, h, part);
+  launch_k(fold_router_mma_kernel<T>, grid, 256, 0, st, w_router, w_sgate, w_up, E, d, h, part);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int64_t n = (int64_t)(E + 1) * h;
-  fold_router_reduce_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(part, n_slices, n, w_rc);
+  launch_k(fold_router_reduce_kernel, (unsigned)ceil_div(n, 256), 256, 0, st, part, n_slices, n, w_rc);
   return cudaGetLastError();
 }
 
@@ -364,6 +368,7 @@ router_topk_kernel(const float* __restrict__ y, int64_t ld, const float* __restr
                    int32_t* __restrict__ idx_out, float* __restrict__ gate_out, float* __restrict__ sgate_out,
                    int32_t* __restrict__ idx_user, float* __restrict__ prob_out, int* __restrict__ status,
                    int check_finite) {
+  pdl_sync();
   extern __shared__ __align__(16) uint8_t rt_smem[];
   const int EP = E + 1;                       // logits per token incl. the shared-gate row
   double* Lp = reinterpret_cast<double*>(rt_smem + router_part_off(E));    // [RT_TOK][EP] this block's partial sums
@@ -597,19 +602,9 @@ inline cudaError_t launch_router_topk(const float* y, int64_t ld, const float* g
       raised[dev] = smem;
     }
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(ceil_div(tokens, RT_TOK) * ROUTE_CLUSTER));
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = ROUTE_CLUSTER;
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, router_topk_kernel, y, ld, gamma, eps, norm_none, w_rc, b_router, tokens, h, E, k,
-                            has_shared, idx_in, idx_out, gate_out, sgate_out, idx_user, prob_out, status, check_finite);
+  return launch_cluster(router_topk_kernel, dim3((unsigned)(ceil_div(tokens, RT_TOK) * ROUTE_CLUSTER)), dim3(ROUTE_CLUSTER),
+                        dim3(256), smem, st, y, ld, gamma, eps, norm_none, w_rc, b_router, tokens, h, E, k, has_shared, idx_in,
+                        idx_out, gate_out, sgate_out, idx_user, prob_out, status, check_finite);
 }
 
 // ---------------------------------------------------------------------------
@@ -640,6 +635,7 @@ inline int map_chunk_tokens(int64_t tokens) {
 __global__ void __launch_bounds__(MAP_THREADS)
 map_rank_kernel(const int32_t* __restrict__ idx, int tokens, int k, int E, int chunk_tokens,
                 int32_t* __restrict__ local_rank, int32_t* __restrict__ chunk_cnt, int* __restrict__ status) {
+  pdl_sync();
   constexpr int WARPS = MAP_THREADS / 32;
   __shared__ int hist[WARPS][MAP_MAX_E];       // counts per warp, then the warps' bases
   __shared__ int run[MAP_MAX_E];
@@ -679,6 +675,7 @@ map_assign_kernel(const int32_t* __restrict__ idx, const float* __restrict__ gat
                   int32_t* __restrict__ expert_cnt, int32_t* __restrict__ expert_off, int32_t* __restrict__ tile_group,
                   int32_t* __restrict__ rows_total, int max_tiles, int4* __restrict__ tok_chunks, int max_chunks,
                   int32_t* __restrict__ tok_row, int32_t* __restrict__ row_tok, float* __restrict__ row_gate) {
+  pdl_sync();
   __shared__ int below[MAP_MAX_E], cnt[MAP_MAX_E];          // this expert's entries in earlier chunks / in all chunks
   __shared__ int off[MAP_MAX_E + 1], coff[MAP_MAX_E + 1];   // first padded row, first token run of an expert
   const int tid = threadIdx.x, lane = tid & 31;
@@ -769,6 +766,7 @@ map_assign_kernel(const int32_t* __restrict__ idx, const float* __restrict__ gat
 template <typename T>
 __global__ void gather_rows_kernel(const T* __restrict__ src, int64_t ld_src, const int32_t* __restrict__ row_tok,
                                    const int32_t* __restrict__ rows_total, int width, T* __restrict__ out) {
+  pdl_sync();
   int row = blockIdx.x;
   if (row >= *rows_total) return;
   int t = row_tok[row];
@@ -795,6 +793,7 @@ __global__ void __launch_bounds__(32 * COMBINE_TOKENS)
 combine_rows_kernel(const T* __restrict__ O, const int32_t* __restrict__ tok_row, int k_rt,
                     const T* __restrict__ S, const float* __restrict__ sgate, int width, int tokens,
                     T* __restrict__ Z) {
+  pdl_sync();
   constexpr int KS = K ? K : 8;
   const int k = K ? K : k_rt;
   const int lane = threadIdx.x & 31;
@@ -839,10 +838,10 @@ inline cudaError_t launch_combine_rows(const T* O, const int32_t* tok_row, int k
   if (tokens <= 0) return cudaSuccess;
   const int blocks = (int)ceil_div(tokens, COMBINE_TOKENS), th = 32 * COMBINE_TOKENS;
   switch (k) {
-    case 1: combine_rows_kernel<T, 1><<<blocks, th, 0, st>>>(O, tok_row, k, S, sgate, width, tokens, Z); break;
-    case 2: combine_rows_kernel<T, 2><<<blocks, th, 0, st>>>(O, tok_row, k, S, sgate, width, tokens, Z); break;
-    case 4: combine_rows_kernel<T, 4><<<blocks, th, 0, st>>>(O, tok_row, k, S, sgate, width, tokens, Z); break;
-    default: combine_rows_kernel<T, 0><<<blocks, th, 0, st>>>(O, tok_row, k, S, sgate, width, tokens, Z); break;
+    case 1: launch_k(combine_rows_kernel<T, 1>, blocks, th, 0, st, O, tok_row, k, S, sgate, width, tokens, Z); break;
+    case 2: launch_k(combine_rows_kernel<T, 2>, blocks, th, 0, st, O, tok_row, k, S, sgate, width, tokens, Z); break;
+    case 4: launch_k(combine_rows_kernel<T, 4>, blocks, th, 0, st, O, tok_row, k, S, sgate, width, tokens, Z); break;
+    default: launch_k(combine_rows_kernel<T, 0>, blocks, th, 0, st, O, tok_row, k, S, sgate, width, tokens, Z); break;
   }
   return cudaGetLastError();
 }
