@@ -6,6 +6,7 @@
 //   softmax_causal    P = softmax(scale * scores) over keys 0..s of query position s
 //   dsoftmax_causal   dS = scale * P * (dP - <P, dP>)
 //   attn_tables       row-block -> key/value group table and group offsets for the grouped products
+//   attn_setup        fused path: rotary table, zeroed padding rows, cleared status word in one launch
 //
 // Head-major buffers pad every (sequence, head) to S_pad = round_up(S, ROW_PAD) rows, so that a
 // 128-row tile of a grouped product never spans two heads; the padding rows are kept at zero.
@@ -15,16 +16,50 @@
 
 namespace revffn {
 
+__device__ __forceinline__ float2 rope_entry(int s, int i, int hd, double theta) {
+  double ang = (double)s * pow(theta, -2.0 * (double)i / (double)hd);
+  double sn, c;
+  sincos(ang, &sn, &c);
+  return make_float2((float)c, (float)sn);
+}
+
 __global__ void rope_table_kernel(int S, int hd, double theta, float2* __restrict__ cs) {
   pdl_sync();
   const int half = hd / 2;
   int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= S * half) return;
-  int s = idx / half, i = idx % half;
-  double ang = (double)s * pow(theta, -2.0 * (double)i / (double)hd);
-  double sn, c;
-  sincos(ang, &sn, &c);
-  cs[idx] = make_float2((float)c, (float)sn);
+  cs[idx] = rope_entry(idx / half, idx % half, hd, theta);
+}
+
+// Everything the fused path needs before its first product, in one launch (it was two kernels and up to five memsets,
+// 4 us each on the stream whatever their size): the rotary table as [pair, position], so that a warp whose lanes are
+// neighbouring positions reads it in whole lines; zeros in the padding rows S .. Sp - 1 of up to four head-major
+// buffers (the attention kernels load whole 128-row tiles); the status word.
+// pad[j]: n_pad_rows[j] padding rows in all, 16 pieces of 16 bytes each (hd = 128, bf16).
+struct AttnPads { bf16* buf[4]; int rows[4]; int n; };
+__global__ void __launch_bounds__(256)
+attn_setup_kernel(int S, int Sp, double theta, float2* __restrict__ cs, const AttnPads pads, int* __restrict__ status) {
+  pdl_sync();
+  int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx == 0 && status) *status = 0;
+  if (cs) {
+    if (idx < (int64_t)S * 64) {
+      const int i = (int)(idx / S), s = (int)(idx % S);
+      cs[idx] = rope_entry(s, i, 128, theta);
+      return;
+    }
+    idx -= (int64_t)S * 64;
+  }
+  const int per = Sp - S;
+  for (int j = 0; j < pads.n; ++j) {
+    const int64_t n = (int64_t)pads.rows[j] * 16;
+    if (idx < n) {
+      const int64_t row = idx / 16, head = row / per, r = row % per;
+      *reinterpret_cast<uint4*>(pads.buf[j] + (head * Sp + S + r) * 128 + (idx % 16) * 8) = make_uint4(0u, 0u, 0u, 0u);
+      return;
+    }
+    idx -= n;
+  }
 }
 
 // RMSNorm of both streams in one launch: warp w < tokens normalises row w of x1, the others row w - tokens of x2;
@@ -35,27 +70,9 @@ __global__ void rmsnorm2_fwd_kernel(const float* __restrict__ x1, const float* _
                                     float* __restrict__ r_out) {
   pdl_sync();
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
   if (warp >= 2 * tokens) return;
   const float* row = warp < tokens ? x1 + (int64_t)warp * ld : x2 + (int64_t)(warp - tokens) * ld;
-  float ss = 0.f;
-  for (int i = lane * 4; i < h; i += 128) {
-    float4 v = *reinterpret_cast<const float4*>(row + i);
-    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-  }
-  ss = warp_sum(ss);
-  const float r = rsqrtf(ss / (float)h + eps);
-  if (lane == 0) r_out[warp] = r;
-  T* out = n_out + (int64_t)warp * h;
-  for (int i = lane * 4; i < h; i += 128) {
-    float4 v = *reinterpret_cast<const float4*>(row + i);
-    float4 g = make_float4(1.f, 1.f, 1.f, 1.f);
-    if (gamma) g = *reinterpret_cast<const float4*>(gamma + i);
-    out[i + 0] = from_f32<T>(v.x * r * g.x);
-    out[i + 1] = from_f32<T>(v.y * r * g.y);
-    out[i + 2] = from_f32<T>(v.z * r * g.z);
-    out[i + 3] = from_f32<T>(v.w * r * g.w);
-  }
+  rmsnorm_row<T>(row, gamma, eps, 0, h, threadIdx.x & 31, n_out + (int64_t)warp * h, r_out + warp);
 }
 
 // One block per token.  in: [T, ld_in] with n heads of hd columns; out: [B, n, S_pad, hd].

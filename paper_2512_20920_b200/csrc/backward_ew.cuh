@@ -330,6 +330,142 @@ inline cudaError_t launch_du_reduce(const T* dUp, const int32_t* tok_row, const 
   return cudaGetLastError();
 }
 
+// RMSNorm backward and the norm scale's gradient in one pass over the rows:
+//   q = gamma * dn;  out = base + r q - y r^3 <q, y> / h;   part[block, c] = sum over the block's rows of dn * y * r
+// (the partial sums are added by colsum_final_kernel).  norm NONE: out = base + dn.  Up to two sets of rows (the two
+// streams of the attention branch, which share the scale); base may be out itself.
+// One warp per row at a time, a row's dn and y in registers between the dot product and the result (h <= 1024), rows
+// dealt out to the grid's warps in turn, so the partial sums are in a fixed order.
+// Bound by HBM: dn, y, base read, out written.  8192 rows of 1024: 31 us + 25 us for the scale's
+// gradient in separate passes, 33 us together.
+struct NormBwdRows { const float* dn; const float* y; const float* r; const float* base; float* out; };
+constexpr int NORM_BWD_MAX_H = 1024;
+constexpr int NORM_BWD_MAX_BLOCKS = 444;
+inline int norm_bwd_blocks(int64_t rows) { return (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(rows, 8), NORM_BWD_MAX_BLOCKS)); }
+
+__global__ void __launch_bounds__(256)
+norm_bwd_kernel(const NormBwdRows s0, const NormBwdRows s1, int64_t ld, const float* __restrict__ gamma, int norm_none,
+                int tokens, int sides, int h, float* __restrict__ part) {
+  pdl_sync();
+  extern __shared__ __align__(16) float nb_smem[];       // [8][h] when part is wanted
+  constexpr int KEEP = NORM_BWD_MAX_H / 128;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float4 acc[KEEP];
+#pragma unroll
+  for (int q = 0; q < KEEP; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int64_t row = (int64_t)blockIdx.x * 8 + warp; row < (int64_t)tokens * sides; row += (int64_t)gridDim.x * 8) {
+    const bool second = row >= tokens;
+    const int64_t t = second ? row - tokens : row;
+    const float* dn = (second ? s1.dn : s0.dn) + t * h;
+    const float* y = (second ? s1.y : s0.y) + t * ld;
+    const float* base = (second ? s1.base : s0.base) + t * ld;
+    float* out = (second ? s1.out : s0.out) + t * ld;
+    const float rt = norm_none ? 1.f : (second ? s1.r : s0.r)[t];
+    float4 d[KEEP], v[KEEP];
+#pragma unroll
+    for (int q = 0; q < KEEP; ++q) {
+      const int i = lane * 4 + q * 128;
+      d[q] = v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < h) {
+        d[q] = *reinterpret_cast<const float4*>(dn + i);
+        if (!norm_none) v[q] = *reinterpret_cast<const float4*>(y + i);
+      }
+    }
+    float dot = 0.f;
+    if (!norm_none) {
+#pragma unroll
+      for (int q = 0; q < KEEP; ++q) {
+        const int i = lane * 4 + q * 128;
+        acc[q].x += d[q].x * v[q].x * rt; acc[q].y += d[q].y * v[q].y * rt;
+        acc[q].z += d[q].z * v[q].z * rt; acc[q].w += d[q].w * v[q].w * rt;
+        if (gamma && i < h) {
+          const float4 g = *reinterpret_cast<const float4*>(gamma + i);
+          d[q].x *= g.x; d[q].y *= g.y; d[q].z *= g.z; d[q].w *= g.w;
+        }
+        dot += d[q].x * v[q].x + d[q].y * v[q].y + d[q].z * v[q].z + d[q].w * v[q].w;
+      }
+      dot = warp_sum(dot);
+    }
+    const float coef = norm_none ? 0.f : rt * rt * rt * dot / (float)h;
+#pragma unroll
+    for (int q = 0; q < KEEP; ++q) {
+      const int i = lane * 4 + q * 128;
+      if (i >= h) continue;
+      float4 o = *reinterpret_cast<const float4*>(base + i);
+      o.x += rt * d[q].x - v[q].x * coef; o.y += rt * d[q].y - v[q].y * coef;
+      o.z += rt * d[q].z - v[q].z * coef; o.w += rt * d[q].w - v[q].w * coef;
+      *reinterpret_cast<float4*>(out + i) = o;
+    }
+  }
+  if (!part) return;
+#pragma unroll
+  for (int q = 0; q < KEEP; ++q) {
+    const int i = lane * 4 + q * 128;
+    if (i < h) *reinterpret_cast<float4*>(nb_smem + warp * h + i) = acc[q];
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < h; c += 256) {
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) v += nb_smem[w * h + c];
+    part[(int64_t)blockIdx.x * h + c] = v;
+  }
+}
+
+// Plain column sums of up to three matrices with the same rows in two launches (partials, then the fixed-order sum):
+// the q, k and v bias gradients.  Column c of the concatenation belongs to the segment whose range holds it; a thread
+// takes four columns (widths and leading dimensions are multiples of 4).
+template <typename T> struct ColSegs { const T* X[3]; int64_t ld[3]; int end[3]; float* out[3]; };
+
+template <typename T>
+__global__ void __launch_bounds__(128)
+colsum_segs_partial_kernel(const ColSegs<T> s, int rows, int cols, int strip, float* __restrict__ part) {
+  pdl_sync();
+  const int c = (blockIdx.x * blockDim.x + threadIdx.x) * 4, b = blockIdx.y;
+  if (c >= cols) return;
+  const int g = c < s.end[0] ? 0 : (c < s.end[1] ? 1 : 2);
+  const int64_t ld = s.ld[g];
+  const T* px = s.X[g] + (c - (g ? s.end[g - 1] : 0));
+  const int t0 = b * strip, t1 = min(rows, t0 + strip);
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+  for (int t = t0; t < t1; ++t) {
+    if constexpr (sizeof(T) == 2) {
+      const uint2 raw = *reinterpret_cast<const uint2*>(px + (int64_t)t * ld);
+      const __nv_bfloat162* hp = reinterpret_cast<const __nv_bfloat162*>(&raw);
+      const float2 u = __bfloat1622float2(hp[0]), v = __bfloat1622float2(hp[1]);
+      acc.x += u.x; acc.y += u.y; acc.z += v.x; acc.w += v.y;
+    } else {
+      const float4 u = *reinterpret_cast<const float4*>(px + (int64_t)t * ld);
+      acc.x += u.x; acc.y += u.y; acc.z += u.z; acc.w += u.w;
+    }
+  }
+  *reinterpret_cast<float4*>(part + (int64_t)b * cols + c) = acc;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+colsum_segs_final_kernel(const float* __restrict__ part, int n_strips, int cols, int accumulate, const ColSegs<T> s) {
+  pdl_sync();
+  __shared__ float red[8][COLSUM_FINAL_COLS];
+  const int cl = threadIdx.x % COLSUM_FINAL_COLS, g = threadIdx.x / COLSUM_FINAL_COLS;
+  const int c = blockIdx.x * COLSUM_FINAL_COLS + cl;
+  float acc = 0.f;
+  if (c < cols)
+    for (int b = g; b < n_strips; b += 8) acc += part[(int64_t)b * cols + c];
+  red[g][cl] = acc;
+  __syncthreads();
+  if (g == 0 && c < cols) {
+    float v = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v += red[i][cl];
+    const int k = c < s.end[0] ? 0 : (c < s.end[1] ? 1 : 2);
+    float* o = s.out[k] + (c - (k ? s.end[k - 1] : 0));
+    *o = (accumulate ? *o : 0.f) + v;
+  }
+}
+
+// The same in separate passes, for rows wider than the one-pass kernel keeps.
 // RMSNorm backward, rows:  q = gamma * dn;  dy = r q - y r^3 <q, y> / h;  dY1 += dy.
 // One warp per token.  norm NONE: dY1 += dn.
 __global__ void rmsnorm_bwd_rows_kernel(const float* __restrict__ dn, const float* __restrict__ y, int64_t ld,

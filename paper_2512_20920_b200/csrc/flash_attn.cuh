@@ -436,7 +436,7 @@ struct FlashBwdParams {
   int64_t ld_out0, ld_out1;
   int col0, col1;
   int heads_own;                  // heads per sequence on the owned side (key/value heads for dK/dV, query heads for dQ)
-  const float2* cs;               // [S, 64] (cos, sin)
+  const float2* cs;               // [64, S] (cos, sin): the lanes' positions are neighbours
   float scale_log2e, scale;
   int* status;
 };
@@ -688,13 +688,13 @@ flash_bwd_dkv_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap
 #pragma unroll
           for (int i = 0; i < 32; ++i) { y0[i] = __uint_as_float(rl[i]); y1[i] = __uint_as_float(rh[i]); }
           if (a == 1) {
-            const float4* cs2 = reinterpret_cast<const float4*>(P.cs + own_pos * 64 + 32 * hh);
+            const float2* cs2 = P.cs + (int64_t)(32 * hh) * P.S + own_pos;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float4 cs = cs2[i];
-              const float a0 = y0[2 * i], b0 = y1[2 * i], a1 = y0[2 * i + 1], b1 = y1[2 * i + 1];
-              y0[2 * i] = a0 * cs.x + b0 * cs.y;         y1[2 * i] = b0 * cs.x - a0 * cs.y;
-              y0[2 * i + 1] = a1 * cs.z + b1 * cs.w;     y1[2 * i + 1] = b1 * cs.z - a1 * cs.w;
+            for (int i = 0; i < 32; ++i) {
+              const float2 cs = cs2[(int64_t)i * P.S];
+              const float a0 = y0[i], b0 = y1[i];
+              y0[i] = a0 * cs.x + b0 * cs.y;
+              y1[i] = b0 * cs.x - a0 * cs.y;
             }
           }
           bf16* dst = (a == 0 ? P.out0 + tok * P.ld_out0 + P.col0 : P.out1 + tok * P.ld_out1 + P.col1) + head * FA_HD + 32 * hh;
@@ -920,14 +920,13 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
       tmem_ld_wait();
       if (row_ok) {
         float y0[32], y1[32];
-        const float4* cs2 = reinterpret_cast<const float4*>(P.cs + own_pos * 64 + 32 * hh);
+        const float2* cs2 = P.cs + (int64_t)(32 * hh) * P.S + own_pos;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const float4 cs = cs2[i];
-          const float a0 = __uint_as_float(rl[2 * i]), b0 = __uint_as_float(rh[2 * i]);
-          const float a1 = __uint_as_float(rl[2 * i + 1]), b1 = __uint_as_float(rh[2 * i + 1]);
-          y0[2 * i] = a0 * cs.x + b0 * cs.y;         y1[2 * i] = b0 * cs.x - a0 * cs.y;
-          y0[2 * i + 1] = a1 * cs.z + b1 * cs.w;     y1[2 * i + 1] = b1 * cs.z - a1 * cs.w;
+        for (int i = 0; i < 32; ++i) {
+          const float2 cs = cs2[(int64_t)i * P.S];
+          const float a0 = __uint_as_float(rl[i]), b0 = __uint_as_float(rh[i]);
+          y0[i] = a0 * cs.x + b0 * cs.y;
+          y1[i] = b0 * cs.x - a0 * cs.y;
         }
         bf16* dst = P.out1 + tok * P.ld_out1 + P.col1 + head * FA_HD + 32 * hh;
         store32_bf16(dst, y0);
@@ -972,9 +971,10 @@ __global__ void attn_rowdot_kernel(const float* __restrict__ o32, const bf16* __
 
 // q, d_o: [B * n_heads * Sp, 128]; k, v: [B * n_kv_heads * Sp, 128] bf16 head-major (rows past the sequence zero).
 // Outputs token-major bf16, rotation undone: dq [T, ld_dq]; dk at column 0 and dv at column dv_col of dkv [T, ld_dkv].
+// The two launches depend on nothing of each other: st_dkv and st_dq may be different streams.
 inline int launch_flash_bwd(const bf16* q, const bf16* k, const bf16* v, const bf16* d_o, const float2* lse_d, const float2* cs,
                             int batch, int n_heads, int n_kv_heads, int S, int Sp, bf16* dq, int64_t ld_dq, bf16* dkv,
-                            int64_t ld_dkv, int dv_col, int* status, cudaStream_t st) {
+                            int64_t ld_dkv, int dv_col, int* status, cudaStream_t st_dkv, cudaStream_t st_dq) {
   TcState& s = tc_state();
   if (!s.ready) return REVFFN_ERR_CUDA;
   if (batch <= 0) return REVFFN_OK;
@@ -988,16 +988,12 @@ inline int launch_flash_bwd(const bf16* q, const bf16* k, const bf16* v, const b
     attr_set[dev] = true;
   }
   const uint64_t q_rows = (uint64_t)batch * n_heads * Sp, kv_rows = (uint64_t)batch * n_kv_heads * Sp;
-  CUtensorMap q128, do128, k128, v128, q64, do64, k64, v64;
+  CUtensorMap k128, v128, q64, do64;
   int r = 0;
-  if (!r) r = tc_make_map(&q128, q, FA_HD, q_rows, FA_HD, 64, 128);
-  if (!r) r = tc_make_map(&do128, d_o, FA_HD, q_rows, FA_HD, 64, 128);
   if (!r) r = tc_make_map(&k128, k, FA_HD, kv_rows, FA_HD, 64, 128);
   if (!r) r = tc_make_map(&v128, v, FA_HD, kv_rows, FA_HD, 64, 128);
   if (!r) r = tc_make_map(&q64, q, FA_HD, q_rows, FA_HD, 64, 64);
   if (!r) r = tc_make_map(&do64, d_o, FA_HD, q_rows, FA_HD, 64, 64);
-  if (!r) r = tc_make_map(&k64, k, FA_HD, kv_rows, FA_HD, 64, 64);
-  if (!r) r = tc_make_map(&v64, v, FA_HD, kv_rows, FA_HD, 64, 64);
   if (r) return r;
   FlashBwdParams P;
   P.S = S; P.Sp = Sp; P.n_heads = n_heads; P.rep = n_heads / n_kv_heads;
@@ -1010,13 +1006,13 @@ inline int launch_flash_bwd(const bf16* q, const bf16* k, const bf16* v, const b
   P.out1 = dkv; P.ld_out1 = ld_dkv; P.col1 = 0;
   P.heads_own = n_kv_heads;
   P.x0 = nullptr; P.x1 = nullptr;
-  launch_k(flash_bwd_dkv_kernel, batch * n_kv_heads * (Sp / FA_BLK), FA_THREADS, FB_SMEM_BYTES, st, P, k128, v128, q64, do64);
+  launch_k(flash_bwd_dkv_kernel, batch * n_kv_heads * (Sp / FA_BLK), FA_THREADS, FB_SMEM_BYTES, st_dkv, P, k128, v128, q64, do64);
   if (cudaGetLastError() != cudaSuccess) return REVFFN_ERR_CUDA;
   P.out0 = nullptr; P.ld_out0 = 0; P.col0 = 0;
   P.out1 = dq; P.ld_out1 = ld_dq; P.col1 = 0;
   P.heads_own = n_heads;
   P.x0 = q; P.x1 = d_o;
-  launch_k(flash_bwd_dq_kernel, batch * n_heads * (Sp / FA_BLK), FA_THREADS, FQ_SMEM_BYTES, st, P, k128, v128);
+  launch_k(flash_bwd_dq_kernel, batch * n_heads * (Sp / FA_BLK), FA_THREADS, FQ_SMEM_BYTES, st_dq, P, k128, v128);
   return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 

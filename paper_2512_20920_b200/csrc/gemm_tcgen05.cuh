@@ -866,7 +866,9 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
         // cannot tell that they do not overlap) and a 32 x 32 block cost eight memory round trips: the fused SGD
         // pass measured 2.4 ms slower than writing the gradients.  (Asking the next tile's lines into the L2 a
         // tile ahead, prefetch.global.L2 per row, changed nothing measurable on top of this.)
-        const bool rmw = EPI == EPI_WGRAD && (wptr != nullptr || p.accumulate);
+        // The coupling's residual rows come the same way (one row per lane, 16 bytes at a time, they cost a line per
+        // lane and load: 384 x 256 outputs over K = 512 took 16 us, a plain store of the same product 9 us).
+        const bool rmw = EPI == EPI_COUPLE || (EPI == EPI_WGRAD && (wptr != nullptr || p.accumulate));
         auto as_f4 = [](const uint4& u) {
           return make_float4(__uint_as_float(u.x), __uint_as_float(u.y), __uint_as_float(u.z), __uint_as_float(u.w));
         };
@@ -887,7 +889,8 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
               const int r = i * 4 + (lane >> 3);
               const int64_t at = (yb + r) * p.ldc + col;
               if (yb + r < y_lim) {
-                if (!wptr) ld[i] = *reinterpret_cast<const uint4*>(cptr + at);
+                if (EPI == EPI_COUPLE) ld[i] = *reinterpret_cast<const uint4*>(p.resid + (yb + r) * p.ld_resid + col);
+                else if (!wptr) ld[i] = *reinterpret_cast<const uint4*>(cptr + at);
                 else if (mptr) ld[i] = *reinterpret_cast<const uint4*>(mptr + at);
                 else { const uint2 w2 = *reinterpret_cast<const uint2*>(wptr + at); ld[i].x = w2.x; ld[i].y = w2.y; }
               }
@@ -899,18 +902,6 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           if constexpr (EPI == EPI_ROWSCALE) {
 #pragma unroll
             for (int i = 0; i < 32; ++i) f[i] *= rs;
-          } else if constexpr (EPI == EPI_COUPLE) {
-            if (m_ok) {
-              const float4* x = reinterpret_cast<const float4*>(p.resid + (int64_t)m * p.ld_resid + n);
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                float4 xv = x[i];
-                f[4 * i] = xv.x + p.resid_sign * f[4 * i];
-                f[4 * i + 1] = xv.y + p.resid_sign * f[4 * i + 1];
-                f[4 * i + 2] = xv.z + p.resid_sign * f[4 * i + 2];
-                f[4 * i + 3] = xv.w + p.resid_sign * f[4 * i + 3];
-              }
-            }
           }
           // bf16 blocks (32 x 32, 2 KB) leave through two alternating staging buffers and TMA stores.
           // fp32 blocks (32 x 32, 4 KB) are transposed through the staging area and written with plain
@@ -973,6 +964,12 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
                   const int64_t at = (yb + r) * p.ldc + col;
                   if (yb + r >= y_lim) continue;
                   const float4 v = *reinterpret_cast<const float4*>(stg + r * 128 + ((piece ^ (r & 7)) << 4));
+                  if (EPI == EPI_COUPLE) {
+                    const float4 o = as_f4(ld[i]);
+                    *reinterpret_cast<float4*>(cptr + at) = make_float4(o.x + p.resid_sign * v.x, o.y + p.resid_sign * v.y,
+                                                                        o.z + p.resid_sign * v.z, o.w + p.resid_sign * v.w);
+                    continue;
+                  }
                   if (!wptr) {          // accumulate into the stored gradient
                     const float4 o = as_f4(ld[i]);
                     *reinterpret_cast<float4*>(cptr + at) = make_float4(o.x + v.x, o.y + v.y, o.z + v.z, o.w + v.w);
@@ -1020,17 +1017,16 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
         uint32_t r1[32];
         const int seq = m_ok ? m / p.hm_S : 0, pos = m_ok ? m % p.hm_S : 0;
         const int n_heads = p.N / 128;
+        const int64_t row_at = ((int64_t)seq * n_heads * p.hm_Sp + pos) * 128;      // this lane's row, head 0
 #pragma unroll 1
         for (int c = half * 32; c < t.ncols; c += 128) {
           if (!slab_ok) continue;      // warp-uniform
           const int n = t.n0 + c;      // first column of the lower half-range; n + 64 is its partner
-          __syncwarp();                // lanes past the last row skipped the previous block's stores: rejoin before the warp-wide loads
           tmem_ld32(taddr + c, r0);
           tmem_ld32(taddr + c + 64, r1);
           tmem_ld_wait();
-          if (!m_ok) continue;
           const int head = n / 128, i0 = n % 128;            // i0 is 0 or 32
-          bf16* dst = reinterpret_cast<bf16*>(p.C) + (((int64_t)seq * n_heads + head) * p.hm_Sp + pos) * 128 + i0;
+          bf16* dst = reinterpret_cast<bf16*>(p.C) + (int64_t)head * p.hm_Sp * 128 + i0;
           float y0[32], y1[32];
 #pragma unroll
           for (int i = 0; i < 32; ++i) { y0[i] = __uint_as_float(r0[i]); y1[i] = __uint_as_float(r1[i]); }
@@ -1045,17 +1041,33 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
             }
           }
           if (p.hm_cs) {
-            const float4* cs2 = reinterpret_cast<const float4*>(p.hm_cs + pos * 64 + i0);   // two (cos, sin) pairs per load
+            // the table is [pair, position]: the lanes' positions are neighbours
+            const float2* cs2 = p.hm_cs + (int64_t)i0 * p.hm_S + pos;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float4 cs = cs2[i];
-              const float a0 = y0[2 * i], b0v = y1[2 * i], a1 = y0[2 * i + 1], b1v = y1[2 * i + 1];
-              y0[2 * i] = a0 * cs.x - b0v * cs.y;         y1[2 * i] = b0v * cs.x + a0 * cs.y;
-              y0[2 * i + 1] = a1 * cs.z - b1v * cs.w;     y1[2 * i + 1] = b1v * cs.z + a1 * cs.w;
+            for (int i = 0; i < 32; ++i) {
+              const float2 cs = cs2[(int64_t)i * p.hm_S];
+              const float a0 = y0[i], b0v = y1[i];
+              y0[i] = a0 * cs.x - b0v * cs.y;
+              y1[i] = b0v * cs.x + a0 * cs.y;
             }
           }
-          store32_bf16(dst, y0);
-          store32_bf16(dst + 64, y1);
+          // out through the staging area, eight rows of 64 bytes per instruction (rows of a slab may belong to two
+          // sequences, so each row's address comes from its lane)
+          stage32_bf16(stg, lane, y0);
+          stage32_bf16(stg + 2048, lane, y1);
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int r = 8 * i + (lane >> 2);
+            const int64_t at = __shfl_sync(0xffffffffu, row_at, r);
+            const int off = r * 64 + (((lane & 3) ^ ((r >> 1) & 3)) << 4);
+            const uint4 v0 = *reinterpret_cast<const uint4*>(stg + off), v1 = *reinterpret_cast<const uint4*>(stg + 2048 + off);
+            if (r < rows_ok) {
+              *reinterpret_cast<uint4*>(dst + at + (lane & 3) * 8) = v0;
+              *reinterpret_cast<uint4*>(dst + at + 64 + (lane & 3) * 8) = v1;
+            }
+          }
+          __syncwarp();
         }
       } else if constexpr (EPI == EPI_SWIGLU) {
         // columns [0, MMA_N/2) hold the gate projection, [MMA_N/2, MMA_N) the up projection.

@@ -10,7 +10,6 @@
 #pragma once
 
 #include "../../include/revffn_attn.h"
-#include "attn.cuh"
 #include "flash_attn.cuh"
 
 namespace revffn {
@@ -18,7 +17,7 @@ namespace revffn {
 struct AttnLayout {
   Buf status, rows_total, tile_group, group_off, cs, n12, r12, u12, raw, qh, kh, vh, lse, sc, p, oh, o, a;
   size_t fwd_bytes = 0;
-  Buf dyb, da, dob, doh, ds, dqh, dkh, dvh, dq, dkv, du12, dn12, part, lse_d;
+  Buf dyb, da, dob, doh, ds, dqh, dkh, dvh, dq, dkv, du12, dn12, part, npart, lse_d;
   size_t bwd_bytes = 0;
   int T = 0, h = 0, hd = 0, d_kv = 0, Sp = 0, n_tiles = 0, groups = 0, strips = 0;
   int64_t rows = 0, kv_rows = 0;
@@ -33,7 +32,7 @@ static AttnLayout plan_attn(const revffn_attn_desc& D) {
   L.rows = B * nh * Sp; L.kv_rows = B * nkv * Sp;
   L.n_tiles = (int)(L.rows / ROW_PAD);
   L.groups = (int)(B * nkv);
-  L.strips = (int)ceil_div(2 * T > 0 ? 2 * T : 1, STRIP);
+  L.strips = (int)ceil_div(T > 0 ? T : 1, STRIP);
   size_t off = 0;
   auto take = [&](Buf& b, size_t bytes) {
     b.off = off; b.bytes = bytes;
@@ -70,7 +69,8 @@ static AttnLayout plan_attn(const revffn_attn_desc& D) {
   take(L.dkv, (size_t)T * 2 * dkv * ts);
   take(L.du12, (size_t)2 * T * d * ts);
   take(L.dn12, (size_t)2 * T * h * 4);
-  take(L.part, (size_t)L.strips * d * 4);
+  take(L.part, (size_t)L.strips * (d + 2 * dkv) * 4);
+  take(L.npart, norm_part_floats(2 * T, (int)h) * 4);
   take(L.lse_d, (size_t)L.rows * 8);
   L.bwd_bytes = off;
   return L;
@@ -90,7 +90,7 @@ static int validate_attn_desc(const revffn_attn_desc* D) {
     return REVFFN_ERR_SHAPE;
   }
   if (!(D->rope_theta > 0.f)) return REVFFN_ERR_SHAPE;
-  if (D->flags & ~(REVFFN_FLAG_FORCE_SIMT | REVFFN_FLAG_REUSE_ACTIVATIONS)) return REVFFN_ERR_UNSUPPORTED;
+  if (D->flags & ~(REVFFN_FLAG_FORCE_SIMT | REVFFN_FLAG_REUSE_ACTIVATIONS | REVFFN_FLAG_SINGLE_STREAM)) return REVFFN_ERR_UNSUPPORTED;
   if (D->ld_stream < h || (D->ld_stream % 4)) return REVFFN_ERR_ALIGN;
   const int64_t Sp = round_up(D->seq_len, ROW_PAD);
   if ((int64_t)D->batch * D->n_heads * Sp > (int64_t)1 << 30 || (int64_t)D->batch * D->seq_len > (int64_t)1 << 28)
@@ -114,13 +114,26 @@ struct ACtx {
   AttnLayout L;
   char* ws;
   cudaStream_t st;
+  int* status;             // device status word: the workspace's own, or that of the block call this one is part of
+  bool clear;              // this call clears it
+  Overlap* ov = nullptr;   // non-null: the second stream is in use for this call
   bool tc;
+  bool fused() const { return std::is_same<T, bf16>::value && tc && L.hd == FA_HD; }      // attention core as tcgen05 kernels
+  // what is queued on `to` from now on follows everything queued on `from` so far (no-op without the second stream)
+  int order(cudaStream_t from, cudaStream_t to) const {
+    if (!ov || from == to) return REVFFN_OK;
+    cudaError_t e;
+    cudaEvent_t x = ov->mark(from, &e);
+    if (e != cudaSuccess || cudaStreamWaitEvent(to, x, 0) != cudaSuccess) return REVFFN_ERR_CUDA;
+    return REVFFN_OK;
+  }
+  ACtx on_side() const { ACtx c = *this; if (ov) c.st = ov->side; return c; }
   template <typename U> U* p(const Buf& b) const { return reinterpret_cast<U*>(ws + b.off); }
 };
 
 template <typename T>
 static int a_gemm(const ACtx<T>& c, GemmProblem p, int tag) {
-  p.status = c.template p<int>(c.L.status);
+  p.status = c.status;
   ProfScope ps(tag, c.st);
   if constexpr (std::is_same<T, bf16>::value) {
     if (c.tc) return launch_gemm_tc(p, c.st);
@@ -128,29 +141,55 @@ static int a_gemm(const ACtx<T>& c, GemmProblem p, int tag) {
   return launch_gemm_simt<T>(p, c.st) == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 
-// Tables of the grouped products, the rotary table, and zeroed padding rows of the head-major buffers.
+// What a pass needs before its first product: rotary table, zeroed padding rows of the head-major buffers, cleared
+// status word; on the materialising path also the tables of the grouped products.  tables: the rotary table and the
+// q / k / v padding (a gradient pass that reuses the key/value side finds them in place); d_o: its padding too.
 template <typename T>
-static int a_setup(const ACtx<T>& c, bool backward) {
+static int a_setup(const ACtx<T>& c, bool tables, bool d_o) {
   const revffn_attn_desc& D = c.D;
   const AttnLayout& L = c.L;
   cudaStream_t st = c.st;
-  const int n_tab = L.n_tiles > L.groups + 1 ? L.n_tiles : L.groups + 1;
-  { ProfScope ps(TG_A_TABLES, st);
-  launch_k(attn_tables_kernel, (unsigned)ceil_div(n_tab, 256), 256, 0, st, 
-      L.n_tiles, L.Sp / ROW_PAD, D.n_heads / D.n_kv_heads, L.groups, (D.n_heads / D.n_kv_heads) * L.Sp,
-      c.template p<int32_t>(L.tile_group), c.template p<int32_t>(L.group_off), c.template p<int32_t>(L.rows_total));
+  const int per = L.Sp - D.seq_len;
+  if constexpr (std::is_same<T, bf16>::value) {
+    if (c.fused()) {
+      AttnPads pads;
+      pads.n = 0;
+      auto pad = [&](const Buf& b, int n_heads) {
+        if (per == 0) return;
+        pads.buf[pads.n] = c.template p<bf16>(b);
+        pads.rows[pads.n++] = D.batch * n_heads * per;
+      };
+      if (tables) { pad(L.qh, D.n_heads); pad(L.kh, D.n_kv_heads); pad(L.vh, D.n_kv_heads); }
+      if (d_o) pad(L.doh, D.n_heads);
+      int64_t n = tables ? (int64_t)D.seq_len * 64 : 0;
+      for (int j = 0; j < pads.n; ++j) n += (int64_t)pads.rows[j] * 16;
+      if (n == 0 && !c.clear) return REVFFN_OK;
+      ProfScope ps(TG_A_TABLES, st);
+      CK(launch_k(attn_setup_kernel, (unsigned)ceil_div(std::max<int64_t>(n, 1), 256), 256, 0, st, D.seq_len, L.Sp,
+                  (double)D.rope_theta, tables ? c.template p<float2>(L.cs) : nullptr, pads, c.clear ? c.status : nullptr));
+      return REVFFN_OK;
+    }
   }
-  CK(cudaGetLastError());
-  { ProfScope ps(TG_A_TABLES, st);
-  launch_k(rope_table_kernel, (unsigned)ceil_div((int64_t)D.seq_len * (L.hd / 2), 256), 256, 0, st, 
-      D.seq_len, L.hd, (double)D.rope_theta, c.template p<float2>(L.cs));
+  if (c.clear) CK(launch_k(clear_status_kernel, 1, 1, 0, st, c.status));
+  if (tables) {
+    const int n_tab = L.n_tiles > L.groups + 1 ? L.n_tiles : L.groups + 1;
+    { ProfScope ps(TG_A_TABLES, st);
+    CK(launch_k(attn_tables_kernel, (unsigned)ceil_div(n_tab, 256), 256, 0, st, L.n_tiles, L.Sp / ROW_PAD,
+                D.n_heads / D.n_kv_heads, L.groups, (D.n_heads / D.n_kv_heads) * L.Sp, c.template p<int32_t>(L.tile_group),
+                c.template p<int32_t>(L.group_off), c.template p<int32_t>(L.rows_total)));
+    }
+    { ProfScope ps(TG_A_TABLES, st);
+    CK(launch_k(rope_table_kernel, (unsigned)ceil_div((int64_t)D.seq_len * (L.hd / 2), 256), 256, 0, st, D.seq_len, L.hd,
+                (double)D.rope_theta, c.template p<float2>(L.cs)));
+    }
   }
-  CK(cudaGetLastError());
-  if (L.Sp != D.seq_len) {
-    CK(cudaMemsetAsync(c.ws + L.qh.off, 0, L.qh.bytes, st));
-    CK(cudaMemsetAsync(c.ws + L.kh.off, 0, L.kh.bytes, st));
-    CK(cudaMemsetAsync(c.ws + L.vh.off, 0, L.vh.bytes, st));
-    if (backward) CK(cudaMemsetAsync(c.ws + L.doh.off, 0, L.doh.bytes, st));
+  if (per != 0) {
+    if (tables) {
+      CK(cudaMemsetAsync(c.ws + L.qh.off, 0, L.qh.bytes, st));
+      CK(cudaMemsetAsync(c.ws + L.kh.off, 0, L.kh.bytes, st));
+      CK(cudaMemsetAsync(c.ws + L.vh.off, 0, L.vh.bytes, st));
+    }
+    if (d_o) CK(cudaMemsetAsync(c.ws + L.doh.off, 0, L.doh.bytes, st));
   }
   return REVFFN_OK;
 }
@@ -186,7 +225,7 @@ static int a_project(const ACtx<T>& c, int side, const void* W, const float* bia
   p.A = c.template p<T>(L.u12) + (int64_t)side * Tn * d; p.lda = d;
   p.B0 = W; p.ldb = d;
   if constexpr (std::is_same<T, bf16>::value) {
-    if (c.tc && L.hd == 128) {
+    if (c.fused()) {
       // bias, rotation and the head-major layout happen in the product's epilogue: no fp32 round trip
       p.epilogue = EPI_HEADS; p.C = heads;
       p.hm_bias = bias; p.hm_cs = rotate ? c.template p<float2>(L.cs) : nullptr; p.hm_S = D.seq_len; p.hm_Sp = L.Sp;
@@ -220,12 +259,12 @@ static int a_core(const ACtx<T>& c, bool need_p, bool keep_o32 = false) {
   const revffn_attn_desc& D = c.D;
   const AttnLayout& L = c.L;
   if constexpr (std::is_same<T, bf16>::value) {
-    if (c.tc && !need_p && L.hd == FA_HD) {
+    if (c.fused() && !need_p) {
       ProfScope ps(TG_A_FLASH, c.st);
       return launch_flash_fwd(c.template p<bf16>(L.qh), c.template p<bf16>(L.kh), c.template p<bf16>(L.vh), D.batch,
                               D.n_heads, D.n_kv_heads, D.seq_len, L.Sp, c.template p<bf16>(L.o), D.d_model,
                               c.template p<float>(L.lse), keep_o32 ? c.template p<float>(L.sc) : nullptr,
-                              c.template p<int>(L.status), c.st);
+                              c.status, c.st);
     }
   }
   {
@@ -288,25 +327,25 @@ static int a_kv_side(const ACtx<T>& c, const float* x2) {
   return a_project(c, 1, c.W.w_v, c.W.b_v, c.D.n_kv_heads, false, c.template p<T>(c.L.vh));
 }
 
+// Query side up to the core's operands: norm, P_up, rotated q.
 template <typename T>
-static int a_query_side(const ACtx<T>& c, const float* x1, bool need_p, bool keep_o32 = false) {
+static int a_query(const ACtx<T>& c, const float* x1) {
   CKR(a_norm_up(c, x1, 0));
-  CKR(a_project(c, 0, c.W.w_q, c.W.b_q, c.D.n_heads, true, c.template p<T>(c.L.qh)));
-  CKR(a_core(c, need_p, keep_o32));
-  return a_wo(c);
+  return a_project(c, 0, c.W.w_q, c.W.b_q, c.D.n_heads, true, c.template p<T>(c.L.qh));
 }
 
-// Forward pass: both streams are known at once, so the norm and P_up run over the 2T rows together.
+// Forward pass: both streams are known at once, so the norm and P_up run over the 2T rows together.  The keys and
+// values are projected on the second stream beside the queries.
 template <typename T>
 static int a_forward(const ACtx<T>& c, const float* x1, const float* x2, float* y1) {
   const revffn_attn_desc& D = c.D;
   const AttnLayout& L = c.L;
-  CKR(a_setup(c, false));
+  const ACtx<T> cs = c.on_side();
+  CKR(a_setup(c, true, false));
   { ProfScope ps(TG_NORM, c.st);
-  launch_k(rmsnorm2_fwd_kernel<T>, (unsigned)ceil_div((int64_t)2 * L.T * 32, 128), 128, 0, c.st, 
-      x1, x2, D.ld_stream, c.W.norm_gamma, D.norm_eps, L.T, L.h, c.template p<T>(L.n12), c.template p<float>(L.r12));
+  CK(launch_k(rmsnorm2_fwd_kernel<T>, (unsigned)ceil_div((int64_t)2 * L.T * 32, 128), 128, 0, c.st, x1, x2, D.ld_stream,
+              c.W.norm_gamma, D.norm_eps, L.T, L.h, c.template p<T>(L.n12), c.template p<float>(L.r12)));
   }
-  CK(cudaGetLastError());
   {
     GemmProblem p = blank_problem();
     p.M = 2 * L.T; p.N = D.d_model; p.K = L.h;
@@ -315,9 +354,11 @@ static int a_forward(const ACtx<T>& c, const float* x1, const float* x2, float* 
     p.epilogue = EPI_STORE; p.C = c.template p<T>(L.u12); p.ldc = D.d_model;
     CKR(a_gemm(c, p, TG_PUP));
   }
-  CKR(a_project(c, 1, c.W.w_k, c.W.b_k, D.n_kv_heads, true, c.template p<T>(L.kh)));
-  CKR(a_project(c, 1, c.W.w_v, c.W.b_v, D.n_kv_heads, false, c.template p<T>(L.vh)));
+  CKR(c.order(c.st, cs.st));
+  CKR(a_project(cs, 1, c.W.w_k, c.W.b_k, D.n_kv_heads, true, c.template p<T>(L.kh)));
+  CKR(a_project(cs, 1, c.W.w_v, c.W.b_v, D.n_kv_heads, false, c.template p<T>(L.vh)));
   CKR(a_project(c, 0, c.W.w_q, c.W.b_q, D.n_heads, true, c.template p<T>(L.qh)));
+  CKR(c.order(cs.st, c.st));
   CKR(a_core(c, false));
   CKR(a_wo(c));
   return a_couple(c, x1, 1.f, y1);
@@ -327,19 +368,24 @@ template <typename T>
 static int a_inverse(const ACtx<T>& c, const float* y1, const float* x2, float* x1, int n_iter) {
   const AttnLayout& L = c.L;
   if (n_iter == 0) {
+    if (c.clear) CK(launch_k(clear_status_kernel, 1, 1, 0, c.st, c.status));
     if (x1 != y1) {
-      launch_k(copy_stream_kernel, (unsigned)ceil_div((int64_t)L.T * L.h, 4 * 256), 256, 0, c.st, y1, c.D.ld_stream, L.T, L.h, x1,
-                                                                                            c.D.ld_stream);
       ++g_prof.launches;
-      CK(cudaGetLastError());
+      CK(launch_k(copy_stream_kernel, (unsigned)ceil_div((int64_t)L.T * L.h, 4 * 256), 256, 0, c.st, y1, c.D.ld_stream, L.T,
+                  L.h, x1, c.D.ld_stream));
     }
     return REVFFN_OK;
   }
-  CKR(a_setup(c, false));
-  CKR(a_kv_side(c, x2));
+  const ACtx<T> cs = c.on_side();
+  CKR(a_setup(c, true, false));
+  CKR(c.order(c.st, cs.st));
+  CKR(a_kv_side(cs, x2));                  // beside the first iteration's query side
   const float* cur = y1;
   for (int it = 0; it < n_iter; ++it) {
-    CKR(a_query_side(c, cur, false));
+    CKR(a_query(c, cur));
+    if (it == 0) CKR(c.order(cs.st, c.st));
+    CKR(a_core(c, false));
+    CKR(a_wo(c));
     CKR(a_couple(c, y1, -1.f, x1));
     cur = x1;
   }
@@ -354,92 +400,78 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
   const int Tn = L.T, d = D.d_model, h = L.h, hd = L.hd, dkv = L.d_kv, Sp = L.Sp;
   const int acc = G.accumulate ? 1 : 0;
   cudaStream_t st = c.st;
+  const ACtx<T> cs = c.on_side();
 
-  // recompute the branch's intermediates (Sec. 3.1: nothing was cached)
-  // REUSE: an inverse call (at least one iteration) on this workspace with the same x2 and weights has left the
-  // tables and the key/value side (n2, u2, k, v head-major) behind; only the query side is evaluated again
-  const bool reuse_kv = (D.flags & REVFFN_FLAG_REUSE_ACTIVATIONS) != 0;
-  if (!reuse_kv) CKR(a_setup(c, true));
-  else if (L.Sp != D.seq_len) CK(cudaMemsetAsync(c.ws + L.doh.off, 0, L.doh.bytes, st));
-  // tcgen05 back end: the attention core runs fused in both directions and P is never written;
-  // otherwise the score matrix is materialised and the gradient pass reads P from memory
-  bool fused = false;
-  if constexpr (std::is_same<T, bf16>::value) fused = c.tc && hd == FA_HD;
-  if (!reuse_kv) CKR(a_kv_side(c, x2));
-  CKR(a_query_side(c, x1, !fused, fused));      // fused: the score buffer holds the unrounded output instead
-
-  auto wgrad = [&](float* out, int M, int N, const void* A, int64_t lda, int a_col0, const void* B, int64_t ldb,
-                   int K, int accumulate) -> int {
+  auto wgrad = [&](const ACtx<T>& on, float* out, int M, int N, const void* A, int64_t lda, int a_col0, const void* B, int64_t ldb,
+                   int K) -> int {
     GemmProblem p = blank_problem();
     p.M = M; p.N = N; p.K = K;
     p.a_mn_major = 1; p.b_mn_major = 1;
     p.A = A; p.lda = lda; p.a_col0 = a_col0;
     p.B0 = B; p.ldb = ldb;
-    p.epilogue = EPI_WGRAD; p.accumulate = accumulate;
+    p.epilogue = EPI_WGRAD; p.accumulate = acc;
     p.C = out; p.ldc = N;
-    return a_gemm(c, p, TG_A_WGRAD);
+    return a_gemm(on, p, TG_A_WGRAD);
   };
-  auto dgrad = [&](int tag, int M, int N, int K, const void* A, int64_t lda, const void* W, int64_t ldw, void* C,
+  auto dgrad = [&](const ACtx<T>& on, int tag, int M, int N, int K, const void* A, int64_t lda, const void* W, int64_t ldw, void* C,
                    bool f32) -> int {
     GemmProblem p = blank_problem();   // C = A W  with W stored [K, N]
     p.M = M; p.N = N; p.K = K;
     p.A = A; p.lda = lda;
     p.B0 = W; p.ldb = ldw; p.b_mn_major = 1;
     p.epilogue = EPI_STORE; p.out_f32 = f32 ? 1 : 0; p.C = C; p.ldc = N;
-    return a_gemm(c, p, tag);
-  };
-  const int strip = STRIP;      // rows per partial sum of the two-pass column reductions
-  auto colsum = [&](const T* X, int64_t ldx, int cols, float* out) -> int {
-    const int strips = (int)ceil_div(Tn, strip);
-    { ProfScope ps(TG_A_BIAS, st);
-    CK(launch_colsum_partial<T>(X, ldx, nullptr, Tn, cols, strip, strips, c.template p<float>(L.part), st));
-    }
-    { ProfScope ps(TG_A_BIAS, st);
-    launch_k(colsum_final_kernel, (unsigned)ceil_div(cols, COLSUM_FINAL_COLS), 256, 0, st, c.template p<float>(L.part), strips, cols, acc, out);
-    }
-    CK(cudaGetLastError());
-    return REVFFN_OK;
+    return a_gemm(on, p, tag);
   };
 
-  // P_down and W_o backward
-  { ProfScope ps(TG_CAST, st);
-  launch_k(cast_stream_kernel<T>, (unsigned)ceil_div((int64_t)Tn * h, 4 * 256), 256, 0, st, dy1, D.ld_stream, Tn, h,
-                                                                                      c.template p<T>(L.dyb));
+  // Recompute the branch's intermediates (Sec. 3.1: nothing was cached).
+  // REUSE: an inverse call (at least one iteration) on this workspace with the same x2 and weights has left the
+  // tables and the key/value side (n2, u2, k, v head-major) behind; only the query side is evaluated again.
+  // tcgen05 back end: the attention core runs fused in both directions and P is never written;
+  // otherwise the score matrix is materialised and the gradient pass reads P from memory.
+  // The upstream gradient's way down to dO needs none of it: it runs on the second stream beside the query side.
+  const bool reuse_kv = (D.flags & REVFFN_FLAG_REUSE_ACTIVATIONS) != 0;
+  const bool fused = c.fused();
+  CKR(a_setup(c, !reuse_kv, true));
+  CKR(c.order(st, cs.st));
+  { ProfScope ps(TG_CAST, cs.st);
+  CK(launch_k(cast_stream_kernel<T>, (unsigned)ceil_div((int64_t)Tn * h, 4 * 256), 256, 0, cs.st, dy1, D.ld_stream, Tn, h,
+              c.template p<T>(L.dyb)));
   }
-  CK(cudaGetLastError());
-  if (G.w_down) CKR(wgrad(G.w_down, h, d, c.template p<T>(L.dyb), h, 0, c.template p<T>(L.a), d, Tn, acc));
-  CKR(dgrad(TG_A_DGRAD, Tn, d, h, c.template p<T>(L.dyb), h, c.W.w_down, d, c.template p<T>(L.da), false));
-  if (G.w_o) CKR(wgrad(G.w_o, d, d, c.template p<T>(L.da), d, 0, c.template p<T>(L.o), d, Tn, acc));
+  CKR(dgrad(cs, TG_A_DGRAD, Tn, d, h, c.template p<T>(L.dyb), h, c.W.w_down, d, c.template p<T>(L.da), false));
   if (fused) {
     GemmProblem p = blank_problem();   // dO = da W_o, written head-major by the product's epilogue
     p.M = Tn; p.N = d; p.K = d;
     p.A = c.template p<T>(L.da); p.lda = d;
     p.B0 = c.W.w_o; p.ldb = d; p.b_mn_major = 1;
     p.epilogue = EPI_HEADS; p.C = c.template p<T>(L.doh); p.hm_S = D.seq_len; p.hm_Sp = Sp;
-    CKR(a_gemm(c, p, TG_A_DGRAD));
+    CKR(a_gemm(cs, p, TG_A_DGRAD));
   } else {
-    CKR(dgrad(TG_A_DGRAD, Tn, d, d, c.template p<T>(L.da), d, c.W.w_o, d, c.template p<T>(L.dob), false));
-    { ProfScope ps(TG_A_HEADS, st);
+    CKR(dgrad(cs, TG_A_DGRAD, Tn, d, d, c.template p<T>(L.da), d, c.W.w_o, d, c.template p<T>(L.dob), false));
+    { ProfScope ps(TG_A_HEADS, cs.st);
     CK((launch_to_heads<T, T>(c.template p<T>(L.dob), d, nullptr, nullptr, Tn, D.seq_len, Sp, D.n_heads, hd,
-                              c.template p<T>(L.doh), st)));
+                              c.template p<T>(L.doh), cs.st)));
     }
   }
+  if (!reuse_kv) CKR(a_kv_side(c, x2));
+  CKR(a_query(c, x1));
+  CKR(a_core(c, !fused, fused));        // fused: the score buffer holds the unrounded output instead
+  CKR(c.order(cs.st, st));
 
   // attention core backward
   if (fused) {
     if constexpr (std::is_same<T, bf16>::value) {
       { ProfScope ps(TG_A_SOFTMAX, st);
-      launch_k(attn_rowdot_kernel, (unsigned)ceil_div(L.rows * 32, 256), 256, 0, st, 
-          c.template p<float>(L.sc), c.template p<bf16>(L.doh), c.template p<float>(L.lse), D.seq_len, Sp, L.rows,
-          1.f / sqrtf((float)hd), c.template p<float2>(L.lse_d));
+      CK(launch_k(attn_rowdot_kernel, (unsigned)ceil_div(L.rows * 32, 256), 256, 0, st, c.template p<float>(L.sc),
+                  c.template p<bf16>(L.doh), c.template p<float>(L.lse), D.seq_len, Sp, L.rows, 1.f / sqrtf((float)hd),
+                  c.template p<float2>(L.lse_d)));
       }
-      CK(cudaGetLastError());
+      CKR(c.order(st, cs.st));
       { ProfScope ps(TG_A_FLASH, st);
       // the two launches also undo the rotation and write dq and dk|dv token-major in the operand type
       CKR(launch_flash_bwd(c.template p<bf16>(L.qh), c.template p<bf16>(L.kh), c.template p<bf16>(L.vh),
                            c.template p<bf16>(L.doh), c.template p<float2>(L.lse_d), c.template p<float2>(L.cs), D.batch,
                            D.n_heads, D.n_kv_heads, D.seq_len, Sp, c.template p<bf16>(L.dq), d, c.template p<bf16>(L.dkv),
-                           2 * (int64_t)dkv, dkv, c.template p<int>(L.status), st));
+                           2 * (int64_t)dkv, dkv, c.status, st, cs.st));
       ++g_prof.launches;
       }
     }
@@ -453,10 +485,9 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
       CKR(a_gemm(c, p, TG_A_DP));
     }
     { ProfScope ps(TG_A_SOFTMAX, st);
-    launch_k(dsoftmax_causal_kernel<T>, (unsigned)ceil_div(L.rows * 32, 256), 256, 0, st, 
-        c.template p<T>(L.p), c.template p<float>(L.sc), D.seq_len, Sp, 1.f / sqrtf((float)hd), L.rows, c.template p<T>(L.ds));
+    CK(launch_k(dsoftmax_causal_kernel<T>, (unsigned)ceil_div(L.rows * 32, 256), 256, 0, st, c.template p<T>(L.p),
+                c.template p<float>(L.sc), D.seq_len, Sp, 1.f / sqrtf((float)hd), L.rows, c.template p<T>(L.ds)));
     }
-    CK(cudaGetLastError());
     auto kv_grad = [&](const T* A, const T* Bm, float* out) -> int {
       GemmProblem p = blank_problem();   // out[g] = A_g^T B_g over the query rows of key/value group g
       p.M = Sp; p.N = hd; p.K = (int)L.rows;
@@ -478,8 +509,6 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
       p.epilogue = EPI_STORE; p.out_f32 = 1; p.C = c.template p<float>(L.dqh); p.ldc = hd;
       CKR(a_gemm(c, p, TG_A_DQ));
     }
-  }
-  if (!fused) {
     // back to token-major; the rotation is undone by its transpose
     { ProfScope ps(TG_A_HEADS, st);
     CK((launch_from_heads<float, T>(c.template p<float>(L.dqh), c.template p<float2>(L.cs), -1.f, Tn, D.seq_len, Sp,
@@ -493,20 +522,18 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
     CK((launch_from_heads<float, T>(c.template p<float>(L.dvh), nullptr, 1.f, Tn, D.seq_len, Sp, D.n_kv_heads, hd,
                                     c.template p<T>(L.dkv), 2 * (int64_t)dkv, dkv, st)));
     }
+    CKR(c.order(st, cs.st));
   }
 
-  // q/k/v projections backward
+  // Input gradients on the caller's stream; every weight gradient is a leaf and goes to the second one (dq is already
+  // there, dk | dv are ordered in).
   const T* u1 = c.template p<T>(L.u12);
   const T* u2 = u1 + (int64_t)Tn * d;
-  if (G.b_q) CKR(colsum(c.template p<T>(L.dq), d, d, G.b_q));
-  if (G.b_k) CKR(colsum(c.template p<T>(L.dkv), 2 * (int64_t)dkv, dkv, G.b_k));
-  if (G.b_v) CKR(colsum(c.template p<T>(L.dkv) + dkv, 2 * (int64_t)dkv, dkv, G.b_v));
-  if (G.w_q) CKR(wgrad(G.w_q, d, d, c.template p<T>(L.dq), d, 0, u1, d, Tn, acc));
-  if (G.w_k) CKR(wgrad(G.w_k, dkv, d, c.template p<T>(L.dkv), 2 * (int64_t)dkv, 0, u2, d, Tn, acc));
-  if (G.w_v) CKR(wgrad(G.w_v, dkv, d, c.template p<T>(L.dkv), 2 * (int64_t)dkv, dkv, u2, d, Tn, acc));
   T* du1 = c.template p<T>(L.du12);
   T* du2 = du1 + (int64_t)Tn * d;
-  CKR(dgrad(TG_A_DGRAD, Tn, d, d, c.template p<T>(L.dq), d, c.W.w_q, d, du1, false));
+  CKR(c.order(cs.st, st));
+  CKR(c.order(st, cs.st));
+  CKR(dgrad(c, TG_A_DGRAD, Tn, d, d, c.template p<T>(L.dq), d, c.W.w_q, d, du1, false));
   {
     GemmProblem p = blank_problem();   // dU2 = dK W_k + dV W_v
     p.M = Tn; p.N = d; p.K = 2 * dkv;
@@ -515,45 +542,49 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
     p.epilogue = EPI_STORE; p.C = du2; p.ldc = d;
     CKR(a_gemm(c, p, TG_A_DGRAD));
   }
-
-  // P_up and the norm, both streams at once where the rows are independent
-  if (G.w_up) CKR(wgrad(G.w_up, d, h, du1, d, 0, c.template p<T>(L.n12), h, 2 * Tn, acc));
-  CKR(dgrad(TG_DN, 2 * Tn, h, d, du1, d, c.W.w_up, h, c.template p<float>(L.dn12), true));
-  if (dx1 != dy1) {
-    launch_k(copy_stream_kernel, (unsigned)ceil_div((int64_t)Tn * h, 4 * 256), 256, 0, st, dy1, D.ld_stream, Tn, h, dx1,
-                                                                                     D.ld_stream);
-    ++g_prof.launches;
-    CK(cudaGetLastError());
+  if (G.w_down) {
+    CKR(a_wo(cs));                     // a = O W_o^T is wanted for this gradient only
+    CKR(wgrad(cs, G.w_down, h, d, c.template p<T>(L.dyb), h, 0, c.template p<T>(L.a), d, Tn));
   }
-  const float* dn1 = c.template p<float>(L.dn12);
-  const float* dn2 = dn1 + (int64_t)Tn * h;
-  const float* r1 = c.template p<float>(L.r12);
-  const float* r2 = r1 + Tn;
-  { ProfScope ps(TG_NORM_BWD, st);
-  launch_k(rmsnorm_bwd_rows_kernel, (unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, st, dn1, x1, D.ld_stream, c.W.norm_gamma, r1,
-                                                                                     0, Tn, h, dx1, D.ld_stream);
-  }
-  CK(cudaGetLastError());
-  { ProfScope ps(TG_NORM_BWD, st);
-  launch_k(rmsnorm_bwd_rows_kernel, (unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, st, dn2, x2, D.ld_stream, c.W.norm_gamma, r2,
-                                                                                     0, Tn, h, dx2, D.ld_stream);
-  }
-  CK(cudaGetLastError());
-  if (G.norm_gamma) {
-    const int strips = (int)ceil_div(Tn, strip);
-    for (int side = 0; side < 2; ++side) {
-      { ProfScope ps(TG_DGAMMA, st);
-      CK(launch_dgamma_partial(side ? dn2 : dn1, side ? x2 : x1, D.ld_stream, side ? r2 : r1, Tn, h, strip, strips,
-                               c.template p<float>(L.part), st));
+  if (G.w_o) CKR(wgrad(cs, G.w_o, d, d, c.template p<T>(L.da), d, 0, c.template p<T>(L.o), d, Tn));
+  if (G.w_q) CKR(wgrad(cs, G.w_q, d, d, c.template p<T>(L.dq), d, 0, u1, d, Tn));
+  if (G.w_k) CKR(wgrad(cs, G.w_k, dkv, d, c.template p<T>(L.dkv), 2 * (int64_t)dkv, 0, u2, d, Tn));
+  if (G.w_v) CKR(wgrad(cs, G.w_v, dkv, d, c.template p<T>(L.dkv), 2 * (int64_t)dkv, dkv, u2, d, Tn));
+  {
+    ColSegs<T> s;
+    int n = 0, cols = 0;
+    auto seg = [&](const T* X, int64_t ld, int width, float* out) {
+      if (!out) return;
+      cols += width;
+      s.X[n] = X; s.ld[n] = ld; s.end[n] = cols; s.out[n++] = out;
+    };
+    seg(c.template p<T>(L.dq), d, d, G.b_q);
+    seg(c.template p<T>(L.dkv), 2 * (int64_t)dkv, dkv, G.b_k);
+    seg(c.template p<T>(L.dkv) + dkv, 2 * (int64_t)dkv, dkv, G.b_v);
+    for (int i = n; i < 3; ++i) { s.X[i] = nullptr; s.ld[i] = 0; s.end[i] = cols; s.out[i] = nullptr; }
+    if (n > 0) {
+      { ProfScope ps(TG_A_BIAS, cs.st);
+      CK(launch_k(colsum_segs_partial_kernel<T>, dim3((unsigned)ceil_div(cols, 4 * 128), (unsigned)L.strips), 128, 0, cs.st, s, Tn,
+                  cols, STRIP, c.template p<float>(L.part)));
       }
-      { ProfScope ps(TG_DGAMMA, st);
-      launch_k(colsum_final_kernel, (unsigned)ceil_div(h, COLSUM_FINAL_COLS), 256, 0, st, c.template p<float>(L.part), strips, h,
-                                                                      side ? 1 : acc, G.norm_gamma);
+      { ProfScope ps(TG_A_BIAS, cs.st);
+      CK(launch_k(colsum_segs_final_kernel<T>, (unsigned)ceil_div(cols, COLSUM_FINAL_COLS), 256, 0, cs.st,
+                  c.template p<float>(L.part), L.strips, cols, acc, s));
       }
-      CK(cudaGetLastError());
     }
   }
-  return REVFFN_OK;
+
+  // P_up and the norm, both streams at once: their rows are independent and share the weights
+  CKR(dgrad(c, TG_DN, 2 * Tn, h, d, du1, d, c.W.w_up, h, c.template p<float>(L.dn12), true));
+  if (G.w_up) {
+    CKR(c.order(st, cs.st));
+    CKR(wgrad(cs, G.w_up, d, h, du1, d, 0, c.template p<T>(L.n12), h, 2 * Tn));
+  }
+  const float* dn1 = c.template p<float>(L.dn12);
+  const float* r1 = c.template p<float>(L.r12);
+  const NormBwdRows s0 = {dn1, x1, r1, dy1, dx1}, s1 = {dn1 + (int64_t)Tn * h, x2, r1 + Tn, dx2, dx2};
+  CKR(norm_backward(st, s0, s1, 2, D.ld_stream, c.W.norm_gamma, 0, Tn, h, G.norm_gamma, acc, c.template p<float>(L.npart)));
+  return c.order(cs.st, st);           // the caller's stream ends after the weight gradients too
 }
 
 enum APass { APASS_FWD = 3, APASS_INV = 4, APASS_BWD = 5 };
@@ -561,14 +592,22 @@ enum APass { APASS_FWD = 3, APASS_INV = 4, APASS_BWD = 5 };
 template <typename T>
 static int a_dispatch(APass pass, const revffn_attn_desc& D, const revffn_attn_weights& W, const AttnLayout& L, void* ws,
                       cudaStream_t st, const float* in1, const float* x2, const float* dy1, float* out1, float* dx2,
-                      int n_iter, const revffn_attn_grads* G) {
+                      int n_iter, const revffn_attn_grads* G, int* status) {
   ACtx<T> c;
   c.D = D; c.W = W; c.L = L; c.ws = reinterpret_cast<char*>(ws); c.st = st;
   g_prof.pass = (int)pass;
   c.tc = std::is_same<T, bf16>::value && !(D.flags & REVFFN_FLAG_FORCE_SIMT);
+  c.status = status ? status : c.template p<int>(L.status);
+  c.clear = status == nullptr;
   if (c.tc) CKR(tc_prepare());
-  CK(cudaMemsetAsync(c.ws + L.status.off, 0, L.status.bytes, st));
-  if (L.T == 0) return REVFFN_OK;
+  if (c.fused() && !g_prof.on && !(D.flags & REVFFN_FLAG_SINGLE_STREAM)) {
+    c.ov = overlap_state();
+    if (!c.ov) return REVFFN_ERR_CUDA;
+  }
+  if (L.T == 0) {
+    if (c.clear) CK(launch_k(clear_status_kernel, 1, 1, 0, st, c.status));
+    return REVFFN_OK;
+  }
   if (pass == APASS_FWD) return a_forward(c, in1, x2, out1);
   if (pass == APASS_INV) return a_inverse(c, in1, x2, out1, n_iter);
   return a_backward(c, in1, x2, dy1, out1, dx2, *G);
@@ -576,7 +615,7 @@ static int a_dispatch(APass pass, const revffn_attn_desc& D, const revffn_attn_w
 
 static int a_entry(APass pass, const revffn_attn_desc* desc, const revffn_attn_weights* w, const float* in1,
                    const float* x2, const float* dy1, float* out1, float* dx2, int n_iter,
-                   const revffn_attn_grads* grads, void* ws, size_t ws_bytes, void* cuda_stream) {
+                   const revffn_attn_grads* grads, void* ws, size_t ws_bytes, void* cuda_stream, int* status = nullptr) {
   CKR(validate_attn_desc(desc));
   CKR(validate_attn_weights(w));
   if (!ws) return REVFFN_ERR_NULL;
@@ -598,8 +637,8 @@ static int a_entry(APass pass, const revffn_attn_desc* desc, const revffn_attn_w
   CKR(check_device());
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   if (desc->weight_dtype == REVFFN_BF16)
-    return a_dispatch<bf16>(pass, *desc, *w, L, ws, st, in1, x2, dy1, out1, dx2, n_iter, grads);
-  return a_dispatch<float>(pass, *desc, *w, L, ws, st, in1, x2, dy1, out1, dx2, n_iter, grads);
+    return a_dispatch<bf16>(pass, *desc, *w, L, ws, st, in1, x2, dy1, out1, dx2, n_iter, grads, status);
+  return a_dispatch<float>(pass, *desc, *w, L, ws, st, in1, x2, dy1, out1, dx2, n_iter, grads, status);
 }
 
 }  // namespace revffn

@@ -30,12 +30,6 @@ static int plan_block(const revffn_block_desc* D, BlockLayout* L) {
   return REVFFN_OK;
 }
 
-// first error wins: keeps the status word of a branch call that a later branch call will clear
-__global__ void status_merge_kernel(int* __restrict__ accum, const int* __restrict__ word) {
-  pdl_sync();
-  if (*accum == 0 && *word != 0) *accum = *word;
-}
-
 // workspace: [status word 256 B | spare stream | the branches' shared workspace]
 struct BlockWs {
   char* ws; size_t sub; float* tmp; int* accum;
@@ -49,19 +43,25 @@ static BlockWs block_ws(void* ws, const BlockLayout& L, size_t ws_bytes) {
   b.sub = ws_bytes - 256 - L.tmp_bytes;
   return b;
 }
-static int block_merge(const BlockWs& b, cudaStream_t st) {
-  launch_k(status_merge_kernel, 1, 1, 0, st, b.accum, reinterpret_cast<const int*>(b.ws));
-  return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
+// The branch calls report into the block's own status word, which the block or stack call clears once.
+static int block_clear(const BlockWs& b, cudaStream_t st) {
+  CK(launch_k(clear_status_kernel, 1, 1, 0, st, b.accum));
+  return REVFFN_OK;
+}
+
+// The attention branch follows the MoE descriptor's choice of streams: the flag speaks of the whole call.
+static revffn_attn_desc block_attn_desc(const revffn_block_desc& D) {
+  revffn_attn_desc a = D.attn;
+  a.flags |= D.moe.flags & REVFFN_FLAG_SINGLE_STREAM;
+  return a;
 }
 
 static int block_forward_one(const revffn_block_desc& D, const revffn_attn_weights* wa, const revffn_moe_weights* wm,
                              const float* x1, const float* x2, float* y1, float* y2, int32_t* idx_out, const BlockWs& b,
                              void* stream) {
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  CKR(revffn_attn_forward(&D.attn, wa, x1, x2, y1, b.ws, b.sub, stream));
-  CKR(block_merge(b, st));
-  CKR(revffn_moe_forward(&D.moe, wm, y1, x2, y2, idx_out, b.ws, b.sub, stream));
-  return block_merge(b, st);
+  const revffn_attn_desc da = block_attn_desc(D);
+  CKR(a_entry(APASS_FWD, &da, wa, x1, x2, nullptr, y1, nullptr, 0, nullptr, b.ws, b.sub, stream, b.accum));
+  return entry(PASS_FWD, &D.moe, wm, y1, x2, y2, nullptr, nullptr, idx_out, b.ws, b.sub, stream, nullptr, b.accum);
 }
 
 static int block_backward_one(const revffn_block_desc& D, const revffn_attn_weights* wa, const revffn_moe_weights* wm,
@@ -72,20 +72,19 @@ static int block_backward_one(const revffn_block_desc& D, const revffn_attn_weig
   d_inv.flags |= REVFFN_FLAG_SAVE_ACTIVATIONS;
   d_bwd.flags |= REVFFN_FLAG_REUSE_ACTIVATIONS;
   // Eq. 2 backwards: X2 = Y2 - MLP(Norm(Y1)), then dY1 += J^T dY2 (dX2 = dY2 so far)
-  CKR(revffn_moe_inverse(&d_inv, wm, s1, s2, s2, idx_in, b.ws, b.sub, stream));
-  CKR(block_merge(b, st));
-  CKR(revffn_moe_backward(&d_bwd, wm, s1, g2, g1, gm, idx_in, b.ws, b.sub, stream));
-  CKR(block_merge(b, st));
-  // Eq. 1 backwards: X1 by fixed-point iteration, then both stream gradients through the attention branch
-  CKR(revffn_attn_inverse(&D.attn, wa, s1, s2, b.tmp, D.inverse_iters, b.ws, b.sub, stream));
-  CKR(block_merge(b, st));
+  CKR(entry(PASS_INV, &d_inv, wm, s1, s2, s2, nullptr, idx_in, nullptr, b.ws, b.sub, stream, nullptr, b.accum));
+  CKR(entry(PASS_BWD, &d_bwd, wm, s1, g2, g1, gm, idx_in, nullptr, b.ws, b.sub, stream, nullptr, b.accum));
+  // Eq. 1 backwards: X1 by fixed-point iteration (in place, unless a second iteration has to read Y1 again), then both
+  // stream gradients through the attention branch
+  const revffn_attn_desc d_ai = block_attn_desc(D);
+  float* x1 = D.inverse_iters > 1 ? b.tmp : s1;
+  CKR(a_entry(APASS_INV, &d_ai, wa, s1, s2, nullptr, x1, nullptr, D.inverse_iters, nullptr, b.ws, b.sub, stream, b.accum));
   // the inverse pass has just evaluated the key/value side from the same X2 in this workspace
-  revffn_attn_desc d_ab = D.attn;
+  revffn_attn_desc d_ab = d_ai;
   if (D.inverse_iters >= 1) d_ab.flags |= REVFFN_FLAG_REUSE_ACTIVATIONS;
-  CKR(revffn_attn_backward(&d_ab, wa, b.tmp, s2, g1, g1, g2, ga, b.ws, b.sub, stream));
-  CKR(block_merge(b, st));
-  if (D.moe.tokens > 0)
-    CK(cudaMemcpy2DAsync(s1, (size_t)D.moe.ld_stream * 4, b.tmp, (size_t)D.moe.ld_stream * 4,
+  CKR(a_entry(APASS_BWD, &d_ab, wa, x1, s2, g1, g1, g2, 0, ga, b.ws, b.sub, stream, b.accum));
+  if (x1 != s1 && D.moe.tokens > 0)
+    CK(cudaMemcpy2DAsync(s1, (size_t)D.moe.ld_stream * 4, x1, (size_t)D.moe.ld_stream * 4,
                          (size_t)(D.moe.d_model / 2) * 4, (size_t)D.moe.tokens, cudaMemcpyDeviceToDevice, st));
   return REVFFN_OK;
 }
@@ -118,7 +117,7 @@ int revffn_block_forward(const revffn_block_desc* desc, const revffn_attn_weight
   int r = block_check(desc, &L, ws, ws_bytes, false);
   if (r != REVFFN_OK) return r;
   BlockWs b = block_ws(ws, L, ws_bytes);
-  CK(cudaMemsetAsync(b.accum, 0, 256, reinterpret_cast<cudaStream_t>(cuda_stream)));
+  CKR(block_clear(b, reinterpret_cast<cudaStream_t>(cuda_stream)));
   return block_forward_one(*desc, wa, wm, x1, x2, y1, y2, topk_idx_out, b, cuda_stream);
 }
 
@@ -130,13 +129,13 @@ int revffn_block_inverse(const revffn_block_desc* desc, const revffn_attn_weight
   if (r != REVFFN_OK) return r;
   BlockWs b = block_ws(ws, L, ws_bytes);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
-  CK(cudaMemsetAsync(b.accum, 0, 256, st));
-  CKR(revffn_moe_inverse(&desc->moe, wm, y1, y2, x2, topk_idx_in, b.ws, b.sub, cuda_stream));
-  CKR(block_merge(b, st));
+  CKR(block_clear(b, st));
+  CKR(entry(PASS_INV, &desc->moe, wm, y1, y2, x2, nullptr, topk_idx_in, nullptr, b.ws, b.sub, cuda_stream, nullptr, b.accum));
   // more than one iteration reads y1 again after x1 has been written: go through the spare stream when they alias
   const bool via_tmp = x1 == y1 && desc->inverse_iters > 1;
-  CKR(revffn_attn_inverse(&desc->attn, wa, y1, x2, via_tmp ? b.tmp : x1, desc->inverse_iters, b.ws, b.sub, cuda_stream));
-  CKR(block_merge(b, st));
+  const revffn_attn_desc da = block_attn_desc(*desc);
+  CKR(a_entry(APASS_INV, &da, wa, y1, x2, nullptr, via_tmp ? b.tmp : x1, nullptr, desc->inverse_iters, nullptr, b.ws, b.sub,
+              cuda_stream, b.accum));
   if (via_tmp && desc->moe.tokens > 0)
     CK(cudaMemcpy2DAsync(x1, (size_t)desc->moe.ld_stream * 4, b.tmp, (size_t)desc->moe.ld_stream * 4,
                          (size_t)(desc->moe.d_model / 2) * 4, (size_t)desc->moe.tokens, cudaMemcpyDeviceToDevice, st));
@@ -151,7 +150,7 @@ int revffn_block_backward(const revffn_block_desc* desc, const revffn_attn_weigh
   int r = block_check(desc, &L, ws, ws_bytes, true);
   if (r != REVFFN_OK) return r;
   BlockWs b = block_ws(ws, L, ws_bytes);
-  CK(cudaMemsetAsync(b.accum, 0, 256, reinterpret_cast<cudaStream_t>(cuda_stream)));
+  CKR(block_clear(b, reinterpret_cast<cudaStream_t>(cuda_stream)));
   return block_backward_one(*desc, wa, wm, s1, s2, g1, g2, ga, gm, topk_idx_in, b, cuda_stream);
 }
 
@@ -164,7 +163,7 @@ int revffn_block_stack_forward(const revffn_block_desc* desc, const revffn_attn_
   if (n_blocks < 0) return REVFFN_ERR_SHAPE;
   if (n_blocks > 0 && (!wa || !wm)) return REVFFN_ERR_NULL;
   BlockWs b = block_ws(ws, L, ws_bytes);
-  CK(cudaMemsetAsync(b.accum, 0, 256, reinterpret_cast<cudaStream_t>(cuda_stream)));
+  CKR(block_clear(b, reinterpret_cast<cudaStream_t>(cuda_stream)));
   const size_t idx_stride = routing_stride(desc->moe);
   for (int l = 0; l < n_blocks; ++l) {
     int32_t* idx = topk_idx ? reinterpret_cast<int32_t*>(reinterpret_cast<char*>(topk_idx) + (size_t)l * idx_stride) : nullptr;
@@ -183,7 +182,7 @@ int revffn_block_stack_backward(const revffn_block_desc* desc, const revffn_attn
   if (n_blocks < 0) return REVFFN_ERR_SHAPE;
   if (n_blocks > 0 && (!wa || !wm || !ga || !gm)) return REVFFN_ERR_NULL;
   BlockWs b = block_ws(ws, L, ws_bytes);
-  CK(cudaMemsetAsync(b.accum, 0, 256, reinterpret_cast<cudaStream_t>(cuda_stream)));
+  CKR(block_clear(b, reinterpret_cast<cudaStream_t>(cuda_stream)));
   const size_t idx_stride = routing_stride(desc->moe);
   for (int l = n_blocks - 1; l >= 0; --l) {
     const int32_t* idx =

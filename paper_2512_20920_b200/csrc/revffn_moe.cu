@@ -19,6 +19,7 @@
 #include "gemm.cuh"
 #include "gemm_tcgen05.cuh"
 #include "fp8.cuh"
+#include "attn.cuh"
 
 namespace revffn {
 
@@ -96,7 +97,7 @@ struct WsLayout {
   size_t fwd_bytes = 0;
   size_t saved_bytes = 0;   // fwd region + SwiGLU pre-activations: what a saved evaluation consists of
   // backward only
-  Buf ab, abs, gb, dz, ds, dl, dop, dg_part, tok_dl, row_dl, dlf, dur, dup, dush, du, dn, part, ksplit;
+  Buf ab, abs, gb, dz, ds, dl, dop, dg_part, tok_dl, row_dl, dlf, dur, dup, dush, du, dn, part, npart, ksplit;
   int ld_dlf = 0;
   size_t bwd_bytes = 0;
   int64_t rows_pad = 0;   // upper bound on padded rows
@@ -108,6 +109,8 @@ struct WsLayout {
 
 constexpr int STRIP = 32;    // tokens per strip in two-pass column reductions
 constexpr int SPLIT_K_MAX = 4;   // most K slices of a dense weight gradient
+
+static size_t norm_part_floats(int64_t rows, int h);
 
 static WsLayout plan_workspace(const revffn_moe_desc& D) {
   WsLayout L;
@@ -184,6 +187,7 @@ static WsLayout plan_workspace(const revffn_moe_desc& D) {
   take(L.du, (size_t)T * d * ts);
   take(L.dn, (size_t)T * h * 4);
   take(L.part, (size_t)L.strips * d * 4);
+  take(L.npart, norm_part_floats(T, (int)h) * 4);
   take(L.ksplit, (size_t)SPLIT_K_MAX * d * h * 4);      // partial sums of the adapters' K-split weight gradients
   L.bwd_bytes = off;
   return L;
@@ -297,11 +301,17 @@ static int guards_fill(const WsLayout& L, size_t limit, char* ws, cudaStream_t s
   launch_k(guard_fill_kernel, g.n, GUARD_BYTES / 4, 0, st, ws, g);
   return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
-static int guards_check(const WsLayout& L, size_t limit, char* ws, cudaStream_t st) {
+static int guards_check(const WsLayout& L, size_t limit, char* ws, cudaStream_t st, int* status) {
   const GuardTable g = guard_table(L, limit);
   if (g.n == 0) return REVFFN_OK;
-  launch_k(guard_check_kernel, g.n, GUARD_BYTES / 4, 0, st, ws, g, reinterpret_cast<int*>(ws + L.status.off));
+  launch_k(guard_check_kernel, g.n, GUARD_BYTES / 4, 0, st, ws, g, status);
   return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
+}
+
+// A kernel and not a memset: it takes part in the programmatic launch chain.
+__global__ void clear_status_kernel(int* __restrict__ status) {
+  pdl_sync();
+  *status = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -348,6 +358,7 @@ struct Ctx {
   WsLayout L;
   char* ws;
   cudaStream_t st;
+  int* status;             // device status word: the workspace's own, or that of the block call this one is part of
   Overlap* ov = nullptr;   // non-null: the second stream is in use for this call
   // what is queued on `to` from now on follows everything queued on `from` so far (no-op without the second stream)
   int order(cudaStream_t from, cudaStream_t to) const {
@@ -365,7 +376,7 @@ struct Ctx {
 
 template <typename T>
 static int run_gemm(const Ctx<T>& c, GemmProblem p, int tag) {
-  p.status = c.template p<int>(c.L.status);
+  p.status = c.status;
   ProfScope ps(tag, c.st);
   if constexpr (std::is_same<T, bf16>::value) {
     if (c.tc) return launch_gemm_tc(p, c.st);
@@ -458,7 +469,7 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
     CK(launch_router_topk(y1, D.ld_stream, c.W.norm_gamma, D.norm_eps, norm_none, c.template p<double>(L.w_rc),
                           c.W.b_router, Tn, h, E, k, Is > 0 ? 1 : 0, idx_in, c.template p<int32_t>(L.idx),
                           c.template p<float>(L.gates), c.template p<float>(L.sgate), idx_user,
-                          gate_all ? c.template p<float>(L.prob) : nullptr, c.template p<int>(L.status),
+                          gate_all ? c.template p<float>(L.prob) : nullptr, c.status,
                           (D.flags & REVFFN_FLAG_DEBUG_CHECKS) ? 1 : 0, rt));
     }
     if (idx_user && records) {      // complete the record the kernel has started with the indices
@@ -472,7 +483,7 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
   const int chunk = map_chunk_tokens(Tn);
   { ProfScope ps(TG_MAP, rt);
   launch_k(map_rank_kernel, L.n_chunks, MAP_THREADS, 0, rt, c.template p<int32_t>(L.idx), Tn, k, E, chunk, c.template p<int32_t>(L.local_rank),
-                                                      c.template p<int32_t>(L.chunk_cnt), c.template p<int>(L.status));
+                                                      c.template p<int32_t>(L.chunk_cnt), c.status);
   }
   CK(cudaGetLastError());
   { ProfScope ps(TG_MAP, rt);
@@ -651,6 +662,49 @@ static int spec_from_adam(const revffn_moe_adam& a, UpdateSpec* u) {
   return REVFFN_OK;
 }
 
+// dX += J^T dn of the norm for one or two sets of rows, and the gradient of the shared scale (d_gamma may be NULL).
+// part: scratch of norm_part_floats() floats.
+static size_t norm_part_floats(int64_t rows, int h) {
+  return h <= NORM_BWD_MAX_H ? (size_t)norm_bwd_blocks(rows) * h : (size_t)ceil_div(rows > 0 ? rows : 1, STRIP) * h;
+}
+static int norm_backward(cudaStream_t st, const NormBwdRows& s0, const NormBwdRows& s1, int sides, int64_t ld, const float* gamma,
+                         int norm_none, int tokens, int h, float* d_gamma, int acc, float* part) {
+  if (norm_none && d_gamma && !acc) CK(cudaMemsetAsync(d_gamma, 0, (size_t)h * 4, st));
+  if (norm_none) d_gamma = nullptr;
+  if (h <= NORM_BWD_MAX_H) {
+    const int blocks = norm_bwd_blocks((int64_t)tokens * sides);
+    { ProfScope ps(TG_NORM_BWD, st);
+    CK(launch_k(norm_bwd_kernel, blocks, 256, d_gamma ? (size_t)8 * h * 4 : 0, st, s0, s1, ld, gamma, norm_none, tokens, sides, h,
+                d_gamma ? part : nullptr));
+    }
+    if (d_gamma) {
+      ProfScope ps(TG_DGAMMA, st);
+      CK(launch_k(colsum_final_kernel, (unsigned)ceil_div(h, COLSUM_FINAL_COLS), 256, 0, st, part, blocks, h, acc, d_gamma));
+    }
+    return REVFFN_OK;
+  }
+  for (int side = 0; side < sides; ++side) {
+    const NormBwdRows& s = side ? s1 : s0;
+    if (s.base != s.out) {
+      ++g_prof.launches;
+      CK(launch_k(copy_stream_kernel, (unsigned)ceil_div((int64_t)tokens * h, 4 * 256), 256, 0, st, s.base, ld, tokens, h, s.out, ld));
+    }
+    { ProfScope ps(TG_NORM_BWD, st);
+    CK(launch_k(rmsnorm_bwd_rows_kernel, (unsigned)ceil_div((int64_t)tokens * 32, 128), 128, 0, st, s.dn, s.y, ld, gamma, s.r,
+                norm_none, tokens, h, s.out, ld));
+    }
+    if (!d_gamma) continue;
+    const int strips = (int)ceil_div(tokens, STRIP);
+    { ProfScope ps(TG_DGAMMA, st);
+    CK(launch_dgamma_partial(s.dn, s.y, ld, s.r, tokens, h, STRIP, strips, part, st));
+    }
+    { ProfScope ps(TG_DGAMMA, st);
+    CK(launch_k(colsum_final_kernel, (unsigned)ceil_div(h, COLSUM_FINAL_COLS), 256, 0, st, part, strips, h, side ? 1 : acc, d_gamma));
+    }
+  }
+  return REVFFN_OK;
+}
+
 template <typename T>
 static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, float* dy1, const revffn_moe_grads& G,
                         const UpdateSpec* sgd, const int32_t* idx_in) {
@@ -793,8 +847,8 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
       }
     }
     if (G.ws_sgate) {
-      // a leaf like the matrix gradients: second stream (which also owns the column-sum scratch `part`: every
-      // user of it, this one, the router bias and the norm scale, is queued there, in order)
+      // a leaf like the matrix gradients: second stream (which also owns the column-sum scratch `part`: both
+      // users of it, this one and the router bias, are queued there, in order)
       CKR(c.order(st, cw.st));
       { ProfScope ps(TG_WG_SGATE, cw.st);
       CK(launch_colsum_partial<T>(c.template p<T>(L.u), d, c.template p<float>(L.dl), Tn, d, STRIP, L.strips,
@@ -928,28 +982,8 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
   }
   CKR(wgrad(TG_WG_PUP, REVFFN_UPD_W_UP, G.w_up, c.W.w_up, S.m_w_up, d, h, c.template p<T>(L.du), d, 0, c.template p<T>(L.n), h,
             false, 0));
-  { ProfScope ps(TG_NORM_BWD, st);
-  launch_k(rmsnorm_bwd_rows_kernel, (unsigned)ceil_div((int64_t)Tn * 32, 128), 128, 0, st, 
-      c.template p<float>(L.dn), y1, D.ld_stream, c.W.norm_gamma, c.template p<float>(L.r), norm_none, Tn, h, dy1,
-      D.ld_stream);
-  }
-  CK(cudaGetLastError());
-  if (G.norm_gamma) {
-    if (norm_none) {
-      if (!acc) CK(cudaMemsetAsync(G.norm_gamma, 0, (size_t)h * 4, st));
-    } else {
-      CKR(c.order(st, cw.st));
-      { ProfScope ps(TG_DGAMMA, cw.st);
-      CK(launch_dgamma_partial(c.template p<float>(L.dn), y1, D.ld_stream, c.template p<float>(L.r), Tn, h, STRIP, L.strips,
-                               c.template p<float>(L.part), cw.st));
-      }
-      { ProfScope ps(TG_DGAMMA, cw.st);
-      launch_k(colsum_final_kernel, (unsigned)ceil_div(h, COLSUM_FINAL_COLS), 256, 0, cw.st, c.template p<float>(L.part), L.strips, h, acc,
-                                                                      G.norm_gamma);
-      }
-      CK(cudaGetLastError());
-    }
-  }
+  const NormBwdRows rows = {c.template p<float>(L.dn), y1, c.template p<float>(L.r), dy1, dy1};
+  CKR(norm_backward(st, rows, rows, 1, D.ld_stream, c.W.norm_gamma, norm_none, Tn, h, G.norm_gamma, acc, c.template p<float>(L.npart)));
   CKR(c.order(cw.st, st));      // the caller's stream ends after the weight gradients too
   return REVFFN_OK;
 }
@@ -962,7 +996,7 @@ enum Pass { PASS_FWD, PASS_INV, PASS_BWD };
 template <typename T>
 static int dispatch(Pass pass, const revffn_moe_desc& D, const revffn_moe_weights& W, const WsLayout& L, void* ws,
                     cudaStream_t st, const float* y1, const float* in2, float* out, const revffn_moe_grads* G,
-                    const UpdateSpec* sgd, const int32_t* idx_in, int32_t* idx_out) {
+                    const UpdateSpec* sgd, const int32_t* idx_in, int32_t* idx_out, int* status) {
   Ctx<T> c;
   c.D = D; c.W = W; c.L = L; c.ws = reinterpret_cast<char*>(ws); c.st = st;
   g_prof.pass = (int)pass;
@@ -974,7 +1008,8 @@ static int dispatch(Pass pass, const revffn_moe_desc& D, const revffn_moe_weight
     if (!c.ov) return REVFFN_ERR_CUDA;
   }
   if (c.tc) CKR(tc_prepare());
-  if (!(D.flags & REVFFN_FLAG_KEEP_STATUS)) CK(cudaMemsetAsync(c.ws + L.status.off, 0, L.status.bytes, st));
+  c.status = status ? status : c.template p<int>(L.status);
+  if (!status && !(D.flags & REVFFN_FLAG_KEEP_STATUS)) CK(launch_k(clear_status_kernel, 1, 1, 0, st, c.status));
   if (D.tokens == 0) return REVFFN_OK;   // empty batch: nothing to compute, gradients untouched
   const bool big_ws = pass == PASS_BWD || (D.flags & REVFFN_FLAG_SAVE_ACTIVATIONS);
   const size_t ws_limit = big_ws ? L.bwd_bytes : L.fwd_bytes;
@@ -985,13 +1020,14 @@ static int dispatch(Pass pass, const revffn_moe_desc& D, const revffn_moe_weight
     CKR(run_branch(c, y1, idx_in, idx_out, (D.flags & REVFFN_FLAG_SAVE_ACTIVATIONS) != 0));
     CKR(run_couple(c, in2, pass == PASS_FWD ? 1.f : -1.f, out));
   }
-  if (L.n_guards) CKR(guards_check(L, ws_limit, c.ws, st));
+  if (L.n_guards) CKR(guards_check(L, ws_limit, c.ws, st, c.status));
   return REVFFN_OK;
 }
 
 static int entry(Pass pass, const revffn_moe_desc* desc, const revffn_moe_weights* w, const float* y1,
                  const float* in2, float* out, const revffn_moe_grads* grads, const int32_t* idx_in,
-                 int32_t* idx_out, void* ws, size_t ws_bytes, void* cuda_stream, const UpdateSpec* sgd = nullptr) {
+                 int32_t* idx_out, void* ws, size_t ws_bytes, void* cuda_stream, const UpdateSpec* sgd = nullptr,
+                 int* status = nullptr) {
   CKR(validate_desc(desc));
   CKR(validate_weights(*desc, w));
   if (!ws) return REVFFN_ERR_NULL;
@@ -1027,8 +1063,8 @@ static int entry(Pass pass, const revffn_moe_desc* desc, const revffn_moe_weight
   CKR(check_device());
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   if (desc->weight_dtype == REVFFN_BF16)
-    return dispatch<bf16>(pass, *desc, *w, L, ws, st, y1, in2, out, grads, sgd, idx_in, idx_out);
-  return dispatch<float>(pass, *desc, *w, L, ws, st, y1, in2, out, grads, sgd, idx_in, idx_out);
+    return dispatch<bf16>(pass, *desc, *w, L, ws, st, y1, in2, out, grads, sgd, idx_in, idx_out, status);
+  return dispatch<float>(pass, *desc, *w, L, ws, st, y1, in2, out, grads, sgd, idx_in, idx_out, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -1560,7 +1596,7 @@ int revffn_dbg_check_guards(const revffn_moe_desc* desc, void* ws, size_t ws_byt
   WsLayout L = plan_workspace(*desc);
   if (ws_bytes < L.fwd_bytes) return REVFFN_ERR_WORKSPACE;
   return guards_check(L, ws_bytes < L.bwd_bytes ? L.fwd_bytes : L.bwd_bytes, reinterpret_cast<char*>(ws),
-                      reinterpret_cast<cudaStream_t>(cuda_stream));
+                      reinterpret_cast<cudaStream_t>(cuda_stream), reinterpret_cast<int*>(reinterpret_cast<char*>(ws) + L.status.off));
 }
 
 int revffn_prof_enable(int on) {
