@@ -94,6 +94,8 @@ typedef struct {
   /* tests: 1 = load MN-major operands as 64 x 64 boxes of 2-D tensor maps, the form the library falls back to when a
    * leading dimension or column offset is not a multiple of 64 (0 = 3-D maps, 128 columns per load, where possible) */
   int32_t mn_boxes;
+  /* tests: columns per tile, 256, 128 or 64 (128 or 64 of each matrix of an N-concatenated pair); 0 = as planned */
+  int32_t tile_n;
 } revffn_dbg_gemm_args;
 int revffn_dbg_gemm(const revffn_dbg_gemm_args* args, int32_t* status_word_dev, void* cuda_stream);
 

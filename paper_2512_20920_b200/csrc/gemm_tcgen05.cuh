@@ -22,7 +22,8 @@
 //               16-byte stores, four 128-byte rows per instruction.  Global writes are whole
 //               lines whatever the row stride.
 // Tile = 128 rows x 256 columns (the last column tile of a row may be 128 wide: N only has
-// to be a multiple of 128), K step 64 (one 128-byte swizzle atom of bf16).
+// to be a multiple of 128), K step 64 (one 128-byte swizzle atom of bf16).  Products that would leave SMs idle with
+// it take tiles of 128 or 64 columns, as tc_plan() reckons.
 // Both operands may be K-major or MN-major; MN-major tiles are fetched 128 columns x 64 K rows at a time through a
 // 3-D view of the matrix (64 x 64 boxes of a 2-D map as the fallback) and described to the tensor core with
 // leading/stride offsets.
@@ -80,7 +81,8 @@ template <int MMA_N, int EPI, bool PAIR> struct TcCfg {
 struct TcParams {
   GemmProblem p;
   int tiles_m, tiles_n;      // GROUP_M: tiles_m is an upper bound, the device value comes from rows_total
-  int tile_n;                // logical output columns per tile
+  int tile_n;                // logical output columns per tile (of each matrix of an N-concatenated pair)
+  int b_box;                 // rows (K-major) or columns (MN-major, 3-D maps) of B that one load brings: 128 or 64
   int k_blocks;              // dense / GROUP_M
   int tr;                    // transposed pair mode: weights on the MMA M side, an expert's token rows on the N side
   int tiles_f;               // tr: 256-wide feature tiles per token chunk
@@ -166,14 +168,15 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
 // matrix {64 columns, K rows, ld / 64 column groups} with a box of two groups; else two 2-D loads of 64 x 64.
 // A tensor load costs its issuing thread a couple of hundred clocks whatever its size, so halving their number
 // matters as much as spreading them over two threads.
-__device__ __forceinline__ void tma_load_mn128(bool mn3d, uint32_t dst, const CUtensorMap* map, int col, int krow, uint32_t bar) {
+__device__ __forceinline__ void tma_load_mn128(bool mn3d, uint32_t dst, const CUtensorMap* map, int col, int krow, uint32_t bar,
+                                               bool second_block = true) {
   if (mn3d) {
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(krow), "r"(col >> 6), "r"(bar) : "memory");
   } else {
     tma_load_2d(dst, map, col, krow, bar);
-    tma_load_2d(dst + 8192, map, col + 64, krow, bar);
+    if (second_block) tma_load_2d(dst + 8192, map, col + 64, krow, bar);
   }
 }
 __device__ __forceinline__ void tma_load_mn128_pair(bool mn3d, uint32_t dst, const CUtensorMap* map, int col, int krow,
@@ -563,8 +566,8 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
             }
             const int nhalf = t.ncols / 2;       // this CTA's share of the tile's columns: 128, or 64 in a ragged last tile
             if (la) {
-              // (a 3-D load of an MN-major B always brings 128 columns, also where this CTA's share is 64)
-              const int b_cols = (p.b_mn_major && P.mn3d) ? 128 : nhalf;
+              // (a 3-D load of an MN-major B brings its whole box, also where this CTA's share of a ragged tile is less)
+              const int b_cols = (p.b_mn_major && P.mn3d) ? P.b_box : nhalf;
               if (crank == 0) mbar_expect_tx(full_bar(stage), 2 * (TC_A_BYTES + b_cols * TC_BK * 2));
               if (!p.a_mn_major) {
                 tma_load_2d_pair(sa, &map_a, kb * TC_BK, t.m0, fbc);
@@ -576,16 +579,16 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
               const bool second = p.concat == CONCAT_K && kb >= k_half;
               const int kbp = second ? kb - k_half : kb;
               if (!p.b_mn_major) {
-                // this CTA's 128 of the 256 accumulator columns: gate rows (rank 0) or up rows (rank 1) of a
-                // SwiGLU pair, else rows n0 + 128 rank .. + 127 of B
+                // this CTA's half of the accumulator columns: gate rows (rank 0) or up rows (rank 1) of a
+                // SwiGLU pair, else rows n0 + nhalf rank .. of B
                 // (the tensor map is named directly in each call: a map chosen through a pointer is slow to issue)
                 if (p.concat == CONCAT_N) {
                   if (crank == 0) tma_load_2d_pair(sb, &map_b0, kbp * TC_BK, t.n0, fbc);
                   else tma_load_2d_pair(sb, &map_b1, kbp * TC_BK, t.n0, fbc);
                 } else if (second) {
-                  tma_load_2d_pair(sb, &map_b1, kbp * TC_BK, t.n0 + 128 * crank, fbc);
+                  tma_load_2d_pair(sb, &map_b1, kbp * TC_BK, t.n0 + nhalf * crank, fbc);
                 } else {
-                  tma_load_2d_pair(sb, &map_b0, kbp * TC_BK, t.n0 + 128 * crank, fbc);
+                  tma_load_2d_pair(sb, &map_b0, kbp * TC_BK, t.n0 + nhalf * crank, fbc);
                 }
               } else {
                 const int krow = t.krow0 + kbp * TC_BK;
@@ -637,7 +640,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
               int row0 = (p.group_mode == GROUP_M ? t.group * p.N : 0) + t.n0;
               if (p.concat == CONCAT_N) {
                 tma_load_2d(sb, &map_b0, kb_b * P.bk, row0, fb);
-                tma_load_2d(sb + 16384, &map_b1, kb_b * P.bk, row0, fb);
+                tma_load_2d(sb + P.tile_n * 128, &map_b1, kb_b * P.bk, row0, fb);
               } else {
 #pragma unroll
                 for (int j = 0; j < MMA_N / 128; ++j) {
@@ -652,7 +655,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
               int krow = (p.group_mode == GROUP_M ? t.group * kdim : t.krow0) + kb_b * TC_BK;
               if (P.mn3d) {
                 if (second) tma_load_mn128(true, sb, &map_b1, p.b_col0 + t.n0, krow, fb);
-                else tma_load_mn128(true, sb, &map_b0, p.b_col0 + t.n0, krow, fb);
+                else tma_load_mn128(true, sb, &map_b0, p.b_col0 + t.n0, krow, fb);      // 64 columns with the narrow box
                 if (!b_mn_split && t.ncols > 128) {
                   if (second) tma_load_mn128(true, sb + 16384, &map_b1, p.b_col0 + t.n0 + 128, krow, fb);
                   else tma_load_mn128(true, sb + 16384, &map_b0, p.b_col0 + t.n0 + 128, krow, fb);
@@ -1070,7 +1073,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           __syncwarp();
         }
       } else if constexpr (EPI == EPI_SWIGLU) {
-        // columns [0, MMA_N/2) hold the gate projection, [MMA_N/2, MMA_N) the up projection.
+        // columns [0, tile_n) hold the gate projection, [tile_n, 2 tile_n) the up projection.
         // H (times the row's scale, when one is given: the routed experts' gate weight) goes out through two
         // alternating 2 KB staging buffers and TMA stores; when the a|b copy is wanted too, a|b and H take turns
         // in the staging area.  (Plain line-wide stores for the a|b copy measured 0.01 ms slower per launch.)
@@ -1078,11 +1081,11 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
         float g[32];
         const float rs = (p.rowscale && m_ok) ? p.rowscale[m] : 1.f;
 #pragma unroll 1
-        for (int c = half * 32; c < MMA_N / 2; c += 64) {
+        for (int c = half * 32; c < P.tile_n; c += 64) {
           const int n = t.n0 + c;
           if (!slab_ok) continue;      // warp-uniform
           tmem_ld32(taddr + c, r0);
-          tmem_ld32(taddr + MMA_N / 2 + c, r1);
+          tmem_ld32(taddr + P.tile_n + c, r1);
           tmem_ld_wait();
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
@@ -1319,10 +1322,10 @@ inline int tc_make_map(CUtensorMap* map, const void* ptr, uint64_t inner, uint64
 
 // Tensor map of an MN-major bf16 operand ([rows, ld] in memory, rows = K) seen as {64 columns, rows, ld / 64
 // column groups}: a box of 64 x 64 x 2 is 128 columns of 64 K rows, delivered as two 8 KB blocks of 64 columns.
-inline int tc_make_map_mn3d(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t ld) {
+inline int tc_make_map_mn3d(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t ld, int box_cols = 128) {
   cuuint64_t dims[3] = {64, rows, ld / 64};
   cuuint64_t strides[2] = {ld * 2u, 128u};
-  cuuint32_t box[3] = {64, 64, 2};
+  cuuint32_t box[3] = {64, 64, (cuuint32_t)box_cols / 64};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = tc_state().encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -1357,6 +1360,63 @@ inline int tc_launch(const TcParams& P, const CUtensorMap& ma, const CUtensorMap
   return e == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 
+// How a product is cut: CTA pairs or single CTAs, columns per tile, and whether it runs transposed.
+struct TcPlan { bool tr, pair; int tile_n; };
+
+// Pair mode is open wherever a 256-row tile cannot straddle two experts, transposed pair mode to expert-grouped plain
+// stores.  (With 256 columns a ragged 128-wide last tile splits into 64-column halves, which only the [K, N] storage
+// of B can load.)  A product whose wide tiles do not fill the GPU once is latency: it takes the narrower tile with the
+// shortest reckoned time (main loop plus fill and epilogue), if that is a fifth shorter.  The constants are clocks measured
+// on the kernel: a K step is bound by its tensor work (2 clk per column; the pair's instructions add about 90) or by the
+// bytes it brings into an SM (about 68 B/clk); an epilogue takes about 10 clk per column of bf16 and 22 of fp32; the
+// first loads and the start take 2500.  Four d = 512 blocks, 384 tokens: 1990 -> PLAN1 us a step; forward of 64 tokens
+// 304 -> 291.  Products that fill the GPU keep wide tiles even where the last round is thin: narrow ones move more
+// bytes per flop, and another stream's kernels use the SMs that are left over (chosen by time alone, a step at 2741
+// tokens went from 2547 to 2689 us, at 512 from 1504 to 1574).
+inline TcPlan tc_plan(const GemmProblem& p, int n_sms) {
+  TcPlan wide;
+  wide.tr = p.group_mode == GROUP_M && p.tok_chunks != nullptr && p.N % 256 == 0 && !p.a_mn_major && p.concat != CONCAT_N &&
+            !p.no_pair && n_sms % 2 == 0 && (p.epilogue == EPI_ROWSCALE || (p.epilogue == EPI_STORE && !p.out_f32));
+  wide.pair = wide.tr || (p.group_mode != GROUP_M && (p.N % 256 == 0 || p.b_mn_major) && !p.no_pair);
+  const bool cat = p.concat == CONCAT_N;
+  wide.tile_n = cat ? 128 : 256;
+  if (p.dbg_tile_n) {
+    wide.tile_n = p.dbg_tile_n;
+    wide.pair = p.group_mode != GROUP_M && !p.no_pair && (cat || (p.dbg_tile_n == 256 ? wide.pair : p.dbg_tile_n >= 128));
+    return wide;
+  }
+  if (wide.tr || p.fp8) return wide;
+  const bool pair_open = p.group_mode != GROUP_M && !p.no_pair && n_sms % 2 == 0;
+  const int64_t groups = p.group_mode == GROUP_K ? (p.n_groups > 0 ? p.n_groups : 1) : 1;
+  int64_t k_steps = ceil_div(p.K, TC_BK);
+  int64_t m_tiles = ceil_div(p.M, TC_BM);
+  if (p.group_mode == GROUP_K) k_steps = std::max<int64_t>(1, k_steps / groups);
+  // padded row space: about half a tile of padding per expert
+  if (p.group_mode == GROUP_M && p.n_groups > 0) m_tiles = std::max<int64_t>(1, (p.M - 127 * (int64_t)p.n_groups) / TC_BM + p.n_groups / 2);
+  auto slots = [&](bool pair) -> int64_t { return pair ? n_sms / 2 : n_sms; };
+  auto tiles = [&](bool pair, int tile_n) { return (pair ? (m_tiles + 1) / 2 : m_tiles) * ceil_div(p.N, tile_n) * groups; };
+  if (tiles(wide.pair, wide.tile_n) > slots(wide.pair)) return wide;
+  const bool f32_out = p.epilogue == EPI_COUPLE || p.epilogue == EPI_WGRAD || p.out_f32;
+  const int epi_clk = p.epilogue == EPI_DSWIGLU ? 70 : (f32_out || cat ? 22 : 10);
+  auto clocks = [&](bool pair, int tile_n) {
+    const int64_t cols = cat ? 2 * tile_n : tile_n;         // accumulator columns
+    const int64_t rounds = ceil_div(tiles(pair, tile_n), slots(pair)), bytes = TC_A_BYTES + cols * (pair ? 64 : 128);
+    const int64_t step = std::max<int64_t>(2 * cols + (pair ? 90 : 0), bytes / 68), epi = epi_clk * cols;
+    return 2500 + rounds * std::max(k_steps * step, epi) + epi;
+  };
+  TcPlan best = wide;
+  int64_t best_clk = clocks(wide.pair, wide.tile_n) * 4 / 5;
+  // a head must not straddle tiles; the sums of <dH, H> are two per 256 columns; 64 columns of both matrices of a pair
+  const int narrowest = p.epilogue == EPI_HEADS ? 128 : (p.epilogue == EPI_DSWIGLU ? (p.dg_part ? 256 : 128) : 64);
+  for (int tile_n = wide.tile_n / 2; tile_n >= narrowest; tile_n /= 2)
+    for (int pair = 1; pair >= 0; --pair) {
+      if (pair && (!pair_open || (cat ? 2 * tile_n : tile_n) < 128)) continue;
+      const int64_t clk = clocks(pair != 0, tile_n);
+      if (clk < best_clk) { best_clk = clk; best.pair = pair != 0; best.tile_n = tile_n; }
+    }
+  return best;
+}
+
 inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   TcState& s = tc_state();
   if (!s.ready) return REVFFN_ERR_CUDA;
@@ -1364,7 +1424,11 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   const int mma_n = 256;
   TcParams P;
   P.p = p;
-  P.tile_n = (p.concat == CONCAT_N) ? mma_n / 2 : mma_n;
+  const TcPlan plan = tc_plan(p, s.n_sms);
+  const bool tr = plan.tr, pair = plan.pair;
+  P.tile_n = plan.tile_n;
+  // what one load of B brings: this CTA's share of a tile's columns, at most 128 of them
+  P.b_box = std::min(128, pair && p.concat != CONCAT_N ? P.tile_n / 2 : P.tile_n);
   P.tiles_m = (int)ceil_div(p.M, TC_BM);
   P.tiles_n = (int)ceil_div(p.N, P.tile_n);
   const bool f8 = p.fp8 != 0;
@@ -1414,16 +1478,16 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
     // B
     if (!p.b_mn_major) {
       uint64_t rows = (p.group_mode == GROUP_M) ? (uint64_t)groups * p.N : (uint64_t)p.N;
-      int r = tc_make_map(&mb0, p.B0, (uint64_t)k_half, rows, (uint64_t)p.ldb, f8 ? 128 : 64, 128, f8);
+      int r = tc_make_map(&mb0, p.B0, (uint64_t)k_half, rows, (uint64_t)p.ldb, f8 ? 128 : 64, tr ? 128 : P.b_box, f8);
       if (r) return r;
-      r = tc_make_map(&mb1, p.B1 ? p.B1 : p.B0, (uint64_t)k_half, rows, (uint64_t)p.ldb, f8 ? 128 : 64, 128, f8);
+      r = tc_make_map(&mb1, p.B1 ? p.B1 : p.B0, (uint64_t)k_half, rows, (uint64_t)p.ldb, f8 ? 128 : 64, tr ? 128 : P.b_box, f8);
       if (r) return r;
     } else {
       uint64_t rows = (p.group_mode == GROUP_M) ? (uint64_t)groups * k_half : (uint64_t)p.K;
-      int r = mn3d ? tc_make_map_mn3d(&mb0, p.B0, rows, (uint64_t)p.ldb)
+      int r = mn3d ? tc_make_map_mn3d(&mb0, p.B0, rows, (uint64_t)p.ldb, tr ? 128 : P.b_box)
                    : tc_make_map(&mb0, p.B0, (uint64_t)p.ldb, rows, (uint64_t)p.ldb, 64, 64);
       if (r) return r;
-      r = mn3d ? tc_make_map_mn3d(&mb1, p.B1 ? p.B1 : p.B0, rows, (uint64_t)p.ldb)
+      r = mn3d ? tc_make_map_mn3d(&mb1, p.B1 ? p.B1 : p.B0, rows, (uint64_t)p.ldb, tr ? 128 : P.b_box)
                : tc_make_map(&mb1, p.B1 ? p.B1 : p.B0, (uint64_t)p.ldb, rows, (uint64_t)p.ldb, 64, 64);
       if (r) return r;
     }
@@ -1483,12 +1547,6 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
       if (r) return r;
     }
   }
-  // Pair mode wherever a 256-row tile cannot straddle two experts and every column tile is 256 wide.
-  // (a ragged 128-wide last tile splits into 64-column halves, which only the [K, N] storage of B can load)
-  const bool tr = p.group_mode == GROUP_M && p.tok_chunks != nullptr && p.N % 256 == 0 && !p.a_mn_major &&
-                  p.concat != CONCAT_N && !p.no_pair && s.n_sms % 2 == 0 &&
-                  (p.epilogue == EPI_ROWSCALE || (p.epilogue == EPI_STORE && !p.out_f32));
-  const bool pair = tr || (p.group_mode != GROUP_M && (p.N % 256 == 0 || p.b_mn_major) && !p.no_pair);
   if (f8 && p.epilogue == EPI_STORE && !tr) return REVFFN_ERR_UNSUPPORTED;      // only the transposed store scales its accumulator
   P.tr = tr ? 1 : 0;
   P.tiles_f = p.N / 256;
