@@ -103,6 +103,13 @@ inline cudaError_t launch_k(void (*kernel)(Params...), dim3 grid, dim3 block, si
   return launch_cluster(kernel, grid, dim3(1, 1, 1), block, smem, st, args...);
 }
 
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool ok) {      // !ok: 16 zero bytes
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+               ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 // 8 elements of T as one vector: loads/stores of 16 bytes for bf16, 2x16 for float.
 // Blocks of `kernel` that are resident on the current device at once (one wave) for this block size and dynamic
 // shared memory: the grid size of the grid-stride kernels.

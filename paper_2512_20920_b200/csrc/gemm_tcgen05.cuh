@@ -68,8 +68,10 @@ constexpr long long TC_WAIT_CYCLES = 4000000000LL;       // ~2 s: bound on any s
 template <int MMA_N, int EPI, bool PAIR> struct TcCfg {
   static constexpr int B_BYTES = (PAIR ? MMA_N / 2 : MMA_N) * TC_BK * 2;
   static constexpr int STAGE_BYTES = TC_A_BYTES + B_BYTES;
-  static constexpr int STAGES = PAIR ? 6 : 4;
-  static constexpr int EPI_WARP_BYTES = 4096;           // staging per epilogue warp: two 32 x 32 bf16 blocks or one fp32 block
+  // The Adam update is bound by what its epilogue reads and writes: it trades half of the operand ring for a ring of
+  // weights and moments in flight (two units of 6 KB per epilogue warp).
+  static constexpr int STAGES = EPI == EPI_WADAM ? (PAIR ? 3 : 2) : (PAIR ? 6 : 4);
+  static constexpr int EPI_WARP_BYTES = EPI == EPI_WADAM ? 16384 : 4096;   // staging per epilogue warp: two 32 x 32 bf16 blocks or one fp32 block
   static constexpr int TMEM_COLS = 2 * MMA_N;           // two accumulators; a power of two >= 32
   // stage ring | epilogue staging | barriers; the ring starts 1024-byte aligned and
   // every stage is a multiple of 1024 bytes, so the staging area is aligned too
@@ -394,6 +396,25 @@ __device__ __forceinline__ float2 sigmoid_approx2(float2 x) {
   return make_float2(r0, r1);
 }
 
+// Where an epilogue warp's 32-row slab of an fp32 result (or of the weights a fused update rewrites) lies.
+struct SlabOut {
+  float* c; bf16* w; float *m, *mom, *var;      // output; updated weight, master copy and moments
+  int64_t at0, ld4, res0;      // this lane's element of row (lane / 8), column piece (lane % 8); four rows; residual element
+  int rows;                    // rows that exist (<= 32)
+};
+__device__ __forceinline__ float4 as_f4(const uint4& u) {
+  return make_float4(__uint_as_float(u.x), __uint_as_float(u.y), __uint_as_float(u.z), __uint_as_float(u.w));
+}
+__device__ __forceinline__ float4 bf4(const uint2& u) {
+  const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+  const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+  return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+__device__ __forceinline__ uint2 pack4(const float4& v) {
+  __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+  return make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+}
+
 // Tile coordinates shared by the three roles.
 struct TcTile {
   int m0, n0, group, k_blocks, krow0;
@@ -461,6 +482,8 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
                const __grid_constant__ CUtensorMap map_b0, const __grid_constant__ CUtensorMap map_b1,
                const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_c1) {
   using Cfg = TcCfg<MMA_N, EPI, PAIR>;
+  constexpr bool RMW = EPI == EPI_COUPLE || EPI == EPI_WRMW;
+  constexpr bool WGRAD = EPI == EPI_WGRAD || EPI == EPI_WADAM || EPI == EPI_WRMW;
   extern __shared__ uint8_t smem_raw[];
   const GemmProblem& p = P.p;
   const uint32_t raw = smem_u32(smem_raw);
@@ -771,11 +794,78 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           blk_load_dist(ds_blk + p.N + half * 32, p.ld_ab, rows_ok, lane, ds_b);
         }
       }
+      // row coordinate of the slab in the output tensor map (rows past its extent are clipped by the store)
+      const int y0 = (p.group_mode == GROUP_K ? t.group * p.M : 0) + t.m0 + q * 32;
+      SlabOut out;
+      uint4 ld_a[8], ld_b[8];     // read-modify-write forms: a block's pieces, four floats or (in .x, .y) four bf16 weights
+      if constexpr (EPI == EPI_COUPLE || WGRAD || EPI == EPI_STORE) {
+        // where this warp's slab of an fp32 result goes
+        int64_t yb = y0;
+        const int64_t y_lim = (p.group_mode == GROUP_K) ? (int64_t)(t.group + 1) * p.M : (p.group_mode == GROUP_M ? (int64_t)m_lim : (int64_t)p.M);
+        out.rows = (int)min((int64_t)32, y_lim - yb);
+        out.c = reinterpret_cast<float*>(p.C);
+        out.w = reinterpret_cast<bf16*>(p.upd_w);
+        out.m = p.upd_m; out.mom = p.upd_mom; out.var = p.upd_var;
+        if (WGRAD && p.split_m > 0) {
+          // two outputs: the slab lies wholly in the first or in the second (split_m is a multiple of 128)
+          int local = t.m0 + q * 32;
+          if (local >= p.split_m) {
+            local -= p.split_m;
+            out.c = reinterpret_cast<float*>(p.C2); out.w = reinterpret_cast<bf16*>(p.upd_w2); out.m = p.upd_m2;
+            out.mom = p.upd_mom2; out.var = p.upd_var2;
+          }
+          yb = (int64_t)t.group * p.split_m + local;
+          out.rows = min(32, p.split_m - local);
+        }
+        out.at0 = (yb + (lane >> 3)) * p.ldc + t.n0 + (lane & 7) * 4;
+        out.ld4 = 4 * p.ldc;
+        out.res0 = EPI == EPI_COUPLE ? (yb + (lane >> 3)) * p.ld_resid + t.n0 + (lane & 7) * 4 : 0;
+      }
+      auto rmw_request = [&](const SlabOut& o, int c, uint4 (&ld)[8]) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          if (i * 4 + (lane >> 3) >= o.rows) continue;
+          const int64_t at = o.at0 + c + i * o.ld4;
+          if (EPI == EPI_COUPLE) ld[i] = *reinterpret_cast<const uint4*>(p.resid + o.res0 + c + i * 4 * p.ld_resid);
+          else if (!o.w) ld[i] = *reinterpret_cast<const uint4*>(o.c + at);
+          else if (o.m) ld[i] = *reinterpret_cast<const uint4*>(o.m + at);
+          else { const uint2 w2 = *reinterpret_cast<const uint2*>(o.w + at); ld[i].x = w2.x; ld[i].y = w2.y; }
+        }
+      };
+      // Adam: unit u of the tile (16 rows of block u / 2) into its half of the ring; always commits a group
+      auto adam_request = [&](const SlabOut& o, int u, int ncols) {
+        const int c = half * 32 + (u >> 1) * 64, r0u = (u & 1) * 16;
+        if (c < ncols) {
+          uint8_t* unit = stg + 4096 + (u & 1) * 6144;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int r = 4 * i + (lane >> 3);
+            const bool in = r0u + r < o.rows;
+            const int64_t at = in ? o.at0 + c + ((r0u >> 2) + i) * o.ld4 : 0;
+            if (o.m) cp_async16(unit + r * 128 + (lane & 7) * 16, o.m + at, in);
+            cp_async16(unit + 2048 + r * 128 + (lane & 7) * 16, o.mom + at, in);
+            cp_async16(unit + 4096 + r * 128 + (lane & 7) * 16, o.var + at, in);
+          }
+          if (!o.m) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {      // 16 rows of 64 bytes: eight rows per instruction, four pieces each
+              const int r = 8 * i + (lane >> 2);
+              const bool in = r0u + r < o.rows;
+              const int64_t at = in ? o.at0 - (int64_t)(lane >> 3) * p.ldc - (lane & 7) * 4 + (int64_t)(r0u + r) * p.ldc + c + (lane & 3) * 8 : 0;
+              cp_async16(unit + r * 64 + (lane & 3) * 16, o.w + at, in);
+            }
+          }
+        }
+        cp_async_commit();
+      };
+      if constexpr (EPI == EPI_WADAM) {
+        if (slab_ok) { adam_request(out, 0, t.ncols); adam_request(out, 1, t.ncols); }
+      } else if constexpr (RMW) {
+        if (slab_ok && half * 32 < t.ncols) rmw_request(out, half * 32, ld_a);
+      }
       if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * MMA_N);
-      // row coordinate of the slab in the output tensor map (rows past its extent are clipped by the store)
-      const int y0 = (p.group_mode == GROUP_K ? t.group * p.M : 0) + t.m0 + q * 32;
       const bool have_acc = t.k_blocks > 0;      // an empty K range leaves the accumulator undefined: use zeros
       uint32_t r0[32];
       float f[32];
@@ -833,184 +923,144 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
             ++n_grp;
           }
         }
-      } else if constexpr (EPI == EPI_STORE || EPI == EPI_ROWSCALE || EPI == EPI_COUPLE || EPI == EPI_WGRAD) {
+      } else if constexpr (EPI == EPI_STORE || EPI == EPI_ROWSCALE || EPI == EPI_COUPLE || WGRAD) {
         float rs = 1.f;
         if (EPI == EPI_ROWSCALE && m_ok) rs = p.rowscale[m];
-        const bool f32_out = (EPI == EPI_COUPLE) || (EPI == EPI_WGRAD) || (EPI == EPI_STORE && p.out_f32);
-        // where this warp's slab of an fp32 result goes
-        const int piece = lane & 7;
-        int64_t y_lim, yb;                                 // row limit and first output row of this warp's slab
-        float* cptr;
-        bf16* wptr;
-        float *mptr, *momptr, *varptr;
-        auto slab_target = [&](const TcTile& tt, int64_t y0_tt) {
-          y_lim = (p.group_mode == GROUP_K) ? (int64_t)(tt.group + 1) * p.M
-                                            : (p.group_mode == GROUP_M ? (int64_t)m_lim : (int64_t)p.M);
-          yb = y0_tt;
-          cptr = reinterpret_cast<float*>(p.C);
-          wptr = reinterpret_cast<bf16*>(p.upd_w);
-          mptr = p.upd_m; momptr = p.upd_mom; varptr = p.upd_var;
-          if (EPI == EPI_WGRAD && p.split_m > 0) {
-            // two outputs: the slab lies wholly in the first or in the second (split_m is a multiple of 128)
-            int local = tt.m0 + q * 32;
-            if (local >= p.split_m) {
-              local -= p.split_m;
-              cptr = reinterpret_cast<float*>(p.C2); wptr = reinterpret_cast<bf16*>(p.upd_w2); mptr = p.upd_m2;
-              momptr = p.upd_mom2; varptr = p.upd_var2;
-            }
-            yb = (int64_t)tt.group * p.split_m + local;
-            y_lim = (int64_t)(tt.group + 1) * p.split_m;
-          }
-        };
-        slab_target(t, y0);
-        // Read-modify-write forms of the weight-gradient epilogue (fused update, accumulation): what the eight
-        // pieces of a block need is requested before the block's accumulator is fetched and staged, and used
-        // after.  Taken piece by piece, each piece's loads waited behind the previous piece's stores (the compiler
-        // cannot tell that they do not overlap) and a 32 x 32 block cost eight memory round trips: the fused SGD
-        // pass measured 2.4 ms slower than writing the gradients.  (Asking the next tile's lines into the L2 a
-        // tile ahead, prefetch.global.L2 per row, changed nothing measurable on top of this.)
-        // The coupling's residual rows come the same way (one row per lane, 16 bytes at a time, they cost a line per
-        // lane and load: 384 x 256 outputs over K = 512 took 16 us, a plain store of the same product 9 us).
-        const bool rmw = EPI == EPI_COUPLE || (EPI == EPI_WGRAD && (wptr != nullptr || p.accumulate));
-        auto as_f4 = [](const uint4& u) {
-          return make_float4(__uint_as_float(u.x), __uint_as_float(u.y), __uint_as_float(u.z), __uint_as_float(u.w));
-        };
-        auto bf_f4 = [](const uint4& u) {
-          const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
-          const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
-          return make_float4(lo.x, lo.y, hi.x, hi.y);
-        };
-#pragma unroll 1
-        for (int c = half * 32; c < t.ncols; c += 64) {
-          const int n = t.n0 + c;
-          if (!slab_ok) continue;      // warp-uniform
-          const int64_t col = n + piece * 4;
-          uint4 ld[8];          // four floats (stored gradient or master copy), or four bf16 weights in .x, .y
-          if (rmw) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int r = i * 4 + (lane >> 3);
-              const int64_t at = (yb + r) * p.ldc + col;
-              if (yb + r < y_lim) {
-                if (EPI == EPI_COUPLE) ld[i] = *reinterpret_cast<const uint4*>(p.resid + (yb + r) * p.ld_resid + col);
-                else if (!wptr) ld[i] = *reinterpret_cast<const uint4*>(cptr + at);
-                else if (mptr) ld[i] = *reinterpret_cast<const uint4*>(mptr + at);
-                else { const uint2 w2 = *reinterpret_cast<const uint2*>(wptr + at); ld[i].x = w2.x; ld[i].y = w2.y; }
-              }
-            }
-          }
-          if (have_acc) { tmem_ld32(taddr + c, r0); tmem_ld_wait(); }
-#pragma unroll
-          for (int i = 0; i < 32; ++i) f[i] = have_acc ? __uint_as_float(r0[i]) : 0.f;
-          if constexpr (EPI == EPI_ROWSCALE) {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) f[i] *= rs;
-          }
+        const bool f32_out = (EPI == EPI_COUPLE) || WGRAD || (EPI == EPI_STORE && p.out_f32);
+        if (!f32_out) {
           // bf16 blocks (32 x 32, 2 KB) leave through two alternating staging buffers and TMA stores.
+          if constexpr (EPI == EPI_STORE || EPI == EPI_ROWSCALE) {
+#pragma unroll 1
+            for (int c = half * 32; c < t.ncols; c += 64) {
+              if (!slab_ok) continue;      // warp-uniform
+              if (have_acc) { tmem_ld32(taddr + c, r0); tmem_ld_wait(); }
+#pragma unroll
+              for (int i = 0; i < 32; ++i) f[i] = have_acc ? __uint_as_float(r0[i]) : 0.f;
+              if constexpr (EPI == EPI_ROWSCALE) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) f[i] *= rs;
+              }
+              const uint32_t off = (n_grp & 1u) * 2048u;
+              if (lane == 0) bulk_wait_read<1>();
+              __syncwarp();
+              stage32_bf16(stg + off, lane, f);
+              fence_async_smem();
+              __syncwarp();
+              if (lane == 0) {
+                tma_store_2d(&map_c, stg_u32 + off, t.n0 + c, y0);
+                bulk_commit();
+              }
+              ++n_grp;
+            }
+          }
+        } else if (slab_ok) {
           // fp32 blocks (32 x 32, 4 KB) are transposed through the staging area and written with plain
           // 16-byte stores, 4 rows x 128 bytes per instruction: whole lines, and nothing to wait for
           // before the area is reused.  (A TMA store of such a block sat behind the producer's operand
           // loads in the copy engine; with the short K of a weight gradient that wait set the pace.)
-          if (f32_out) {
-            if (lane == 0) bulk_wait_read<0>();     // no bulk store of this warp reads the area any more
+          // A block's accumulator is fetched while the block before it is written: F32NUMS
+          const int rsub = lane >> 3;
+          const bool all_rows = out.rows >= 32;
+          auto fetch = [&](int c) { if (have_acc && c < t.ncols) tmem_ld32(taddr + c, r0); };
+          auto stage = [&]() {
+            tmem_ld_wait();
+            uint8_t* row = stg + lane * 128;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              *reinterpret_cast<uint4*>(row + ((j ^ (lane & 7)) << 4)) =
+                  have_acc ? make_uint4(r0[4 * j], r0[4 * j + 1], r0[4 * j + 2], r0[4 * j + 3]) : make_uint4(0u, 0u, 0u, 0u);
             __syncwarp();
-            {
-              uint8_t* row = stg + lane * 128;
+          };
+          auto staged = [&](int i) -> float4 {           // this lane's piece of row 4 i + rsub
+            const int r = i * 4 + rsub;
+            return *reinterpret_cast<const float4*>(stg + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
+          };
+          auto row_ok = [&](int i) -> bool { return all_rows || i * 4 + rsub < out.rows; };
+          fetch(half * 32);
+          if constexpr (EPI == EPI_WADAM) {
+            // Adam: weight (or master copy) and the two moments of a unit of 16 rows x 32 columns come by cp.async into
+            // a ring of two units; a lane asks for exactly the pieces it will use, so nothing but its own copies
+            // has to have landed.
+            int u = 0;
+#pragma unroll 1
+            for (int c = half * 32; c < t.ncols; c += 64) {
+              stage();
+              fetch(c + 64);
+#pragma unroll 1
+              for (int h2 = 0; h2 < 2; ++h2, ++u) {
+                cp_async_wait<1>();
+                if (!out.m) __syncwarp();      // bf16 weights: a 16-byte piece serves two lanes
+                const uint8_t* unit = stg + 4096 + (u & 1) * 6144;
+                float4 w4[4], mo[4], va[4];
 #pragma unroll
-              for (int j = 0; j < 8; ++j)
-                *reinterpret_cast<float4*>(row + ((j ^ (lane & 7)) << 4)) =
-                    make_float4(f[4 * j], f[4 * j + 1], f[4 * j + 2], f[4 * j + 3]);
-            }
-            __syncwarp();
-            if (rmw) {
-              if (wptr && p.upd.kind != 0) {
-                // Adam: the element's two moments live beside the weight (fp32, same layout), 16 bytes each per lane;
-                // two passes of four pieces keep the registers in bounds
-#pragma unroll
-                for (int h4 = 0; h4 < 8; h4 += 4) {
-                  float4 mo[4], va[4];
-#pragma unroll
-                  for (int i = 0; i < 4; ++i) {
-                    const int r = (h4 + i) * 4 + (lane >> 3);
-                    const int64_t at = (yb + r) * p.ldc + col;
-                    if (yb + r < y_lim) {
-                      mo[i] = *reinterpret_cast<const float4*>(momptr + at);
-                      va[i] = *reinterpret_cast<const float4*>(varptr + at);
-                    }
-                  }
-#pragma unroll
-                  for (int i = 0; i < 4; ++i) {
-                    const int r = (h4 + i) * 4 + (lane >> 3);
-                    const int64_t at = (yb + r) * p.ldc + col;
-                    if (yb + r >= y_lim) continue;
-                    const float4 v = *reinterpret_cast<const float4*>(stg + r * 128 + ((piece ^ (r & 7)) << 4));
-                    float4 w4 = mptr ? as_f4(ld[h4 + i]) : bf_f4(ld[h4 + i]);
-                    w4.x = upd_step(p.upd, w4.x, v.x, &mo[i].x, &va[i].x);
-                    w4.y = upd_step(p.upd, w4.y, v.y, &mo[i].y, &va[i].y);
-                    w4.z = upd_step(p.upd, w4.z, v.z, &mo[i].z, &va[i].z);
-                    w4.w = upd_step(p.upd, w4.w, v.w, &mo[i].w, &va[i].w);
-                    *reinterpret_cast<float4*>(momptr + at) = mo[i];
-                    *reinterpret_cast<float4*>(varptr + at) = va[i];
-                    if (mptr) *reinterpret_cast<float4*>(mptr + at) = w4;
-                    uint2 out;
-                    __nv_bfloat162 h2 = __floats2bfloat162_rn(w4.x, w4.y);
-                    out.x = *reinterpret_cast<uint32_t*>(&h2);
-                    h2 = __floats2bfloat162_rn(w4.z, w4.w);
-                    out.y = *reinterpret_cast<uint32_t*>(&h2);
-                    *reinterpret_cast<uint2*>(wptr + at) = out;
-                  }
+                for (int i = 0; i < 4; ++i) {
+                  const int at = (4 * i + rsub) * 128 + (lane & 7) * 16;
+                  if (out.m) w4[i] = *reinterpret_cast<const float4*>(unit + at);
+                  else w4[i] = bf4(*reinterpret_cast<const uint2*>(unit + (4 * i + rsub) * 64 + (lane & 7) * 8));
+                  mo[i] = *reinterpret_cast<const float4*>(unit + 2048 + at);
+                  va[i] = *reinterpret_cast<const float4*>(unit + 4096 + at);
                 }
-              } else {
+                if (!out.m) __syncwarp();
+                adam_request(out, u + 2, t.ncols);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                  const int r = i * 4 + (lane >> 3);
-                  const int64_t at = (yb + r) * p.ldc + col;
-                  if (yb + r >= y_lim) continue;
-                  const float4 v = *reinterpret_cast<const float4*>(stg + r * 128 + ((piece ^ (r & 7)) << 4));
-                  if (EPI == EPI_COUPLE) {
-                    const float4 o = as_f4(ld[i]);
-                    *reinterpret_cast<float4*>(cptr + at) = make_float4(o.x + p.resid_sign * v.x, o.y + p.resid_sign * v.y,
-                                                                        o.z + p.resid_sign * v.z, o.w + p.resid_sign * v.w);
-                    continue;
-                  }
-                  if (!wptr) {          // accumulate into the stored gradient
-                    const float4 o = as_f4(ld[i]);
-                    *reinterpret_cast<float4*>(cptr + at) = make_float4(o.x + v.x, o.y + v.y, o.z + v.z, o.w + v.w);
-                    continue;
-                  }
-                  // fused SGD step on the weight tile this gradient tile belongs to; the gradient is not stored
-                  float4 w4 = mptr ? as_f4(ld[i]) : bf_f4(ld[i]);
-                  w4.x -= p.upd.lr * v.x; w4.y -= p.upd.lr * v.y; w4.z -= p.upd.lr * v.z; w4.w -= p.upd.lr * v.w;
-                  if (mptr) *reinterpret_cast<float4*>(mptr + at) = w4;
-                  uint2 out;
-                  __nv_bfloat162 h2 = __floats2bfloat162_rn(w4.x, w4.y);
-                  out.x = *reinterpret_cast<uint32_t*>(&h2);
-                  h2 = __floats2bfloat162_rn(w4.z, w4.w);
-                  out.y = *reinterpret_cast<uint32_t*>(&h2);
-                  *reinterpret_cast<uint2*>(wptr + at) = out;
+                for (int i = 0; i < 4; ++i) {
+                  if (!row_ok(4 * h2 + i)) continue;
+                  const float4 v = staged(4 * h2 + i);
+                  w4[i].x = upd_step(p.upd, w4[i].x, v.x, &mo[i].x, &va[i].x);
+                  w4[i].y = upd_step(p.upd, w4[i].y, v.y, &mo[i].y, &va[i].y);
+                  w4[i].z = upd_step(p.upd, w4[i].z, v.z, &mo[i].z, &va[i].z);
+                  w4[i].w = upd_step(p.upd, w4[i].w, v.w, &mo[i].w, &va[i].w);
+                  const int64_t at = out.at0 + c + (4 * h2 + i) * out.ld4;
+                  *reinterpret_cast<float4*>(out.mom + at) = mo[i];
+                  *reinterpret_cast<float4*>(out.var + at) = va[i];
+                  if (out.m) *reinterpret_cast<float4*>(out.m + at) = w4[i];
+                  *reinterpret_cast<uint2*>(out.w + at) = pack4(w4[i]);
                 }
               }
-            } else {
+              __syncwarp();
+            }
+          } else {
+            // Read-modify-write forms (coupling, accumulation, SGD step): what a block needs is requested a block
+            // ahead, the first one before the wait for the accumulator.
+            auto write = [&](int c, const uint4 (&ld)[8]) {
 #pragma unroll
               for (int i = 0; i < 8; ++i) {
-                const int r = i * 4 + (lane >> 3);
-                const float4 v = *reinterpret_cast<const float4*>(stg + r * 128 + ((piece ^ (r & 7)) << 4));
-                if (yb + r < y_lim) *reinterpret_cast<float4*>(cptr + (yb + r) * p.ldc + col) = v;
+                if (!row_ok(i)) continue;
+                float4 v = staged(i);
+                const int64_t at = out.at0 + c + i * out.ld4;
+                if (EPI == EPI_COUPLE) {
+                  const float4 o = as_f4(ld[i]);
+                  v = make_float4(o.x + p.resid_sign * v.x, o.y + p.resid_sign * v.y, o.z + p.resid_sign * v.z, o.w + p.resid_sign * v.w);
+                } else if (EPI == EPI_WRMW) {
+                  if (!out.w) {          // accumulate into the stored gradient
+                    const float4 o = as_f4(ld[i]);
+                    v = make_float4(o.x + v.x, o.y + v.y, o.z + v.z, o.w + v.w);
+                  } else {
+                    // fused SGD step on the weight tile this gradient tile belongs to; the gradient is not stored
+                    float4 w4 = out.m ? as_f4(ld[i]) : bf4(make_uint2(ld[i].x, ld[i].y));
+                    w4.x -= p.upd.lr * v.x; w4.y -= p.upd.lr * v.y; w4.z -= p.upd.lr * v.z; w4.w -= p.upd.lr * v.w;
+                    if (out.m) *reinterpret_cast<float4*>(out.m + at) = w4;
+                    *reinterpret_cast<uint2*>(out.w + at) = pack4(w4);
+                    continue;
+                  }
+                }
+                *reinterpret_cast<float4*>(out.c + at) = v;
               }
+            };
+#pragma unroll 1
+            for (int c = half * 32; c < t.ncols; c += 128) {
+              stage();
+              fetch(c + 64);
+              if (RMW && c + 64 < t.ncols) rmw_request(out, c + 64, ld_b);
+              write(c, ld_a);
+              __syncwarp();
+              if (c + 64 >= t.ncols) break;
+              stage();
+              fetch(c + 128);
+              if (RMW && c + 128 < t.ncols) rmw_request(out, c + 128, ld_a);
+              write(c + 64, ld_b);
+              __syncwarp();
             }
-            __syncwarp();
-          } else {
-            const uint32_t off = (n_grp & 1u) * 2048u;
-            if (lane == 0) bulk_wait_read<1>();
-            __syncwarp();
-            stage32_bf16(stg + off, lane, f);
-            fence_async_smem();
-            __syncwarp();
-            if (lane == 0) {
-              tma_store_2d(&map_c, stg_u32 + off, n, y0);
-              bulk_commit();
-            }
-            ++n_grp;
           }
         }
       } else if constexpr (EPI == EPI_HEADS) {
@@ -1200,6 +1250,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
     }
     // this lane's stores must be complete (shared memory read, global memory written) before the CTA exits
     if (lane == 0) bulk_wait_all();
+    if constexpr (EPI == EPI_WADAM) cp_async_wait<0>();
   }
 
   // ------------------------------------------------------------------ teardown
@@ -1300,6 +1351,8 @@ inline int tc_prepare() {
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_COUPLE>();
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_DSWIGLU>();
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_WGRAD>();
+  if (e == cudaSuccess) e = tc_set_attr<256, EPI_WADAM>();
+  if (e == cudaSuccess) e = tc_set_attr<256, EPI_WRMW>();
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_HEADS>();
   if (e != cudaSuccess) return REVFFN_ERR_CUDA;
   s.ready = true;
@@ -1566,9 +1619,11 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   if (grid <= 0) return REVFFN_OK;
 
 #define TC_CASE(N_, E_) \
-  if (mma_n == N_ && p.epilogue == E_) return tc_launch<N_, E_>(P, ma, mb0, mb1, mc, mc1, grid, pair, st);
+  if (mma_n == N_ && epi == E_) return tc_launch<N_, E_>(P, ma, mb0, mb1, mc, mc1, grid, pair, st);
+  const int epi = p.epilogue != EPI_WGRAD ? p.epilogue : (p.upd_w ? (p.upd.kind != 0 ? EPI_WADAM : EPI_WRMW) : (p.accumulate ? EPI_WRMW : EPI_WGRAD));
   TC_CASE(256, EPI_STORE) TC_CASE(256, EPI_SWIGLU) TC_CASE(256, EPI_ROWSCALE) TC_CASE(256, EPI_COUPLE)
-  TC_CASE(256, EPI_DSWIGLU) TC_CASE(256, EPI_WGRAD) TC_CASE(256, EPI_HEADS)
+  TC_CASE(256, EPI_DSWIGLU) TC_CASE(256, EPI_WGRAD) TC_CASE(256, EPI_WADAM) TC_CASE(256, EPI_WRMW)
+  TC_CASE(256, EPI_HEADS)
 #undef TC_CASE
   return REVFFN_ERR_UNSUPPORTED;
 }

@@ -347,13 +347,6 @@ __device__ __forceinline__ double ld_cluster_f64(const double* p, uint32_t rank)
   asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
   return v;
 }
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool ok) {      // !ok: 16 zero bytes
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
-               ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // D (8x8) += A (8x4, row-major fragment) * B (4x8, column-major fragment), fp64.
 // Lane l holds A[l/4][l%4], B[l%4][l/4] and D[l/4][2*(l%4) + {0,1}].
 __device__ __forceinline__ void dmma_8x8x4(double& d0, double& d1, double a, double b) {
