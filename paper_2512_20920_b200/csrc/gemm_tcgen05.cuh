@@ -68,10 +68,10 @@ constexpr long long TC_WAIT_CYCLES = 4000000000LL;       // ~2 s: bound on any s
 template <int MMA_N, int EPI, bool PAIR> struct TcCfg {
   static constexpr int B_BYTES = (PAIR ? MMA_N / 2 : MMA_N) * TC_BK * 2;
   static constexpr int STAGE_BYTES = TC_A_BYTES + B_BYTES;
-  // The Adam update is bound by what its epilogue reads and writes: it trades half of the operand ring for a ring of
-  // weights and moments in flight (two units of 6 KB per epilogue warp).
-  static constexpr int STAGES = EPI == EPI_WADAM ? (PAIR ? 3 : 2) : (PAIR ? 6 : 4);
-  static constexpr int EPI_WARP_BYTES = EPI == EPI_WADAM ? 16384 : 4096;   // staging per epilogue warp: two 32 x 32 bf16 blocks or one fp32 block
+  // The fused updates of grouped products are bound by what their epilogue reads and writes: they trade most of the
+  // operand ring for a row-wise staging area (8 KB per epilogue warp) and a ring of weights and moments in flight (12 KB).
+  static constexpr int STAGES = EPI == EPI_WUPD ? (PAIR ? 2 : 1) : (PAIR ? 6 : 4);
+  static constexpr int EPI_WARP_BYTES = EPI == EPI_WUPD ? 20480 : 4096;   // staging per epilogue warp: two 32 x 32 bf16 blocks or one fp32 block
   static constexpr int TMEM_COLS = 2 * MMA_N;           // two accumulators; a power of two >= 32
   // stage ring | epilogue staging | barriers; the ring starts 1024-byte aligned and
   // every stage is a multiple of 1024 bytes, so the staging area is aligned too
@@ -397,9 +397,10 @@ __device__ __forceinline__ float2 sigmoid_approx2(float2 x) {
 }
 
 // Where an epilogue warp's 32-row slab of an fp32 result (or of the weights a fused update rewrites) lies.
+// at0: this lane's element of row (lane / 8), column piece (lane % 8); in EPI_WUPD of the warp's first row, piece `lane`.
 struct SlabOut {
   float* c; bf16* w; float *m, *mom, *var;      // output; updated weight, master copy and moments
-  int64_t at0, ld4, res0;      // this lane's element of row (lane / 8), column piece (lane % 8); four rows; residual element
+  int64_t at0, ld4, res0;      // ...; four rows; residual element
   int rows;                    // rows that exist (<= 32)
 };
 __device__ __forceinline__ float4 as_f4(const uint4& u) {
@@ -415,48 +416,150 @@ __device__ __forceinline__ uint2 pack4(const float4& v) {
   return make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
 }
 
+// Fused update of a grouped product's tile (EPI_WUPD): a warp's 16 rows x 128 columns, eight units of two rows.  Weights (the
+// fp32 master copy, or the bf16 weights themselves) and Adam's moments of a unit come by cp.async into a ring of UpdRing
+// units per warp behind the 8 KB staging area.  Everything that does not change is a compile-time constant or a running
+// offset: with two epilogue warps per scheduler an instruction costs its latency, and the first form of this loop
+// (kind and ring depth looked up at run time) took 950 clk per unit before any memory traffic.
+template <bool ADAM, bool MASTER> struct UpdRing {
+  static constexpr int W = MASTER ? 1024 : 512;                    // bytes of weights in a unit
+  static constexpr int UNIT = W + (ADAM ? 2048 : 0);
+  static constexpr int DEPTH = ADAM ? 4 : 8;
+  static_assert(DEPTH * UNIT <= 12288, "ring");
+};
+template <bool ADAM, bool MASTER>
+__device__ __forceinline__ void upd_ask(const SlabOut& o, uint8_t* unit, int lane, int64_t at, int64_t ldc) {      // at: the unit's first row
+  using R = UpdRing<ADAM, MASTER>;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    if (MASTER) cp_async16(unit + i * 512 + lane * 16, o.m + at + i * ldc, true);
+    if (ADAM) {
+      cp_async16(unit + R::W + i * 512 + lane * 16, o.mom + at + i * ldc, true);
+      cp_async16(unit + R::W + 1024 + i * 512 + lane * 16, o.var + at + i * ldc, true);
+    }
+  }
+  // 256 bytes of bf16 weights per row: half a warp each (at points at column 4 lane)
+  if (!MASTER) cp_async16(unit + lane * 16, o.w + at - lane * 4 + (lane >> 4) * ldc + (lane & 15) * 8, true);
+}
+template <bool ADAM, bool MASTER>
+__device__ __forceinline__ void upd_first(const SlabOut& o, uint8_t* stg, int lane, int64_t ldc) {
+  using R = UpdRing<ADAM, MASTER>;
+#pragma unroll
+  for (int u = 0; u < R::DEPTH; ++u) {
+    upd_ask<ADAM, MASTER>(o, stg + 8192 + u * R::UNIT, lane, o.at0 + 2 * u * ldc, ldc);
+    cp_async_commit();
+  }
+}
+template <bool ADAM, bool MASTER>
+__device__ __forceinline__ void upd_half(const UpdRule& rule, const SlabOut& o, uint8_t* stg, int lane, int64_t ldc, int cb, bool last) {
+  using R = UpdRing<ADAM, MASTER>;
+  int64_t at = o.at0 + cb * 128;
+#pragma unroll
+  for (int u = 0; u < 8; ++u, at += 2 * ldc) {
+    uint8_t* unit = stg + 8192 + u % R::DEPTH * R::UNIT;
+    cp_async_wait<R::DEPTH - 1>();
+    if (!MASTER) __syncwarp();      // a 16-byte piece of bf16 weights serves two lanes
+    float4 w[2], mo[2], va[2], g[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      w[i] = MASTER ? *reinterpret_cast<const float4*>(unit + i * 512 + lane * 16) : bf4(*reinterpret_cast<const uint2*>(unit + i * 256 + lane * 8));
+      if (ADAM) {
+        mo[i] = *reinterpret_cast<const float4*>(unit + R::W + i * 512 + lane * 16);
+        va[i] = *reinterpret_cast<const float4*>(unit + R::W + 1024 + i * 512 + lane * 16);
+      }
+      g[i] = *reinterpret_cast<const float4*>(stg + (2 * u + i) * 512 + ((lane ^ ((2 * u + i) & 7)) << 4));
+    }
+    if (!MASTER) __syncwarp();
+    if (u + R::DEPTH < 8) upd_ask<ADAM, MASTER>(o, unit, lane, at + 2 * R::DEPTH * ldc, ldc);
+    else if (!last) upd_ask<ADAM, MASTER>(o, unit, lane, at + 2 * (R::DEPTH - 8) * ldc + 128, ldc);
+    cp_async_commit();
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      if (ADAM) {
+        w[i].x = upd_step(rule, w[i].x, g[i].x, &mo[i].x, &va[i].x);
+        w[i].y = upd_step(rule, w[i].y, g[i].y, &mo[i].y, &va[i].y);
+        w[i].z = upd_step(rule, w[i].z, g[i].z, &mo[i].z, &va[i].z);
+        w[i].w = upd_step(rule, w[i].w, g[i].w, &mo[i].w, &va[i].w);
+        *reinterpret_cast<float4*>(o.mom + at + i * ldc) = mo[i];
+        *reinterpret_cast<float4*>(o.var + at + i * ldc) = va[i];
+      } else {
+        w[i].x -= rule.lr * g[i].x; w[i].y -= rule.lr * g[i].y; w[i].z -= rule.lr * g[i].z; w[i].w -= rule.lr * g[i].w;
+      }
+      if (MASTER) *reinterpret_cast<float4*>(o.m + at + i * ldc) = w[i];
+      *reinterpret_cast<uint2*>(o.w + at + i * ldc) = pack4(w[i]);
+    }
+  }
+}
+
 // Tile coordinates shared by the three roles.
 struct TcTile {
   int m0, n0, group, k_blocks, krow0;
-  int ncols;      // accumulator columns in use: 256, or 128 in the last column tile of an odd multiple of 128
-  bool valid;
+  int ncols;      // accumulator columns in use: the tile's, or 128 in the last column tile of an odd multiple of 128
 };
 
-// pair_rank < 0: one CTA per 128-row tile.  pair_rank 0 / 1: w counts 256-row tiles worked by two CTAs,
-// this CTA takes rows 128 * pair_rank .. + 127 of it (rows past M are loaded as zeros and never stored).
-__device__ __forceinline__ TcTile tc_tile(const TcParams& P, int w, int tiles_m_dev, int pair_rank = -1) {
-  TcTile t;
+// A tile's index split into its parts, and the table entries that the rest of its description comes from.  The roles
+// ask for the next tile's entries (tc_ask) when they begin a tile and look at them (tc_tile) when they begin the next: the
+// loads are then long done.  Looked up when needed, each of the three roles spent 1200-2000 clk per tile on them, the
+// tensor core idle for most of that (expert weight gradients at 512 tokens, one K step per tile: ASKNUMS).
+struct TcAsk { int tm, tn, group; int4 e; };
+
+// Tiles of this launch, known once the kernel runs (row tiles or token chunks of the grouped forms are counted on the device).
+__device__ __forceinline__ int tc_total(const TcParams& P, int tiles_m_dev, int pair_rank) {
   const GemmProblem& p = P.p;
+  if (P.tr) return p.rows_total[1] * P.tiles_f;
+  const int tiles_m = pair_rank >= 0 ? (tiles_m_dev + 1) / 2 : tiles_m_dev;
+  return tiles_m * P.tiles_n * (p.group_mode == GROUP_K ? p.n_groups : 1);
+}
+
+__device__ __forceinline__ TcAsk tc_ask(const TcParams& P, int w, int total, int tiles_m_dev, int pair_rank) {
+  TcAsk a;
+  const GemmProblem& p = P.p;
+  a.tm = a.tn = a.group = 0;
+  a.e = make_int4(0, 0, 0, 0);
+  if (w >= total) return a;
   if (P.tr) {
-    // w = token chunk * tiles_f + feature tile; m0 = first token row, ncols = token rows (the MMA N),
-    // n0 = first feature of this CTA's 128
-    const int ci = w / P.tiles_f, ft = w - ci * P.tiles_f;
-    t.group = 0; t.krow0 = 0; t.k_blocks = P.k_blocks; t.ncols = 0; t.m0 = t.n0 = 0;
-    t.valid = ci < p.rows_total[1];
-    if (!t.valid) return t;
-    const int4 ch = p.tok_chunks[ci];
-    t.group = ch.x; t.m0 = ch.y; t.ncols = ch.z;
-    t.n0 = ft * 2 * TC_BM + pair_rank * TC_BM;
-    return t;
+    // w = token chunk * tiles_f + feature tile
+    a.tm = w / P.tiles_f;
+    a.tn = w - a.tm * P.tiles_f;
+    a.e = p.tok_chunks[a.tm];
+    return a;
   }
   if (pair_rank >= 0) tiles_m_dev = (tiles_m_dev + 1) / 2;
-  int per_group = tiles_m_dev * P.tiles_n;
-  t.group = 0;
-  t.krow0 = 0;
-  t.k_blocks = P.k_blocks;
-  int total = (p.group_mode == GROUP_K) ? per_group * p.n_groups : per_group;
-  t.valid = w < total;
-  t.ncols = 0;
-  if (!t.valid) { t.m0 = t.n0 = 0; return t; }
   int r = w;
   if (p.group_mode == GROUP_K) {
-    t.group = w / per_group;
-    r = w - t.group * per_group;
+    const int per_group = tiles_m_dev * P.tiles_n;
+    a.group = w / per_group;
+    r = w - a.group * per_group;
     if (p.group_off) {
-      int k0 = p.group_off[t.group], k1 = p.group_off[t.group + 1];
-      t.krow0 = k0;
-      t.k_blocks = (k1 - k0) / TC_BK;
-      if (p.group_cnt) t.k_blocks = min(t.k_blocks, (p.group_cnt[t.group] + TC_BK - 1) / TC_BK);   // skip all-zero K blocks
+      a.e.x = p.group_off[a.group];
+      a.e.y = p.group_off[a.group + 1];
+      a.e.z = p.group_cnt ? p.group_cnt[a.group] : 0x7fffff00;
+    }
+  }
+  a.tm = r / P.tiles_n;
+  a.tn = r - a.tm * P.tiles_n;
+  if (p.group_mode == GROUP_M) a.e.x = p.tile_group[a.tm];
+  return a;
+}
+
+// pair_rank < 0: one CTA per 128-row tile.  pair_rank 0 / 1: a tile is 256 rows worked by two CTAs,
+// this CTA takes rows 128 * pair_rank .. + 127 of it (rows past M are loaded as zeros and never stored).
+__device__ __forceinline__ TcTile tc_tile(const TcParams& P, const TcAsk& a, int pair_rank = -1) {
+  TcTile t;
+  const GemmProblem& p = P.p;
+  t.krow0 = 0;
+  t.k_blocks = P.k_blocks;
+  if (P.tr) {
+    // m0 = first token row, ncols = token rows (the MMA N), n0 = first feature of this CTA's 128
+    t.group = a.e.x; t.m0 = a.e.y; t.ncols = a.e.z;
+    t.n0 = a.tn * 2 * TC_BM + pair_rank * TC_BM;
+    return t;
+  }
+  t.group = a.group;
+  if (p.group_mode == GROUP_K) {
+    if (p.group_off) {
+      t.krow0 = a.e.x;
+      t.k_blocks = min((a.e.y - a.e.x) / TC_BK, (a.e.z + TC_BK - 1) / TC_BK);   // skip all-zero K blocks
     } else {
       // equal slices of a dense K (split-K): rows past K in the last K step load as zeros
       const int slice = (int)split_k_rows(p.K, p.n_groups);
@@ -465,11 +568,10 @@ __device__ __forceinline__ TcTile tc_tile(const TcParams& P, int w, int tiles_m_
       t.k_blocks = (k1 - k0 + TC_BK - 1) / TC_BK;
     }
   }
-  int tm = r / P.tiles_n, tn = r - tm * P.tiles_n;
-  t.m0 = (pair_rank >= 0) ? tm * 2 * TC_BM + pair_rank * TC_BM : tm * TC_BM;
-  t.n0 = tn * P.tile_n;
+  t.m0 = (pair_rank >= 0) ? a.tm * 2 * TC_BM + pair_rank * TC_BM : a.tm * TC_BM;
+  t.n0 = a.tn * P.tile_n;
   t.ncols = (p.concat == CONCAT_N) ? 2 * P.tile_n : min(P.tile_n, p.N - t.n0);
-  if (p.group_mode == GROUP_M) t.group = p.tile_group[tm];
+  if (p.group_mode == GROUP_M) t.group = a.e.x;
   return t;
 }
 
@@ -483,7 +585,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
                const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_c1) {
   using Cfg = TcCfg<MMA_N, EPI, PAIR>;
   constexpr bool RMW = EPI == EPI_COUPLE || EPI == EPI_WRMW;
-  constexpr bool WGRAD = EPI == EPI_WGRAD || EPI == EPI_WADAM || EPI == EPI_WRMW;
+  constexpr bool WGRAD = EPI == EPI_WGRAD || EPI == EPI_WUPD || EPI == EPI_WRMW;
   extern __shared__ uint8_t smem_raw[];
   const GemmProblem& p = P.p;
   const uint32_t raw = smem_u32(smem_raw);
@@ -534,6 +636,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
 
   int tiles_m_dev = P.tiles_m;
   if (p.group_mode == GROUP_M) tiles_m_dev = min(P.tiles_m, *p.rows_total / TC_BM);
+  const int total = tc_total(P, tiles_m_dev, prank);
 
   if (warp == 0 || warp == TC_LOAD_WARP_B) {
     // ------------------------------------------------------------------ operand loads
@@ -554,9 +657,10 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int w = w0; ok; w += wstride) {
-        TcTile t = tc_tile(P, w, tiles_m_dev, prank);
-        if (!t.valid) break;
+      TcAsk ask = tc_ask(P, w0, total, tiles_m_dev, prank);
+      for (int w = w0; ok && w < total; w += wstride) {
+        const TcTile t = tc_tile(P, ask, prank);
+        ask = tc_ask(P, w + wstride, total, tiles_m_dev, prank);
         const int k_half = t.k_blocks / 2;
         for (int kb = 0; kb < t.k_blocks; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
@@ -720,9 +824,10 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       const uint32_t b_step = n_mn ? (2048u >> 4) : (32u >> 4);
       constexpr uint32_t SB16 = (uint32_t)Cfg::STAGE_BYTES >> 4;  // the whole ring stays below 256 KB: no carry out of the field
       uint32_t a_lo = a_lo0, b_lo = b_lo0, fbar = full_bar(0), ebar = empty_bar(0);
-      for (int w = w0; ok && crank == 0; w += wstride, ++it) {
-        TcTile t = tc_tile(P, w, tiles_m_dev, prank);
-        if (!t.valid) break;
+      TcAsk ask = tc_ask(P, w0, total, tiles_m_dev, prank);
+      for (int w = w0; ok && crank == 0 && w < total; w += wstride, ++it) {
+        const TcTile t = tc_tile(P, ask, prank);
+        ask = tc_ask(P, w + wstride, total, tiles_m_dev, prank);
         const int acc = it & 1;
         const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
         if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
@@ -773,9 +878,10 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
     bool ok = true;
     int it = 0;
     uint32_t n_grp = 0;                          // bulk groups committed so far (same in every lane)
-    for (int w = w0; ok; w += wstride, ++it) {
-      TcTile t = tc_tile(P, w, tiles_m_dev, prank);
-      if (!t.valid) break;
+    TcAsk ask = tc_ask(P, w0, total, tiles_m_dev, prank);
+    for (int w = w0; ok && w < total; w += wstride, ++it) {
+      const TcTile t = tc_tile(P, ask, prank);
+      ask = tc_ask(P, w + wstride, total, tiles_m_dev, prank);
       const int acc = it & 1;
       const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
       const int m = t.m0 + row_in_tile;
@@ -797,7 +903,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       // row coordinate of the slab in the output tensor map (rows past its extent are clipped by the store)
       const int y0 = (p.group_mode == GROUP_K ? t.group * p.M : 0) + t.m0 + q * 32;
       SlabOut out;
-      uint4 ld_a[8], ld_b[8];     // read-modify-write forms: a block's pieces, four floats or (in .x, .y) four bf16 weights
+      uint4 ld[8];     // read-modify-write forms: a block's pieces, four floats or (in .x, .y) four bf16 weights
       if constexpr (EPI == EPI_COUPLE || WGRAD || EPI == EPI_STORE) {
         // where this warp's slab of an fp32 result goes
         int64_t yb = y0;
@@ -817,7 +923,8 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           yb = (int64_t)t.group * p.split_m + local;
           out.rows = min(32, p.split_m - local);
         }
-        out.at0 = (yb + (lane >> 3)) * p.ldc + t.n0 + (lane & 7) * 4;
+        if (EPI == EPI_WUPD) out.at0 = (yb + half * 16) * p.ldc + t.n0 + lane * 4;
+        else out.at0 = (yb + (lane >> 3)) * p.ldc + t.n0 + (lane & 7) * 4;
         out.ld4 = 4 * p.ldc;
         out.res0 = EPI == EPI_COUPLE ? (yb + (lane >> 3)) * p.ld_resid + t.n0 + (lane & 7) * 4 : 0;
       }
@@ -832,40 +939,27 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           else { const uint2 w2 = *reinterpret_cast<const uint2*>(o.w + at); ld[i].x = w2.x; ld[i].y = w2.y; }
         }
       };
-      // Adam: unit u of the tile (16 rows of block u / 2) into its half of the ring; always commits a group
-      auto adam_request = [&](const SlabOut& o, int u, int ncols) {
-        const int c = half * 32 + (u >> 1) * 64, r0u = (u & 1) * 16;
-        if (c < ncols) {
-          uint8_t* unit = stg + 4096 + (u & 1) * 6144;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int r = 4 * i + (lane >> 3);
-            const bool in = r0u + r < o.rows;
-            const int64_t at = in ? o.at0 + c + ((r0u >> 2) + i) * o.ld4 : 0;
-            if (o.m) cp_async16(unit + r * 128 + (lane & 7) * 16, o.m + at, in);
-            cp_async16(unit + 2048 + r * 128 + (lane & 7) * 16, o.mom + at, in);
-            cp_async16(unit + 4096 + r * 128 + (lane & 7) * 16, o.var + at, in);
-          }
-          if (!o.m) {
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {      // 16 rows of 64 bytes: eight rows per instruction, four pieces each
-              const int r = 8 * i + (lane >> 2);
-              const bool in = r0u + r < o.rows;
-              const int64_t at = in ? o.at0 - (int64_t)(lane >> 3) * p.ldc - (lane & 7) * 4 + (int64_t)(r0u + r) * p.ldc + c + (lane & 3) * 8 : 0;
-              cp_async16(unit + r * 64 + (lane & 3) * 16, o.w + at, in);
-            }
+      if constexpr (EPI == EPI_WUPD) {
+        if (slab_ok) {
+          if (out.mom) {
+            if (out.m) upd_first<true, true>(out, stg, lane, p.ldc); else upd_first<true, false>(out, stg, lane, p.ldc);
+          } else {
+            if (out.m) upd_first<false, true>(out, stg, lane, p.ldc); else upd_first<false, false>(out, stg, lane, p.ldc);
           }
         }
-        cp_async_commit();
-      };
-      if constexpr (EPI == EPI_WADAM) {
-        if (slab_ok) { adam_request(out, 0, t.ncols); adam_request(out, 1, t.ncols); }
-      } else if constexpr (RMW) {
-        if (slab_ok && half * 32 < t.ncols) rmw_request(out, half * 32, ld_a);
       }
       if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * MMA_N);
+      // accumulator may be overwritten by the MMA warp
+      auto release = [&]() {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          if constexpr (PAIR) mbar_arrive_cluster(mapa_u32(tempty_bar(acc), 0));   // the even CTA's MMA warp waits for both
+          else mbar_arrive(tempty_bar(acc));
+        }
+      };
       const bool have_acc = t.k_blocks > 0;      // an empty K range leaves the accumulator undefined: use zeros
       uint32_t r0[32];
       float f[32];
@@ -976,52 +1070,67 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
             return *reinterpret_cast<const float4*>(stg + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
           };
           auto row_ok = [&](int i) -> bool { return all_rows || i * 4 + rsub < out.rows; };
-          fetch(half * 32);
-          if constexpr (EPI == EPI_WADAM) {
-            // Adam: weight (or master copy) and the two moments of a unit of 16 rows x 32 columns come by cp.async into
-            // a ring of two units; a lane asks for exactly the pieces it will use, so nothing but its own copies
-            // has to have landed.
-            int u = 0;
+          if (!RMW && EPI != EPI_WUPD) fetch(half * 32);
+          if constexpr (EPI == EPI_WUPD) {
+            // Fused update of the grouped products, whose short K leaves the kernel bound by what this reads and writes.
+            // HBM serves the four arrays' 128-byte pieces of the block-wise form at 4.1 TB/s, 512-byte pieces at 5.3
+            // (a bare read-modify-write kernel, 26 bytes per element, 148 CTAs; bf16 weights alone: 64-byte pieces 3.9,
+            // 256-byte 5.3).  So a warp takes 16 whole rows of its quadrant, 128 columns at a time: the accumulator goes
+            // through a 16 x 128 staging area, weights and moments of two rows at a time come by cp.async into
+            // a ring, one instruction is one row.
+            for (int cb = 0; cb * 128 < t.ncols; ++cb) {
 #pragma unroll 1
-            for (int c = half * 32; c < t.ncols; c += 64) {
-              stage();
-              fetch(c + 64);
+              for (int jj = 0; jj < 4; ++jj) {
+                if (have_acc) { tmem_ld32(taddr + cb * 128 + jj * 32, r0); tmem_ld_wait(); }
+                if ((lane >> 4) == half) {
+                  uint8_t* row = stg + (lane & 15) * 512;
+#pragma unroll
+                  for (int j = 0; j < 8; ++j)
+                    *reinterpret_cast<uint4*>(row + ((jj * 8 + (j ^ (lane & 7))) << 4)) =
+                        have_acc ? make_uint4(r0[4 * j], r0[4 * j + 1], r0[4 * j + 2], r0[4 * j + 3]) : make_uint4(0u, 0u, 0u, 0u);
+                }
+                __syncwarp();
+              }
+              const bool last = cb * 128 + 128 >= t.ncols;
+              if (last) release();      // the tile's last columns are out of tensor memory
+              if (out.mom) {
+                if (out.m) upd_half<true, true>(p.upd, out, stg, lane, p.ldc, cb, last); else upd_half<true, false>(p.upd, out, stg, lane, p.ldc, cb, last);
+              } else {
+                if (out.m) upd_half<false, true>(p.upd, out, stg, lane, p.ldc, cb, last); else upd_half<false, false>(p.upd, out, stg, lane, p.ldc, cb, last);
+              }
+              __syncwarp();
+            }
+          } else {
+            // Read-modify-write forms (coupling, accumulation, fused updates of dense products, whose long K hides them):
+            // all a block needs is requested before its accumulator is fetched.
+            auto write_adam = [&](int c) {
 #pragma unroll 1
-              for (int h2 = 0; h2 < 2; ++h2, ++u) {
-                cp_async_wait<1>();
-                if (!out.m) __syncwarp();      // bf16 weights: a 16-byte piece serves two lanes
-                const uint8_t* unit = stg + 4096 + (u & 1) * 6144;
+              for (int h4 = 0; h4 < 8; h4 += 4) {      // four pieces at a time keep the registers in bounds
                 float4 w4[4], mo[4], va[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                  const int at = (4 * i + rsub) * 128 + (lane & 7) * 16;
-                  if (out.m) w4[i] = *reinterpret_cast<const float4*>(unit + at);
-                  else w4[i] = bf4(*reinterpret_cast<const uint2*>(unit + (4 * i + rsub) * 64 + (lane & 7) * 8));
-                  mo[i] = *reinterpret_cast<const float4*>(unit + 2048 + at);
-                  va[i] = *reinterpret_cast<const float4*>(unit + 4096 + at);
+                  if (!row_ok(h4 + i)) continue;
+                  const int64_t at = out.at0 + c + (h4 + i) * out.ld4;
+                  w4[i] = out.m ? *reinterpret_cast<const float4*>(out.m + at) : bf4(*reinterpret_cast<const uint2*>(out.w + at));
+                  mo[i] = *reinterpret_cast<const float4*>(out.mom + at);
+                  va[i] = *reinterpret_cast<const float4*>(out.var + at);
                 }
-                if (!out.m) __syncwarp();
-                adam_request(out, u + 2, t.ncols);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                  if (!row_ok(4 * h2 + i)) continue;
-                  const float4 v = staged(4 * h2 + i);
+                  if (!row_ok(h4 + i)) continue;
+                  const float4 v = staged(h4 + i);
+                  const int64_t at = out.at0 + c + (h4 + i) * out.ld4;
                   w4[i].x = upd_step(p.upd, w4[i].x, v.x, &mo[i].x, &va[i].x);
                   w4[i].y = upd_step(p.upd, w4[i].y, v.y, &mo[i].y, &va[i].y);
                   w4[i].z = upd_step(p.upd, w4[i].z, v.z, &mo[i].z, &va[i].z);
                   w4[i].w = upd_step(p.upd, w4[i].w, v.w, &mo[i].w, &va[i].w);
-                  const int64_t at = out.at0 + c + (4 * h2 + i) * out.ld4;
                   *reinterpret_cast<float4*>(out.mom + at) = mo[i];
                   *reinterpret_cast<float4*>(out.var + at) = va[i];
                   if (out.m) *reinterpret_cast<float4*>(out.m + at) = w4[i];
                   *reinterpret_cast<uint2*>(out.w + at) = pack4(w4[i]);
                 }
               }
-              __syncwarp();
-            }
-          } else {
-            // Read-modify-write forms (coupling, accumulation, SGD step): what a block needs is requested a block
-            // ahead, the first one before the wait for the accumulator.
+            };
             auto write = [&](int c, const uint4 (&ld)[8]) {
 #pragma unroll
               for (int i = 0; i < 8; ++i) {
@@ -1036,7 +1145,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
                     const float4 o = as_f4(ld[i]);
                     v = make_float4(o.x + v.x, o.y + v.y, o.z + v.z, o.w + v.w);
                   } else {
-                    // fused SGD step on the weight tile this gradient tile belongs to; the gradient is not stored
+                    // fused update on the weight tile this gradient tile belongs to; the gradient is not stored
                     float4 w4 = out.m ? as_f4(ld[i]) : bf4(make_uint2(ld[i].x, ld[i].y));
                     w4.x -= p.upd.lr * v.x; w4.y -= p.upd.lr * v.y; w4.z -= p.upd.lr * v.z; w4.w -= p.upd.lr * v.w;
                     if (out.m) *reinterpret_cast<float4*>(out.m + at) = w4;
@@ -1048,17 +1157,13 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
               }
             };
 #pragma unroll 1
-            for (int c = half * 32; c < t.ncols; c += 128) {
+            for (int c = half * 32; c < t.ncols; c += 64) {
+              const bool adam = EPI == EPI_WRMW && out.w && out.mom;
+              if (RMW && !adam) rmw_request(out, c, ld);
+              if (RMW) fetch(c);
               stage();
-              fetch(c + 64);
-              if (RMW && c + 64 < t.ncols) rmw_request(out, c + 64, ld_b);
-              write(c, ld_a);
-              __syncwarp();
-              if (c + 64 >= t.ncols) break;
-              stage();
-              fetch(c + 128);
-              if (RMW && c + 128 < t.ncols) rmw_request(out, c + 128, ld_a);
-              write(c + 64, ld_b);
+              if (!RMW) fetch(c + 64);
+              if (adam) write_adam(c); else write(c, ld);
               __syncwarp();
             }
           }
@@ -1240,17 +1345,11 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
         }
         if (p.dg_part && m_ok) p.dg_part[(int64_t)m * p.dg_ld + 2 * (t.n0 / P.tile_n) + half] = dg2.x + dg2.y;
       }
-      // accumulator may be overwritten by the MMA warp
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        if constexpr (PAIR) mbar_arrive_cluster(mapa_u32(tempty_bar(acc), 0));   // the even CTA's MMA warp waits for both
-        else mbar_arrive(tempty_bar(acc));
-      }
+      if (EPI != EPI_WUPD || !slab_ok) release();
     }
     // this lane's stores must be complete (shared memory read, global memory written) before the CTA exits
     if (lane == 0) bulk_wait_all();
-    if constexpr (EPI == EPI_WADAM) cp_async_wait<0>();
+    if constexpr (EPI == EPI_WUPD) cp_async_wait<0>();
   }
 
   // ------------------------------------------------------------------ teardown
@@ -1351,7 +1450,7 @@ inline int tc_prepare() {
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_COUPLE>();
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_DSWIGLU>();
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_WGRAD>();
-  if (e == cudaSuccess) e = tc_set_attr<256, EPI_WADAM>();
+  if (e == cudaSuccess) e = tc_set_attr<256, EPI_WUPD>();
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_WRMW>();
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_HEADS>();
   if (e != cudaSuccess) return REVFFN_ERR_CUDA;
@@ -1438,7 +1537,7 @@ inline TcPlan tc_plan(const GemmProblem& p, int n_sms) {
     wide.pair = p.group_mode != GROUP_M && !p.no_pair && (cat || (p.dbg_tile_n == 256 ? wide.pair : p.dbg_tile_n >= 128));
     return wide;
   }
-  if (wide.tr || p.fp8) return wide;
+  if (wide.tr || p.fp8 || p.upd_w) return wide;
   const bool pair_open = p.group_mode != GROUP_M && !p.no_pair && n_sms % 2 == 0;
   const int64_t groups = p.group_mode == GROUP_K ? (p.n_groups > 0 ? p.n_groups : 1) : 1;
   int64_t k_steps = ceil_div(p.K, TC_BK);
@@ -1620,9 +1719,9 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
 
 #define TC_CASE(N_, E_) \
   if (mma_n == N_ && epi == E_) return tc_launch<N_, E_>(P, ma, mb0, mb1, mc, mc1, grid, pair, st);
-  const int epi = p.epilogue != EPI_WGRAD ? p.epilogue : (p.upd_w ? (p.upd.kind != 0 ? EPI_WADAM : EPI_WRMW) : (p.accumulate ? EPI_WRMW : EPI_WGRAD));
+  const int epi = p.epilogue != EPI_WGRAD ? p.epilogue : (p.upd_w && p.group_off ? EPI_WUPD : (p.upd_w || p.accumulate ? EPI_WRMW : EPI_WGRAD));
   TC_CASE(256, EPI_STORE) TC_CASE(256, EPI_SWIGLU) TC_CASE(256, EPI_ROWSCALE) TC_CASE(256, EPI_COUPLE)
-  TC_CASE(256, EPI_DSWIGLU) TC_CASE(256, EPI_WGRAD) TC_CASE(256, EPI_WADAM) TC_CASE(256, EPI_WRMW)
+  TC_CASE(256, EPI_DSWIGLU) TC_CASE(256, EPI_WGRAD) TC_CASE(256, EPI_WUPD) TC_CASE(256, EPI_WRMW)
   TC_CASE(256, EPI_HEADS)
 #undef TC_CASE
   return REVFFN_ERR_UNSUPPORTED;
