@@ -68,10 +68,11 @@ constexpr long long TC_WAIT_CYCLES = 4000000000LL;       // ~2 s: bound on any s
 template <int MMA_N, int EPI, bool PAIR> struct TcCfg {
   static constexpr int B_BYTES = (PAIR ? MMA_N / 2 : MMA_N) * TC_BK * 2;
   static constexpr int STAGE_BYTES = TC_A_BYTES + B_BYTES;
-  // The fused updates of grouped products are bound by what their epilogue reads and writes: they trade most of the
-  // operand ring for a row-wise staging area (8 KB per epilogue warp) and a ring of weights and moments in flight (12 KB).
-  static constexpr int STAGES = EPI == EPI_WUPD ? (PAIR ? 2 : 1) : (PAIR ? 6 : 4);
-  static constexpr int EPI_WARP_BYTES = EPI == EPI_WUPD ? 20480 : 4096;   // staging per epilogue warp: two 32 x 32 bf16 blocks or one fp32 block
+  // The fused updates of grouped products are bound by what their epilogue reads and writes: they trade part of the
+  // operand ring for a row-wise staging area (8 KB per epilogue warp) and a ring of weights and moments in flight.
+  static constexpr int STAGES = EPI == EPI_WADAM ? (PAIR ? 2 : 1) : EPI == EPI_WSGD ? (PAIR ? 3 : 2) : (PAIR ? 6 : 4);
+  // staging per epilogue warp: two 32 x 32 bf16 blocks or one fp32 block
+  static constexpr int EPI_WARP_BYTES = EPI == EPI_WADAM ? 20480 : EPI == EPI_WSGD ? 16384 : 4096;
   static constexpr int TMEM_COLS = 2 * MMA_N;           // two accumulators; a power of two >= 32
   // stage ring | epilogue staging | barriers; the ring starts 1024-byte aligned and
   // every stage is a multiple of 1024 bytes, so the staging area is aligned too
@@ -397,7 +398,7 @@ __device__ __forceinline__ float2 sigmoid_approx2(float2 x) {
 }
 
 // Where an epilogue warp's 32-row slab of an fp32 result (or of the weights a fused update rewrites) lies.
-// at0: this lane's element of row (lane / 8), column piece (lane % 8); in EPI_WUPD of the warp's first row, piece `lane`.
+// at0: this lane's element of row (lane / 8), column piece (lane % 8); in the row-wise updates of the warp's first row, piece `lane`.
 struct SlabOut {
   float* c; bf16* w; float *m, *mom, *var;      // output; updated weight, master copy and moments
   int64_t at0, ld4, res0;      // ...; four rows; residual element
@@ -416,16 +417,18 @@ __device__ __forceinline__ uint2 pack4(const float4& v) {
   return make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
 }
 
-// Fused update of a grouped product's tile (EPI_WUPD): a warp's 16 rows x 128 columns, eight units of two rows.  Weights (the
+// Fused update of a grouped product's tile (EPI_WADAM, EPI_WSGD): a warp's 16 rows x 128 columns, eight units of two rows.  Weights (the
 // fp32 master copy, or the bf16 weights themselves) and Adam's moments of a unit come by cp.async into a ring of UpdRing
 // units per warp behind the 8 KB staging area.  Everything that does not change is a compile-time constant or a running
 // offset: with two epilogue warps per scheduler an instruction costs its latency, and the first form of this loop
-// (kind and ring depth looked up at run time) took 950 clk per unit before any memory traffic.
+// (kind and ring depth looked up at run time) took 950 clk per unit before any memory traffic.  Adam's last
+// units of a tile ask for the first ones of the next, so that reads go on while its accumulator is staged (experts'
+// gate | up at 1024 tokens, 9.0 GB: 2088 -> 1965 us; the SGD step, 1.4 GB, got slower by it, 309 -> 362).
 template <bool ADAM, bool MASTER> struct UpdRing {
   static constexpr int W = MASTER ? 1024 : 512;                    // bytes of weights in a unit
   static constexpr int UNIT = W + (ADAM ? 2048 : 0);
   static constexpr int DEPTH = ADAM ? 4 : 8;
-  static_assert(DEPTH * UNIT <= 12288, "ring");
+  static_assert(DEPTH * UNIT <= (ADAM ? 12288 : 8192), "ring");
 };
 template <bool ADAM, bool MASTER>
 __device__ __forceinline__ void upd_ask(const SlabOut& o, uint8_t* unit, int lane, int64_t at, int64_t ldc) {      // at: the unit's first row
@@ -451,7 +454,8 @@ __device__ __forceinline__ void upd_first(const SlabOut& o, uint8_t* stg, int la
   }
 }
 template <bool ADAM, bool MASTER>
-__device__ __forceinline__ void upd_half(const UpdRule& rule, const SlabOut& o, uint8_t* stg, int lane, int64_t ldc, int cb, bool last) {
+__device__ __forceinline__ void upd_half(const UpdRule& rule, const SlabOut& o, const SlabOut& next, uint8_t* stg, int lane, int64_t ldc,
+                                         int cb, bool last, bool more) {
   using R = UpdRing<ADAM, MASTER>;
   int64_t at = o.at0 + cb * 128;
 #pragma unroll
@@ -472,6 +476,7 @@ __device__ __forceinline__ void upd_half(const UpdRule& rule, const SlabOut& o, 
     if (!MASTER) __syncwarp();
     if (u + R::DEPTH < 8) upd_ask<ADAM, MASTER>(o, unit, lane, at + 2 * R::DEPTH * ldc, ldc);
     else if (!last) upd_ask<ADAM, MASTER>(o, unit, lane, at + 2 * (R::DEPTH - 8) * ldc + 128, ldc);
+    else if (more) upd_ask<ADAM, MASTER>(next, unit, lane, next.at0 + 2 * (u + R::DEPTH - 8) * ldc, ldc);
     cp_async_commit();
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
@@ -585,7 +590,8 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
                const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_c1) {
   using Cfg = TcCfg<MMA_N, EPI, PAIR>;
   constexpr bool RMW = EPI == EPI_COUPLE || EPI == EPI_WRMW;
-  constexpr bool WGRAD = EPI == EPI_WGRAD || EPI == EPI_WUPD || EPI == EPI_WRMW;
+  constexpr bool UPD = EPI == EPI_WADAM || EPI == EPI_WSGD;
+  constexpr bool WGRAD = EPI == EPI_WGRAD || EPI == EPI_WRMW || UPD;
   extern __shared__ uint8_t smem_raw[];
   const GemmProblem& p = P.p;
   const uint32_t raw = smem_u32(smem_raw);
@@ -878,6 +884,36 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
     bool ok = true;
     int it = 0;
     uint32_t n_grp = 0;                          // bulk groups committed so far (same in every lane)
+    // where this warp's slab of an fp32 result goes
+    auto slab_of = [&](const TcTile& t) -> SlabOut {
+      SlabOut out;
+      const int y0 = (p.group_mode == GROUP_K ? t.group * p.M : 0) + t.m0 + q * 32;
+      const int m_lim = (p.group_mode == GROUP_M) ? tiles_m_dev * TC_BM : p.M;
+      int64_t yb = y0;
+      const int64_t y_lim = (p.group_mode == GROUP_K) ? (int64_t)(t.group + 1) * p.M : (p.group_mode == GROUP_M ? (int64_t)m_lim : (int64_t)p.M);
+      out.rows = (int)min((int64_t)32, y_lim - yb);
+      out.c = reinterpret_cast<float*>(p.C);
+      out.w = reinterpret_cast<bf16*>(p.upd_w);
+      out.m = p.upd_m; out.mom = p.upd_mom; out.var = p.upd_var;
+      if (WGRAD && p.split_m > 0) {
+        // two outputs: the slab lies wholly in the first or in the second (split_m is a multiple of 128)
+        int local = t.m0 + q * 32;
+        if (local >= p.split_m) {
+          local -= p.split_m;
+          out.c = reinterpret_cast<float*>(p.C2); out.w = reinterpret_cast<bf16*>(p.upd_w2); out.m = p.upd_m2;
+          out.mom = p.upd_mom2; out.var = p.upd_var2;
+        }
+        yb = (int64_t)t.group * p.split_m + local;
+        out.rows = min(32, p.split_m - local);
+      }
+      if (UPD) out.at0 = (yb + half * 16) * p.ldc + t.n0 + lane * 4;
+      else out.at0 = (yb + (lane >> 3)) * p.ldc + t.n0 + (lane & 7) * 4;
+      out.ld4 = 4 * p.ldc;
+      out.res0 = EPI == EPI_COUPLE ? (yb + (lane >> 3)) * p.ld_resid + t.n0 + (lane & 7) * 4 : 0;
+      return out;
+    };
+    SlabOut next_out;      // Adam, row-wise: the next tile's slab, whose first units this tile has asked for (primed)
+    bool primed = false;
     TcAsk ask = tc_ask(P, w0, total, tiles_m_dev, prank);
     for (int w = w0; ok && w < total; w += wstride, ++it) {
       const TcTile t = tc_tile(P, ask, prank);
@@ -902,32 +938,9 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       }
       // row coordinate of the slab in the output tensor map (rows past its extent are clipped by the store)
       const int y0 = (p.group_mode == GROUP_K ? t.group * p.M : 0) + t.m0 + q * 32;
-      SlabOut out;
       uint4 ld[8];     // read-modify-write forms: a block's pieces, four floats or (in .x, .y) four bf16 weights
-      if constexpr (EPI == EPI_COUPLE || WGRAD || EPI == EPI_STORE) {
-        // where this warp's slab of an fp32 result goes
-        int64_t yb = y0;
-        const int64_t y_lim = (p.group_mode == GROUP_K) ? (int64_t)(t.group + 1) * p.M : (p.group_mode == GROUP_M ? (int64_t)m_lim : (int64_t)p.M);
-        out.rows = (int)min((int64_t)32, y_lim - yb);
-        out.c = reinterpret_cast<float*>(p.C);
-        out.w = reinterpret_cast<bf16*>(p.upd_w);
-        out.m = p.upd_m; out.mom = p.upd_mom; out.var = p.upd_var;
-        if (WGRAD && p.split_m > 0) {
-          // two outputs: the slab lies wholly in the first or in the second (split_m is a multiple of 128)
-          int local = t.m0 + q * 32;
-          if (local >= p.split_m) {
-            local -= p.split_m;
-            out.c = reinterpret_cast<float*>(p.C2); out.w = reinterpret_cast<bf16*>(p.upd_w2); out.m = p.upd_m2;
-            out.mom = p.upd_mom2; out.var = p.upd_var2;
-          }
-          yb = (int64_t)t.group * p.split_m + local;
-          out.rows = min(32, p.split_m - local);
-        }
-        if (EPI == EPI_WUPD) out.at0 = (yb + half * 16) * p.ldc + t.n0 + lane * 4;
-        else out.at0 = (yb + (lane >> 3)) * p.ldc + t.n0 + (lane & 7) * 4;
-        out.ld4 = 4 * p.ldc;
-        out.res0 = EPI == EPI_COUPLE ? (yb + (lane >> 3)) * p.ld_resid + t.n0 + (lane & 7) * 4 : 0;
-      }
+      SlabOut out;
+      if constexpr (EPI == EPI_COUPLE || WGRAD || EPI == EPI_STORE) out = slab_of(t);
       auto rmw_request = [&](const SlabOut& o, int c, uint4 (&ld)[8]) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -939,13 +952,10 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           else { const uint2 w2 = *reinterpret_cast<const uint2*>(o.w + at); ld[i].x = w2.x; ld[i].y = w2.y; }
         }
       };
-      if constexpr (EPI == EPI_WUPD) {
-        if (slab_ok) {
-          if (out.mom) {
-            if (out.m) upd_first<true, true>(out, stg, lane, p.ldc); else upd_first<true, false>(out, stg, lane, p.ldc);
-          } else {
-            if (out.m) upd_first<false, true>(out, stg, lane, p.ldc); else upd_first<false, false>(out, stg, lane, p.ldc);
-          }
+      if constexpr (UPD) {
+        if (slab_ok && !primed) {
+          if (out.m) upd_first<EPI == EPI_WADAM, true>(out, stg, lane, p.ldc);
+          else upd_first<EPI == EPI_WADAM, false>(out, stg, lane, p.ldc);
         }
       }
       if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
@@ -1070,8 +1080,8 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
             return *reinterpret_cast<const float4*>(stg + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
           };
           auto row_ok = [&](int i) -> bool { return all_rows || i * 4 + rsub < out.rows; };
-          if (!RMW && EPI != EPI_WUPD) fetch(half * 32);
-          if constexpr (EPI == EPI_WUPD) {
+          if (!RMW && !UPD) fetch(half * 32);
+          if constexpr (UPD) {
             // Fused update of the grouped products, whose short K leaves the kernel bound by what this reads and writes.
             // HBM serves the four arrays' 128-byte pieces of the block-wise form at 4.1 TB/s, 512-byte pieces at 5.3
             // (a bare read-modify-write kernel, 26 bytes per element, 148 CTAs; bf16 weights alone: 64-byte pieces 3.9,
@@ -1093,11 +1103,16 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
               }
               const bool last = cb * 128 + 128 >= t.ncols;
               if (last) release();      // the tile's last columns are out of tensor memory
-              if (out.mom) {
-                if (out.m) upd_half<true, true>(p.upd, out, stg, lane, p.ldc, cb, last); else upd_half<true, false>(p.upd, out, stg, lane, p.ldc, cb, last);
-              } else {
-                if (out.m) upd_half<false, true>(p.upd, out, stg, lane, p.ldc, cb, last); else upd_half<false, false>(p.upd, out, stg, lane, p.ldc, cb, last);
+              if (last) {
+                primed = EPI == EPI_WADAM && w + wstride < total;
+                if (primed) {
+                  const TcTile tn = tc_tile(P, ask, prank);
+                  next_out = slab_of(tn);
+                  primed = next_out.rows > 0;
+                }
               }
+              if (out.m) upd_half<EPI == EPI_WADAM, true>(p.upd, out, next_out, stg, lane, p.ldc, cb, last, primed);
+              else upd_half<EPI == EPI_WADAM, false>(p.upd, out, next_out, stg, lane, p.ldc, cb, last, primed);
               __syncwarp();
             }
           } else {
@@ -1345,11 +1360,11 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
         }
         if (p.dg_part && m_ok) p.dg_part[(int64_t)m * p.dg_ld + 2 * (t.n0 / P.tile_n) + half] = dg2.x + dg2.y;
       }
-      if (EPI != EPI_WUPD || !slab_ok) release();
+      if (!UPD || !slab_ok) release();
     }
     // this lane's stores must be complete (shared memory read, global memory written) before the CTA exits
     if (lane == 0) bulk_wait_all();
-    if constexpr (EPI == EPI_WUPD) cp_async_wait<0>();
+    if constexpr (UPD) cp_async_wait<0>();
   }
 
   // ------------------------------------------------------------------ teardown
@@ -1450,7 +1465,8 @@ inline int tc_prepare() {
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_COUPLE>();
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_DSWIGLU>();
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_WGRAD>();
-  if (e == cudaSuccess) e = tc_set_attr<256, EPI_WUPD>();
+  if (e == cudaSuccess) e = tc_set_attr<256, EPI_WADAM>();
+  if (e == cudaSuccess) e = tc_set_attr<256, EPI_WSGD>();
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_WRMW>();
   if (e == cudaSuccess) e = tc_set_attr<256, EPI_HEADS>();
   if (e != cudaSuccess) return REVFFN_ERR_CUDA;
@@ -1719,9 +1735,16 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
 
 #define TC_CASE(N_, E_) \
   if (mma_n == N_ && epi == E_) return tc_launch<N_, E_>(P, ma, mb0, mb1, mc, mc1, grid, pair, st);
-  const int epi = p.epilogue != EPI_WGRAD ? p.epilogue : (p.upd_w && p.group_off ? EPI_WUPD : (p.upd_w || p.accumulate ? EPI_WRMW : EPI_WGRAD));
+  // A fused update of a grouped product runs in its own form while the K range of a group is short (rows of K on average):
+  // beyond, the operand ring that the form gives up is worth more than its reads and writes.  Per 256 x 256 tile: a K step costs
+  // about 1400 clk with two stages, 1000 with three and 600 with six, the row-wise epilogue 46 k (Adam) or 9 k (SGD),
+  // the block-wise one 57 k or 17 k.
+  const int64_t k_group = p.K / groups;
+  const int epi = p.epilogue != EPI_WGRAD ? p.epilogue
+                  : p.upd_w && p.group_off && k_group <= (p.upd.kind ? 2560 : 1152) ? (p.upd.kind ? EPI_WADAM : EPI_WSGD)
+                  : p.upd_w || p.accumulate ? EPI_WRMW : EPI_WGRAD;
   TC_CASE(256, EPI_STORE) TC_CASE(256, EPI_SWIGLU) TC_CASE(256, EPI_ROWSCALE) TC_CASE(256, EPI_COUPLE)
-  TC_CASE(256, EPI_DSWIGLU) TC_CASE(256, EPI_WGRAD) TC_CASE(256, EPI_WUPD) TC_CASE(256, EPI_WRMW)
+  TC_CASE(256, EPI_DSWIGLU) TC_CASE(256, EPI_WGRAD) TC_CASE(256, EPI_WADAM) TC_CASE(256, EPI_WSGD) TC_CASE(256, EPI_WRMW)
   TC_CASE(256, EPI_HEADS)
 #undef TC_CASE
   return REVFFN_ERR_UNSUPPORTED;
