@@ -54,5 +54,5 @@ def test_update_equals_the_update_of_the_written_gradient(rv, tokens, E, k, mast
                 assert torch.allclose(ms[n].double(), want, rtol=1e-6, atol=2e-6 * lr + 1e-8)
                 assert torch.equal(blk.weights[n], ms[n].to(torch.bfloat16))
             else:
-                # bf16 weights: half an ulp, 2^-9 relative, plus the step's own error
-                assert torch.allclose(blk.weights[n].double(), want, rtol=2.0 ** -8.9, atol=1e-6)
+                # bf16 weights (8 significant bits): half an ulp is at most 2^-8 of the value, plus the step's own error
+                assert torch.allclose(blk.weights[n].double(), want, rtol=2.0 ** -7.99, atol=1e-6)
