@@ -502,54 +502,52 @@ struct TcTile {
   int ncols;      // accumulator columns in use: the tile's, or 128 in the last column tile of an odd multiple of 128
 };
 
-// A tile's index split into its parts, and the table entries that the rest of its description comes from.  The roles
-// ask for the next tile's entries (tc_ask) when they begin a tile and look at them (tc_tile) when they begin the next: the
-// loads are then long done.  Looked up when needed, each of the three roles spent 1200-2000 clk per tile on them, the
-// tensor core idle for most of that (expert weight gradients at 512 tokens, one K step per tile: ASKNUMS).
-struct TcAsk { int tm, tn, group; int4 e; };
-
-// Tiles of this launch, known once the kernel runs (row tiles or token chunks of the grouped forms are counted on the device).
-__device__ __forceinline__ int tc_total(const TcParams& P, int tiles_m_dev, int pair_rank) {
-  const GemmProblem& p = P.p;
-  if (P.tr) return p.rows_total[1] * P.tiles_f;
-  const int tiles_m = pair_rank >= 0 ? (tiles_m_dev + 1) / 2 : tiles_m_dev;
-  return tiles_m * P.tiles_n * (p.group_mode == GROUP_K ? p.n_groups : 1);
-}
-
-__device__ __forceinline__ TcAsk tc_ask(const TcParams& P, int w, int total, int tiles_m_dev, int pair_rank) {
-  TcAsk a;
-  const GemmProblem& p = P.p;
-  a.tm = a.tn = a.group = 0;
-  a.e = make_int4(0, 0, 0, 0);
-  if (w >= total) return a;
-  if (P.tr) {
-    // w = token chunk * tiles_f + feature tile
-    a.tm = w / P.tiles_f;
-    a.tn = w - a.tm * P.tiles_f;
-    a.e = p.tok_chunks[a.tm];
-    return a;
-  }
-  if (pair_rank >= 0) tiles_m_dev = (tiles_m_dev + 1) / 2;
-  int r = w;
-  if (p.group_mode == GROUP_K) {
-    const int per_group = tiles_m_dev * P.tiles_n;
-    a.group = w / per_group;
-    r = w - a.group * per_group;
-    if (p.group_off) {
-      a.e.x = p.group_off[a.group];
-      a.e.y = p.group_off[a.group + 1];
-      a.e.z = p.group_cnt ? p.group_cnt[a.group] : 0x7fffff00;
+// A role's walk over the tiles w0, w0 + stride, ...: the tile's index split into its parts, and the table entries that the
+// rest of its description comes from.  step() moves on by additions and asks for the next tile's entries; tc_tile() looks
+// at them when the role begins that tile, the loads are then long done.  Divided and looked up when needed, each of the
+// three roles spent 1200-2000 clk per tile on this, the tensor core idle for most of it (experts' gate | up weight
+// gradient, one K step per tile: 285 -> 269 us).
+struct TcWalk {
+  int tm, tn, group;                 // row tile (tr: token chunk), column tile (tr: feature tile), group
+  int left;                          // tiles of this role that are left, this one included
+  int dm, dn, dg, tiles_m, tiles_n;  // what a step adds; how far the parts count
+  int4 e;
+  __device__ __forceinline__ void ask(const GemmProblem& p, bool tr) {
+    if (left <= 0) return;
+    if (tr) e = p.tok_chunks[tm];
+    else if (p.group_mode == GROUP_M) e.x = p.tile_group[tm];
+    else if (p.group_mode == GROUP_K && p.group_off) {
+      e.x = p.group_off[group];
+      e.y = p.group_off[group + 1];
+      e.z = p.group_cnt ? p.group_cnt[group] : 0x7fffff00;
     }
   }
-  a.tm = r / P.tiles_n;
-  a.tn = r - a.tm * P.tiles_n;
-  if (p.group_mode == GROUP_M) a.e.x = p.tile_group[a.tm];
-  return a;
-}
+  // tiles_m_dev: 128-row tiles as counted on the device (row tiles or token chunks of the grouped forms)
+  __device__ __forceinline__ void begin(const TcParams& P, int w0, int stride, int tiles_m_dev, int pair_rank) {
+    const GemmProblem& p = P.p;
+    tiles_n = P.tr ? P.tiles_f : P.tiles_n;
+    tiles_m = P.tr ? p.rows_total[1] : (pair_rank >= 0 ? (tiles_m_dev + 1) / 2 : tiles_m_dev);
+    const int per = tiles_m * tiles_n, total = per * (p.group_mode == GROUP_K ? p.n_groups : 1);
+    e = make_int4(0, 0, 0, 0);
+    left = w0 < total ? (total - w0 + stride - 1) / stride : 0;
+    tm = tn = group = dm = dn = dg = 0;
+    if (left == 0) return;
+    group = w0 / per; tm = (w0 - group * per) / tiles_n; tn = w0 - group * per - tm * tiles_n;
+    dg = stride / per; dm = (stride - dg * per) / tiles_n; dn = stride - dg * per - dm * tiles_n;
+    ask(p, P.tr);
+  }
+  __device__ __forceinline__ void step(const TcParams& P) {
+    --left;
+    tn += dn; tm += dm; group += dg;
+    if (tn >= tiles_n) { tn -= tiles_n; ++tm; }
+    if (tm >= tiles_m) { tm -= tiles_m; ++group; }
+    ask(P.p, P.tr);
+  }
+};
 
 // pair_rank < 0: one CTA per 128-row tile.  pair_rank 0 / 1: a tile is 256 rows worked by two CTAs,
 // this CTA takes rows 128 * pair_rank .. + 127 of it (rows past M are loaded as zeros and never stored).
-__device__ __forceinline__ TcTile tc_tile(const TcParams& P, const TcAsk& a, int pair_rank = -1) {
+__device__ __forceinline__ TcTile tc_tile(const TcParams& P, const TcWalk& a, int pair_rank = -1) {
   TcTile t;
   const GemmProblem& p = P.p;
   t.krow0 = 0;
@@ -642,7 +640,6 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
 
   int tiles_m_dev = P.tiles_m;
   if (p.group_mode == GROUP_M) tiles_m_dev = min(P.tiles_m, *p.rows_total / TC_BM);
-  const int total = tc_total(P, tiles_m_dev, prank);
 
   if (warp == 0 || warp == TC_LOAD_WARP_B) {
     // ------------------------------------------------------------------ operand loads
@@ -663,10 +660,11 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      TcAsk ask = tc_ask(P, w0, total, tiles_m_dev, prank);
-      for (int w = w0; ok && w < total; w += wstride) {
-        const TcTile t = tc_tile(P, ask, prank);
-        ask = tc_ask(P, w + wstride, total, tiles_m_dev, prank);
+      TcWalk walk;
+      walk.begin(P, w0, wstride, tiles_m_dev, prank);
+      while (ok && walk.left > 0) {
+        const TcTile t = tc_tile(P, walk, prank);
+        walk.step(P);
         const int k_half = t.k_blocks / 2;
         for (int kb = 0; kb < t.k_blocks; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
@@ -830,10 +828,11 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       const uint32_t b_step = n_mn ? (2048u >> 4) : (32u >> 4);
       constexpr uint32_t SB16 = (uint32_t)Cfg::STAGE_BYTES >> 4;  // the whole ring stays below 256 KB: no carry out of the field
       uint32_t a_lo = a_lo0, b_lo = b_lo0, fbar = full_bar(0), ebar = empty_bar(0);
-      TcAsk ask = tc_ask(P, w0, total, tiles_m_dev, prank);
-      for (int w = w0; ok && crank == 0 && w < total; w += wstride, ++it) {
-        const TcTile t = tc_tile(P, ask, prank);
-        ask = tc_ask(P, w + wstride, total, tiles_m_dev, prank);
+      TcWalk walk;
+      walk.begin(P, w0, wstride, tiles_m_dev, prank);
+      for (; ok && crank == 0 && walk.left > 0; ++it) {
+        const TcTile t = tc_tile(P, walk, prank);
+        walk.step(P);
         const int acc = it & 1;
         const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
         if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
@@ -914,10 +913,11 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
     };
     SlabOut next_out;      // Adam, row-wise: the next tile's slab, whose first units this tile has asked for (primed)
     bool primed = false;
-    TcAsk ask = tc_ask(P, w0, total, tiles_m_dev, prank);
-    for (int w = w0; ok && w < total; w += wstride, ++it) {
-      const TcTile t = tc_tile(P, ask, prank);
-      ask = tc_ask(P, w + wstride, total, tiles_m_dev, prank);
+    TcWalk walk;
+    walk.begin(P, w0, wstride, tiles_m_dev, prank);
+    for (; ok && walk.left > 0; ++it) {
+      const TcTile t = tc_tile(P, walk, prank);
+      walk.step(P);
       const int acc = it & 1;
       const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
       const int m = t.m0 + row_in_tile;
@@ -1104,9 +1104,9 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
               const bool last = cb * 128 + 128 >= t.ncols;
               if (last) release();      // the tile's last columns are out of tensor memory
               if (last) {
-                primed = EPI == EPI_WADAM && w + wstride < total;
+                primed = EPI == EPI_WADAM && walk.left > 0;
                 if (primed) {
-                  const TcTile tn = tc_tile(P, ask, prank);
+                  const TcTile tn = tc_tile(P, walk, prank);
                   next_out = slab_of(tn);
                   primed = next_out.rows > 0;
                 }
