@@ -2,22 +2,21 @@
 //   O = softmax(scale * Q K^T, keys <= query position) V   per (sequence, head),
 // without materialising the score matrix.
 //
-// One CTA per (sequence, head, block of 128 query positions); it walks the key/value blocks
-// 0 .. its own diagonal block.  320 threads:
-//   warp 0      TMA producer: Q once, then K and V blocks into two-stage rings
-//   warp 1      MMA issuer and TMEM owner.  TMEM (512 columns): two score accumulators S0/S1 and two
-//               output accumulators O0/O1 of 128 fp32 columns each.
-//               S_j = Q K_j^T is issued one block ahead of O_j = P_j V_j, so the tensor pipe computes
-//               the next scores while the softmax warps work on the current ones.  P_j is the A operand
-//               of the second product straight from tensor memory.
-//   warps 2..9  softmax: two threads per query row (= TMEM lane), 64 keys each.  Per block: the scores
-//               into registers, row maximum (the halves exchange theirs through shared memory),
-//               p = exp2((s - m) * scale * log2 e), P as bf16 pairs over the first 64 columns of the
-//               score accumulator it came from (tcgen05.st; no shared-memory round trip, and the
-//               tensor core reads 4 KB less per instruction), then the PREVIOUS block's O_j (this
-//               thread's 64 columns) is added into a register accumulator,
-//               acc = acc * exp2((m_old - m_new) ...) + O_j.  Every O_j is a fresh TMEM accumulator, so
-//               no rescaling pass over TMEM is needed and P_j V_j never waits for a correction.
+// Forward: one CTA per (sequence, head, 256 query positions = two tiles of 128); it walks the key/value blocks
+// 0 .. the second tile's diagonal block.  320 threads:
+//   warp 0      TMA producer: the Q tiles once, then K and V blocks into two-stage rings, each used by both tiles
+//   warp 1      MMA issuer and TMEM owner.  TMEM (512 columns): a score and an output accumulator of 128 fp32
+//               columns for each tile.  Per block and tile: O += P_j V_j, then S_{j+1} = Q K_{j+1}^T over the scores that
+//               P_j came from.  While one tile's softmax runs, the tensor pipe works for the other.
+//   warps 2..9  softmax: four warps per tile, one thread per query row (= TMEM lane), all 128 scores of a block in
+//               registers: row maximum, p = exp2((s - m) * scale * log2 e), P as bf16 pairs over the first 64
+//               columns of the score accumulator, from where the second product takes it as its A operand.
+//               O stays in tensor memory.  The row's reference m follows the maximum only when that has grown by more
+//               than a factor 2^8 (p then stays below 2^8, exact in the same number of bits); the warp then rescales
+//               its rows of O, which is at rest: S_j complete means P_{j-1} V_{j-1} complete, both come from one
+//               in-order queue, and P_j V_j waits for this warp.
+// What bounds it: the exponentials (two warps per scheduler on a unit of four a clock: 2048 clk per block of both
+// tiles) beside as much tensor work.  FWDNUMS
 // Operands: q, k, v head-major [.., S_pad, hd] bf16 with hd = 128 (rows past the sequence are zero);
 // output token-major [T, ld_o] bf16, plus the row log-sum-exp (natural log, of the scaled scores).
 // Every wait is bounded; a wait that runs out sets the status word and all roles leave.
@@ -31,13 +30,12 @@ constexpr int FA_THREADS = 320;
 constexpr int FA_BLK = 128;                       // query rows per CTA and keys per block
 constexpr int FA_HD = 128;                        // head dimension
 constexpr int FA_TILE = FA_BLK * 64 * 2;          // one 64-wide K block of an operand tile: 16 KB
-constexpr int FA_Q_OFF = 0;                       // Q: 2 tiles
-constexpr int FA_K_OFF = 2 * FA_TILE;             // K: 2 stages x 2 tiles
+constexpr int FA_Q_OFF = 0;                       // Q: two query tiles of 2 tiles each
+constexpr int FA_K_OFF = 4 * FA_TILE;             // K: 2 stages x 2 tiles
 constexpr int FA_V_OFF = FA_K_OFF + 4 * FA_TILE;  // V: 2 stages x 2 k-blocks (each 2 chunks of 8 KB)
 constexpr int FA_BAR_OFF = FA_V_OFF + 4 * FA_TILE;
-constexpr int FA_XMAX_OFF = FA_BAR_OFF + 256;             // row maxima exchanged between the two halves: [2][2][128] floats
-constexpr int FA_XSUM_OFF = FA_XMAX_OFF + 2048;           // row sums exchanged at the end: [2][128] floats
-constexpr int FA_SMEM_BYTES = FA_XSUM_OFF + 1024 + 1024;  // + alignment slack
+constexpr int FA_SMEM_BYTES = FA_BAR_OFF + 256 + 1024;      // + alignment slack
+constexpr float FA_RESCALE_LOG2 = 8.f;            // growth of a row's maximum (log2) that its reference does not follow
 
 __device__ __forceinline__ float fa_exp2(float x) {
   float y;
@@ -45,36 +43,18 @@ __device__ __forceinline__ float fa_exp2(float x) {
   return y;
 }
 
-// Row maximum over this thread's 64 scores.  DIAG: the diagonal block, where key c of the block is masked
-// for query row `row` when c > row (col0 = first key of this thread's half).
-template <bool DIAG>
-__device__ __forceinline__ float fa_row_max(const uint32_t (&r0)[32], const uint32_t (&r1)[32], int col0, int row) {
-  float mx = -INFINITY;
+// p = exp2(s * cl - mc) for 64 scores of this thread's row, packed to bf16; returns their sum in two halves.
+__device__ __forceinline__ float2 fa_probs64(const uint32_t (&r0)[32], const uint32_t (&r1)[32], float cl, float mc, uint32_t (&pw)[32]) {
+  float2 sum = make_float2(0.f, 0.f);
+  const float2 c2 = make_float2(cl, cl), m2 = make_float2(-mc, -mc);
 #pragma unroll
   for (int i = 0; i < 32; ++i) {
-    if (!DIAG || col0 + i <= row) mx = fmaxf(mx, __uint_as_float(r0[i]));
-    if (!DIAG || col0 + 32 + i <= row) mx = fmaxf(mx, __uint_as_float(r1[i]));
-  }
-  return mx;
-}
-
-// p = exp2(s * cl - mc) for this thread's 64 scores, packed to bf16 (eight 16-byte pieces); returns their sum.
-template <bool DIAG>
-__device__ __forceinline__ float fa_probs(const uint32_t (&r0)[32], const uint32_t (&r1)[32], float cl, float mc, int col0,
-                                          int row, uint4 (&pk)[8]) {
-  float sum = 0.f;
-#pragma unroll
-  for (int g = 0; g < 8; ++g) {
-    float pv[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int kk = 8 * g + i;
-      float p = fa_exp2(__uint_as_float(kk < 32 ? r0[kk] : r1[kk - 32]) * cl - mc);
-      if (DIAG && col0 + kk > row) p = 0.f;
-      pv[i] = p;
-      sum += p;
-    }
-    pk[g] = pack8(pv);
+    const uint32_t* r = i < 16 ? &r0[2 * i] : &r1[2 * i - 32];
+    const float2 t = __ffma2_rn(make_float2(__uint_as_float(r[0]), __uint_as_float(r[1])), c2, m2);
+    const float2 e = make_float2(fa_exp2(t.x), fa_exp2(t.y));
+    sum = __fadd2_rn(sum, e);
+    const __nv_bfloat162 h = __floats2bfloat162_rn(e.x, e.y);
+    pw[i] = *reinterpret_cast<const uint32_t*>(&h);
   }
   return sum;
 }
@@ -119,22 +99,21 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
   const uint32_t bars = base + FA_BAR_OFF;
   // barrier slots (8 bytes each)
   auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
-  enum { B_QFULL = 0, B_KFULL = 1, B_KEMPTY = 3, B_VFULL = 5, B_VEMPTY = 7, B_SFULL = 9, B_SEMPTY = 11, B_PFULL = 13,
-         B_OFULL = 15, B_OEMPTY = 17, B_COUNT = 19 };
+  enum { B_QFULL = 0, B_KFULL = 1, B_KEMPTY = 3, B_VFULL = 5, B_VEMPTY = 7, B_SFULL = 9, B_PFULL = 11, B_OFULL = 13, B_DRAIN = 15,
+         B_COUNT = 16 };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen_base + FA_BAR_OFF + 8 * B_COUNT);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(gen_base + FA_BAR_OFF + 8 * B_COUNT + 8);
   int* issued = reinterpret_cast<int*>(gen_base + FA_BAR_OFF + 8 * B_COUNT + 16);   // [5]: q, k0, k1, v0, v1 -> phase + 1
-  float* xmax = reinterpret_cast<float*>(gen_base + FA_XMAX_OFF);
-  float* xsum = reinterpret_cast<float*>(gen_base + FA_XSUM_OFF);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_qblk = P.Sp / FA_BLK;
-  // heavy work first: the last query block of every (sequence, head) has the most key blocks
-  const int bh_count = (int)gridDim.x / n_qblk;
-  const int qblk = n_qblk - 1 - (int)blockIdx.x / bh_count;
+  const int n_qblk = P.Sp / FA_BLK, n_pair = (n_qblk + 1) / 2;
+  // heavy work first: the last query tiles of every (sequence, head) have the most key blocks
+  const int bh_count = (int)gridDim.x / n_pair;
+  const int qp = n_pair - 1 - (int)blockIdx.x / bh_count;
   const int bh = (int)blockIdx.x % bh_count;           // sequence * n_heads + head
-  const int n_blk = qblk + 1;
-  const int q_row0 = bh * P.Sp + qblk * FA_BLK;
+  const bool two = 2 * qp + 1 < n_qblk;                // the last pair of an odd number of tiles has one
+  const int n_blk = 2 * qp + (two ? 2 : 1);            // key blocks of the CTA; tile x needs 2 qp + x + 1 of them
+  const int q_row0 = bh * P.Sp + 2 * qp * FA_BLK;
   const int kv_row0 = (bh / P.rep) * P.Sp;             // (sequence * n_kv_heads + head / rep) * S_pad
 
   if (threadIdx.x == 0) {
@@ -142,9 +121,9 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
     for (int s = 0; s < 2; ++s) {
       mbar_init(bar(B_KFULL + s), 1); mbar_init(bar(B_KEMPTY + s), 1);
       mbar_init(bar(B_VFULL + s), 1); mbar_init(bar(B_VEMPTY + s), 1);
-      mbar_init(bar(B_SFULL + s), 1); mbar_init(bar(B_SEMPTY + s), 1); mbar_init(bar(B_PFULL + s), 8);
-      mbar_init(bar(B_OFULL + s), 1); mbar_init(bar(B_OEMPTY + s), 8);
+      mbar_init(bar(B_SFULL + s), 1); mbar_init(bar(B_PFULL + s), 4); mbar_init(bar(B_OFULL + s), 1);
     }
+    mbar_init(bar(B_DRAIN), 1);
     for (int i = 0; i < 5; ++i) issued[i] = 0;
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -160,6 +139,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // TMEM columns: scores of tile x at 128 x, output of tile x at 256 + 128 x
   // instruction descriptors: fp32 accumulate, bf16 operands, M = 128, N = 128; V is stored [key, hd] (N contiguous)
   const uint32_t idesc_qk = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(FA_BLK >> 3) << 17) | ((uint32_t)(FA_BLK >> 4) << 24);
   const uint32_t idesc_pv = idesc_qk | (1u << 16);
@@ -167,9 +147,11 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
   if (warp == 0) {
     // ------------------------------------------------------------------ producer
     if (lane == 0) {
-      mbar_expect_tx(bar(B_QFULL), 2 * FA_TILE);
+      const int nq = two ? 4 : 2;
+      mbar_expect_tx(bar(B_QFULL), nq * FA_TILE);
       issued[0] = 1;
-      for (int kb = 0; kb < 2; ++kb) tma_load_2d(base + FA_Q_OFF + kb * FA_TILE, &map_q, 64 * kb, q_row0, bar(B_QFULL));
+      for (int i = 0; i < nq; ++i)
+        tma_load_2d(base + FA_Q_OFF + i * FA_TILE, &map_q, 64 * (i & 1), q_row0 + (i >> 1) * FA_BLK, bar(B_QFULL));
       for (int j = 0; j < n_blk; ++j) {
         const int s = j & 1;
         const uint32_t ph = (uint32_t)(j >> 1) & 1u;
@@ -192,156 +174,171 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
     // ------------------------------------------------------------------ MMA issuer
     if (lane == 0) {
       bool ok = mbar_wait(bar(B_QFULL), 0u, abort_flag, P.status);
-      tc_fence_after();
-      auto issue_qk = [&](int j) -> bool {
+      // S_j of tile x; the block's K has been waited for
+      auto issue_qk = [&](int j, int x) {
         const int b = j & 1;
-        const uint32_t ph = (uint32_t)(j >> 1) & 1u;
-        if (!mbar_wait(bar(B_KFULL + b), ph, abort_flag, P.status)) return false;
-        if (!mbar_wait(bar(B_SEMPTY + b), ph ^ 1u, abort_flag, P.status)) return false;
-        tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)(b * FA_BLK);
 #pragma unroll
         for (int kb = 0; kb < 2; ++kb) {
-          const uint64_t a_desc = make_smem_desc(base + FA_Q_OFF + kb * FA_TILE, 16, 1024);
+          const uint64_t a_desc = make_smem_desc(base + FA_Q_OFF + (2 * x + kb) * FA_TILE, 16, 1024);
           const uint64_t b_desc = make_smem_desc(base + FA_K_OFF + (2 * b + kb) * FA_TILE, 16, 1024);
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks)
-            tc_mma(d, a_desc + (uint64_t)(2 * ks), b_desc + (uint64_t)(2 * ks), idesc_qk, (kb | ks) != 0 ? 1u : 0u);
+            tc_mma(tmem_base + (uint32_t)(128 * x), a_desc + (uint64_t)(2 * ks), b_desc + (uint64_t)(2 * ks), idesc_qk,
+                   (kb | ks) != 0 ? 1u : 0u);
         }
-        tc_commit(bar(B_KEMPTY + b));
-        tc_commit(bar(B_SFULL + b));
-        return true;
+        tc_commit(bar(B_SFULL + x));
       };
-      if (ok) ok = issue_qk(0);
+      if (ok) ok = mbar_wait(bar(B_KFULL), 0u, abort_flag, P.status);
+      if (ok) {
+        tc_fence_after();
+        issue_qk(0, 0);
+        if (two) issue_qk(0, 1);
+        tc_commit(bar(B_KEMPTY));
+      }
       for (int j = 0; ok && j < n_blk; ++j) {
-        if (j + 1 < n_blk && !issue_qk(j + 1)) { ok = false; break; }
         const int b = j & 1;
         const uint32_t ph = (uint32_t)(j >> 1) & 1u;
-        if (!mbar_wait(bar(B_VFULL + b), ph, abort_flag, P.status)) { ok = false; break; }
-        if (!mbar_wait(bar(B_OEMPTY + b), ph ^ 1u, abort_flag, P.status)) { ok = false; break; }
-        if (!mbar_wait(bar(B_PFULL + b), ph, abort_flag, P.status)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)(2 * FA_BLK + b * FA_BLK);
-        const uint32_t a_tmem = tmem_base + (uint32_t)(b * FA_BLK);      // P over the first 64 columns of S
+        bool have_k = false;
+        for (int x = 0; ok && x < (two ? 2 : 1); ++x) {
+          const int n_x = 2 * qp + x + 1;
+          if (j >= n_x) continue;
+          // P_j (its columns may then be read), and V_j once for both tiles
+          if (!mbar_wait(bar(B_PFULL + x), (uint32_t)j & 1u, abort_flag, P.status)) { ok = false; break; }
+          if (!mbar_wait(bar(B_VFULL + b), ph, abort_flag, P.status)) { ok = false; break; }
+          tc_fence_after();
 #pragma unroll
-        for (int kb = 0; kb < 2; ++kb) {
-          const uint64_t b_desc = make_smem_desc(base + FA_V_OFF + (2 * b + kb) * FA_TILE, 8192, 1024);
+          for (int kb = 0; kb < 2; ++kb) {
+            const uint64_t b_desc = make_smem_desc(base + FA_V_OFF + (2 * b + kb) * FA_TILE, 8192, 1024);
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks)
-            tc_mma_ta(d, a_tmem + (uint32_t)(8 * (4 * kb + ks)), b_desc + (uint64_t)(128 * ks), idesc_pv, (kb | ks) != 0 ? 1u : 0u);
+            for (int ks = 0; ks < 4; ++ks)
+              tc_mma_ta(tmem_base + (uint32_t)(256 + 128 * x), tmem_base + (uint32_t)(128 * x + 8 * (4 * kb + ks)),
+                        b_desc + (uint64_t)(128 * ks), idesc_pv, (j | kb | ks) != 0 ? 1u : 0u);
+          }
+          if (j + 1 == n_x) tc_commit(bar(B_OFULL + x));
+          if (j + 1 < n_x) {
+            if (!have_k) {
+              if (!mbar_wait(bar(B_KFULL + (b ^ 1)), (uint32_t)((j + 1) >> 1) & 1u, abort_flag, P.status)) { ok = false; break; }
+              tc_fence_after();
+              have_k = true;
+            }
+            issue_qk(j + 1, x);
+          }
         }
+        if (!ok) break;
         tc_commit(bar(B_VEMPTY + b));
-        tc_commit(bar(B_OFULL + b));
-        tc_commit(bar(B_SEMPTY + b));      // the scores' columns (now holding P) are free again
+        if (have_k) tc_commit(bar(B_KEMPTY + (b ^ 1)));
+      }
+      if (!ok) {
+        // an abandoned wait: products issued so far must have finished before the teardown frees what they use
+        tc_commit(bar(B_DRAIN));
+        const long long t0 = clock64();
+        while (!mbar_try_wait(bar(B_DRAIN), 0u) && clock64() - t0 < TC_WAIT_CYCLES) {}
       }
     }
   } else {
     // ------------------------------------------------------------------ softmax (warps 2..9)
-    // Two threads per query row: warps 2..5 take keys (and output columns) 0..63 of a block, warps 6..9
-    // take 64..127.  The two halves of a row exchange their maxima through shared memory once per block;
-    // every thread passes the named barrier in every iteration, also after an abandoned wait, so that
-    // nobody is left waiting at it.
     const int q = warp & 3;                      // TMEM lane quadrant this warp may access
-    const int half = (warp - 2) >> 2;
-    const int row = q * 32 + lane;               // query row within the block
-    const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(64 * half);
-    float acc[64];
-#pragma unroll
-    for (int i = 0; i < 64; ++i) acc[i] = 0.f;
-    float m = -INFINITY, l = 0.f, alpha_pending = 0.f;
+    const int x = (warp - 2) >> 2;               // query tile
+    const int row = q * 32 + lane;               // query row within the tile
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+    const uint32_t s_addr = lane_addr + (uint32_t)(128 * x), o_addr = lane_addr + (uint32_t)(256 + 128 * x);
+    const int n_x = (x == 0 || two) ? 2 * qp + x + 1 : 0;
+    float m = 0.f, l = 0.f;
     const float cl = P.scale_log2e;
     bool ok = true;
-    // acc = acc * alpha + O_j (this thread's 64 columns); the caller has seen O_j complete
-    auto add_block = [&](int j, float alpha) {
-      const int b = j & 1;
-      uint32_t r0[32], r1[32];
-      tmem_ld32(lane_addr + (uint32_t)(2 * FA_BLK + b * FA_BLK), r0);
-      tmem_ld32(lane_addr + (uint32_t)(2 * FA_BLK + b * FA_BLK + 32), r1);
+    for (int j = 0; j < n_x; ++j) {
+      ok = __all_sync(0xffffffffu, mbar_wait(bar(B_SFULL + x), (uint32_t)j & 1u, abort_flag, P.status));
+      if (!ok) break;
+      tc_fence_after();
+      uint32_t r0[32], r1[32], r2[32], r3[32];
+      tmem_ld32(s_addr, r0);
+      tmem_ld32(s_addr + 32, r1);
+      tmem_ld32(s_addr + 64, r2);
+      tmem_ld32(s_addr + 96, r3);
       tmem_ld_wait();
+      if (j + 1 == n_x) {      // the diagonal block: keys past the query position
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        acc[i] = acc[i] * alpha + __uint_as_float(r0[i]);
-        acc[32 + i] = acc[32 + i] * alpha + __uint_as_float(r1[i]);
+        for (int i = 0; i < 32; ++i) {
+          if (i > row) r0[i] = 0xff800000u;
+          if (32 + i > row) r1[i] = 0xff800000u;
+          if (64 + i > row) r2[i] = 0xff800000u;
+          if (96 + i > row) r3[i] = 0xff800000u;
+        }
       }
+      float a0 = __uint_as_float(r0[0]), a1 = __uint_as_float(r1[0]), a2 = __uint_as_float(r2[0]), a3 = __uint_as_float(r3[0]);
+#pragma unroll
+      for (int i = 1; i < 32; ++i) {
+        a0 = fmaxf(a0, __uint_as_float(r0[i])); a1 = fmaxf(a1, __uint_as_float(r1[i]));
+        a2 = fmaxf(a2, __uint_as_float(r2[i])); a3 = fmaxf(a3, __uint_as_float(r3[i]));
+      }
+      const float mx = fmaxf(fmaxf(a0, a1), fmaxf(a2, a3));
+      if (j == 0) {
+        m = mx;
+      } else if (__any_sync(0xffffffffu, (mx - m) * cl > FA_RESCALE_LOG2)) {
+        const float m_new = fmaxf(m, mx), alpha = fa_exp2((m - m_new) * cl);
+        l *= alpha;
+        m = m_new;
+#pragma unroll 1
+        for (int c = 0; c < 128; c += 32) {
+          uint32_t o[32];
+          tmem_ld32(o_addr + c, o);
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+          tmem_st32(o_addr + c, o);
+        }
+      }
+      const float mc = m * cl;
+      uint32_t pw[32];
+      const float2 s0 = fa_probs64(r0, r1, cl, mc, pw);
+      tmem_st32(s_addr, pw);
+      const float2 s1 = fa_probs64(r2, r3, cl, mc, pw);
+      tmem_st32(s_addr + 32, pw);
+      l += (s0.x + s0.y) + (s1.x + s1.y);
+      tmem_st_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(B_OEMPTY + b));
-    };
-    auto wait_o = [&](int j) -> bool {           // O_j = P_j V_j complete (P's buffer is free again)
-      if (!mbar_wait(bar(B_OFULL + (j & 1)), (uint32_t)(j >> 1) & 1u, abort_flag, P.status)) return false;
-      tc_fence_after();
-      return true;
-    };
-    for (int j = 0; j < n_blk; ++j) {
-      const int b = j & 1;
-      const uint32_t ph = (uint32_t)(j >> 1) & 1u;
-      const bool diag = j == qblk;               // keys past the query position exist only in the diagonal block
-      uint32_t r0[32], r1[32];
-      float mx = -INFINITY;
-      if (ok && !mbar_wait(bar(B_SFULL + b), ph, abort_flag, P.status)) ok = false;
-      if (ok) {
-        tc_fence_after();
-        tmem_ld32(lane_addr + (uint32_t)(b * FA_BLK), r0);
-        tmem_ld32(lane_addr + (uint32_t)(b * FA_BLK + 32), r1);
-        tmem_ld_wait();
-        mx = diag ? fa_row_max<true>(r0, r1, 64 * half, row) : fa_row_max<false>(r0, r1, 64 * half, row);
-        xmax[(b * 2 + half) * FA_BLK + row] = mx;
-      }
-      asm volatile("bar.sync 1, 256;" ::: "memory");
-      if (ok) {
-        const float m_new = fmaxf(m, fmaxf(mx, xmax[(b * 2 + (half ^ 1)) * FA_BLK + row]));
-        const float alpha = fa_exp2((m - m_new) * cl);        // first block: exp2(-inf) = 0
-        const float mc = m_new * cl;
-        uint4 pk[8];                             // this thread's 64 probabilities as bf16
-        const float sum = diag ? fa_probs<true>(r0, r1, cl, mc, 64 * half, row, pk)
-                               : fa_probs<false>(r0, r1, cl, mc, 64 * half, row, pk);
-        l = l * alpha + sum;
-        m = m_new;
-        {
-          // P over the scores in tensor memory: this thread's 64 keys are 32 columns of packed pairs.  Both halves
-          // of the row have their scores in registers (they met at the barrier above).
-          uint32_t pw[32];
-#pragma unroll
-          for (int g = 0; g < 8; ++g) { pw[4 * g] = pk[g].x; pw[4 * g + 1] = pk[g].y; pw[4 * g + 2] = pk[g].z; pw[4 * g + 3] = pk[g].w; }
-          tmem_st32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * FA_BLK + 32 * half), pw);
-          tmem_st_wait();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar(B_PFULL + b));
-          if (j >= 1 && !wait_o(j - 1)) ok = false;
-        }
-        if (ok) {
-          if (j >= 1) add_block(j - 1, alpha_pending);
-          alpha_pending = alpha;
-        }
-      }
+      if (lane == 0) mbar_arrive(bar(B_PFULL + x));
     }
-    if (ok) ok = wait_o(n_blk - 1);
-    if (ok) add_block(n_blk - 1, alpha_pending);
-    // the row's denominator is the sum of the two halves' partial sums (both are relative to the same maximum)
-    xsum[half * FA_BLK + row] = l;
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-    l += xsum[(half ^ 1) * FA_BLK + row];
-    const int s_pos = qblk * FA_BLK + row;
-    if (ok && s_pos < P.S) {
+    if (n_x > 0 && ok) ok = __all_sync(0xffffffffu, mbar_wait(bar(B_OFULL + x), 0u, abort_flag, P.status));
+    if (n_x > 0 && ok) {
+      tc_fence_after();
+      // out through this tile's Q area (its products are complete), 64- and 128-byte row pieces per instruction
+      const int s_pos0 = (2 * qp + x) * FA_BLK + q * 32, s_pos = s_pos0 + lane;
+      const int rows_ok = min(32, P.S - s_pos0);
       const float inv = 1.f / l;
       const int seq = bh / P.n_heads, head = bh % P.n_heads;
-      bf16* dst = P.o + ((int64_t)seq * P.S + s_pos) * P.ld_o + (int64_t)head * FA_HD + 64 * half;
+      uint8_t* stg = gen_base + FA_Q_OFF + x * 2 * FA_TILE + q * 8192;
+      bf16* dst = P.o + ((int64_t)seq * P.S + s_pos0) * P.ld_o + (int64_t)head * FA_HD;
+#pragma unroll 1
+      for (int c = 0; c < 128; c += 32) {
+        uint32_t o[32];
+        float f[32];
+        tmem_ld32(o_addr + c, o);
+        tmem_ld_wait();
 #pragma unroll
-      for (int g = 0; g < 8; ++g) {
-        float f[8];
+        for (int i = 0; i < 32; ++i) f[i] = __uint_as_float(o[i]) * inv;
+        stage32_bf16(stg, lane, f);
+        if (P.o32) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) f[i] = acc[8 * g + i] * inv;
-        *reinterpret_cast<uint4*>(dst + 8 * g) = pack8(f);
+          for (int g = 0; g < 8; ++g)
+            *reinterpret_cast<float4*>(stg + 4096 + lane * 128 + ((g ^ (lane & 7)) << 4)) =
+                make_float4(f[4 * g], f[4 * g + 1], f[4 * g + 2], f[4 * g + 3]);
+        }
+        __syncwarp();
+        blk_stage_to_global(stg, lane, dst + c, P.ld_o, rows_ok);
+        if (P.o32) {
+          float* d32 = P.o32 + ((int64_t)bh * P.Sp + s_pos0) * FA_HD + c;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int r = 4 * i + (lane >> 3);
+            const float4 v = *reinterpret_cast<const float4*>(stg + 4096 + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
+            if (r < rows_ok) *reinterpret_cast<float4*>(d32 + (int64_t)r * FA_HD + (lane & 7) * 4) = v;
+          }
+        }
+        __syncwarp();
       }
-      if (P.lse && half == 0) P.lse[(int64_t)bh * P.Sp + s_pos] = m * P.scale + logf(l);
-      if (P.o32) {
-        float* d32 = P.o32 + ((int64_t)bh * P.Sp + s_pos) * FA_HD + 64 * half;
-#pragma unroll
-        for (int g = 0; g < 16; ++g)
-          *reinterpret_cast<float4*>(d32 + 4 * g) =
-              make_float4(acc[4 * g] * inv, acc[4 * g + 1] * inv, acc[4 * g + 2] * inv, acc[4 * g + 3] * inv);
-      }
+      if (P.lse && lane < rows_ok) P.lse[(int64_t)bh * P.Sp + s_pos] = m * P.scale + logf(l);
     }
   }
 
@@ -391,7 +388,7 @@ inline int launch_flash_fwd(const bf16* q, const bf16* k, const bf16* v, int bat
   P.scale = 1.f / sqrtf((float)FA_HD);
   P.scale_log2e = P.scale * 1.4426950408889634f;
   P.status = status;
-  const int grid = batch * n_heads * (Sp / FA_BLK);
+  const int grid = batch * n_heads * ((Sp / FA_BLK + 1) / 2);
   launch_k(flash_fwd_kernel, grid, FA_THREADS, FA_SMEM_BYTES, st, P, mq, mk, mv);
   return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }

@@ -1,0 +1,43 @@
+"""The attention core at the edges of its query tiles, through the branch, against the oracle.
+
+A forward block holds two tiles of 128 query positions and walks the key blocks that they need: sequence lengths on
+both sides of one, two, three and four tiles (an odd number of tiles leaves the last block one), grouped key/value
+heads; and weights large enough that row maxima grow by more than 2^8 along the keys, which the softmax's running
+reference has to follow.  Tolerance: the path's stated 2e-2 (bf16 operands, P rounded to bf16, fp32 sums).  The scores
+have a standard deviation of (16 std)^2 sqrt(128) = 18.5 at std 0.08; q and k rounded to bf16 (2^-9 / sqrt(3) relative
+each) move a score by 18.5 * 2^-9 * sqrt(2/3) = 0.03 and so each unsaturated weight by 3 %, which the sum over keys
+brings below 2e-2; at std 0.12 it would be 6.6 %, too much for that tolerance whatever the kernel."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import revffn_attn_oracle as orc
+from workloads.generate import AttnConfig, make_attn_streams, make_attn_weights
+
+from helpers import dev, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("std", [0.05, 0.08])
+@pytest.mark.parametrize("seq_len", [1, 127, 128, 129, 256, 257, 384, 385, 512, 600])
+def test_forward_and_backward_at_tile_edges(seq_len, std):
+    import paper_2512_20920_b200 as rv
+    cfg = AttnConfig("edge", batch=2, seq_len=seq_len, d_model=512, n_heads=4, n_kv_heads=2, weight_dtype="bf16")
+    w, s = make_attn_weights(cfg, 5, std=std, bias_std=std), make_attn_streams(cfg, 5)
+    f32 = ("norm_gamma", "b_q", "b_k", "b_v")
+    dw = {n: torch.from_numpy(np.ascontiguousarray(v)).to("cuda", torch.float32 if n in f32 else torch.bfloat16) for n, v in w.items()}
+    br = rv.AttnBranch(batch=2, seq_len=seq_len, d_model=512, n_heads=4, n_kv_heads=2, weight_dtype=rv.BF16, weights=dw,
+                       norm_eps=cfg.norm_eps, rope_theta=cfg.rope_theta)
+    oa = dict(S=seq_len, n_heads=4, n_kv_heads=2, eps=cfg.norm_eps, theta=cfg.rope_theta)
+    x1, x2 = dev(s["x1"]), dev(s["x2"])
+    y1 = br.forward(x1, x2)
+    assert br.status() == 0
+    want = orc.forward(w, s["x1"], s["x2"], **oa) - s["x1"]
+    assert rel_l2(y1.cpu().numpy() - s["x1"], want) < 2e-2
+    if std < 0.06:
+        dx2 = torch.zeros_like(x2)
+        dx1 = br.backward(x1, x2, dev(s["dy1"]), dx2)
+        assert br.status() == 0
+        g1, g2, _ = orc.backward(w, s["x1"], s["x2"], s["dy1"], **oa)
+        assert rel_l2(dx1.cpu().numpy() - s["dy1"], g1 - s["dy1"]) < 2e-2 and rel_l2(dx2.cpu().numpy(), g2) < 2e-2
