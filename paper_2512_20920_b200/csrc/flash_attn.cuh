@@ -35,7 +35,7 @@ constexpr int FA_K_OFF = 4 * FA_TILE;             // K: 2 stages x 2 tiles
 constexpr int FA_V_OFF = FA_K_OFF + 4 * FA_TILE;  // V: 2 stages x 2 k-blocks (each 2 chunks of 8 KB)
 constexpr int FA_BAR_OFF = FA_V_OFF + 4 * FA_TILE;
 constexpr int FA_SMEM_BYTES = FA_BAR_OFF + 256 + 1024;      // + alignment slack
-constexpr float FA_RESCALE_LOG2 = 8.f;            // growth of a row's maximum (log2) that its reference does not follow
+constexpr float FA_SUM_MAX = 1048576.f;           // sum of a row's weights in a block above which the row's reference follows
 
 __device__ __forceinline__ float fa_exp2(float x) {
   float y;
@@ -80,6 +80,14 @@ __device__ __forceinline__ void tc_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
 }
 
+// One lane of a converged warp.  The issuing warp walks its loop with all lanes and elects one for each group of
+// instructions: a loop in one lane alone is divergent code, where every operand is moved to a uniform register first.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 struct FlashParams {
   int S, Sp, n_heads, rep;        // rep = query heads per key/value head
   bf16* o; int64_t ld_o;          // [T, ld_o]
@@ -105,7 +113,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
   volatile int* abort_flag = reinterpret_cast<volatile int*>(gen_base + FA_BAR_OFF + 8 * B_COUNT + 8);
   int* issued = reinterpret_cast<int*>(gen_base + FA_BAR_OFF + 8 * B_COUNT + 16);   // [5]: q, k0, k1, v0, v1 -> phase + 1
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int n_qblk = P.Sp / FA_BLK, n_pair = (n_qblk + 1) / 2;
   // heavy work first: the last query tiles of every (sequence, head) have the most key blocks
   const int bh_count = (int)gridDim.x / n_pair;
@@ -172,69 +180,72 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      bool ok = mbar_wait(bar(B_QFULL), 0u, abort_flag, P.status);
-      // S_j of tile x; the block's K has been waited for
-      auto issue_qk = [&](int j, int x) {
-        const int b = j & 1;
+    const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0), sb = __shfl_sync(0xffffffffu, base, 0);
+    auto wait = [&](int i, uint32_t parity) -> bool {
+      const bool got = __all_sync(0xffffffffu, mbar_wait(bar(i), parity, abort_flag, P.status));
+      tc_fence_after();
+      return got;
+    };
+    // S_j of tile x; the block's K has been waited for
+    auto issue_qk = [&](int j, int x) {
+      const uint64_t a_desc = make_smem_desc(sb + FA_Q_OFF + 2 * x * FA_TILE, 16, 1024);
+      const uint64_t b_desc = make_smem_desc(sb + FA_K_OFF + 2 * (j & 1) * FA_TILE, 16, 1024);
+      if (elect_one()) {
 #pragma unroll
-        for (int kb = 0; kb < 2; ++kb) {
-          const uint64_t a_desc = make_smem_desc(base + FA_Q_OFF + (2 * x + kb) * FA_TILE, 16, 1024);
-          const uint64_t b_desc = make_smem_desc(base + FA_K_OFF + (2 * b + kb) * FA_TILE, 16, 1024);
-#pragma unroll
-          for (int ks = 0; ks < 4; ++ks)
-            tc_mma(tmem_base + (uint32_t)(128 * x), a_desc + (uint64_t)(2 * ks), b_desc + (uint64_t)(2 * ks), idesc_qk,
-                   (kb | ks) != 0 ? 1u : 0u);
-        }
+        for (int k = 0; k < 8; ++k)       // two 16 KB tiles of 64 columns, 16 columns an instruction
+          tc_mma(tb + (uint32_t)(128 * x), a_desc + (uint64_t)((k >> 2) * (FA_TILE >> 4) + 2 * (k & 3)),
+                 b_desc + (uint64_t)((k >> 2) * (FA_TILE >> 4) + 2 * (k & 3)), idesc_qk, k != 0 ? 1u : 0u);
         tc_commit(bar(B_SFULL + x));
-      };
-      if (ok) ok = mbar_wait(bar(B_KFULL), 0u, abort_flag, P.status);
-      if (ok) {
-        tc_fence_after();
-        issue_qk(0, 0);
-        if (two) issue_qk(0, 1);
-        tc_commit(bar(B_KEMPTY));
       }
-      for (int j = 0; ok && j < n_blk; ++j) {
-        const int b = j & 1;
-        const uint32_t ph = (uint32_t)(j >> 1) & 1u;
-        bool have_k = false;
-        for (int x = 0; ok && x < (two ? 2 : 1); ++x) {
-          const int n_x = 2 * qp + x + 1;
-          if (j >= n_x) continue;
-          // P_j (its columns may then be read), and V_j once for both tiles
-          if (!mbar_wait(bar(B_PFULL + x), (uint32_t)j & 1u, abort_flag, P.status)) { ok = false; break; }
-          if (!mbar_wait(bar(B_VFULL + b), ph, abort_flag, P.status)) { ok = false; break; }
-          tc_fence_after();
+      __syncwarp();
+    };
+    auto commit = [&](int i) {
+      if (elect_one()) tc_commit(bar(i));
+      __syncwarp();
+    };
+    bool ok = wait(B_QFULL, 0u);
+    if (ok) ok = wait(B_KFULL, 0u);
+    if (ok) {
+      issue_qk(0, 0);
+      if (two) issue_qk(0, 1);
+      commit(B_KEMPTY);
+    }
+    for (int j = 0; ok && j < n_blk; ++j) {
+      const int b = j & 1;
+      const uint32_t ph = (uint32_t)(j >> 1) & 1u;
+      const bool more = j + 1 < n_blk;
+      if (!(ok = wait(B_VFULL + b, ph))) break;                                    // V_j and K_{j+1}, once for both tiles
+      if (more && !(ok = wait(B_KFULL + (b ^ 1), (uint32_t)((j + 1) >> 1) & 1u))) break;
 #pragma unroll
-          for (int kb = 0; kb < 2; ++kb) {
-            const uint64_t b_desc = make_smem_desc(base + FA_V_OFF + (2 * b + kb) * FA_TILE, 8192, 1024);
+      for (int x = 0; x < 2; ++x) {
+        const int n_x = (x == 0 || two) ? 2 * qp + x + 1 : 0;
+        if (j < n_x && ok) {
+          ok = wait(B_PFULL + x, (uint32_t)j & 1u);                                // P_j: its columns may be read
+          if (ok) {
+            const uint64_t b_desc = make_smem_desc(sb + FA_V_OFF + 2 * b * FA_TILE, 8192, 1024);
+            if (elect_one()) {
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-              tc_mma_ta(tmem_base + (uint32_t)(256 + 128 * x), tmem_base + (uint32_t)(128 * x + 8 * (4 * kb + ks)),
-                        b_desc + (uint64_t)(128 * ks), idesc_pv, (j | kb | ks) != 0 ? 1u : 0u);
-          }
-          if (j + 1 == n_x) tc_commit(bar(B_OFULL + x));
-          if (j + 1 < n_x) {
-            if (!have_k) {
-              if (!mbar_wait(bar(B_KFULL + (b ^ 1)), (uint32_t)((j + 1) >> 1) & 1u, abort_flag, P.status)) { ok = false; break; }
-              tc_fence_after();
-              have_k = true;
+              for (int k = 0; k < 8; ++k)
+                tc_mma_ta(tb + (uint32_t)(256 + 128 * x), tb + (uint32_t)(128 * x + 8 * k),
+                          b_desc + (uint64_t)((k >> 2) * (FA_TILE >> 4) + 128 * (k & 3)), idesc_pv, (j | k) != 0 ? 1u : 0u);
+              if (j + 1 == n_x) tc_commit(bar(B_OFULL + x));
             }
-            issue_qk(j + 1, x);
+            __syncwarp();
+            if (j + 1 < n_x) issue_qk(j + 1, x);
           }
         }
-        if (!ok) break;
-        tc_commit(bar(B_VEMPTY + b));
-        if (have_k) tc_commit(bar(B_KEMPTY + (b ^ 1)));
       }
-      if (!ok) {
-        // an abandoned wait: products issued so far must have finished before the teardown frees what they use
-        tc_commit(bar(B_DRAIN));
-        const long long t0 = clock64();
-        while (!mbar_try_wait(bar(B_DRAIN), 0u) && clock64() - t0 < TC_WAIT_CYCLES) {}
-      }
+      if (!ok) break;
+      commit(B_VEMPTY + b);
+      if (more) commit(B_KEMPTY + (b ^ 1));
     }
+    if (!ok) {
+      // an abandoned wait: products issued so far must have finished before the teardown frees what they use
+      commit(B_DRAIN);
+      const long long t0 = clock64();
+      while (!mbar_try_wait(bar(B_DRAIN), 0u) && clock64() - t0 < TC_WAIT_CYCLES) {}
+    }
+    __syncwarp();
   } else {
     // ------------------------------------------------------------------ softmax (warps 2..9)
     const int q = warp & 3;                      // TMEM lane quadrant this warp may access
@@ -243,58 +254,63 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     const uint32_t s_addr = lane_addr + (uint32_t)(128 * x), o_addr = lane_addr + (uint32_t)(256 + 128 * x);
     const int n_x = (x == 0 || two) ? 2 * qp + x + 1 : 0;
-    float m = 0.f, l = 0.f;
+    float m = -INFINITY, l = 0.f;
     const float cl = P.scale_log2e;
     bool ok = true;
     for (int j = 0; j < n_x; ++j) {
       ok = __all_sync(0xffffffffu, mbar_wait(bar(B_SFULL + x), (uint32_t)j & 1u, abort_flag, P.status));
       if (!ok) break;
       tc_fence_after();
-      uint32_t r0[32], r1[32], r2[32], r3[32];
-      tmem_ld32(s_addr, r0);
-      tmem_ld32(s_addr + 32, r1);
-      tmem_ld32(s_addr + 64, r2);
-      tmem_ld32(s_addr + 96, r3);
-      tmem_ld_wait();
-      if (j + 1 == n_x) {      // the diagonal block: keys past the query position
+      uint32_t p0[32], p1[32];
+      float sum;
+      bool ref = j == 0;        // take the reference from this block's maxima
+      while (true) {
+        uint32_t r0[32], r1[32], r2[32], r3[32];
+        tmem_ld32(s_addr, r0);
+        tmem_ld32(s_addr + 32, r1);
+        tmem_ld32(s_addr + 64, r2);
+        tmem_ld32(s_addr + 96, r3);
+        tmem_ld_wait();
+        if (j + 1 == n_x) {      // the diagonal block: keys past the query position
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          if (i > row) r0[i] = 0xff800000u;
-          if (32 + i > row) r1[i] = 0xff800000u;
-          if (64 + i > row) r2[i] = 0xff800000u;
-          if (96 + i > row) r3[i] = 0xff800000u;
+          for (int i = 0; i < 32; ++i) {
+            if (i > row) r0[i] = 0xff800000u;
+            if (32 + i > row) r1[i] = 0xff800000u;
+            if (64 + i > row) r2[i] = 0xff800000u;
+            if (96 + i > row) r3[i] = 0xff800000u;
+          }
         }
-      }
-      float a0 = __uint_as_float(r0[0]), a1 = __uint_as_float(r1[0]), a2 = __uint_as_float(r2[0]), a3 = __uint_as_float(r3[0]);
+        if (ref) {
+          float a0 = m, a1 = m, a2 = m, a3 = m;
 #pragma unroll
-      for (int i = 1; i < 32; ++i) {
-        a0 = fmaxf(a0, __uint_as_float(r0[i])); a1 = fmaxf(a1, __uint_as_float(r1[i]));
-        a2 = fmaxf(a2, __uint_as_float(r2[i])); a3 = fmaxf(a3, __uint_as_float(r3[i]));
-      }
-      const float mx = fmaxf(fmaxf(a0, a1), fmaxf(a2, a3));
-      if (j == 0) {
-        m = mx;
-      } else if (__any_sync(0xffffffffu, (mx - m) * cl > FA_RESCALE_LOG2)) {
-        const float m_new = fmaxf(m, mx), alpha = fa_exp2((m - m_new) * cl);
-        l *= alpha;
-        m = m_new;
+          for (int i = 0; i < 32; ++i) {
+            a0 = fmaxf(a0, __uint_as_float(r0[i])); a1 = fmaxf(a1, __uint_as_float(r1[i]));
+            a2 = fmaxf(a2, __uint_as_float(r2[i])); a3 = fmaxf(a3, __uint_as_float(r3[i]));
+          }
+          const float m_new = fmaxf(fmaxf(a0, a1), fmaxf(a2, a3));
+          if (j > 0) {
+            const float alpha = fa_exp2((m - m_new) * cl);
+            l *= alpha;
 #pragma unroll 1
-        for (int c = 0; c < 128; c += 32) {
-          uint32_t o[32];
-          tmem_ld32(o_addr + c, o);
-          tmem_ld_wait();
+            for (int c = 0; c < 128; c += 32) {
+              uint32_t o[32];
+              tmem_ld32(o_addr + c, o);
+              tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-          tmem_st32(o_addr + c, o);
+              for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+              tmem_st32(o_addr + c, o);
+            }
+          }
+          m = m_new;
         }
+        const float2 s0 = fa_probs64(r0, r1, cl, m * cl, p0), s1 = fa_probs64(r2, r3, cl, m * cl, p1);
+        sum = (s0.x + s0.y) + (s1.x + s1.y);
+        if (ref || !__any_sync(0xffffffffu, !(sum <= FA_SUM_MAX))) break;
+        ref = true;
       }
-      const float mc = m * cl;
-      uint32_t pw[32];
-      const float2 s0 = fa_probs64(r0, r1, cl, mc, pw);
-      tmem_st32(s_addr, pw);
-      const float2 s1 = fa_probs64(r2, r3, cl, mc, pw);
-      tmem_st32(s_addr + 32, pw);
-      l += (s0.x + s0.y) + (s1.x + s1.y);
+      tmem_st32(s_addr, p0);
+      tmem_st32(s_addr + 32, p1);
+      l += sum;
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
@@ -496,7 +512,7 @@ flash_bwd_dkv_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap
   volatile int* abort_flag = reinterpret_cast<volatile int*>(gen_base + FB_BAR_OFF + 8 * B_COUNT + 8);
   int* issued = reinterpret_cast<int*>(gen_base + FB_BAR_OFF + 8 * B_COUNT + 16);   // [1 + NS]: x, y stages -> phase + 1
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int n_blk = P.Sp / FA_BLK;                  // 128-row blocks per head
   const int n_t64 = P.Sp / 64;                      // 64-row tiles per head
   // heavy work first: low key blocks see the most query tiles
@@ -564,57 +580,54 @@ flash_bwd_dkv_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      bool ok = mbar_wait(bar(B_XFULL), 0u, abort_flag, P.status);
+    const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0), sb = __shfl_sync(0xffffffffu, base, 0);
+    auto wait = [&](int i, uint32_t parity) -> bool {
+      const bool got = __all_sync(0xffffffffu, mbar_wait(bar(i), parity, abort_flag, P.status));
       tc_fence_after();
-      auto issue_sd = [&](int s) -> bool {
-        const int b = s & 1, st = s % NS;
-        const uint32_t ph = (uint32_t)(s >> 1) & 1u;
-        if (!mbar_wait(bar(B_YFULL + st), (uint32_t)(s / NS) & 1u, abort_flag, P.status)) return false;
-        if (!mbar_wait(bar(B_SDEMPTY + b), ph ^ 1u, abort_flag, P.status)) return false;
-        tc_fence_after();
-        const uint32_t ys = base + Y_OFF + st * FB_STAGE;
+      return got;
+    };
+    bool ok = wait(B_XFULL, 0u);
+    auto issue_sd = [&](int s) -> bool {
+      const int b = s & 1, st = s % NS;
+      const uint32_t ph = (uint32_t)(s >> 1) & 1u;
+      if (!wait(B_YFULL + st, (uint32_t)(s / NS) & 1u)) return false;
+      if (!wait(B_SDEMPTY + b, ph ^ 1u)) return false;
+      const uint64_t a_desc = make_smem_desc(sb + FB_X_OFF, 16, 1024);
+      const uint64_t b_desc = make_smem_desc(sb + Y_OFF + st * FB_STAGE, 16, 1024);
+      if (elect_one()) {
 #pragma unroll
         for (int w = 0; w < 2; ++w) {            // w = 0: S' = X0 Y0^T, w = 1: dP' = X1 Y1^T
-          const uint32_t d = tmem_base + (uint32_t)(b * 128 + w * 64);
 #pragma unroll
-          for (int kb = 0; kb < 2; ++kb) {
-            const uint64_t a_desc = make_smem_desc(base + FB_X_OFF + (2 * w + kb) * FA_TILE, 16, 1024);
-            const uint64_t b_desc = make_smem_desc(ys + w * FA_TILE + kb * 8192, 16, 1024);
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-              tc_mma(d, a_desc + (uint64_t)(2 * ks), b_desc + (uint64_t)(2 * ks), idesc_sd, (kb | ks) != 0 ? 1u : 0u);
-          }
+          for (int k = 0; k < 8; ++k)            // 64-column tiles of 16 KB (X) and 8 KB (Y), 16 columns an instruction
+            tc_mma(tb + (uint32_t)(b * 128 + w * 64), a_desc + (uint64_t)((2 * w + (k >> 2)) * (FA_TILE >> 4) + 2 * (k & 3)),
+                   b_desc + (uint64_t)((2 * w + (k >> 2)) * (8192 >> 4) + 2 * (k & 3)), idesc_sd, k != 0 ? 1u : 0u);
         }
         tc_commit(bar(B_SDFULL + b));
-        return true;
-      };
-      if (ok) ok = issue_sd(0);
-      for (int s = 0; ok && s < n_steps; ++s) {
-        if (s + 1 < n_steps && !issue_sd(s + 1)) { ok = false; break; }
-        const int st = s % NS;
-        if (!mbar_wait(bar(B_PDFULL), (uint32_t)s & 1u, abort_flag, P.status)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t ys = base + Y_OFF + st * FB_STAGE;
-        // the walked tiles again, now as [64 rows (K), 128 columns (N)] operands: the two 64-column halves are 8 KB apart
-        {
-          const uint64_t a_desc = make_smem_desc(base + FB_P_OFF, 16, 1024);
-          const uint64_t b_desc = make_smem_desc(ys + FA_TILE, 8192, 1024);
+      }
+      __syncwarp();
+      return true;
+    };
+    if (ok) ok = issue_sd(0);
+    for (int s = 0; ok && s < n_steps; ++s) {
+      if (s + 1 < n_steps && !issue_sd(s + 1)) { ok = false; break; }
+      const int st = s % NS;
+      if (!(ok = wait(B_PDFULL, (uint32_t)s & 1u))) break;
+      // the walked tiles again, now as [64 rows (K), 128 columns (N)] operands: the two 64-column halves are 8 KB apart
+      const uint64_t a_desc = make_smem_desc(sb + FB_P_OFF, 16, 1024);
+      const uint64_t b_desc = make_smem_desc(sb + Y_OFF + st * FB_STAGE, 8192, 1024);
+      if (elect_one()) {
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks)
-            tc_mma(tmem_base + 256u, a_desc + (uint64_t)(2 * ks), b_desc + (uint64_t)(128 * ks), idesc_acc, (s | ks) != 0 ? 1u : 0u);
-        }
-        {
-          const uint64_t a_desc = make_smem_desc(base + FB_DS_OFF, 16, 1024);
-          const uint64_t b_desc = make_smem_desc(ys, 8192, 1024);
+        for (int ks = 0; ks < 4; ++ks)
+          tc_mma(tb + 256u, a_desc + (uint64_t)(2 * ks), b_desc + (uint64_t)((FA_TILE >> 4) + 128 * ks), idesc_acc, (s | ks) != 0 ? 1u : 0u);
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks)
-            tc_mma(tmem_base + 384u, a_desc + (uint64_t)(2 * ks), b_desc + (uint64_t)(128 * ks), idesc_acc, (s | ks) != 0 ? 1u : 0u);
-        }
+        for (int ks = 0; ks < 4; ++ks)
+          tc_mma(tb + 384u, a_desc + (uint64_t)(((FB_DS_OFF - FB_P_OFF) >> 4) + 2 * ks), b_desc + (uint64_t)(128 * ks), idesc_acc,
+                 (s | ks) != 0 ? 1u : 0u);
         tc_commit(bar(B_YEMPTY + st));
         tc_commit(bar(B_PDEMPTY));
+        if (s + 1 == n_steps) tc_commit(bar(B_ACCFULL));
       }
-      if (ok) tc_commit(bar(B_ACCFULL));
+      __syncwarp();
     }
   } else {
     // ------------------------------------------------------------------ P' / dS' (warps 2..9)
@@ -745,7 +758,7 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
   volatile int* abort_flag = reinterpret_cast<volatile int*>(gen_base + FQ_BAR_OFF + 8 * B_COUNT + 8);
   int* issued = reinterpret_cast<int*>(gen_base + FQ_BAR_OFF + 8 * B_COUNT + 16);   // [FQ_NS]: stage -> phase + 1
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int n_blk = P.Sp / FA_BLK;
   const int per = (int)gridDim.x / n_blk;
   const int blk = n_blk - 1 - (int)blockIdx.x / per;     // heavy work first: high query blocks see the most key tiles
@@ -798,46 +811,49 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      bool ok = mbar_wait(bar(B_XFULL), 0u, abort_flag, P.status);
+    const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0), sb = __shfl_sync(0xffffffffu, base, 0);
+    auto wait = [&](int i, uint32_t parity) -> bool {
+      const bool got = __all_sync(0xffffffffu, mbar_wait(bar(i), parity, abort_flag, P.status));
       tc_fence_after();
-      auto issue_sd = [&](int s) -> bool {
-        const int st = s % FQ_NS;
-        if (!mbar_wait(bar(B_YFULL + st), (uint32_t)(s / FQ_NS) & 1u, abort_flag, P.status)) return false;
-        if (!mbar_wait(bar(B_SDEMPTY), ((uint32_t)s & 1u) ^ 1u, abort_flag, P.status)) return false;
-        tc_fence_after();
-        const uint32_t ys = base + st * FQ_STAGE;
+      return got;
+    };
+    bool ok = wait(B_XFULL, 0u);
+    auto issue_sd = [&](int s) -> bool {
+      const int st = s % FQ_NS;
+      if (!wait(B_YFULL + st, (uint32_t)(s / FQ_NS) & 1u)) return false;
+      if (!wait(B_SDEMPTY, ((uint32_t)s & 1u) ^ 1u)) return false;
+      const uint64_t b_desc = make_smem_desc(sb + st * FQ_STAGE, 16, 1024);
+      if (elect_one()) {
 #pragma unroll
         for (int w = 0; w < 2; ++w) {            // w = 0: S' = Q_i K_t^T, w = 1: dP' = dO_i V_t^T
 #pragma unroll
-          for (int kb = 0; kb < 2; ++kb) {
-            const uint64_t b_desc = make_smem_desc(ys + (2 * w + kb) * FA_TILE, 16, 1024);
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-              tc_mma_ta(tmem_base + (uint32_t)(128 * w), tmem_base + (uint32_t)(256 + 64 * w + 8 * (4 * kb + ks)),
-                        b_desc + (uint64_t)(2 * ks), idesc_sd, (kb | ks) != 0 ? 1u : 0u);
-          }
+          for (int k = 0; k < 8; ++k)
+            tc_mma_ta(tb + (uint32_t)(128 * w), tb + (uint32_t)(256 + 64 * w + 8 * k),
+                      b_desc + (uint64_t)((2 * w + (k >> 2)) * (FA_TILE >> 4) + 2 * (k & 3)), idesc_sd, k != 0 ? 1u : 0u);
         }
         tc_commit(bar(B_SDFULL));
-        return true;
-      };
-      if (ok) ok = issue_sd(0);
-      for (int s = 0; ok && s < n_steps; ++s) {
-        if (s + 1 < n_steps && !issue_sd(s + 1)) { ok = false; break; }
-        const int st = s % FQ_NS;
-        if (!mbar_wait(bar(B_PDFULL), (uint32_t)s & 1u, abort_flag, P.status)) { ok = false; break; }
-        tc_fence_after();
-        // dQ += dS' K_t: K_t's two 64-column tiles read as one [128 keys, 128 columns] operand, halves 16 KB apart
-        const uint64_t b_desc = make_smem_desc(base + st * FQ_STAGE, 2 * 8192, 1024);
+      }
+      __syncwarp();
+      return true;
+    };
+    if (ok) ok = issue_sd(0);
+    for (int s = 0; ok && s < n_steps; ++s) {
+      if (s + 1 < n_steps && !issue_sd(s + 1)) { ok = false; break; }
+      const int st = s % FQ_NS;
+      if (!(ok = wait(B_PDFULL, (uint32_t)s & 1u))) break;
+      // dQ += dS' K_t: K_t's two 64-column tiles read as one [128 keys, 128 columns] operand, halves 16 KB apart
+      const uint64_t a_desc = make_smem_desc(sb + FQ_DS_OFF, 16, 1024);
+      const uint64_t b_desc = make_smem_desc(sb + st * FQ_STAGE, 2 * 8192, 1024);
+      if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const uint64_t a_desc = make_smem_desc(base + FQ_DS_OFF + (kk >> 2) * FA_TILE, 16, 1024);
-          tc_mma(tmem_base + 384u, a_desc + (uint64_t)(2 * (kk & 3)), b_desc + (uint64_t)(128 * kk), idesc_acc, (s | kk) != 0 ? 1u : 0u);
-        }
+        for (int k = 0; k < 8; ++k)
+          tc_mma(tb + 384u, a_desc + (uint64_t)((k >> 2) * (FA_TILE >> 4) + 2 * (k & 3)), b_desc + (uint64_t)(128 * k), idesc_acc,
+                 (s | k) != 0 ? 1u : 0u);
         tc_commit(bar(B_YEMPTY + st));
         tc_commit(bar(B_PDEMPTY));
+        if (s + 1 == n_steps) tc_commit(bar(B_ACCFULL));
       }
-      if (ok) tc_commit(bar(B_ACCFULL));
+      __syncwarp();
     }
   } else {
     // ------------------------------------------------------------------ dS' (warps 2..9)
