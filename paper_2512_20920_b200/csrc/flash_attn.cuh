@@ -80,14 +80,6 @@ __device__ __forceinline__ void tc_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
 }
 
-// One lane of a converged warp.  The issuing warp walks its loop with all lanes and elects one for each group of
-// instructions: a loop in one lane alone is divergent code, where every operand is moved to a uniform register first.
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
-}
-
 struct FlashParams {
   int S, Sp, n_heads, rep;        // rep = query heads per key/value head
   bf16* o; int64_t ld_o;          // [T, ld_o]
@@ -182,7 +174,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
     // ------------------------------------------------------------------ MMA issuer
     const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0), sb = __shfl_sync(0xffffffffu, base, 0);
     auto wait = [&](int i, uint32_t parity) -> bool {
-      const bool got = __all_sync(0xffffffffu, mbar_wait(bar(i), parity, abort_flag, P.status));
+      const bool got = mbar_wait_warp(bar(i), parity, abort_flag, P.status);
       tc_fence_after();
       return got;
     };
@@ -582,7 +574,7 @@ flash_bwd_dkv_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap
     // ------------------------------------------------------------------ MMA issuer
     const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0), sb = __shfl_sync(0xffffffffu, base, 0);
     auto wait = [&](int i, uint32_t parity) -> bool {
-      const bool got = __all_sync(0xffffffffu, mbar_wait(bar(i), parity, abort_flag, P.status));
+      const bool got = mbar_wait_warp(bar(i), parity, abort_flag, P.status);
       tc_fence_after();
       return got;
     };
@@ -813,7 +805,7 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
     // ------------------------------------------------------------------ MMA issuer
     const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0), sb = __shfl_sync(0xffffffffu, base, 0);
     auto wait = [&](int i, uint32_t parity) -> bool {
-      const bool got = __all_sync(0xffffffffu, mbar_wait(bar(i), parity, abort_flag, P.status));
+      const bool got = mbar_wait_warp(bar(i), parity, abort_flag, P.status);
       tc_fence_after();
       return got;
     };

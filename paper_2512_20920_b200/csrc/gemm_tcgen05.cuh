@@ -140,6 +140,20 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// The same for a whole warp that stays converged (the result is the same in every lane).
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
+                                               long long limit = TC_WAIT_CYCLES) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, limit));
+}
+// One lane of a converged warp.  The issuing warp walks its loop with all lanes and elects one for each group of
+// instructions: a loop in one lane alone is divergent code, where every operand is moved to a uniform register first.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
@@ -606,7 +620,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
   int* issued = reinterpret_cast<int*>(tmem_slot + 2);   // [STAGES] parity+1 of the last load issued per stage
   int* issued_b = issued + Cfg::STAGES;                  // the same for the second load warp: nonzero once it has issued
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int crank = PAIR ? (int)cluster_ctarank() : 0;     // rank in the pair; rank 0 issues the MMAs
   const int prank = PAIR ? crank : -1;
   const int w0 = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;       // first tile and tile stride of this CTA / pair
@@ -813,15 +827,16 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
     // 60, against 512 clocks of tensor work in a 128 x 256 x 64 step.  Everything that does not change inside a
     // tile (descriptor high words, layout steps, barrier addresses) is therefore set up outside the loop, and a
     // K step costs the wait, two additions, the four products and the commit.
-    if (lane == 0) {
+    if (crank == 0) {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
       int it = 0;
       // the M-side slot holds A (or, transposed, the weights B); the N-side slot the other operand
       const int m_mn = P.tr ? p.b_mn_major : p.a_mn_major, n_mn = P.tr ? p.a_mn_major : p.b_mn_major;
-      const uint64_t a_desc0 = m_mn ? make_smem_desc(base, 8192, 1024) : make_smem_desc(base, 16, 1024);
-      const uint64_t b_desc0 = n_mn ? make_smem_desc(base + TC_A_BYTES, 8192, 1024) : make_smem_desc(base + TC_A_BYTES, 16, 1024);
+      const uint32_t sb = __shfl_sync(0xffffffffu, base, 0), tb = __shfl_sync(0xffffffffu, tmem_base, 0);
+      const uint64_t a_desc0 = m_mn ? make_smem_desc(sb, 8192, 1024) : make_smem_desc(sb, 16, 1024);
+      const uint64_t b_desc0 = n_mn ? make_smem_desc(sb + TC_A_BYTES, 8192, 1024) : make_smem_desc(sb + TC_A_BYTES, 16, 1024);
       const uint32_t a_hi = (uint32_t)(a_desc0 >> 32), b_hi = (uint32_t)(b_desc0 >> 32);
       const uint32_t a_lo0 = (uint32_t)a_desc0, b_lo0 = (uint32_t)b_desc0;    // address field (bits 0..13, 16-byte units) + leading offset
       const uint32_t a_step = m_mn ? (2048u >> 4) : (32u >> 4);   // 16 k-elements per instruction
@@ -830,44 +845,49 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       uint32_t a_lo = a_lo0, b_lo = b_lo0, fbar = full_bar(0), ebar = empty_bar(0);
       TcWalk walk;
       walk.begin(P, w0, wstride, tiles_m_dev, prank);
-      for (; ok && crank == 0 && walk.left > 0; ++it) {
+      for (; ok && walk.left > 0; ++it) {
         const TcTile t = tc_tile(P, walk, prank);
         walk.step(P);
         const int acc = it & 1;
         const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
-        if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
+        if (!mbar_wait_warp(tempty_bar(acc), acc_phase ^ 1u, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * MMA_N);
+        const uint32_t d_tmem = tb + (uint32_t)(acc * MMA_N);
         const uint32_t idesc = (P.idesc & ~(0x3Fu << 17)) | ((uint32_t)(t.ncols >> 3) << 17);   // N of this tile
         const int nk = t.k_blocks;
         for (int kb = 0; kb < nk; ++kb) {
-          if (!mbar_wait(fbar, phase, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
+          if (!mbar_wait_warp(fbar, phase, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
           tc_fence_after();
-          if (p.fp8) {
-            tc_mma_lohi_f8<PAIR>(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, kb != 0 ? 1u : 0u);
-            tc_mma_lohi_f8<PAIR>(d_tmem, a_lo + a_step, a_hi, b_lo + b_step, b_hi, idesc, 1u);
-            tc_mma_lohi_f8<PAIR>(d_tmem, a_lo + 2 * a_step, a_hi, b_lo + 2 * b_step, b_hi, idesc, 1u);
-            tc_mma_lohi_f8<PAIR>(d_tmem, a_lo + 3 * a_step, a_hi, b_lo + 3 * b_step, b_hi, idesc, 1u);
-          } else {
-            tc_mma_lohi<PAIR>(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, kb != 0 ? 1u : 0u);
-            tc_mma_lohi<PAIR>(d_tmem, a_lo + a_step, a_hi, b_lo + b_step, b_hi, idesc, 1u);
-            tc_mma_lohi<PAIR>(d_tmem, a_lo + 2 * a_step, a_hi, b_lo + 2 * b_step, b_hi, idesc, 1u);
-            tc_mma_lohi<PAIR>(d_tmem, a_lo + 3 * a_step, a_hi, b_lo + 3 * b_step, b_hi, idesc, 1u);
+          if (elect_one()) {
+            if (p.fp8) {
+              tc_mma_lohi_f8<PAIR>(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, kb != 0 ? 1u : 0u);
+              tc_mma_lohi_f8<PAIR>(d_tmem, a_lo + a_step, a_hi, b_lo + b_step, b_hi, idesc, 1u);
+              tc_mma_lohi_f8<PAIR>(d_tmem, a_lo + 2 * a_step, a_hi, b_lo + 2 * b_step, b_hi, idesc, 1u);
+              tc_mma_lohi_f8<PAIR>(d_tmem, a_lo + 3 * a_step, a_hi, b_lo + 3 * b_step, b_hi, idesc, 1u);
+            } else {
+              tc_mma_lohi<PAIR>(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, kb != 0 ? 1u : 0u);
+              tc_mma_lohi<PAIR>(d_tmem, a_lo + a_step, a_hi, b_lo + b_step, b_hi, idesc, 1u);
+              tc_mma_lohi<PAIR>(d_tmem, a_lo + 2 * a_step, a_hi, b_lo + 2 * b_step, b_hi, idesc, 1u);
+              tc_mma_lohi<PAIR>(d_tmem, a_lo + 3 * a_step, a_hi, b_lo + 3 * b_step, b_hi, idesc, 1u);
+            }
+            // stage reusable once these MMAs have read it (in both CTAs of a pair)
+            if constexpr (PAIR) tc_commit_pair(ebar); else tc_commit(ebar);
           }
-          // stage reusable once these MMAs have read it (in both CTAs of a pair)
-          if constexpr (PAIR) tc_commit_pair(ebar); else tc_commit(ebar);
+          __syncwarp();
           a_lo += SB16; b_lo += SB16; fbar += 8u; ebar += 8u;
           if (++stage == Cfg::STAGES) { stage = 0; phase ^= 1u; a_lo = a_lo0; b_lo = b_lo0; fbar = full_bar(0); ebar = empty_bar(0); }
         }
         if (!ok) break;
-        if constexpr (PAIR) tc_commit_pair(tfull_bar(acc)); else tc_commit(tfull_bar(acc));   // accumulator complete
+        if (elect_one()) { if constexpr (PAIR) tc_commit_pair(tfull_bar(acc)); else tc_commit(tfull_bar(acc)); }   // accumulator complete
+        __syncwarp();
       }
       if (!ok && !PAIR) {
         // A wait was abandoned.  Products issued before it may still be running: they read the stage ring and
         // write tensor memory, so they must have finished before the teardown below releases either.  A commit
         // on a barrier of its own completes once every product issued so far is done (products wait for
         // nothing themselves, so this ends; the wait is bounded all the same).
-        tc_commit(drain_bar);
+        if (elect_one()) tc_commit(drain_bar);
+        __syncwarp();
         const long long t0 = clock64();
         while (!mbar_try_wait(drain_bar, 0u) && clock64() - t0 < P.wait_cycles) {}
       }
