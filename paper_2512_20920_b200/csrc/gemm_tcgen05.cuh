@@ -670,151 +670,154 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
     // la: this thread loads the first operand's share (and announces the stage); lb: the second operand's.
     // Without split_loads the first warp's thread does both and the second warp has nothing to do.
     const bool la = warp == 0, lb = P.split_loads ? warp != 0 : warp == 0;
-    if (lane == 0 && !P.starve && (la || lb)) {
+    if (!P.starve && (la || lb)) {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
       TcWalk walk;
       walk.begin(P, w0, wstride, tiles_m_dev, prank);
+      // this warp's loads of K step kb of tile t, by one elected lane
+      auto issue = [&](const TcTile& t, int kb, int k_half) {
+        const uint32_t sa = base + stage * Cfg::STAGE_BYTES;
+        const uint32_t sb = sa + TC_A_BYTES;
+        if constexpr (PAIR) {
+          // both CTAs' loads complete on the even CTA's barrier, which expects the bytes of both
+          const uint32_t fbc = mapa_u32(full_bar(stage), 0);
+          if (P.tr) {
+            // M side: 128 rows of the expert's weights; N side: this CTA's half of the chunk's token rows
+            // (a full 128-row box either way; rows past the half are loaded and not used)
+            if (la) {
+              if (crank == 0) mbar_expect_tx(full_bar(stage), 2 * Cfg::STAGE_BYTES);
+              int kw = kb;
+              const bool second = p.concat == CONCAT_K && kb >= k_half;
+              if (second) kw = kb - k_half;
+              if (!p.b_mn_major) {
+                if (second) tma_load_2d_pair(sa, &map_b1, kw * P.bk, t.group * p.N + t.n0, fbc);
+                else tma_load_2d_pair(sa, &map_b0, kw * P.bk, t.group * p.N + t.n0, fbc);
+              } else {
+                const int kdim = (p.concat == CONCAT_K) ? k_half * TC_BK : t.k_blocks * TC_BK;
+                const int krow = t.group * kdim + kw * TC_BK;
+                if (second) tma_load_mn128_pair(P.mn3d, sa, &map_b1, p.b_col0 + t.n0, krow, fbc);
+                else tma_load_mn128_pair(P.mn3d, sa, &map_b0, p.b_col0 + t.n0, krow, fbc);
+              }
+            }
+            if (lb) tma_load_2d_pair(sb, &map_a, kb * P.bk, t.m0 + crank * (t.ncols / 2), fbc);
+            return;
+          }
+          const int nhalf = t.ncols / 2;       // this CTA's share of the tile's columns: 128, or 64 in a ragged last tile
+          if (la) {
+            // (a 3-D load of an MN-major B brings its whole box, also where this CTA's share of a ragged tile is less)
+            const int b_cols = (p.b_mn_major && P.mn3d) ? P.b_box : nhalf;
+            if (crank == 0) mbar_expect_tx(full_bar(stage), 2 * (TC_A_BYTES + b_cols * TC_BK * 2));
+            if (!p.a_mn_major) {
+              tma_load_2d_pair(sa, &map_a, kb * TC_BK, t.m0, fbc);
+            } else {
+              tma_load_mn128_pair(P.mn3d, sa, &map_a, p.a_col0 + t.m0, t.krow0 + kb * TC_BK, fbc);
+            }
+          }
+          if (lb) {
+            const bool second = p.concat == CONCAT_K && kb >= k_half;
+            const int kbp = second ? kb - k_half : kb;
+            if (!p.b_mn_major) {
+              // this CTA's half of the accumulator columns: gate rows (rank 0) or up rows (rank 1) of a
+              // SwiGLU pair, else rows n0 + nhalf rank .. of B
+              // (the tensor map is named directly in each call: a map chosen through a pointer is slow to issue)
+              if (p.concat == CONCAT_N) {
+                if (crank == 0) tma_load_2d_pair(sb, &map_b0, kbp * TC_BK, t.n0, fbc);
+                else tma_load_2d_pair(sb, &map_b1, kbp * TC_BK, t.n0, fbc);
+              } else if (second) {
+                tma_load_2d_pair(sb, &map_b1, kbp * TC_BK, t.n0 + nhalf * crank, fbc);
+              } else {
+                tma_load_2d_pair(sb, &map_b0, kbp * TC_BK, t.n0 + nhalf * crank, fbc);
+              }
+            } else {
+              const int krow = t.krow0 + kbp * TC_BK;
+              if (second) tma_load_mn128_pair(P.mn3d, sb, &map_b1, p.b_col0 + t.n0 + nhalf * crank, krow, fbc, nhalf > 64);
+              else tma_load_mn128_pair(P.mn3d, sb, &map_b0, p.b_col0 + t.n0 + nhalf * crank, krow, fbc, nhalf > 64);
+            }
+          }
+          return;
+        }
+        const uint32_t fb = full_bar(stage);
+        const bool second = p.concat == CONCAT_K && kb >= k_half;
+        const int kb_b = second ? kb - k_half : kb;
+        // An MN-major B tile is four 64 x 64 boxes against one or two loads for A: with two load threads the
+        // first takes B's last boxes too (3 + 2 loads, or 3 + 3 when A is MN-major as well).
+        const int b_mn_split = !p.b_mn_major ? 0 : (!P.split_loads ? 0 : ((p.a_mn_major && !P.mn3d) ? 3 : 2));
+        if (la) {
+          mbar_expect_tx(fb, TC_A_BYTES + t.ncols * TC_BK * 2);
+          issued[stage] = (int)phase + 1;
+          // A tile
+          if (!p.a_mn_major) {
+            tma_load_2d(sa, &map_a, kb * P.bk, t.m0, fb);
+          } else {
+            tma_load_mn128(P.mn3d, sa, &map_a, p.a_col0 + t.m0, t.krow0 + kb * TC_BK, fb);
+          }
+          if (b_mn_split) {
+            int kdim = (p.concat == CONCAT_K) ? k_half * TC_BK : t.k_blocks * TC_BK;
+            int krow = (p.group_mode == GROUP_M ? t.group * kdim : t.krow0) + kb_b * TC_BK;
+            if (P.mn3d) {          // the second 128 columns
+              if (t.ncols > 128) {
+                if (second) tma_load_mn128(true, sb + 16384, &map_b1, p.b_col0 + t.n0 + 128, krow, fb);
+                else tma_load_mn128(true, sb + 16384, &map_b0, p.b_col0 + t.n0 + 128, krow, fb);
+              }
+            } else {
+#pragma unroll
+              for (int j = 2; j < MMA_N / 64; ++j) {
+                if (j < b_mn_split || 64 * j >= t.ncols) continue;
+                if (second) tma_load_2d(sb + j * 8192, &map_b1, p.b_col0 + t.n0 + 64 * j, krow, fb);
+                else tma_load_2d(sb + j * 8192, &map_b0, p.b_col0 + t.n0 + 64 * j, krow, fb);
+              }
+            }
+          }
+        }
+        if (lb) {
+          issued_b[stage] = (int)phase + 1;
+          // B tile
+          if (!p.b_mn_major) {
+            // rows of the flattened [groups * N, K] weight tensor
+            int row0 = (p.group_mode == GROUP_M ? t.group * p.N : 0) + t.n0;
+            if (p.concat == CONCAT_N) {
+              tma_load_2d(sb, &map_b0, kb_b * P.bk, row0, fb);
+              tma_load_2d(sb + P.tile_n * 128, &map_b1, kb_b * P.bk, row0, fb);
+            } else {
+#pragma unroll
+              for (int j = 0; j < MMA_N / 128; ++j) {
+                if (128 * j >= t.ncols) continue;
+                if (second) tma_load_2d(sb + j * 16384, &map_b1, kb_b * P.bk, row0 + 128 * j, fb);
+                else tma_load_2d(sb + j * 16384, &map_b0, kb_b * P.bk, row0 + 128 * j, fb);
+              }
+            }
+          } else {
+            // rows of the flattened [groups * Kdim, N] weight tensor, or token rows (GROUP_K / dense wgrad)
+            int kdim = (p.concat == CONCAT_K) ? k_half * TC_BK : t.k_blocks * TC_BK;
+            int krow = (p.group_mode == GROUP_M ? t.group * kdim : t.krow0) + kb_b * TC_BK;
+            if (P.mn3d) {
+              if (second) tma_load_mn128(true, sb, &map_b1, p.b_col0 + t.n0, krow, fb);
+              else tma_load_mn128(true, sb, &map_b0, p.b_col0 + t.n0, krow, fb);      // 64 columns with the narrow box
+              if (!b_mn_split && t.ncols > 128) {
+                if (second) tma_load_mn128(true, sb + 16384, &map_b1, p.b_col0 + t.n0 + 128, krow, fb);
+                else tma_load_mn128(true, sb + 16384, &map_b0, p.b_col0 + t.n0 + 128, krow, fb);
+              }
+            } else {
+#pragma unroll
+              for (int j = 0; j < MMA_N / 64; ++j) {
+                if ((b_mn_split && j >= b_mn_split) || 64 * j >= t.ncols) continue;
+                if (second) tma_load_2d(sb + j * 8192, &map_b1, p.b_col0 + t.n0 + 64 * j, krow, fb);
+                else tma_load_2d(sb + j * 8192, &map_b0, p.b_col0 + t.n0 + 64 * j, krow, fb);
+              }
+            }
+          }
+        }
+      };
       while (ok && walk.left > 0) {
         const TcTile t = tc_tile(P, walk, prank);
         walk.step(P);
         const int k_half = t.k_blocks / 2;
         for (int kb = 0; kb < t.k_blocks; ++kb) {
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
-          const uint32_t sa = base + stage * Cfg::STAGE_BYTES;
-          const uint32_t sb = sa + TC_A_BYTES;
-          if constexpr (PAIR) {
-            // both CTAs' loads complete on the even CTA's barrier, which expects the bytes of both
-            const uint32_t fbc = mapa_u32(full_bar(stage), 0);
-            if (P.tr) {
-              // M side: 128 rows of the expert's weights; N side: this CTA's half of the chunk's token rows
-              // (a full 128-row box either way; rows past the half are loaded and not used)
-              if (la) {
-                if (crank == 0) mbar_expect_tx(full_bar(stage), 2 * Cfg::STAGE_BYTES);
-                int kw = kb;
-                const bool second = p.concat == CONCAT_K && kb >= k_half;
-                if (second) kw = kb - k_half;
-                if (!p.b_mn_major) {
-                  if (second) tma_load_2d_pair(sa, &map_b1, kw * P.bk, t.group * p.N + t.n0, fbc);
-                  else tma_load_2d_pair(sa, &map_b0, kw * P.bk, t.group * p.N + t.n0, fbc);
-                } else {
-                  const int kdim = (p.concat == CONCAT_K) ? k_half * TC_BK : t.k_blocks * TC_BK;
-                  const int krow = t.group * kdim + kw * TC_BK;
-                  if (second) tma_load_mn128_pair(P.mn3d, sa, &map_b1, p.b_col0 + t.n0, krow, fbc);
-                  else tma_load_mn128_pair(P.mn3d, sa, &map_b0, p.b_col0 + t.n0, krow, fbc);
-                }
-              }
-              if (lb) tma_load_2d_pair(sb, &map_a, kb * P.bk, t.m0 + crank * (t.ncols / 2), fbc);
-              if (++stage == Cfg::STAGES) { stage = 0; phase ^= 1u; }
-              continue;
-            }
-            const int nhalf = t.ncols / 2;       // this CTA's share of the tile's columns: 128, or 64 in a ragged last tile
-            if (la) {
-              // (a 3-D load of an MN-major B brings its whole box, also where this CTA's share of a ragged tile is less)
-              const int b_cols = (p.b_mn_major && P.mn3d) ? P.b_box : nhalf;
-              if (crank == 0) mbar_expect_tx(full_bar(stage), 2 * (TC_A_BYTES + b_cols * TC_BK * 2));
-              if (!p.a_mn_major) {
-                tma_load_2d_pair(sa, &map_a, kb * TC_BK, t.m0, fbc);
-              } else {
-                tma_load_mn128_pair(P.mn3d, sa, &map_a, p.a_col0 + t.m0, t.krow0 + kb * TC_BK, fbc);
-              }
-            }
-            if (lb) {
-              const bool second = p.concat == CONCAT_K && kb >= k_half;
-              const int kbp = second ? kb - k_half : kb;
-              if (!p.b_mn_major) {
-                // this CTA's half of the accumulator columns: gate rows (rank 0) or up rows (rank 1) of a
-                // SwiGLU pair, else rows n0 + nhalf rank .. of B
-                // (the tensor map is named directly in each call: a map chosen through a pointer is slow to issue)
-                if (p.concat == CONCAT_N) {
-                  if (crank == 0) tma_load_2d_pair(sb, &map_b0, kbp * TC_BK, t.n0, fbc);
-                  else tma_load_2d_pair(sb, &map_b1, kbp * TC_BK, t.n0, fbc);
-                } else if (second) {
-                  tma_load_2d_pair(sb, &map_b1, kbp * TC_BK, t.n0 + nhalf * crank, fbc);
-                } else {
-                  tma_load_2d_pair(sb, &map_b0, kbp * TC_BK, t.n0 + nhalf * crank, fbc);
-                }
-              } else {
-                const int krow = t.krow0 + kbp * TC_BK;
-                if (second) tma_load_mn128_pair(P.mn3d, sb, &map_b1, p.b_col0 + t.n0 + nhalf * crank, krow, fbc, nhalf > 64);
-                else tma_load_mn128_pair(P.mn3d, sb, &map_b0, p.b_col0 + t.n0 + nhalf * crank, krow, fbc, nhalf > 64);
-              }
-            }
-            if (++stage == Cfg::STAGES) { stage = 0; phase ^= 1u; }
-            continue;
-          }
-          const uint32_t fb = full_bar(stage);
-          const bool second = p.concat == CONCAT_K && kb >= k_half;
-          const int kb_b = second ? kb - k_half : kb;
-          // An MN-major B tile is four 64 x 64 boxes against one or two loads for A: with two load threads the
-          // first takes B's last boxes too (3 + 2 loads, or 3 + 3 when A is MN-major as well).
-          const int b_mn_split = !p.b_mn_major ? 0 : (!P.split_loads ? 0 : ((p.a_mn_major && !P.mn3d) ? 3 : 2));
-          if (la) {
-            mbar_expect_tx(fb, TC_A_BYTES + t.ncols * TC_BK * 2);
-            issued[stage] = (int)phase + 1;
-            // A tile
-            if (!p.a_mn_major) {
-              tma_load_2d(sa, &map_a, kb * P.bk, t.m0, fb);
-            } else {
-              tma_load_mn128(P.mn3d, sa, &map_a, p.a_col0 + t.m0, t.krow0 + kb * TC_BK, fb);
-            }
-            if (b_mn_split) {
-              int kdim = (p.concat == CONCAT_K) ? k_half * TC_BK : t.k_blocks * TC_BK;
-              int krow = (p.group_mode == GROUP_M ? t.group * kdim : t.krow0) + kb_b * TC_BK;
-              if (P.mn3d) {          // the second 128 columns
-                if (t.ncols > 128) {
-                  if (second) tma_load_mn128(true, sb + 16384, &map_b1, p.b_col0 + t.n0 + 128, krow, fb);
-                  else tma_load_mn128(true, sb + 16384, &map_b0, p.b_col0 + t.n0 + 128, krow, fb);
-                }
-              } else {
-#pragma unroll
-                for (int j = 2; j < MMA_N / 64; ++j) {
-                  if (j < b_mn_split || 64 * j >= t.ncols) continue;
-                  if (second) tma_load_2d(sb + j * 8192, &map_b1, p.b_col0 + t.n0 + 64 * j, krow, fb);
-                  else tma_load_2d(sb + j * 8192, &map_b0, p.b_col0 + t.n0 + 64 * j, krow, fb);
-                }
-              }
-            }
-          }
-          if (lb) {
-            issued_b[stage] = (int)phase + 1;
-            // B tile
-            if (!p.b_mn_major) {
-              // rows of the flattened [groups * N, K] weight tensor
-              int row0 = (p.group_mode == GROUP_M ? t.group * p.N : 0) + t.n0;
-              if (p.concat == CONCAT_N) {
-                tma_load_2d(sb, &map_b0, kb_b * P.bk, row0, fb);
-                tma_load_2d(sb + P.tile_n * 128, &map_b1, kb_b * P.bk, row0, fb);
-              } else {
-#pragma unroll
-                for (int j = 0; j < MMA_N / 128; ++j) {
-                  if (128 * j >= t.ncols) continue;
-                  if (second) tma_load_2d(sb + j * 16384, &map_b1, kb_b * P.bk, row0 + 128 * j, fb);
-                  else tma_load_2d(sb + j * 16384, &map_b0, kb_b * P.bk, row0 + 128 * j, fb);
-                }
-              }
-            } else {
-              // rows of the flattened [groups * Kdim, N] weight tensor, or token rows (GROUP_K / dense wgrad)
-              int kdim = (p.concat == CONCAT_K) ? k_half * TC_BK : t.k_blocks * TC_BK;
-              int krow = (p.group_mode == GROUP_M ? t.group * kdim : t.krow0) + kb_b * TC_BK;
-              if (P.mn3d) {
-                if (second) tma_load_mn128(true, sb, &map_b1, p.b_col0 + t.n0, krow, fb);
-                else tma_load_mn128(true, sb, &map_b0, p.b_col0 + t.n0, krow, fb);      // 64 columns with the narrow box
-                if (!b_mn_split && t.ncols > 128) {
-                  if (second) tma_load_mn128(true, sb + 16384, &map_b1, p.b_col0 + t.n0 + 128, krow, fb);
-                  else tma_load_mn128(true, sb + 16384, &map_b0, p.b_col0 + t.n0 + 128, krow, fb);
-                }
-              } else {
-#pragma unroll
-                for (int j = 0; j < MMA_N / 64; ++j) {
-                  if ((b_mn_split && j >= b_mn_split) || 64 * j >= t.ncols) continue;
-                  if (second) tma_load_2d(sb + j * 8192, &map_b1, p.b_col0 + t.n0 + 64 * j, krow, fb);
-                  else tma_load_2d(sb + j * 8192, &map_b0, p.b_col0 + t.n0 + 64 * j, krow, fb);
-                }
-              }
-            }
-          }
+          if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
+          if (elect_one()) issue(t, kb, k_half);
+          __syncwarp();
           if (++stage == Cfg::STAGES) { stage = 0; phase ^= 1u; }
         }
       }
