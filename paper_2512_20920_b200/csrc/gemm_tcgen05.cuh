@@ -62,6 +62,7 @@ constexpr int TC_BK = 64;
 constexpr int TC_THREADS = 352;      // warp 0, 10: operand loads; warp 1: products; warps 2..9: epilogue
 constexpr int TC_LOAD_WARP_B = 10;   // the second load warp
 constexpr int TC_EPI_WARPS = 8;
+constexpr int TR_SMALL = 64;            // transposed: halves of a token chunk up to here come in 32-row boxes (experts of 4 rows: 66.7 -> 64.3 us)
 constexpr int TC_A_BYTES = TC_BM * TC_BK * 2;            // 16 KB
 constexpr long long TC_WAIT_CYCLES = 4000000000LL;       // ~2 s: bound on any single wait
 
@@ -684,10 +685,11 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           // both CTAs' loads complete on the even CTA's barrier, which expects the bytes of both
           const uint32_t fbc = mapa_u32(full_bar(stage), 0);
           if (P.tr) {
-            // M side: 128 rows of the expert's weights; N side: this CTA's half of the chunk's token rows
-            // (a full 128-row box either way; rows past the half are loaded and not used)
+            // M side: 128 rows of the expert's weights; N side: this CTA's half of the chunk's token rows, one
+            // 128-row box or up to two 32-row boxes (rows past the half are loaded and not used)
+            const int half = t.ncols / 2, n32 = half <= TR_SMALL ? (half + 31) / 32 : 0;
             if (la) {
-              if (crank == 0) mbar_expect_tx(full_bar(stage), 2 * Cfg::STAGE_BYTES);
+              if (crank == 0) mbar_expect_tx(full_bar(stage), 2 * (TC_A_BYTES + (n32 ? n32 * 4096 : 16384)));
               int kw = kb;
               const bool second = p.concat == CONCAT_K && kb >= k_half;
               if (second) kw = kb - k_half;
@@ -701,7 +703,10 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
                 else tma_load_mn128_pair(P.mn3d, sa, &map_b0, p.b_col0 + t.n0, krow, fbc);
               }
             }
-            if (lb) tma_load_2d_pair(sb, &map_a, kb * P.bk, t.m0 + crank * (t.ncols / 2), fbc);
+            if (lb) {
+              if (n32 == 0) tma_load_2d_pair(sb, &map_a, kb * P.bk, t.m0 + crank * half, fbc);
+              else for (int i = 0; i < n32; ++i) tma_load_2d_pair(sb + i * 4096, &map_c1, kb * P.bk, t.m0 + crank * half + 32 * i, fbc);
+            }
             return;
           }
           const int nhalf = t.ncols / 2;       // this CTA's share of the tile's columns: 128, or 64 in a ragged last tile
@@ -1737,6 +1742,10 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
       r = tc_make_out_map(&mc1, p.C1, false, (uint64_t)2 * p.N, (uint64_t)p.M, (uint64_t)p.ldc1);
       if (r) return r;
     }
+  }
+  if (tr) {
+    const int r = tc_make_map(&mc1, p.A, (uint64_t)p.K, (uint64_t)p.M, (uint64_t)p.lda, f8 ? 128 : 64, 32, f8);
+    if (r) return r;
   }
   if (f8 && p.epilogue == EPI_STORE && !tr) return REVFFN_ERR_UNSUPPORTED;      // only the transposed store scales its accumulator
   P.tr = tr ? 1 : 0;
