@@ -89,7 +89,8 @@ struct TcParams {
   int b_box;                 // rows (K-major) or columns (MN-major, 3-D maps) of B that one load brings: 128 or 64
   int k_blocks;              // dense / GROUP_M
   int tr;                    // transposed pair mode: weights on the MMA M side, an expert's token rows on the N side
-  int tiles_f;               // tr: 256-wide feature tiles per token chunk
+  int tiles_f;               // tr: feature tiles per token chunk, 256 wide (128 of each matrix of a pair)
+  int tr_swap;               // tr, matrix pair: the second matrix lies first in memory and in each group of 32 lanes
   uint32_t idesc;
   long long wait_cycles;     // bound on every wait of the kernel (clock cycles)
   int starve;                // failure-path test: the load warp issues nothing, so the first wait for operands runs out
@@ -207,6 +208,12 @@ __device__ __forceinline__ void tma_load_mn128_pair(bool mn3d, uint32_t dst, con
     tma_load_2d_pair(dst, map, col, krow, bar_cluster);
     if (second_block) tma_load_2d_pair(dst + 8192, map, col + 64, krow, bar_cluster);
   }
+}
+// 16 rows of both matrices of a pair, four times: {64 columns (128 bytes), 16 rows, 2 matrices, 4 groups of rows}.
+__device__ __forceinline__ void tma_load_rows16_pair(uint32_t dst, const CUtensorMap* map, int col, int group, uint32_t bar_cluster) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(col), "r"(0), "r"(0), "r"(group), "r"(bar_cluster) : "memory");
 }
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
@@ -515,6 +522,7 @@ __device__ __forceinline__ void upd_half(const UpdRule& rule, const SlabOut& o, 
 struct TcTile {
   int m0, n0, group, k_blocks, krow0;
   int ncols;      // accumulator columns in use: the tile's, or 128 in the last column tile of an odd multiple of 128
+  int pad;        // tr: rows of the expert's zero padding after the chunk's (its last chunk only)
 };
 
 // A role's walk over the tiles w0, w0 + stride, ...: the tile's index split into its parts, and the table entries that the
@@ -566,11 +574,13 @@ __device__ __forceinline__ TcTile tc_tile(const TcParams& P, const TcWalk& a, in
   TcTile t;
   const GemmProblem& p = P.p;
   t.krow0 = 0;
+  t.pad = 0;
   t.k_blocks = P.k_blocks;
   if (P.tr) {
     // m0 = first token row, ncols = token rows (the MMA N), n0 = first feature of this CTA's 128
     t.group = a.e.x; t.m0 = a.e.y; t.ncols = a.e.z;
-    t.n0 = a.tn * 2 * TC_BM + pair_rank * TC_BM;
+    t.n0 = (a.tn * 2 + pair_rank) * (p.concat == CONCAT_N ? TC_BM / 2 : TC_BM);
+    t.pad = a.e.w;
     return t;
   }
   t.group = a.group;
@@ -693,7 +703,9 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
               int kw = kb;
               const bool second = p.concat == CONCAT_K && kb >= k_half;
               if (second) kw = kb - k_half;
-              if (!p.b_mn_major) {
+              if (EPI == EPI_SWIGLU) {
+                tma_load_rows16_pair(sa, &map_b0, kb * P.bk, (t.group * p.N + t.n0) / 16, fbc);
+              } else if (!p.b_mn_major) {
                 if (second) tma_load_2d_pair(sa, &map_b1, kw * P.bk, t.group * p.N + t.n0, fbc);
                 else tma_load_2d_pair(sa, &map_b0, kw * P.bk, t.group * p.N + t.n0, fbc);
               } else {
@@ -1053,6 +1065,100 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
               bulk_commit();
             }
             ++n_grp;
+          }
+        }
+        if constexpr (PAIR && EPI == EPI_SWIGLU) {
+          // Transposed SwiGLU: of this warp's 32 lanes 16 hold gate rows, 16 the up rows of the same features, for 32
+          // token rows per block.  Lanes l and l + 16 trade halves, each finishes 16 tokens of one feature; then, as
+          // above, lanes 2i and 2i+1 trade so that feature pairs go to the staging area ([32 tokens][16 features], and
+          // [32 tokens][16 + 16] for the a|b copy) and rows of 32 bytes from there to memory by plain stores.  The rows
+          // of an expert's padding are written as zeros: products over rows (weight gradients) read them.
+          // Against 128 token rows x 128 columns of both matrices on one CTA, a pair brings 32 instead of 48 KB into
+          // each SM per K step and pads a run of rows to 32 instead of 128 (experts' gate | up at 8192 tokens 302 -> 279 us,
+          // with the copy 334 -> 295; at 2741 tokens 155 -> 138 and 167 -> 148)
+          const bool odd = lane & 1, hi = lane >= 16, up_lane = hi != (P.tr_swap != 0);
+          const int fw = t.n0 + q * 16;            // first feature of the warp
+          float sw = 1.f;
+          if (p.fp8) sw = (up_lane ? p.b_scale1 : p.b_scale0)[(int64_t)t.group * p.N + fw + (lane & 15)];
+          bf16* const h_out = reinterpret_cast<bf16*>(p.C) + (int64_t)t.m0 * p.ldc + fw;
+          bf16* const ab_out = reinterpret_cast<bf16*>(p.C1) + (int64_t)t.m0 * p.ldc1 + fw;
+#pragma unroll 1
+          for (int c = half * 32; c < t.ncols + t.pad; c += 64) {
+            if (c < t.ncols) {
+              tmem_ld32(taddr + c, r0);
+              tmem_ld_wait();
+            } else {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) r0[i] = 0u;
+            }
+#pragma unroll
+            for (int i = 0; i < 32; ++i) f[i] = __uint_as_float(r0[i]);
+            if (p.fp8) {
+              const float4* a4 = reinterpret_cast<const float4*>(p.a_scale + t.m0 + c);    // the same for every lane
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const float4 a = a4[i];
+                f[4 * i] *= sw * a.x; f[4 * i + 1] *= sw * a.y; f[4 * i + 2] *= sw * a.z; f[4 * i + 3] *= sw * a.w;
+              }
+            }
+            // two tokens of one feature in, one token of two features out
+            auto trade = [&](float t0, float t1) -> uint32_t {
+              const __nv_bfloat162 v = __floats2bfloat162_rn(t0, t1);
+              const uint32_t own = *reinterpret_cast<const uint32_t*>(&v);
+              const uint32_t other = __shfl_xor_sync(0xffffffffu, own, 1);
+              return odd ? __byte_perm(other, own, 0x7632) : __byte_perm(own, other, 0x5410);
+            };
+            if (p.C1) {
+              const int within = ((lane >> 1) & 3) * 4;
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const int tok = 2 * j + (odd ? 1 : 0);
+                *reinterpret_cast<uint32_t*>(stg + tok * 64 + (((lane >> 3) ^ ((tok >> 1) & 3)) << 4) + within) = trade(f[2 * j], f[2 * j + 1]);
+              }
+            }
+            float h[16], rs[16];
+            if (p.rowscale) {
+              const float4* g4 = reinterpret_cast<const float4*>(p.rowscale + t.m0 + c + (hi ? 16 : 0));
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const float4 g = g4[i];
+                rs[4 * i] = g.x; rs[4 * i + 1] = g.y; rs[4 * i + 2] = g.z; rs[4 * i + 3] = g.w;
+              }
+            } else {
+#pragma unroll
+              for (int i = 0; i < 16; ++i) rs[i] = 1.f;
+            }
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) {
+              const float2 own = hi ? make_float2(f[16 + i], f[17 + i]) : make_float2(f[i], f[i + 1]);
+              const float2 send = hi ? make_float2(f[i], f[i + 1]) : make_float2(f[16 + i], f[17 + i]);
+              const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, send.x, 16), __shfl_xor_sync(0xffffffffu, send.y, 16));
+              const float2 A = up_lane ? got : own, B = up_lane ? own : got;
+              const float2 Hh = __fmul2_rn(__fmul2_rn(__fmul2_rn(A, sigmoid_approx2(A)), B), make_float2(rs[i], rs[i + 1]));
+              h[i] = Hh.x; h[i + 1] = Hh.y;
+            }
+            // a token's row of 32 bytes; the rows of tokens 16.. change places in pairs, away from the banks of tokens 0..
+            auto slot = [](int tok) -> int { return (tok ^ ((tok >> 4) << 1)) * 32; };
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              *reinterpret_cast<uint32_t*>(stg + 2048 + slot((hi ? 16 : 0) + 2 * j + (odd ? 1 : 0)) + ((lane & 15) >> 1) * 4) = trade(h[2 * j], h[2 * j + 1]);
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              const int tok = 16 * i + (lane >> 1);
+              *reinterpret_cast<uint4*>(h_out + (int64_t)(c + tok) * p.ldc + (lane & 1) * 8) =
+                  *reinterpret_cast<const uint4*>(stg + 2048 + slot(tok) + (lane & 1) * 16);
+            }
+            if (p.C1) {
+              bf16* const dst = ab_out + ((((lane >> 1) & 1) != P.tr_swap) ? p.N : 0) + (lane & 1) * 8;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const int tok = 8 * i + (lane >> 2);
+                *reinterpret_cast<uint4*>(dst + (int64_t)(c + tok) * p.ldc1) =
+                    *reinterpret_cast<const uint4*>(stg + tok * 64 + (((lane & 3) ^ ((tok >> 1) & 3)) << 4));
+              }
+            }
+            __syncwarp();
           }
         }
       } else if constexpr (EPI == EPI_STORE || EPI == EPI_ROWSCALE || EPI == EPI_COUPLE || WGRAD) {
@@ -1529,6 +1635,23 @@ inline int tc_make_map_mn3d(CUtensorMap* map, const void* ptr, uint64_t rows, ui
   return r == CUDA_SUCCESS ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 
+// Two [groups * N, K] weight matrices of one layout seen as {K, 16 rows, 2 matrices, groups of 16 rows}: a box of
+// 128 bytes x 16 x 2 x 4 is 64 rows of both, 16 of one and 16 of the other in turn.  The step between the matrices is the
+// distance of their addresses.
+inline int tc_make_map_rows16(CUtensorMap* map, const GemmProblem& p) {
+  const uintptr_t b0 = reinterpret_cast<uintptr_t>(p.B0), b1 = reinterpret_cast<uintptr_t>(p.B1);
+  const uint64_t es = p.fp8 ? 1 : 2, dist = b0 < b1 ? b1 - b0 : b0 - b1, rows = (uint64_t)(p.n_groups > 0 ? p.n_groups : 1) * p.N;
+  if (!p.B0 || !p.B1 || dist == 0 || dist % 16 != 0 || dist >= (1ull << 40)) return REVFFN_ERR_UNSUPPORTED;
+  cuuint64_t dims[4] = {(cuuint64_t)p.K, 16, 2, rows / 16};
+  cuuint64_t strides[3] = {(cuuint64_t)p.ldb * es, dist, 16 * (cuuint64_t)p.ldb * es};
+  cuuint32_t box[4] = {p.fp8 ? 128u : 64u, 16, 2, 4};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = tc_state().encode(map, p.fp8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
+                                 reinterpret_cast<void*>(b0 < b1 ? b0 : b1), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                 CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? REVFFN_OK : REVFFN_ERR_CUDA;
+}
+
 // Tensor map of an epilogue output: boxes of 32 rows x 64 bytes (32 bf16 or 16 fp32 columns),
 // 64-byte swizzle.
 inline int tc_make_out_map(CUtensorMap* map, const void* ptr, bool f32, uint64_t inner, uint64_t outer, uint64_t ld) {
@@ -1571,16 +1694,20 @@ struct TcPlan { bool tr, pair; int tile_n; };
 // tokens went from 2547 to 2689 us, at 512 from 1504 to 1574).
 inline TcPlan tc_plan(const GemmProblem& p, int n_sms) {
   TcPlan wide;
-  wide.tr = p.group_mode == GROUP_M && p.tok_chunks != nullptr && p.N % 256 == 0 && !p.a_mn_major && p.concat != CONCAT_N &&
-            !p.no_pair && n_sms % 2 == 0 && (p.epilogue == EPI_ROWSCALE || (p.epilogue == EPI_STORE && !p.out_f32));
-  wide.pair = wide.tr || (p.group_mode != GROUP_M && (p.N % 256 == 0 || p.b_mn_major) && !p.no_pair);
   const bool cat = p.concat == CONCAT_N;
+  wide.tr = p.group_mode == GROUP_M && p.tok_chunks != nullptr && !p.a_mn_major && !p.no_pair && n_sms % 2 == 0 &&
+            (cat ? p.epilogue == EPI_SWIGLU && !p.b_mn_major
+                 : p.N % 256 == 0 && (p.epilogue == EPI_ROWSCALE || (p.epilogue == EPI_STORE && !p.out_f32)));
+  wide.pair = wide.tr || (p.group_mode != GROUP_M && (p.N % 256 == 0 || p.b_mn_major) && !p.no_pair);
   wide.tile_n = cat ? 128 : 256;
   if (p.dbg_tile_n) {
     wide.tile_n = p.dbg_tile_n;
     wide.pair = p.group_mode != GROUP_M && !p.no_pair && (cat || (p.dbg_tile_n == 256 ? wide.pair : p.dbg_tile_n >= 128));
     return wide;
   }
+  // a pair of matrices whose transposed tiles leave SMs idle is better off with the row tiles below, which can be narrow
+  // (four d = 512 blocks, eight experts of 144 rows: 1663 us a step with transposed tiles, 1630 without)
+  if (wide.tr && cat && ((p.M - 127 * (int64_t)p.n_groups) / 256 + p.n_groups / 2) * (p.N / 128) < n_sms / 2) wide.tr = wide.pair = false;
   if (wide.tr || p.fp8 || p.upd_w) return wide;
   const bool pair_open = p.group_mode != GROUP_M && !p.no_pair && n_sms % 2 == 0;
   const int64_t groups = p.group_mode == GROUP_K ? (p.n_groups > 0 ? p.n_groups : 1) : 1;
@@ -1622,6 +1749,12 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   P.p = p;
   const TcPlan plan = tc_plan(p, s.n_sms);
   const bool tr = plan.tr, pair = plan.pair;
+  CUtensorMap m_gu;
+  if (tr && p.concat == CONCAT_N && tc_make_map_rows16(&m_gu, p) != REVFFN_OK) {      // the driver does not take the view
+    GemmProblem q = p;
+    q.tok_chunks = nullptr;
+    return launch_gemm_tc(q, st);
+  }
   P.tile_n = plan.tile_n;
   // what one load of B brings: this CTA's share of a tile's columns, at most 128 of them
   P.b_box = std::min(128, pair && p.concat != CONCAT_N ? P.tile_n / 2 : P.tile_n);
@@ -1749,7 +1882,9 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   }
   if (f8 && p.epilogue == EPI_STORE && !tr) return REVFFN_ERR_UNSUPPORTED;      // only the transposed store scales its accumulator
   P.tr = tr ? 1 : 0;
-  P.tiles_f = p.N / 256;
+  P.tiles_f = p.N / (p.concat == CONCAT_N ? 128 : 256);
+  P.tr_swap = tr && p.concat == CONCAT_N && reinterpret_cast<uintptr_t>(p.B1) < reinterpret_cast<uintptr_t>(p.B0);
+  if (tr && p.concat == CONCAT_N) mb0 = m_gu;
   int64_t total = (int64_t)P.tiles_m * P.tiles_n * (p.group_mode == GROUP_K ? groups : 1);
   int grid = (int)(total < s.n_sms ? total : s.n_sms);
   if (tr) {

@@ -434,7 +434,7 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
   // other's way: a product CTA needs a whole SM and its tiles are dealt out in advance, so SMs that the router
   // gives up late hold up the whole product.  At 8192 tokens, in the inverse pass: beside each other 104-148 us for
   // P_up, maps ready after 150 us; one after the other 42 us and after 128 us.  The line is two router blocks per SM.
-  const bool pup_first = rt != st && ceil_div(Tn, RT_TOK) * ROUTE_CLUSTER > 2 * tc_state().n_sms;
+  const bool router_fills = ceil_div(Tn, RT_TOK) * ROUTE_CLUSTER > 2 * tc_state().n_sms, pup_first = rt != st && router_fills;
 
   // Router: fold through P_up, logits, top-k, gates -- or everything from a routing record.  The router reads y1
   // and the permutation maps read the router's result: neither needs the norm or P_up, so with the second stream
@@ -497,11 +497,24 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
   CK(cudaGetLastError());
 
   if (!pup_first || from_record) CKR(p_up());
-  CKR(c.order(rt, st));            // the permutation needs the maps
   // The shared expert needs u and nothing else of this pass: on the second stream it runs beside the routed experts.
+  // Where the router leaves most SMs idle, its first product runs beside the router instead, on the main stream, which
+  // waits for the maps anyway (step at 512 tokens 1432 -> 1412 us, forward of 64 tokens 284 -> 279).
   Ctx<T> cs = c;
   cs.st = c.side();
+  auto shared_gate_up = [&](const Ctx<T>& on) -> int {
+    GemmProblem p = blank_problem();
+    p.M = Tn; p.N = Is; p.K = d;
+    p.A = c.template p<T>(L.u); p.lda = d;
+    p.B0 = c.W.ws_gate; p.B1 = c.W.ws_up; p.ldb = d; p.concat = CONCAT_N;
+    p.epilogue = EPI_SWIGLU; p.C = c.template p<T>(L.hs); p.ldc = Is;
+    if (save_ab) { p.C1 = c.template p<T>(L.abs); p.ldc1 = 2 * (int64_t)Is; }
+    return run_gemm(on, p, TG_SH_GATEUP);
+  };
+  const bool shared_early = rt != st && !router_fills;
+  if (Is > 0 && shared_early) CKR(shared_gate_up(c));
   if (Is > 0) CKR(c.order(st, cs.st));
+  CKR(c.order(rt, st));            // the permutation needs the maps
 
   const bool fp8 = (D.flags & REVFFN_FLAG_FP8_EXPERTS) != 0;
   if constexpr (std::is_same<T, bf16>::value) {
@@ -522,6 +535,7 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
         p.group_mode = GROUP_M; p.n_groups = E; p.b_group_stride = (int64_t)I * d;
         p.group_off = c.template p<int32_t>(L.expert_off); p.tile_group = c.template p<int32_t>(L.tile_group);
         p.rows_total = c.template p<int32_t>(L.rows_total);
+        p.tok_chunks = c.template p<int4>(L.tok_chunks);
         p.epilogue = EPI_SWIGLU; p.C = c.template p<T>(L.hmid); p.ldc = I;
         p.rowscale = c.template p<float>(L.row_gate);
         CKR(run_gemm(c, p, TG_EXP_GATEUP));
@@ -565,6 +579,7 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
       p.group_mode = GROUP_M; p.n_groups = E; p.b_group_stride = (int64_t)I * d;
       p.group_off = c.template p<int32_t>(L.expert_off); p.tile_group = c.template p<int32_t>(L.tile_group);
       p.rows_total = c.template p<int32_t>(L.rows_total);
+      p.tok_chunks = c.template p<int4>(L.tok_chunks);
       p.epilogue = EPI_SWIGLU; p.C = c.template p<T>(L.hmid); p.ldc = I;
       p.rowscale = c.template p<float>(L.row_gate);
       if (save_ab) { p.C1 = c.template p<T>(L.ab); p.ldc1 = 2 * (int64_t)I; }
@@ -587,13 +602,7 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
 
   // Shared expert: S = (silu(U Wsg^T) * (U Wsu^T)) Wsd^T
   if (Is > 0) {
-    GemmProblem p = blank_problem();
-    p.M = Tn; p.N = Is; p.K = d;
-    p.A = c.template p<T>(L.u); p.lda = d;
-    p.B0 = c.W.ws_gate; p.B1 = c.W.ws_up; p.ldb = d; p.concat = CONCAT_N;
-    p.epilogue = EPI_SWIGLU; p.C = c.template p<T>(L.hs); p.ldc = Is;
-    if (save_ab) { p.C1 = c.template p<T>(L.abs); p.ldc1 = 2 * (int64_t)Is; }
-    CKR(run_gemm(cs, p, TG_SH_GATEUP));
+    if (!shared_early) CKR(shared_gate_up(cs));
     GemmProblem q = blank_problem();
     q.M = Tn; q.N = d; q.K = Is;
     q.A = c.template p<T>(L.hs); q.lda = Is;

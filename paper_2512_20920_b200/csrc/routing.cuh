@@ -738,12 +738,12 @@ map_assign_kernel(const int32_t* __restrict__ idx, const float* __restrict__ gat
     for (int t = off[e] / ROW_PAD; t < off[e + 1] / ROW_PAD && t < max_tiles; ++t) tile_group[t] = e;
     // Token runs for the products that put tokens on the MMA N side: per expert, runs of up to TOK_CHUNK rows
     // covering its real rows rounded up to 32 (the rounding stays inside the expert's zero padding).
-    // Entry = (expert, first row, rows, 0).
+    // Entry = (expert, first row, rows, rows of padding after them: nonzero in the expert's last run only).
     // (Runs of equal length, 3 x 192 instead of 256 + 256 + 64 for 546 rows, stay within 2 % either way: the two
     // products that use the table measured 2 % faster alone and the whole step 1-2 % slower.)
     const int real = (int)round_up(cnt[e], 32);
     for (int r = 0, c = coff[e]; r < real && c < max_chunks; r += TOK_CHUNK, ++c)
-      tok_chunks[c] = make_int4(e, off[e] + r, min(TOK_CHUNK, real - r), 0);
+      tok_chunks[c] = make_int4(e, off[e] + r, min(TOK_CHUNK, real - r), r + TOK_CHUNK >= real ? off[e + 1] - off[e] - real : 0);
   }
   if (tid == 0) {
     rows_total[0] = off[E];
