@@ -370,26 +370,11 @@ __device__ __forceinline__ void stage32_bf16(uint8_t* buf, int r, const float* f
   for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(row + ((j ^ ((r >> 1) & 3)) << 4)) = pack8(f + 8 * j);
 }
 
-// A warp's 32-row x 32-column bf16 block (rows of 64 bytes, row stride ld elements) between global memory and
-// the staging layout above, in "distributed" form: instruction i of four moves rows 8i .. 8i+7, lane l the
+// A warp's 32-row x 32-column bf16 block (rows of 64 bytes, row stride ld elements) from the staging layout above to
+// global memory, in "distributed" form: instruction i of four moves rows 8i .. 8i+7, lane l the
 // 16-byte piece l & 3 of row 8i + (l >> 2).  Eight lanes cover four whole 64-byte row segments, so every
 // 32-byte sector a request touches is used in full, and the 512 contiguous staging bytes an instruction
-// touches spread over all banks.  rows_ok: rows of the block that exist (the rest read as zeros / are not stored).
-__device__ __forceinline__ void blk_load_dist(const bf16* g, int64_t ld, int rows_ok, int lane, uint4 (&raw)[4]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = 8 * i + (lane >> 2);
-    raw[i] = (r < rows_ok) ? __ldcg(reinterpret_cast<const uint4*>(g + (int64_t)r * ld + (lane & 3) * 8))
-                           : make_uint4(0u, 0u, 0u, 0u);
-  }
-}
-__device__ __forceinline__ void blk_dist_to_stage(uint8_t* buf, int lane, const uint4 (&raw)[4]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = 8 * i + (lane >> 2);
-    *reinterpret_cast<uint4*>(buf + r * 64 + (((lane & 3) ^ ((r >> 1) & 3)) << 4)) = raw[i];
-  }
-}
+// touches spread over all banks.  rows_ok: rows of the block that exist (the rest are not stored).
 __device__ __forceinline__ void blk_stage_to_global(const uint8_t* buf, int lane, bf16* g, int64_t ld, int rows_ok) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -966,14 +951,36 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       const bool slab_ok = t.m0 + q * 32 < m_lim;             // this warp's 32 rows hold at least one real row
       const int rows_ok = min(32, m_lim - (t.m0 + q * 32));   // real rows among them (<= 0: none)
       // SwiGLU backward: the a|b operands of the warp's first block do not depend on the accumulator, so
-      // their loads go out before the wait for it (ds_a / ds_b: one block in distributed form)
+      // their loads go out before the wait for it.  A lane takes 16-byte pieces lane % 4 of rows lane / 4 + 8 i of a block
+      // of 32 rows x 32 columns (ds_a, ds_b; ds_rs: the rows' scales).
+      const bool ds_tr = EPI == EPI_DSWIGLU && PAIR && P.tr;
       uint4 ds_a[4], ds_b[4];
-      bf16* ds_blk = nullptr;
+      float ds_rs[4];
+      bf16* ds_at = nullptr;          // this lane's piece of the row lane / 4 of the block at column (tr: token row) 0
+      int64_t ds_step = 0, ds_row8 = 0;
+      int ds_rows = 0;                // real rows of a block
+      auto ds_load = [&](int i, int c) {
+        const bool in = 8 * i + (lane >> 2) < ds_rows;
+        const bf16* at = ds_at + c * ds_step + i * ds_row8;
+        ds_a[i] = in ? __ldcg(reinterpret_cast<const uint4*>(at)) : make_uint4(0u, 0u, 0u, 0u);
+        ds_b[i] = in ? __ldcg(reinterpret_cast<const uint4*>(at + p.N)) : make_uint4(0u, 0u, 0u, 0u);
+      };
+      auto ds_scale = [&](int row0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int row = 8 * i + (lane >> 2);
+          ds_rs[i] = p.rowscale && row < ds_rows ? p.rowscale[row0 + row] : 1.f;
+        }
+      };
       if constexpr (EPI == EPI_DSWIGLU) {
-        ds_blk = reinterpret_cast<bf16*>(p.ab) + (int64_t)(t.m0 + q * 32) * p.ld_ab + t.n0;
-        if (slab_ok && half * 32 < t.ncols) {
-          blk_load_dist(ds_blk + half * 32, p.ld_ab, rows_ok, lane, ds_a);
-          blk_load_dist(ds_blk + p.N + half * 32, p.ld_ab, rows_ok, lane, ds_b);
+        ds_rows = ds_tr ? (t.n0 < p.N ? 32 : 0) : max(0, rows_ok);      // a pair's second half can lie past the last feature
+        ds_step = ds_tr ? p.ld_ab : 1;
+        ds_row8 = 8 * p.ld_ab;
+        ds_at = reinterpret_cast<bf16*>(p.ab) + (int64_t)(t.m0 + (ds_tr ? 0 : q * 32) + (lane >> 2)) * p.ld_ab + t.n0 + (ds_tr ? q * 32 : 0) + (lane & 3) * 8;
+        if (half * 32 < t.ncols) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) ds_load(i, half * 32);
+          ds_scale(ds_tr ? t.m0 + half * 32 : t.m0 + q * 32);
         }
       }
       // row coordinate of the slab in the output tensor map (rows past its extent are clipped by the store)
@@ -1014,7 +1021,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       uint32_t r0[32];
       float f[32];
 
-      if (PAIR && P.tr) {
+      if (PAIR && P.tr && EPI != EPI_DSWIGLU) {
         if constexpr (PAIR && (EPI == EPI_STORE || EPI == EPI_ROWSCALE)) {
           // Transposed tile: this lane holds output feature t.n0 + 32 q + lane for 32 token rows per block.
           // Lanes 2i and 2i+1 trade halves so that each ends up with feature PAIRS of single tokens (the even
@@ -1442,57 +1449,88 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           ++n_grp;
         }
       } else {   // EPI_DSWIGLU
-        // Per 32-column block: a|b arrive in distributed form by plain 16-byte loads (the next block's are in
-        // flight during this block's arithmetic), pass through the staging area into row-per-lane form, da|db are
-        // written over them there and leave by plain line-wide stores.  Nothing in this path queues behind the
-        // load warp's operand traffic in the copy engine or waits for a bulk store to drain, which is what
-        // bounded the first version of this epilogue (a|b by TMA, two sets, three bulk stores per block).
-        const float rs = (p.rowscale && m_ok) ? p.rowscale[m] : 1.f;
-        float2 dg2 = make_float2(0.f, 0.f);
+        // The accumulator block goes through the staging area as fp32 into the distributed form in which a|b
+        // arrive and da|db leave, straight from and to memory in rows of 64 bytes (transposed tiles: lane = feature,
+        // so the staging write transposes).  A piece of the next block is requested as soon as this one's registers
+        // are free, the next block's accumulator while this one is worked on.
+        // (With a|b and da|db through the staging area and the accumulator in place, and the experts' rows in 128-row
+        // tiles: experts' product 231 us at 8192 tokens, 112 at 2741, 93 at 512, now 210, 99, 77; the shared expert's at 8192
+        // 166 -> 147.  It still sets the pace, 3.6k clk per block of the warp beside 18.6k of main loop per tile: without its
+        // stores a block takes 2.7k, without its loads 2.0k, without exponentials as long as with them.  Asking a tile
+        // ahead for L2 prefetches or a whole block ahead into other registers changes nothing.)
+        const bool any = ds_rows > 0;            // warp-uniform
+        float dg[4] = {0.f, 0.f, 0.f, 0.f};
+        // sums over the four lanes of a row; lane (row, i) ends up with the row 8 i + lane / 4
+        auto dg_out = [&](int row0, int rows, int part) {
+          float mine = 0.f;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float v = dg[i];
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            if ((lane & 3) == i) mine = v;
+            dg[i] = 0.f;
+          }
+          const int row = 8 * (lane & 3) + (lane >> 2);
+          if (row < rows) p.dg_part[(int64_t)(row0 + row) * p.dg_ld + part] = mine;
+        };
+        if (any && half * 32 < t.ncols) tmem_ld32(taddr + half * 32, r0);
 #pragma unroll 1
         for (int c = half * 32; c < t.ncols; c += 64) {
-          if (!slab_ok) continue;      // warp-uniform
-          blk_dist_to_stage(stg, lane, ds_a);
-          blk_dist_to_stage(stg + 2048, lane, ds_b);
-          __syncwarp();
-          if (c + 64 < t.ncols) {
-            blk_load_dist(ds_blk + c + 64, p.ld_ab, rows_ok, lane, ds_a);
-            blk_load_dist(ds_blk + p.N + c + 64, p.ld_ab, rows_ok, lane, ds_b);
-          }
-          tmem_ld32(taddr + c, r0);
+          if (!any) continue;
+          const bool more = c + 64 < t.ncols;
           tmem_ld_wait();
-          uint8_t* row_a = stg + lane * 64;
-          uint8_t* row_b = stg + 2048 + lane * 64;
-          const int sw = (lane >> 1) & 3;
+          if (ds_tr) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+            for (int i = 0; i < 32; ++i)
+              *reinterpret_cast<uint32_t*>(stg + i * 128 + (((lane >> 2) ^ (i & 7)) << 4) + (lane & 3) * 4) = r0[i];
+          } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              *reinterpret_cast<uint4*>(stg + lane * 128 + ((j ^ (lane & 7)) << 4)) =
+                  make_uint4(r0[4 * j], r0[4 * j + 1], r0[4 * j + 2], r0[4 * j + 3]);
+          }
+          __syncwarp();
+          if (more) tmem_ld32(taddr + c + 64, r0);
+          bf16* const out_at = ds_at + c * ds_step;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int row = 8 * i + (lane >> 2);
+            const float4 v0 = *reinterpret_cast<const float4*>(stg + row * 128 + (((2 * (lane & 3)) ^ (row & 7)) << 4));
+            const float4 v1 = *reinterpret_cast<const float4*>(stg + row * 128 + (((2 * (lane & 3) + 1) ^ (row & 7)) << 4));
+            const float v[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
             float a[8], b[8];
-            unpack8(*reinterpret_cast<const uint4*>(row_a + ((j ^ sw) << 4)), a);
-            unpack8(*reinterpret_cast<const uint4*>(row_b + ((j ^ sw) << 4)), b);
+            unpack8(ds_a[i], a);
+            unpack8(ds_b[i], b);
+            if (more) ds_load(i, c + 64);
+            float2 dg2 = make_float2(0.f, 0.f);
             // two elements at a time on the packed fp32 pipe (half the instructions of the scalar form)
 #pragma unroll
-            for (int i = 0; i < 8; i += 2) {
-              const float2 A = make_float2(a[i], a[i + 1]), B = make_float2(b[i], b[i + 1]);
-              const float2 V = make_float2(__uint_as_float(r0[8 * j + i]), __uint_as_float(r0[8 * j + i + 1]));
+            for (int e = 0; e < 8; e += 2) {
+              const float2 A = make_float2(a[e], a[e + 1]), B = make_float2(b[e], b[e + 1]), V = make_float2(v[e], v[e + 1]);
               const float2 S = sigmoid_approx2(A);
               const float2 SI = __fmul2_rn(A, S);                         // silu(a)
-              const float2 DH = __fmul2_rn(make_float2(rs, rs), V);       // dL/dH of this row
+              const float2 DH = __fmul2_rn(make_float2(ds_rs[i], ds_rs[i]), V);       // dL/dH of this row
               dg2 = __ffma2_rn(V, __fmul2_rn(SI, B), dg2);                // <dH', H>: gradient of the row's gate weight
               // da = dh b silu'(a), silu'(a) = s (1 + a (1 - s)) = s (1 + a - silu(a));  db = dh silu(a)
               const float2 T1 = __fadd2_rn(__fadd2_rn(A, make_float2(1.f, 1.f)), make_float2(-SI.x, -SI.y));
               const float2 DA = __fmul2_rn(__fmul2_rn(DH, B), __fmul2_rn(S, T1));
               const float2 DB = __fmul2_rn(DH, SI);
-              a[i] = DA.x; a[i + 1] = DA.y; b[i] = DB.x; b[i + 1] = DB.y;
+              a[e] = DA.x; a[e + 1] = DA.y; b[e] = DB.x; b[e + 1] = DB.y;
             }
-            *reinterpret_cast<uint4*>(row_a + ((j ^ sw) << 4)) = pack8(a);
-            *reinterpret_cast<uint4*>(row_b + ((j ^ sw) << 4)) = pack8(b);
+            dg[i] += dg2.x + dg2.y;
+            if (row < ds_rows) {
+              *reinterpret_cast<uint4*>(out_at + i * ds_row8) = pack8(a);
+              *reinterpret_cast<uint4*>(out_at + i * ds_row8 + p.N) = pack8(b);
+            }
+          }
+          if (ds_tr) {
+            if (p.dg_part) dg_out(t.m0 + c, 32, t.n0 / 32 + q);
+            if (more) ds_scale(t.m0 + c + 64);
           }
           __syncwarp();
-          blk_stage_to_global(stg, lane, ds_blk + c, p.ld_ab, rows_ok);
-          blk_stage_to_global(stg + 2048, lane, ds_blk + p.N + c, p.ld_ab, rows_ok);
-          __syncwarp();
         }
-        if (p.dg_part && m_ok) p.dg_part[(int64_t)m * p.dg_ld + 2 * (t.n0 / P.tile_n) + half] = dg2.x + dg2.y;
+        if (!ds_tr && any && p.dg_part) dg_out(t.m0 + q * 32, ds_rows, 2 * (t.n0 / P.tile_n) + half);
       }
       if (!UPD || !slab_ok) release();
     }
@@ -1666,7 +1704,6 @@ inline int tc_make_out_map(CUtensorMap* map, const void* ptr, bool f32, uint64_t
   return r == CUDA_SUCCESS ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 
-inline int tc_dg_parts(int N) { return 2 * (int)ceil_div(N, 256); }   // two epilogue warps per row and column tile
 
 template <int MMA_N, int EPI>
 inline int tc_launch(const TcParams& P, const CUtensorMap& ma, const CUtensorMap& mb0, const CUtensorMap& mb1,
@@ -1697,6 +1734,7 @@ inline TcPlan tc_plan(const GemmProblem& p, int n_sms) {
   const bool cat = p.concat == CONCAT_N;
   wide.tr = p.group_mode == GROUP_M && p.tok_chunks != nullptr && !p.a_mn_major && !p.no_pair && n_sms % 2 == 0 &&
             (cat ? p.epilogue == EPI_SWIGLU && !p.b_mn_major
+                 : p.epilogue == EPI_DSWIGLU ? p.b_mn_major && p.concat == CONCAT_NONE
                  : p.N % 256 == 0 && (p.epilogue == EPI_ROWSCALE || (p.epilogue == EPI_STORE && !p.out_f32)));
   wide.pair = wide.tr || (p.group_mode != GROUP_M && (p.N % 256 == 0 || p.b_mn_major) && !p.no_pair);
   wide.tile_n = cat ? 128 : 256;
@@ -1707,7 +1745,9 @@ inline TcPlan tc_plan(const GemmProblem& p, int n_sms) {
   }
   // a pair of matrices whose transposed tiles leave SMs idle is better off with the row tiles below, which can be narrow
   // (four d = 512 blocks, eight experts of 144 rows: 1663 us a step with transposed tiles, 1630 without)
-  if (wide.tr && cat && ((p.M - 127 * (int64_t)p.n_groups) / 256 + p.n_groups / 2) * (p.N / 128) < n_sms / 2) wide.tr = wide.pair = false;
+  if (wide.tr && (cat || p.epilogue == EPI_DSWIGLU) &&
+      ((p.M - 127 * (int64_t)p.n_groups) / 256 + p.n_groups / 2) * ceil_div(p.N, cat ? 128 : 256) < n_sms / 2)
+    wide.tr = wide.pair = false;
   if (wide.tr || p.fp8 || p.upd_w) return wide;
   const bool pair_open = p.group_mode != GROUP_M && !p.no_pair && n_sms % 2 == 0;
   const int64_t groups = p.group_mode == GROUP_K ? (p.n_groups > 0 ? p.n_groups : 1) : 1;
@@ -1739,6 +1779,9 @@ inline TcPlan tc_plan(const GemmProblem& p, int n_sms) {
     }
   return best;
 }
+
+// Partial sums of <dH, H> per row that a SwiGLU backward product writes: one per epilogue warp that holds columns of it.
+inline int tc_dg_parts(const GemmProblem& p) { return tc_plan(p, tc_state().n_sms).tr ? p.N / 32 : 2 * (int)ceil_div(p.N, 256); }
 
 inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   TcState& s = tc_state();
@@ -1882,7 +1925,7 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   }
   if (f8 && p.epilogue == EPI_STORE && !tr) return REVFFN_ERR_UNSUPPORTED;      // only the transposed store scales its accumulator
   P.tr = tr ? 1 : 0;
-  P.tiles_f = p.N / (p.concat == CONCAT_N ? 128 : 256);
+  P.tiles_f = (int)ceil_div(p.N, p.concat == CONCAT_N ? 128 : 256);
   P.tr_swap = tr && p.concat == CONCAT_N && reinterpret_cast<uintptr_t>(p.B1) < reinterpret_cast<uintptr_t>(p.B0);
   if (tr && p.concat == CONCAT_N) mb0 = m_gu;
   int64_t total = (int64_t)P.tiles_m * P.tiles_n * (p.group_mode == GROUP_K ? groups : 1);

@@ -120,7 +120,7 @@ static WsLayout plan_workspace(const revffn_moe_desc& D) {
   L.rows_pad = max_padded_rows(T, (int)k, (int)E);
   L.n_chunks = (int)ceil_div(T > 0 ? T : 1, map_chunk_tokens(T));
   L.max_tiles = (int)(L.rows_pad / ROW_PAD);
-  L.dg_ld = (int)ceil_div(I, SIMT_BN);
+  L.dg_ld = (int)ceil_div(I, 32);      // most partial sums per row of any back end and tiling
   L.strips = (int)ceil_div(T > 0 ? T : 1, STRIP);
   const int64_t Rp = L.rows_pad;
   size_t off = 0;
@@ -385,11 +385,11 @@ static int run_gemm(const Ctx<T>& c, GemmProblem p, int tag) {
 }
 
 template <typename T>
-static int dg_parts(const Ctx<T>& c, int N) {
+static int dg_parts(const Ctx<T>& c, const GemmProblem& p) {
   if constexpr (std::is_same<T, bf16>::value) {
-    if (c.tc) return tc_dg_parts(N);
+    if (c.tc) return tc_dg_parts(p);
   }
-  return simt_dg_parts(N);
+  return simt_dg_parts(p.N);
 }
 
 static GemmProblem blank_problem() {
@@ -877,7 +877,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
                                                       c.template p<int32_t>(L.rows_total), d, c.template p<T>(L.dop));
   }
   CK(cudaGetLastError());
-  const int n_part = dg_parts(c, I);
+  int n_part = 0;
   {
     GemmProblem p = blank_problem();   // dH' = dO Wd; SwiGLU backward in place on a|b; dg partials
     p.M = Rp; p.N = I; p.K = d;
@@ -886,9 +886,11 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
     p.group_mode = GROUP_M; p.n_groups = E; p.b_group_stride = (int64_t)d * I;
     p.group_off = c.template p<int32_t>(L.expert_off); p.tile_group = c.template p<int32_t>(L.tile_group);
     p.rows_total = c.template p<int32_t>(L.rows_total);
+    p.tok_chunks = c.template p<int4>(L.tok_chunks);
     p.epilogue = EPI_DSWIGLU; p.ab = c.template p<T>(L.ab); p.ld_ab = 2 * (int64_t)I;
     p.rowscale = c.template p<float>(L.row_gate);
     p.dg_part = c.template p<float>(L.dg_part); p.dg_ld = L.dg_ld;
+    n_part = dg_parts(c, p);
     CKR(run_gemm(c, p, TG_EXP_DH));
   }
   {
@@ -924,7 +926,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
   const bool dense_gate = (D.flags & REVFFN_FLAG_GATE_SOFTMAX_ALL) != 0;
   if (!dense_gate) {
     { ProfScope ps(TG_ROUTER_BWD, st);
-    launch_k(router_bwd_kernel, (unsigned)ceil_div(Tn, 128), 128, 0, st, 
+    launch_k(router_bwd_kernel, (unsigned)ceil_div(Tn, 256 / ROUTER_BWD_LANES), 256, 0, st, 
         c.template p<float>(L.dg_part), L.dg_ld, n_part, c.template p<float>(L.gates), c.template p<int32_t>(L.tok_row),
         Tn, k, c.template p<float>(L.tok_dl), c.template p<float>(L.row_dl));
     }
@@ -942,7 +944,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
   } else {
     // every logit carries a gradient: dL is a dense [T, E] matrix and its products are matrix products
     { ProfScope ps(TG_ROUTER_BWD, st);
-    launch_k(router_bwd_dense_kernel<T>, (unsigned)ceil_div(Tn, 128), 128, 0, st, 
+    launch_k(router_bwd_dense_kernel<T>, (unsigned)ceil_div(Tn, 256 / ROUTER_BWD_LANES), 256, 0, st, 
         c.template p<float>(L.dg_part), L.dg_ld, n_part, c.template p<float>(L.prob), c.template p<int32_t>(L.idx),
         c.template p<int32_t>(L.tok_row), Tn, k, E, L.ld_dlf, c.template p<T>(L.dlf));
     }
