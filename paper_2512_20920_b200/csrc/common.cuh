@@ -103,6 +103,11 @@ inline cudaError_t launch_k(void (*kernel)(Params...), dim3 grid, dim3 block, si
   return launch_cluster(kernel, grid, dim3(1, 1, 1), block, smem, st, args...);
 }
 
+// Padded expert-major rows: every row of the 64 around `row` is padding (row_tok < 0; an expert's real rows come first).
+__device__ __forceinline__ bool padding_group(const int32_t* __restrict__ row_tok, int64_t row) {
+  return row_tok[row & ~static_cast<int64_t>(63)] < 0;
+}
+
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool ok) {      // !ok: 16 zero bytes
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
                ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");

@@ -35,15 +35,17 @@ __device__ __forceinline__ uint2 e4m3_pack8(const float* f, float inv) {
 // between the maximum and the conversion, so the row is read once and nothing goes through shared memory.
 // row_map == NULL: out[r] = quantised in[r].  row_map != NULL (the permutation into the padded expert-major row
 // space): out[r] = quantised in[row_map[r]], zeros with scale 1 for padding rows (row_map[r] < 0); rows at or beyond
-// *rows_total are skipped.  width a multiple of 8, at most 2048.
+// *rows_total are skipped, and with row_tok (the padded row space) groups of 64 padding rows, which nobody reads.  width a
+// multiple of 8, at most 2048.
 __global__ void __launch_bounds__(256)
 quantize_rows_e4m3_kernel(const bf16* __restrict__ in, int64_t ld_in, const int32_t* __restrict__ row_map,
-                          const int32_t* __restrict__ rows_total, int64_t rows, int width, uint8_t* __restrict__ out,
+                          const int32_t* __restrict__ row_tok, const int32_t* __restrict__ rows_total, int64_t rows, int width, uint8_t* __restrict__ out,
                           float* __restrict__ scale) {
   pdl_sync();
   const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows || (rows_total && row >= *rows_total)) return;
+  if (row_tok && row_tok[row] < 0 && padding_group(row_tok, row)) return;      // nobody reads it
   int64_t src = row;
   if (row_map) src = row_map[row];
   Vec8<bf16> v[8];
@@ -77,11 +79,11 @@ quantize_rows_e4m3_kernel(const bf16* __restrict__ in, int64_t ld_in, const int3
   }
 }
 
-inline cudaError_t launch_quantize_rows(const bf16* in, int64_t ld_in, const int32_t* row_map, const int32_t* rows_total,
+inline cudaError_t launch_quantize_rows(const bf16* in, int64_t ld_in, const int32_t* row_map, const int32_t* row_tok, const int32_t* rows_total,
                                         int64_t rows, int width, uint8_t* out, float* scale, cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
   if (width % 8 != 0 || width > 2048) return cudaErrorInvalidValue;
-  launch_k(quantize_rows_e4m3_kernel, (unsigned)ceil_div(rows, 8), 256, 0, st, in, ld_in, row_map, rows_total, rows, width, out, scale);
+  launch_k(quantize_rows_e4m3_kernel, (unsigned)ceil_div(rows, 8), 256, 0, st, in, ld_in, row_map, row_tok, rows_total, rows, width, out, scale);
   return cudaGetLastError();
 }
 

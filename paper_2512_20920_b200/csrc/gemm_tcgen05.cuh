@@ -507,7 +507,7 @@ __device__ __forceinline__ void upd_half(const UpdRule& rule, const SlabOut& o, 
 struct TcTile {
   int m0, n0, group, k_blocks, krow0;
   int ncols;      // accumulator columns in use: the tile's, or 128 in the last column tile of an odd multiple of 128
-  int pad;        // tr: rows of the expert's zero padding after the chunk's (its last chunk only)
+  int pad;        // tr: rows of zero padding after the chunk's, to the next multiple of 64 (an expert's last chunk only)
 };
 
 // A role's walk over the tiles w0, w0 + stride, ...: the tile's index split into its parts, and the table entries that the
@@ -1079,7 +1079,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           // token rows per block.  Lanes l and l + 16 trade halves, each finishes 16 tokens of one feature; then, as
           // above, lanes 2i and 2i+1 trade so that feature pairs go to the staging area ([32 tokens][16 features], and
           // [32 tokens][16 + 16] for the a|b copy) and rows of 32 bytes from there to memory by plain stores.  The rows
-          // of an expert's padding are written as zeros: products over rows (weight gradients) read them.
+          // of padding up to the next multiple of 64 are written as zeros: products over rows (weight gradients) read them.
           // Against 128 token rows x 128 columns of both matrices on one CTA, a pair brings 32 instead of 48 KB into
           // each SM per K step and pads a run of rows to 32 instead of 128 (experts' gate | up at 8192 tokens 302 -> 279 us,
           // with the copy 334 -> 295; at 2741 tokens 155 -> 138 and 167 -> 148)

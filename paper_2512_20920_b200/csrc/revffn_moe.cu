@@ -523,8 +523,8 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
       // product's epilogue applies the scales before the SwiGLU, g*H is quantised row by row, and the down
       // projection (tokens on the MMA N side) applies its scales before it stores.
       { ProfScope ps(TG_GATHER, st);
-      CK(launch_quantize_rows(c.template p<bf16>(L.u), d, c.template p<int32_t>(L.row_tok), c.template p<int32_t>(L.rows_total),
-                              L.rows_pad, d, c.template p<uint8_t>(L.upq), c.template p<float>(L.up_scale), st));
+      CK(launch_quantize_rows(c.template p<bf16>(L.u), d, c.template p<int32_t>(L.row_tok), c.template p<int32_t>(L.row_tok),
+                              c.template p<int32_t>(L.rows_total), L.rows_pad, d, c.template p<uint8_t>(L.upq), c.template p<float>(L.up_scale), st));
       }
       {
         GemmProblem p = blank_problem();
@@ -541,7 +541,7 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
         CKR(run_gemm(c, p, TG_EXP_GATEUP));
       }
       { ProfScope ps(TG_GATHER, st);
-      CK(launch_quantize_rows(c.template p<bf16>(L.hmid), I, nullptr, c.template p<int32_t>(L.rows_total), L.rows_pad, I,
+      CK(launch_quantize_rows(c.template p<bf16>(L.hmid), I, nullptr, c.template p<int32_t>(L.row_tok), c.template p<int32_t>(L.rows_total), L.rows_pad, I,
                               c.template p<uint8_t>(L.hq), c.template p<float>(L.h_scale), st));
       }
       {
@@ -562,9 +562,8 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
   if (!fp8) {
     // Permute: Up[row] = U[token(row)]
     { ProfScope ps(TG_GATHER, st);
-    launch_k(gather_rows_kernel<T>, (unsigned)L.rows_pad, 256, 0, st, c.template p<T>(L.u), d, c.template p<int32_t>(L.row_tok),
-                                                                c.template p<int32_t>(L.rows_total), d,
-                                                                c.template p<T>(L.up));
+    launch_k(gather_rows_kernel<T>, (unsigned)ceil_div(L.rows_pad, GATHER_ROWS), 32 * GATHER_ROWS, 0, st, c.template p<T>(L.u), d,
+             c.template p<int32_t>(L.row_tok), c.template p<int32_t>(L.rows_total), d, c.tc ? 0 : 1, c.template p<T>(L.up));
     }
     CK(cudaGetLastError());
   
@@ -873,8 +872,8 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
 
   // Routed experts backward
   { ProfScope ps(TG_GATHER_DZ, st);
-  launch_k(gather_rows_kernel<T>, (unsigned)Rp, 256, 0, st, c.template p<T>(L.dz), d, c.template p<int32_t>(L.row_tok),
-                                                      c.template p<int32_t>(L.rows_total), d, c.template p<T>(L.dop));
+  launch_k(gather_rows_kernel<T>, (unsigned)ceil_div(Rp, GATHER_ROWS), 32 * GATHER_ROWS, 0, st, c.template p<T>(L.dz), d,
+           c.template p<int32_t>(L.row_tok), c.template p<int32_t>(L.rows_total), d, c.tc ? 0 : 1, c.template p<T>(L.dop));
   }
   CK(cudaGetLastError());
   int n_part = 0;
@@ -1177,7 +1176,7 @@ int revffn_moe_quantize_experts(const revffn_moe_desc* desc, const revffn_moe_we
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   const int64_t E = desc->n_experts, I = desc->d_expert, d = desc->d_model;
   auto q = [&](const void* in, int64_t rows, int width, const void* out, const float* scale) {
-    return launch_quantize_rows(reinterpret_cast<const bf16*>(in), width, nullptr, nullptr, rows, width,
+    return launch_quantize_rows(reinterpret_cast<const bf16*>(in), width, nullptr, nullptr, nullptr, rows, width,
                                 reinterpret_cast<uint8_t*>(const_cast<void*>(out)), const_cast<float*>(scale), st);
   };
   CK(q(w->w_gate, E * I, (int)d, w->q_gate, w->s_gate));
