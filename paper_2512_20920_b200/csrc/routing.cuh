@@ -299,8 +299,8 @@ inline cudaError_t launch_fold_router_mma(const T* w_router, const T* w_sgate, c
 //            over the k selected logits, sigmoid of the shared-gate logit.
 // The split is the same whatever the number of tokens, so a token's logits do not depend on the batch it is in.
 // What bounds it: the serial walk over K at small batches, where splitting K gives eight times the blocks (64 tokens:
-// 47 -> 15 us; 512: 47 -> 15), and at large ones the fp64 tensor pipe at the occupancy of three blocks an SM (8192 tokens:
-// 76 -> 71 us; 8192 x 61 x 1024 multiply-adds are 29 us of the pipe).
+// 47 us with a run of tokens in one block, now 12; 512: 47, now 20), and at large ones the fp64 tensor pipe, idle while the
+// blocks of an SM start and finish (8192 tokens: 76, now 65; 8192 x 61 x 1024 multiply-adds are 29 us of the pipe).
 // idx_in != NULL: expert sets are taken from it (gates are still recomputed).
 // prob_out != NULL: gates are the selected entries of the softmax over ALL experts (not
 // renormalised), and that softmax is written to prob_out[T, E].
@@ -338,14 +338,36 @@ __device__ __forceinline__ void route_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// The double at the same shared-memory place in block `rank` of the cluster.
-__device__ __forceinline__ double ld_cluster_f64(const double* p, uint32_t rank) {
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+// Cluster-wide address of the same shared-memory place in block `rank`, and the double at such an address.
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
   uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ double ld_cluster_f64(uint32_t addr) {
   double v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
   return v;
+}
+// Integers in the order of the doubles, for comparisons beside an fp64 pipe that other blocks keep busy: equal for equal
+// values (both zeros included), NaN as -inf, never 0.
+__device__ __forceinline__ unsigned long long order_key(double v) {
+  long long b = __double_as_longlong(v);
+  if ((b & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL) b = (long long)0xfff0000000000000ULL;
+  if (b == (long long)0x8000000000000000ULL) b = 0;
+  return b < 0 ? ~(unsigned long long)b : (unsigned long long)b | 0x8000000000000000ULL;
+}
+__device__ __forceinline__ double from_order_key(unsigned long long key) {
+  return __longlong_as_double((long long)(key >> 63 ? key & 0x7fffffffffffffffULL : ~key));
+}
+// x^-1/2 to the last places of fp64: two Newton steps, y (3 - x y^2) / 2, from the fp32 value (2^-22 -> 2^-43 -> rounding),
+// nine dependent fp64 operations where a square root and a division take several times as many.
+__device__ __forceinline__ double rsqrt_f64(double x) {
+  if (!(x > 1e-30 && x < 1e30)) return 1.0 / sqrt(x);
+  double y = (double)rsqrtf((float)x);
+  const double hx = 0.5 * x;
+  y = y * fma(-hx * y, y, 1.5);
+  return y * fma(-hx * y, y, 1.5);
 }
 // D (8x8) += A (8x4, row-major fragment) * B (4x8, column-major fragment), fp64.
 // Lane l holds A[l/4][l%4], B[l%4][l/4] and D[l/4][2*(l%4) + {0,1}].
@@ -360,7 +382,7 @@ router_topk_kernel(const float* __restrict__ y, int64_t ld, const float* __restr
                    int tokens, int h, int E, int k, int has_shared, const int32_t* __restrict__ idx_in,
                    int32_t* __restrict__ idx_out, float* __restrict__ gate_out, float* __restrict__ sgate_out,
                    int32_t* __restrict__ idx_user, float* __restrict__ prob_out, int* __restrict__ status,
-                   int check_finite) {
+                   int check_finite, double inv_h) {
   pdl_sync();
   extern __shared__ __align__(16) uint8_t rt_smem[];
   const int EP = E + 1;                       // logits per token incl. the shared-gate row
@@ -461,82 +483,98 @@ router_topk_kernel(const float* __restrict__ y, int64_t ld, const float* __restr
           if (e < EP) Lp[tt * EP + e] = acc[a][b][c];
         }
   }
+  const int tt = (int)rank * 8 + warp, t = t0 + tt;
+  // this lane's biases (columns lane, lane + 32) and, with idx_in, the index of its slot, in flight across the barrier
+  const float bias0 = b_router && lane < E ? b_router[lane] : 0.f, bias1 = b_router && lane + 32 < E ? b_router[lane + 32] : 0.f;
+  const int idx_lane = idx_in && t < tokens && lane < k ? idx_in[(int64_t)t * k + lane] : -1;
   route_cluster_sync();
 
-  // phase 2: top-k and gates; one warp per token
-  const int tt = (int)rank * 8 + warp, t = t0 + tt;
+  // phase 2: top-k and gates; one warp per token.  Each block runs this once, from a cold instruction cache: it is kept
+  // short, its loops rolled (8 rounds of a 5-step shuffle reduction in fp64, unrolled, and a square root and a division
+  // took 13k clk of a block's 45k; now about 6k, 2k of them the other blocks' partial sums: kernel at 8192 tokens 82 -> 65
+  // us, at 512 24 -> 20, at 64 14.1 -> 11.8).
   if (t < tokens) {
     double* L = Lrow + warp * EP;
-    double ss = 0.0;
+    // Partial sums of the squares and of this lane's first two logits, slices in ascending order, all asked for before any
+    // is used.
+    double part[ROUTE_CLUSTER], p0[ROUTE_CLUSTER], p1[ROUTE_CLUSTER];
 #pragma unroll
-    for (int r = 0; r < ROUTE_CLUSTER; ++r) ss += ld_cluster_f64(sq + tt, (uint32_t)r);
-    const double rt = norm_none ? 1.0 : 1.0 / sqrt(ss / (double)h + (double)eps);
-    for (int e = lane; e < EP; e += 32) {
+    for (int r = 0; r < ROUTE_CLUSTER; ++r) {
+      const uint32_t base = cluster_addr(rt_smem, (uint32_t)r);
+      const uint32_t row = base + (uint32_t)(reinterpret_cast<uint8_t*>(Lp + tt * EP) - rt_smem);
+      part[r] = ld_cluster_f64(base + (uint32_t)(reinterpret_cast<uint8_t*>(sq + tt) - rt_smem));
+      p0[r] = ld_cluster_f64(row + 8 * min(lane, EP - 1));
+      p1[r] = ld_cluster_f64(row + 8 * min(lane + 32, EP - 1));
+    }
+    double ss = 0.0, v0 = 0.0, v1 = 0.0;
+#pragma unroll
+    for (int r = 0; r < ROUTE_CLUSTER; ++r) { ss += part[r]; v0 += p0[r]; v1 += p1[r]; }
+    const double rt = norm_none ? 1.0 : rsqrt_f64(ss * inv_h + (double)eps);
+    v0 *= rt; v1 *= rt;
+    if (b_router && lane < E) v0 += (double)bias0;
+    if (b_router && lane + 32 < E) v1 += (double)bias1;
+    if (lane < EP) L[lane] = v0;
+    if (lane + 32 < EP) L[lane + 32] = v1;
+#pragma unroll 1
+    for (int e = lane + 64; e < EP; e += 32) {
       double v = 0.0;
 #pragma unroll
-      for (int r = 0; r < ROUTE_CLUSTER; ++r) v += ld_cluster_f64(Lp + tt * EP + e, (uint32_t)r);
+      for (int r = 0; r < ROUTE_CLUSTER; ++r) v += ld_cluster_f64(cluster_addr(Lp + tt * EP + e, (uint32_t)r));
       v *= rt;
       if (e < E && b_router) v += (double)b_router[e];
       L[e] = v;
     }
     __syncwarp();
-    double sel[8];
-    int seli[8];
     if (check_finite) {
       // a NaN or infinite logit (non-finite input or weight) makes the selection meaningless: report it
       bool bad = false;
       for (int e = lane; e < EP; e += 32) bad |= !isfinite(L[e]);
       if (__any_sync(0xffffffffu, bad) && lane == 0) set_status(status, REVFFN_ERR_NONFINITE);
     }
+    // Lane s < k ends up with the logit (mine) and index of slot s, every lane with the largest selected logit (m).  The
+    // softmax runs in fp32 on the fp64 differences to it (the decision is fp64; the weights are fp32 outputs).
+    const double minus_inf = __longlong_as_double(0xfff0000000000000LL);
+    double m = minus_inf, mine = minus_inf;
+    int mine_i = -1;
     if (idx_in) {
       // Expert sets from the caller.  An index outside [0, E) is reported and kept as -1: the
       // permutation maps skip such an entry, and its gate weight is zero.
-#pragma unroll
-      for (int s = 0; s < 8; ++s)
-        if (s < k) {
-          const int e = idx_in[(int64_t)t * k + s];
-          const bool in_range = (unsigned)e < (unsigned)E;
-          if (!in_range && lane == 0) set_status(status, REVFFN_ERR_INDEX);
-          seli[s] = in_range ? e : -1;
-          sel[s] = in_range ? L[e] : __longlong_as_double(0xfff0000000000000LL);
-        }
-    } else {
-      // candidates of this lane: e = lane + 32 j
-      unsigned taken = 0u;                    // bit j set: candidate j already selected
-#pragma unroll
-      for (int s = 0; s < 8; ++s) {
-        if (s >= k) break;
-        double best = __longlong_as_double(0xfff0000000000000LL);   // -inf
-        int besti = 0x7fffffff;
-        for (int j = 0; lane + 32 * j < E; ++j) {
-          if (taken & (1u << j)) continue;
-          double v = L[lane + 32 * j];
-          if (v != v) v = __longlong_as_double(0xfff0000000000000LL);   // NaN orders as -inf: the comparisons below stay a
-                                                                        // total order and every lane names the same winner
-          int e = lane + 32 * j;
-          if (v > best || (v == best && e < besti) || besti == 0x7fffffff) { best = v; besti = e; }
-        }
-        // warp arg-max: larger value wins, equal values -> lower index
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          double ov = __shfl_xor_sync(0xffffffffu, best, o);
-          int oi = __shfl_xor_sync(0xffffffffu, besti, o);
-          bool take = (oi != 0x7fffffff) && (besti == 0x7fffffff || ov > best || (ov == best && oi < besti));
-          if (take) { best = ov; besti = oi; }
-        }
-        sel[s] = best; seli[s] = besti;
-        if ((besti & 31) == lane) taken |= 1u << (besti >> 5);
+      if (lane < k) {
+        if ((unsigned)idx_lane < (unsigned)E) { mine_i = idx_lane; mine = L[idx_lane]; }
+        else set_status(status, REVFFN_ERR_INDEX);
       }
-    }
-    // gates: lane s < k takes slot s, lane k the shared gate.  The softmax runs in fp32 on the fp64
-    // differences to the largest selected logit (the decision above is fp64; the weights are fp32 outputs).
-    double m = sel[0], mine = sel[0];
-    int mine_i = seli[0];
-#pragma unroll
-    for (int s = 1; s < 8; ++s) {
-      if (s < k) {
-        m = fmax(m, sel[s]);
-        if (lane == s) { mine = sel[s]; mine_i = seli[s]; }
+      m = mine;
+#pragma unroll 1
+      for (int o = 4; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));      // k <= 8
+      m = __shfl_sync(0xffffffffu, m, 0);
+    } else {
+      // k rounds of the warp's arg-max in integers: the upper halves of the keys, among the lanes that hold the maximum the
+      // lower halves, and among equals the lowest index
+      unsigned taken = 0u;                    // bit j set: candidate lane + 32 j already selected
+      const unsigned long long key0 = lane < E ? order_key(v0) : 0ull, key1 = lane + 32 < E ? order_key(v1) : 0ull;
+#pragma unroll 1
+      for (int s = 0; s < k; ++s) {
+        unsigned long long best = taken & 1u ? 0ull : key0;       // 0: below every key
+        int bj = 0;
+        if (!(taken & 2u) && key1 > best) { best = key1; bj = 1; }
+        if (E > 64) {
+#pragma unroll 1
+          for (int j = 2; 32 * j < E; ++j) {
+            const unsigned long long key = lane + 32 * j < E ? order_key(L[lane + 32 * j]) : 0ull;
+            if (!(taken >> j & 1u) && key > best) { best = key; bj = j; }
+          }
+        }
+        const unsigned hi = (unsigned)(best >> 32), lo = (unsigned)best;
+        const unsigned top = __reduce_max_sync(0xffffffffu, hi);
+        const unsigned low = __reduce_max_sync(0xffffffffu, hi == top ? lo : 0u);
+        const unsigned e = (hi == top && lo == low) ? (unsigned)(lane + 32 * bj) : 0xffffffffu;
+        const unsigned win = __reduce_min_sync(0xffffffffu, e);
+        if (e == win) taken |= 1u << bj;
+        if (lane == s || s == 0) {
+          const double v = from_order_key((unsigned long long)top << 32 | low);
+          if (s == 0) m = v;                  // selected in descending order
+          if (lane == s) { mine = v; mine_i = (int)win; }
+        }
       }
     }
     float den;
@@ -597,7 +635,7 @@ inline cudaError_t launch_router_topk(const float* y, int64_t ld, const float* g
   }
   return launch_cluster(router_topk_kernel, dim3((unsigned)(ceil_div(tokens, RT_TOK) * ROUTE_CLUSTER)), dim3(ROUTE_CLUSTER),
                         dim3(256), smem, st, y, ld, gamma, eps, norm_none, w_rc, b_router, tokens, h, E, k, has_shared, idx_in,
-                        idx_out, gate_out, sgate_out, idx_user, prob_out, status, check_finite);
+                        idx_out, gate_out, sgate_out, idx_user, prob_out, status, check_finite, 1.0 / (double)h);
 }
 
 // ---------------------------------------------------------------------------
