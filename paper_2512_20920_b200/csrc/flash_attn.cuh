@@ -9,14 +9,18 @@
 //               columns for each tile.  Per block and tile: O += P_j V_j, then S_{j+1} = Q K_{j+1}^T over the scores that
 //               P_j came from.  While one tile's softmax runs, the tensor pipe works for the other.
 //   warps 2..9  softmax: four warps per tile, one thread per query row (= TMEM lane), all 128 scores of a block in
-//               registers: row maximum, p = exp2((s - m) * scale * log2 e), P as bf16 pairs over the first 64
-//               columns of the score accumulator, from where the second product takes it as its A operand.
-//               O stays in tensor memory.  The row's reference m follows the maximum only when that has grown by more
-//               than a factor 2^8 (p then stays below 2^8, exact in the same number of bits); the warp then rescales
-//               its rows of O, which is at rest: S_j complete means P_{j-1} V_{j-1} complete, both come from one
-//               in-order queue, and P_j V_j waits for this warp.
-// What bounds it: the exponentials (two warps per scheduler on a unit of four a clock: 2048 clk per block of both
-// tiles) beside as much tensor work.  FWDNUMS
+//               registers: p = exp2((s - m) * scale * log2 e), P as bf16 pairs over the first 64 columns of the score
+//               accumulator, from where the second product takes it as its A operand.  O stays in tensor memory.
+//               The row's reference m is its maximum in the first block; later blocks take no maximum, and only when
+//               the weights of a row add up to more than 2^20 in a block (p, P and the sums are floating point: no bit
+//               is lost below that) does the warp take m from that block's maxima and rescale its rows of O, which is
+//               at rest: S_j complete means P_{j-1} V_{j-1} complete, both come from one in-order queue, and P_j V_j
+//               waits for this warp.
+// What bounds it: a pair of blocks takes 3.6k clk, the chain of one tile (softmax 1.85k, products 1.2k, barriers); the
+// exponentials alone are 2.0k (two warps per scheduler on a unit of four a clock), the products 2.3k; a CTA starts and
+// ends in 5-8k.  4 sequences of 2048 x 16 heads: 120 us with one query tile per CTA, the output in registers and maxima
+// exchanged through shared memory; 97 with two tiles; 88 with products issued by a converged warp (the row maxima left
+// out beside that: no difference).  7 x 613: 37 us, as with one tile: five query tiles make three pairs.
 // Operands: q, k, v head-major [.., S_pad, hd] bf16 with hd = 128 (rows past the sequence are zero);
 // output token-major [T, ld_o] bf16, plus the row log-sum-exp (natural log, of the scaled scores).
 // Every wait is bounded; a wait that runs out sets the status word and all roles leave.

@@ -4,10 +4,9 @@
 //   warps 0, 10 TMA producers: cp.async.bulk.tensor loads (128-byte swizzle) of
 //               A and B tiles into a ring of shared-memory stages, completion on
 //               mbarriers (no multicast LOADS anywhere: every CTA fetches its own operands; the only
-//               cluster-wide instruction is the pair mode's tcgen05.commit, a barrier arrive).  One thread
-//               of warp 0 announces a stage's bytes and loads the first operand's share, one thread of
-//               warp 10 loads the second operand's: a single thread cannot issue a stage's loads as fast
-//               as the tensor core consumes them.
+//               cluster-wide instruction is the pair mode's tcgen05.commit, a barrier arrive).  Warp 0
+//               announces a stage's bytes and loads the first operand's share, warp 10 loads the second
+//               operand's: one warp cannot issue a stage's loads as fast as the tensor core consumes them.
 //   warp 1      MMA issuer: owns the TMEM allocation (two accumulators, so the
 //               epilogue of tile i overlaps the main loop of tile i+1); one
 //               elected lane issues tcgen05.mma kind::f16 (bf16 x bf16 -> fp32),
@@ -38,8 +37,8 @@
 // arrive on the barriers of both CTAs, both CTAs' loads complete on its "full" barriers, and
 // both CTAs' epilogue warps release its accumulator barriers.
 //
-// Transposed pair mode (expert-grouped products with bf16 store or gate-scale epilogue): the
-// pair computes C^T.  The MMA M side holds 256 output features (rows of the expert's weight
+// Transposed pair mode (expert-grouped products with bf16 store, gate-scale, SwiGLU or SwiGLU
+// backward epilogue): the pair computes C^T.  The MMA M side holds 256 output features (rows of the expert's weight
 // matrix, 128 per CTA), the N side a run of up to 256 of the expert's token rows, real rows
 // only (rounded up to 32), taken from a chunk table built with the permutation.  Padding rows
 // then cost no tensor-core time, and these products get the pair mode's operand savings, which
@@ -653,18 +652,18 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
 
   if (warp == 0 || warp == TC_LOAD_WARP_B) {
     // ------------------------------------------------------------------ operand loads
-    // Two threads, one in each load warp, walk the same tiles and stages.  A tensor load takes the issuing thread
-    // 150-250 clocks (more in the pair form, whose completion is signalled in the partner CTA), and a stage needs
-    // two to six of them: issued by one thread they took 500-850 clocks per stage, more than the 512 clocks of
-    // tensor work in a stage, and the MMA thread waited for operands in every product.  Thread A announces the
-    // stage's bytes and loads the first operand's share of the stage, thread B loads the second operand's; the
-    // bytes may arrive before they are announced (the barrier's phase cannot complete before the announcing
-    // arrival).
+    // Two warps walk the same tiles and stages, all lanes together, and one elected lane of each issues a K step's loads:
+    // in a loop that one lane runs alone every operand of a load is moved to a uniform register first (forward of 64
+    // tokens 286 -> 277 us, fp8 forward at 8192 1048 -> 1023, step at 8192 5328 -> 5267 by this alone).  A K step's loads
+    // still take a warp 260-310 clocks, of which all of them in one warp would be more than the 512 clocks of tensor
+    // work in a stage.  Warp A announces the stage's bytes and loads the first operand's share of the stage, warp B
+    // loads the second operand's; the bytes may arrive before they are announced (the barrier's phase cannot complete
+    // before the announcing arrival).
     // (A version of this loop that kept per-tile "load slots" -- tensor-map pointer, destination, coordinates --
     // in registers and issued one load per slot measured 15-40 % slower: a load whose tensor map is named through
     // a pointer chosen at run time, rather than as the kernel parameter itself, is slow to issue.)
-    // la: this thread loads the first operand's share (and announces the stage); lb: the second operand's.
-    // Without split_loads the first warp's thread does both and the second warp has nothing to do.
+    // la: this warp loads the first operand's share (and announces the stage); lb: the second operand's.
+    // Without split_loads the first warp does both and the second warp has nothing to do.
     const bool la = warp == 0, lb = P.split_loads ? warp != 0 : warp == 0;
     if (!P.starve && (la || lb)) {
       int stage = 0;
@@ -827,11 +826,12 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    // One thread issues every product of the CTA (pair), so the cycles this loop spends per K step bound the
-    // kernel as surely as the tensor pipe does: four products take about 300 clocks to issue and the commit
-    // 60, against 512 clocks of tensor work in a 128 x 256 x 64 step.  Everything that does not change inside a
-    // tile (descriptor high words, layout steps, barrier addresses) is therefore set up outside the loop, and a
-    // K step costs the wait, two additions, the four products and the commit.
+    // One lane issues every product of the CTA (pair), so the cycles this loop spends per K step bound the
+    // kernel as surely as the tensor pipe does: 512 clocks of tensor work in a 128 x 256 x 64 step, less in narrow
+    // tiles.  The warp walks the loop converged and elects the lane, which keeps operands in uniform registers (a loop
+    // in one lane: about 300 clocks for four products and 60 for the commit; steps at 512 and 8192 tokens 1496 -> 1480
+    // and 5479 -> 5416 us, fp8 forward at 8192 1083 -> 1056).  Everything that does not change inside a tile (descriptor
+    // high words, layout steps, barrier addresses) is set up outside the loop.
     if (crank == 0) {
       int stage = 0;
       uint32_t phase = 0;
@@ -1203,7 +1203,9 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           // 16-byte stores, 4 rows x 128 bytes per instruction: whole lines, and nothing to wait for
           // before the area is reused.  (A TMA store of such a block sat behind the producer's operand
           // loads in the copy engine; with the short K of a weight gradient that wait set the pace.)
-          // A block's accumulator is fetched while the block before it is written: F32NUMS
+          // A block's accumulator is fetched while the block before it is written.  With one K step per tile the kernel
+          // writes 6 TB/s (experts' gate | up gradient at 512 tokens, 1.38 GB: 240 us); at 8192 tokens a tile's four blocks
+          // take 6.5k clk beside 5k of main loop, 410 us.
           const int rsub = lane >> 3;
           const bool all_rows = out.rows >= 32;
           auto fetch = [&](int c) { if (have_acc && c < t.ncols) tmem_ld32(taddr + c, r0); };
@@ -1725,7 +1727,7 @@ struct TcPlan { bool tr, pair; int tile_n; };
 // shortest reckoned time (main loop plus fill and epilogue), if that is a fifth shorter.  The constants are clocks measured
 // on the kernel: a K step is bound by its tensor work (2 clk per column; the pair's instructions add about 90) or by the
 // bytes it brings into an SM (about 68 B/clk); an epilogue takes about 10 clk per column of bf16 and 22 of fp32; the
-// first loads and the start take 2500.  Four d = 512 blocks, 384 tokens: 1990 -> PLAN1 us a step; forward of 64 tokens
+// first loads and the start take 2500.  Four d = 512 blocks, 384 tokens: 1990 -> 1738 us a step; forward of 64 tokens
 // 304 -> 291.  Products that fill the GPU keep wide tiles even where the last round is thin: narrow ones move more
 // bytes per flop, and another stream's kernels use the SMs that are left over (chosen by time alone, a step at 2741
 // tokens went from 2547 to 2689 us, at 512 from 1504 to 1574).
