@@ -11,16 +11,18 @@
 //   warps 2..9  softmax: four warps per tile, one thread per query row (= TMEM lane), all 128 scores of a block in
 //               registers: p = exp2((s - m) * scale * log2 e), P as bf16 pairs over the first 64 columns of the score
 //               accumulator, from where the second product takes it as its A operand.  O stays in tensor memory.
-//               The row's reference m is its maximum in the first block; later blocks take no maximum, and only when
-//               the weights of a row add up to more than 2^20 in a block (p, P and the sums are floating point: no bit
-//               is lost below that) does the warp take m from that block's maxima and rescale its rows of O, which is
-//               at rest: S_j complete means P_{j-1} V_{j-1} complete, both come from one in-order queue, and P_j V_j
-//               waits for this warp.
-// What bounds it: a pair of blocks takes 3.6k clk, the chain of one tile (softmax 1.85k, products 1.2k, barriers); the
-// exponentials alone are 2.0k (two warps per scheduler on a unit of four a clock), the products 2.3k; a CTA starts and
-// ends in 5-8k.  4 sequences of 2048 x 16 heads: 120 us with one query tile per CTA, the output in registers and maxima
-// exchanged through shared memory; 97 with two tiles; 88 with products issued by a converged warp (the row maxima left
-// out beside that: no difference).  7 x 613: 37 us, as with one tile: five query tiles make three pairs.
+//               The row's reference m is its maximum in the first block.  It is taken anew from a block's maxima, and
+//               the warp's rows of O rescaled, only when the weights of the block's first 64 keys add up to more than
+//               2^20 or one of the others passes 2^14 (p, P and the sums are floating point: no bit is lost below that).
+//               O is at rest then: S_j complete means P_{j-1} V_{j-1} complete, both come from one in-order queue, and
+//               P_j V_j waits for this warp.  P goes out in halves of 64 keys, so that P V starts under the exponentials
+//               of the second half.
+// What bounds it: a pair of blocks takes about 3.5k clk, the chain of one tile (softmax 1.85k, products 1.2k, of which a
+// quarter k lies under the softmax, barriers); the exponentials alone are 2.0k (two warps per scheduler on a unit of four a
+// clock), the products 2.3k; a CTA starts and ends in 5-8k.  4 sequences of 2048 x 16 heads: 120 us with one query tile per
+// CTA, the output in registers and maxima exchanged through shared memory; 97 with two tiles; 88 with products issued by a
+// converged warp (the row maxima left out beside that: no difference); P in halves 92 -> 88 on another box.  7 x 613: 38 ->
+// 36 us: five query tiles make three pairs.
 // Operands: q, k, v head-major [.., S_pad, hd] bf16 with hd = 128 (rows past the sequence are zero);
 // output token-major [T, ld_o] bf16, plus the row log-sum-exp (natural log, of the scaled scores).
 // Every wait is bounded; a wait that runs out sets the status word and all roles leave.
@@ -39,7 +41,8 @@ constexpr int FA_K_OFF = 4 * FA_TILE;             // K: 2 stages x 2 tiles
 constexpr int FA_V_OFF = FA_K_OFF + 4 * FA_TILE;  // V: 2 stages x 2 k-blocks (each 2 chunks of 8 KB)
 constexpr int FA_BAR_OFF = FA_V_OFF + 4 * FA_TILE;
 constexpr int FA_SMEM_BYTES = FA_BAR_OFF + 256 + 1024;      // + alignment slack
-constexpr float FA_SUM_MAX = 1048576.f;           // sum of a row's weights in a block above which the row's reference follows
+constexpr float FA_SUM_MAX = 1048576.f;           // sum of a row's weights of 64 keys above which the row's reference follows
+constexpr float FA_LOG2_MAX = 14.f;               // log2 of a single weight above which it does
 
 __device__ __forceinline__ float fa_exp2(float x) {
   float y;
@@ -104,7 +107,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
   // barrier slots (8 bytes each)
   auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
   enum { B_QFULL = 0, B_KFULL = 1, B_KEMPTY = 3, B_VFULL = 5, B_VEMPTY = 7, B_SFULL = 9, B_PFULL = 11, B_OFULL = 13, B_DRAIN = 15,
-         B_COUNT = 16 };
+         B_PHALF = 16, B_COUNT = 18 };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen_base + FA_BAR_OFF + 8 * B_COUNT);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(gen_base + FA_BAR_OFF + 8 * B_COUNT + 8);
   int* issued = reinterpret_cast<int*>(gen_base + FA_BAR_OFF + 8 * B_COUNT + 16);   // [5]: q, k0, k1, v0, v1 -> phase + 1
@@ -125,7 +128,8 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
     for (int s = 0; s < 2; ++s) {
       mbar_init(bar(B_KFULL + s), 1); mbar_init(bar(B_KEMPTY + s), 1);
       mbar_init(bar(B_VFULL + s), 1); mbar_init(bar(B_VEMPTY + s), 1);
-      mbar_init(bar(B_SFULL + s), 1); mbar_init(bar(B_PFULL + s), 4); mbar_init(bar(B_OFULL + s), 1);
+      mbar_init(bar(B_SFULL + s), 1); mbar_init(bar(B_PHALF + s), 4); mbar_init(bar(B_PFULL + s), 4);
+      mbar_init(bar(B_OFULL + s), 1);
     }
     mbar_init(bar(B_DRAIN), 1);
     for (int i = 0; i < 5; ++i) issued[i] = 0;
@@ -216,19 +220,20 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
       for (int x = 0; x < 2; ++x) {
         const int n_x = (x == 0 || two) ? 2 * qp + x + 1 : 0;
         if (j < n_x && ok) {
-          ok = wait(B_PFULL + x, (uint32_t)j & 1u);                                // P_j: its columns may be read
-          if (ok) {
-            const uint64_t b_desc = make_smem_desc(sb + FA_V_OFF + 2 * b * FA_TILE, 8192, 1024);
-            if (elect_one()) {
+          const uint64_t b_desc = make_smem_desc(sb + FA_V_OFF + 2 * b * FA_TILE, 8192, 1024);
 #pragma unroll
-              for (int k = 0; k < 8; ++k)
+          for (int h = 0; h < 2; ++h) {         // 64 keys each, as P_j's columns become readable
+            if (ok) ok = wait((h ? B_PFULL : B_PHALF) + x, (uint32_t)j & 1u);
+            if (ok && elect_one()) {
+#pragma unroll
+              for (int k = 4 * h; k < 4 * h + 4; ++k)
                 tc_mma_ta(tb + (uint32_t)(256 + 128 * x), tb + (uint32_t)(128 * x + 8 * k),
                           b_desc + (uint64_t)((k >> 2) * (FA_TILE >> 4) + 128 * (k & 3)), idesc_pv, (j | k) != 0 ? 1u : 0u);
-              if (j + 1 == n_x) tc_commit(bar(B_OFULL + x));
+              if (h == 1 && j + 1 == n_x) tc_commit(bar(B_OFULL + x));
             }
             __syncwarp();
-            if (j + 1 < n_x) issue_qk(j + 1, x);
           }
+          if (ok && j + 1 < n_x) issue_qk(j + 1, x);
         }
       }
       if (!ok) break;
@@ -257,11 +262,11 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
       ok = __all_sync(0xffffffffu, mbar_wait(bar(B_SFULL + x), (uint32_t)j & 1u, abort_flag, P.status));
       if (!ok) break;
       tc_fence_after();
-      uint32_t p0[32], p1[32];
-      float sum;
+      uint32_t pw[32], r2[32], r3[32];
+      float2 s0;
       bool ref = j == 0;        // take the reference from this block's maxima
       while (true) {
-        uint32_t r0[32], r1[32], r2[32], r3[32];
+        uint32_t r0[32], r1[32];
         tmem_ld32(s_addr, r0);
         tmem_ld32(s_addr + 32, r1);
         tmem_ld32(s_addr + 64, r2);
@@ -299,14 +304,25 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
           }
           m = m_new;
         }
-        const float2 s0 = fa_probs64(r0, r1, cl, m * cl, p0), s1 = fa_probs64(r2, r3, cl, m * cl, p1);
-        sum = (s0.x + s0.y) + (s1.x + s1.y);
-        if (ref || !__any_sync(0xffffffffu, !(sum <= FA_SUM_MAX))) break;
+        // the first half's weights; of the second half only that they will not be too large (the maximum hides under the
+        // exponentials), so that the product may start on the first
+        s0 = fa_probs64(r0, r1, cl, m * cl, pw);
+        if (ref) break;
+        float b0 = __uint_as_float(r2[0]), b1 = __uint_as_float(r3[0]);
+#pragma unroll
+        for (int i = 1; i < 32; ++i) { b0 = fmaxf(b0, __uint_as_float(r2[i])); b1 = fmaxf(b1, __uint_as_float(r3[i])); }
+        const bool fits = s0.x + s0.y <= FA_SUM_MAX && (fmaxf(b0, b1) - m) * cl <= FA_LOG2_MAX;
+        if (!__any_sync(0xffffffffu, !fits)) break;
         ref = true;
       }
-      tmem_st32(s_addr, p0);
-      tmem_st32(s_addr + 32, p1);
-      l += sum;
+      tmem_st32(s_addr, pw);
+      tmem_st_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(B_PHALF + x));
+      const float2 s1 = fa_probs64(r2, r3, cl, m * cl, pw);
+      tmem_st32(s_addr + 32, pw);
+      l += (s0.x + s0.y) + (s1.x + s1.y);
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();

@@ -41,3 +41,25 @@ def test_forward_and_backward_at_tile_edges(seq_len, std):
         assert br.status() == 0
         g1, g2, _ = orc.backward(w, s["x1"], s["x2"], s["dy1"], **oa)
         assert rel_l2(dx1.cpu().numpy() - s["dy1"], g1 - s["dy1"]) < 2e-2 and rel_l2(dx2.cpu().numpy(), g2) < 2e-2
+
+
+@pytest.mark.parametrize("seq_len", [200, 256, 600, 1100])
+def test_row_maxima_that_grow_along_the_keys(seq_len):
+    """Biases in one slowly rotating pair of q and k add 20 cos(0.0029 distance) to every score: towards a late query the
+    scores grow by 16 to 39 (23 to 56 in log2) from the first block to its own (600 and 1100 positions), past what the first block's reference may stay.
+    q and k rounded to bf16 move such a score by 20 * 2^-9 * sqrt(2/3) = 0.03, which the sum over some hundred keys of
+    like weight brings below the path's 2e-2."""
+    import paper_2512_20920_b200 as rv
+    cfg = AttnConfig("grow", batch=1, seq_len=seq_len, d_model=512, n_heads=4, n_kv_heads=2, weight_dtype="bf16")
+    w, s = make_attn_weights(cfg, 6, std=0.03, bias_std=0.03), make_attn_streams(cfg, 6)
+    for n in ("b_q", "b_k"):
+        w[n] = w[n].copy()
+        w[n][27::128] = 15.0
+    f32 = ("norm_gamma", "b_q", "b_k", "b_v")
+    dw = {n: torch.from_numpy(np.ascontiguousarray(v)).to("cuda", torch.float32 if n in f32 else torch.bfloat16) for n, v in w.items()}
+    br = rv.AttnBranch(batch=1, seq_len=seq_len, d_model=512, n_heads=4, n_kv_heads=2, weight_dtype=rv.BF16, weights=dw,
+                       norm_eps=cfg.norm_eps, rope_theta=cfg.rope_theta)
+    y1 = br.forward(dev(s["x1"]), dev(s["x2"]))
+    assert br.status() == 0
+    want = orc.forward(w, s["x1"], s["x2"], S=seq_len, n_heads=4, n_kv_heads=2, eps=cfg.norm_eps, theta=cfg.rope_theta) - s["x1"]
+    assert rel_l2(y1.cpu().numpy() - s["x1"], want) < 2e-2
