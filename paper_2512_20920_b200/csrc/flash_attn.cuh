@@ -14,6 +14,10 @@
 //               The row's reference m is its maximum in the first block.  It is taken anew from a block's maxima, and
 //               the warp's rows of O rescaled, only when the weights of the block's first 64 keys add up to more than
 //               2^20 or one of the others passes 2^14 (p, P and the sums are floating point: no bit is lost below that).
+//               O is divided by the sum of the weights as P holds them: relative to the first block's maximum a row's
+//               largest weight is not a power of two, and its rounding to bf16 would scale the whole row by up to 2^-8.
+//               (Against fp64, 4 x 2048 and 7 x 613: the branch's error is 0.2 % below that of the exact sum relative to a running maximum;
+//               divided by the exact sum of these weights 0.05 % above, with scores of a standard deviation of 3 0.9 %.)
 //               O is at rest then: S_j complete means P_{j-1} V_{j-1} complete, both come from one in-order queue, and
 //               P_j V_j waits for this warp.  P goes out in halves of 64 keys, so that P V starts under the exponentials
 //               of the second half.
@@ -21,8 +25,10 @@
 // quarter k lies under the softmax, barriers); the exponentials alone are 2.0k (two warps per scheduler on a unit of four a
 // clock), the products 2.3k; a CTA starts and ends in 5-8k.  4 sequences of 2048 x 16 heads: 120 us with one query tile per
 // CTA, the output in registers and maxima exchanged through shared memory; 97 with two tiles; 88 with products issued by a
-// converged warp (the row maxima left out beside that: no difference); P in halves 92 -> 88 on another box.  7 x 613: 38 ->
-// 36 us: five query tiles make three pairs.
+// converged warp (the row maxima left out beside that: no difference); P in halves 92 -> 88 on another box.  The second sum
+// costs 4 us there, 82 -> 86, in two unpackings and an addition per pair of weights; a gradient pass, which wants both sums,
+// fetches the second half's scores twice instead of spilling registers (117 -> 103).  7 x 613: 38 -> 36 us when five query
+// tiles made three pairs; 33 -> 35 by the second sum.
 // Operands: q, k, v head-major [.., S_pad, hd] bf16 with hd = 128 (rows past the sequence are zero);
 // output token-major [T, ld_o] bf16, plus the row log-sum-exp (natural log, of the scaled scores).
 // Every wait is bounded; a wait that runs out sets the status word and all roles leave.
@@ -50,20 +56,23 @@ __device__ __forceinline__ float fa_exp2(float x) {
   return y;
 }
 
-// p = exp2(s * cl - mc) for 64 scores of this thread's row, packed to bf16; returns their sum in two halves.
+// p = exp2(s * cl - mc) for 64 scores of this thread's row, packed to bf16.  Returns the sum of the packed values (.y) and,
+// with SUM, of the weights themselves (.x).
+template <bool SUM>
 __device__ __forceinline__ float2 fa_probs64(const uint32_t (&r0)[32], const uint32_t (&r1)[32], float cl, float mc, uint32_t (&pw)[32]) {
-  float2 sum = make_float2(0.f, 0.f);
+  float2 sum = make_float2(0.f, 0.f), rounded = make_float2(0.f, 0.f);
   const float2 c2 = make_float2(cl, cl), m2 = make_float2(-mc, -mc);
 #pragma unroll
   for (int i = 0; i < 32; ++i) {
     const uint32_t* r = i < 16 ? &r0[2 * i] : &r1[2 * i - 32];
     const float2 t = __ffma2_rn(make_float2(__uint_as_float(r[0]), __uint_as_float(r[1])), c2, m2);
     const float2 e = make_float2(fa_exp2(t.x), fa_exp2(t.y));
-    sum = __fadd2_rn(sum, e);
+    if (SUM) sum = __fadd2_rn(sum, e);
     const __nv_bfloat162 h = __floats2bfloat162_rn(e.x, e.y);
+    rounded = __fadd2_rn(rounded, __bfloat1622float2(h));
     pw[i] = *reinterpret_cast<const uint32_t*>(&h);
   }
-  return sum;
+  return make_float2(sum.x + sum.y, rounded.x + rounded.y);
 }
 
 // 32 consecutive 32-bit columns of this thread's TMEM lane, written from registers.
@@ -90,12 +99,14 @@ __device__ __forceinline__ void tc_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint
 struct FlashParams {
   int S, Sp, n_heads, rep;        // rep = query heads per key/value head
   bf16* o; int64_t ld_o;          // [T, ld_o]
-  float* lse;                     // [B * n_heads * Sp] or NULL
-  float* o32;                     // [B * n_heads * Sp, 128] or NULL: the output before rounding, head-major
+  float* lse;                     // GRAD: [B * n_heads * Sp]
+  float* o32;                     // GRAD: [B * n_heads * Sp, 128], the output before rounding, head-major
   float scale_log2e, scale;
   int* status;
 };
 
+// GRAD: for a gradient pass, which also wants the row log-sum-exp and the output before rounding.
+template <bool GRAD>
 __global__ void __launch_bounds__(FA_THREADS, 1)
 flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v) {
@@ -255,7 +266,11 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     const uint32_t s_addr = lane_addr + (uint32_t)(128 * x), o_addr = lane_addr + (uint32_t)(256 + 128 * x);
     const int n_x = (x == 0 || two) ? 2 * qp + x + 1 : 0;
-    float m = -INFINITY, l = 0.f;
+    // l.x: sum of the weights, for the row's log-sum-exp.  l.y: of the rounded weights that P V uses, which O is divided
+    // by: a weight that outweighs all others then cancels whatever its rounding (it is exact only when the reference is
+    // its own score), and the others' errors act on their values' distance from the mean.
+    float m = -INFINITY;
+    float2 l = make_float2(0.f, 0.f);
     const float cl = P.scale_log2e;
     bool ok = true;
     for (int j = 0; j < n_x; ++j) {
@@ -265,33 +280,36 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
       uint32_t pw[32], r2[32], r3[32];
       float2 s0;
       bool ref = j == 0;        // take the reference from this block's maxima
+      auto load64 = [&](int c, uint32_t (&a)[32], uint32_t (&b)[32]) {
+        tmem_ld32(s_addr + c, a);
+        tmem_ld32(s_addr + c + 32, b);
+        tmem_ld_wait();
+        if (j + 1 < n_x) return;
+        // the diagonal block: keys past the query position
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          if (c + i > row) a[i] = 0xff800000u;
+          if (c + 32 + i > row) b[i] = 0xff800000u;
+        }
+      };
       while (true) {
         uint32_t r0[32], r1[32];
-        tmem_ld32(s_addr, r0);
-        tmem_ld32(s_addr + 32, r1);
-        tmem_ld32(s_addr + 64, r2);
-        tmem_ld32(s_addr + 96, r3);
-        tmem_ld_wait();
-        if (j + 1 == n_x) {      // the diagonal block: keys past the query position
+        load64(64, r2, r3);
+        float b0 = __uint_as_float(r2[0]), b1 = __uint_as_float(r3[0]);
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            if (i > row) r0[i] = 0xff800000u;
-            if (32 + i > row) r1[i] = 0xff800000u;
-            if (64 + i > row) r2[i] = 0xff800000u;
-            if (96 + i > row) r3[i] = 0xff800000u;
-          }
-        }
+        for (int i = 1; i < 32; ++i) { b0 = fmaxf(b0, __uint_as_float(r2[i])); b1 = fmaxf(b1, __uint_as_float(r3[i])); }
+        float b = fmaxf(b0, b1);
+        if (GRAD) asm volatile("" : "+f"(b));      // the second half's registers are free from here: it is fetched again below
+        load64(0, r0, r1);
         if (ref) {
-          float a0 = m, a1 = m, a2 = m, a3 = m;
+          float a0 = m, a1 = b;
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            a0 = fmaxf(a0, __uint_as_float(r0[i])); a1 = fmaxf(a1, __uint_as_float(r1[i]));
-            a2 = fmaxf(a2, __uint_as_float(r2[i])); a3 = fmaxf(a3, __uint_as_float(r3[i]));
-          }
-          const float m_new = fmaxf(fmaxf(a0, a1), fmaxf(a2, a3));
+          for (int i = 0; i < 32; ++i) { a0 = fmaxf(a0, __uint_as_float(r0[i])); a1 = fmaxf(a1, __uint_as_float(r1[i])); }
+          const float m_new = fmaxf(a0, a1);
           if (j > 0) {
             const float alpha = fa_exp2((m - m_new) * cl);
-            l *= alpha;
+            if (GRAD) l.x *= alpha;
+            l.y *= alpha;
 #pragma unroll 1
             for (int c = 0; c < 128; c += 32) {
               uint32_t o[32];
@@ -306,12 +324,9 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
         }
         // the first half's weights; of the second half only that they will not be too large (the maximum hides under the
         // exponentials), so that the product may start on the first
-        s0 = fa_probs64(r0, r1, cl, m * cl, pw);
+        s0 = fa_probs64<GRAD>(r0, r1, cl, m * cl, pw);
         if (ref) break;
-        float b0 = __uint_as_float(r2[0]), b1 = __uint_as_float(r3[0]);
-#pragma unroll
-        for (int i = 1; i < 32; ++i) { b0 = fmaxf(b0, __uint_as_float(r2[i])); b1 = fmaxf(b1, __uint_as_float(r3[i])); }
-        const bool fits = s0.x + s0.y <= FA_SUM_MAX && (fmaxf(b0, b1) - m) * cl <= FA_LOG2_MAX;
+        const bool fits = s0.y <= FA_SUM_MAX && (b - m) * cl <= FA_LOG2_MAX;
         if (!__any_sync(0xffffffffu, !fits)) break;
         ref = true;
       }
@@ -320,9 +335,11 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(B_PHALF + x));
-      const float2 s1 = fa_probs64(r2, r3, cl, m * cl, pw);
+      if (GRAD) load64(64, r2, r3);
+      const float2 s1 = fa_probs64<GRAD>(r2, r3, cl, m * cl, pw);
       tmem_st32(s_addr + 32, pw);
-      l += (s0.x + s0.y) + (s1.x + s1.y);
+      if (GRAD) l.x += s0.x + s1.x;
+      l.y += s0.y + s1.y;
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
@@ -334,7 +351,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
       // out through this tile's Q area (its products are complete), 64- and 128-byte row pieces per instruction
       const int s_pos0 = (2 * qp + x) * FA_BLK + q * 32, s_pos = s_pos0 + lane;
       const int rows_ok = min(32, P.S - s_pos0);
-      const float inv = 1.f / l;
+      const float inv = 1.f / l.y;
       const int seq = bh / P.n_heads, head = bh % P.n_heads;
       uint8_t* stg = gen_base + FA_Q_OFF + x * 2 * FA_TILE + q * 8192;
       bf16* dst = P.o + ((int64_t)seq * P.S + s_pos0) * P.ld_o + (int64_t)head * FA_HD;
@@ -347,7 +364,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
 #pragma unroll
         for (int i = 0; i < 32; ++i) f[i] = __uint_as_float(o[i]) * inv;
         stage32_bf16(stg, lane, f);
-        if (P.o32) {
+        if (GRAD) {
 #pragma unroll
           for (int g = 0; g < 8; ++g)
             *reinterpret_cast<float4*>(stg + 4096 + lane * 128 + ((g ^ (lane & 7)) << 4)) =
@@ -355,7 +372,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
         }
         __syncwarp();
         blk_stage_to_global(stg, lane, dst + c, P.ld_o, rows_ok);
-        if (P.o32) {
+        if (GRAD) {
           float* d32 = P.o32 + ((int64_t)bh * P.Sp + s_pos0) * FA_HD + c;
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
@@ -366,7 +383,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
         }
         __syncwarp();
       }
-      if (P.lse && lane < rows_ok) P.lse[(int64_t)bh * P.Sp + s_pos] = m * P.scale + logf(l);
+      if (GRAD && lane < rows_ok) P.lse[(int64_t)bh * P.Sp + s_pos] = m * P.scale + logf(l.x);
     }
   }
 
@@ -389,7 +406,8 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
   }
 }
 
-// q: [B * n_heads * Sp, 128], k, v: [B * n_kv_heads * Sp, 128] bf16 head-major; o: [B * S, ld_o] bf16.
+// q: [B * n_heads * Sp, 128], k, v: [B * n_kv_heads * Sp, 128] bf16 head-major; o: [B * S, ld_o] bf16.  lse and o32 are
+// written when o32 is given.
 inline int launch_flash_fwd(const bf16* q, const bf16* k, const bf16* v, int batch, int n_heads, int n_kv_heads, int S, int Sp,
                             bf16* o, int64_t ld_o, float* lse, float* o32, int* status, cudaStream_t st) {
   TcState& s = tc_state();
@@ -399,7 +417,8 @@ inline int launch_flash_fwd(const bf16* q, const bf16* k, const bf16* v, int bat
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return REVFFN_ERR_CUDA;
   if (!attr_set[dev]) {
-    if (cudaFuncSetAttribute(flash_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FA_SMEM_BYTES) != cudaSuccess)
+    if (cudaFuncSetAttribute(flash_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FA_SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(flash_fwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FA_SMEM_BYTES) != cudaSuccess)
       return REVFFN_ERR_CUDA;
     attr_set[dev] = true;
   }
@@ -417,7 +436,7 @@ inline int launch_flash_fwd(const bf16* q, const bf16* k, const bf16* v, int bat
   P.scale_log2e = P.scale * 1.4426950408889634f;
   P.status = status;
   const int grid = batch * n_heads * ((Sp / FA_BLK + 1) / 2);
-  launch_k(flash_fwd_kernel, grid, FA_THREADS, FA_SMEM_BYTES, st, P, mq, mk, mv);
+  launch_k(o32 ? flash_fwd_kernel<true> : flash_fwd_kernel<false>, grid, FA_THREADS, FA_SMEM_BYTES, st, P, mq, mk, mv);
   return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 

@@ -63,3 +63,35 @@ def test_row_maxima_that_grow_along_the_keys(seq_len):
     assert br.status() == 0
     want = orc.forward(w, s["x1"], s["x2"], S=seq_len, n_heads=4, n_kv_heads=2, eps=cfg.norm_eps, theta=cfg.rope_theta) - s["x1"]
     assert rel_l2(y1.cpu().numpy() - s["x1"], want) < 2e-2
+
+
+@pytest.mark.parametrize("key", [20, 150, 200, 400, 601])
+def test_a_dominating_weight_keeps_its_value(key):
+    """One key's weight is 2^13.007 times every other one's, a number that bf16 holds to 0.3 % only, and the row's reference
+    stays that of the first block when the key comes later.  The weight's rounding must cancel in the output.
+
+    Identities for P_up, W_v, W_o and P_down make Y1 - X1 the first head's output in bf16; X1 = 0 makes the queries b_q, one
+    nearly unturned pair (1.2e-6 per position) reads one feature of the keys, and X2 holds +-1.  With w the dominating
+    weight's share, rounded weights p (1 + e), |e| <= 2^-8, move the weighted mean of values in [-1, 1] by at most
+    2 * 2^-8 * 2 (1 - w), and its rounding to bf16 (below 1) by 2^-9; 1e-4 covers the table, the norm's eps and fp32."""
+    import paper_2512_20920_b200 as rv
+    S, d, h = 640, 256, 128
+    rng = np.random.default_rng(8)
+    x2 = np.where(rng.random((S, h)) < 0.5, -1.0, 1.0).astype(np.float32)
+    x2[:, 0] = -1.0
+    x2[key, 0] = 1.0
+    eye = torch.eye(d)
+    w = dict(w_up=eye[:, :h], w_down=eye[:h], w_q=torch.zeros(d, d), w_k=torch.zeros(d, d), w_v=eye.clone(), w_o=eye.clone())
+    w["w_k"][63, 0] = 1.0
+    w = {n: t.to("cuda", torch.bfloat16).contiguous() for n, t in w.items()}
+    w["b_q"] = torch.zeros(d, device="cuda")
+    w["b_q"][63] = 51.0
+    br = rv.AttnBranch(batch=1, seq_len=S, d_model=d, n_heads=2, n_kv_heads=2, weight_dtype=rv.BF16, weights=w, norm_eps=1e-12)
+    y1 = br.forward(torch.zeros(S, h, device="cuda"), dev(x2)).cpu().numpy().astype(np.float64)
+    assert br.status() == 0
+    p = np.exp(51.0 / np.sqrt(128.0) * (x2[:, 0].astype(np.float64) - 1.0))
+    want = np.cumsum(p[:, None] * x2, 0) / np.cumsum(p)[:, None]
+    share = 1.0 / np.cumsum(p)                  # of the dominating key, for the queries that see it
+    err = np.abs(y1 - want).max(1)
+    bound = 4 * 2.0 ** -8 * (1 - share) + 2.0 ** -9 + 1e-4
+    assert (err[key:] < bound[key:]).all(), (err[key:] / bound[key:]).max()
