@@ -114,7 +114,8 @@ int revffn_attn_inverse(const revffn_attn_desc* desc, const revffn_attn_weights*
  * With REVFFN_FLAG_REUSE_ACTIVATIONS the call takes the key/value side (which depends on x2 and the
  * weights only) from the workspace, where a revffn_attn_inverse call with n_iter >= 1, the same x2,
  * weights and descriptor has left it, and evaluates only the query side again: in reversible
- * back-propagation the inverse pass of a block runs right before its gradient pass.
+ * back-propagation the inverse pass of a block runs right before its gradient pass.  The two calls may
+ * differ in REVFFN_FLAG_FORCE_SIMT.
  */
 int revffn_attn_backward(const revffn_attn_desc* desc, const revffn_attn_weights* w,
                          const float* x1, const float* x2, const float* dy1,

@@ -99,7 +99,8 @@ enum { REVFFN_NORM_RMS = 0, REVFFN_NORM_NONE = 1 }; /* norm_kind                
  *   REUSE_ACTIVATIONS  backward: ws still holds everything a forward / inverse call with
  *                      SAVE_ACTIVATIONS wrote for the same y1, weights and descriptor; the
  *                      recomputation is skipped.  The backward pass overwrites some of it,
- *                      so one saved evaluation serves one backward call.               */
+ *                      so one saved evaluation serves one backward call.  The two calls
+ *                      may differ in REVFFN_FLAG_FORCE_SIMT.                           */
 #define REVFFN_FLAG_SAVE_ACTIVATIONS 2u
 #define REVFFN_FLAG_REUSE_ACTIVATIONS 4u
 /* Gate weights without renormalisation: g_e = softmax(L over all E experts)_e for the k selected

@@ -15,7 +15,7 @@
 namespace revffn {
 
 struct AttnLayout {
-  Buf status, rows_total, tile_group, group_off, cs, n12, r12, u12, raw, qh, kh, vh, lse, sc, p, oh, o, a;
+  Buf status, rows_total, tile_group, group_off, cs, cs_t, n12, r12, u12, raw, qh, kh, vh, lse, sc, p, oh, o, a;
   size_t fwd_bytes = 0;
   Buf dyb, da, dob, doh, ds, dqh, dkh, dvh, dq, dkv, du12, dn12, part, npart, lse_d;
   size_t bwd_bytes = 0;
@@ -43,6 +43,8 @@ static AttnLayout plan_attn(const revffn_attn_desc& D) {
   take(L.tile_group, (size_t)L.n_tiles * 4);
   take(L.group_off, (size_t)(L.groups + 1) * 4);
   take(L.cs, (size_t)S * (hd / 2) * 8);
+  // the fused kernels' own table, [pair, position]: a backward call may take up what a call on the other back end left
+  take(L.cs_t, D.weight_dtype == REVFFN_BF16 && hd == FA_HD ? (size_t)S * (hd / 2) * 8 : 0);
   take(L.n12, (size_t)2 * T * h * ts);
   take(L.r12, (size_t)2 * T * 4);
   take(L.u12, (size_t)2 * T * d * ts);
@@ -144,6 +146,9 @@ static int a_gemm(const ACtx<T>& c, GemmProblem p, int tag) {
 // What a pass needs before its first product: rotary table, zeroed padding rows of the head-major buffers, cleared
 // status word; on the materialising path also the tables of the grouped products.  tables: the rotary table and the
 // q / k / v padding (a gradient pass that reuses the key/value side finds them in place); d_o: its padding too.
+// The two back ends have rotary tables of their own, and only the materialising path has tables of groups.  Where both can
+// run (bf16, heads of 128) the slow one sees to both: it writes the fused kernels' table too, and makes its own
+// tables again when it takes up a key/value side, which the fused path may have left.
 template <typename T>
 static int a_setup(const ACtx<T>& c, bool tables, bool d_o) {
   const revffn_attn_desc& D = c.D;
@@ -166,12 +171,20 @@ static int a_setup(const ACtx<T>& c, bool tables, bool d_o) {
       if (n == 0 && !c.clear) return REVFFN_OK;
       ProfScope ps(TG_A_TABLES, st);
       CK(launch_k(attn_setup_kernel, (unsigned)ceil_div(std::max<int64_t>(n, 1), 256), 256, 0, st, D.seq_len, L.Sp,
-                  (double)D.rope_theta, tables ? c.template p<float2>(L.cs) : nullptr, pads, c.clear ? c.status : nullptr));
+                  (double)D.rope_theta, tables ? c.template p<float2>(L.cs_t) : nullptr, pads, c.clear ? c.status : nullptr));
       return REVFFN_OK;
     }
   }
   if (c.clear) CK(launch_k(clear_status_kernel, 1, 1, 0, st, c.status));
-  if (tables) {
+  const bool both = std::is_same<T, bf16>::value && L.hd == FA_HD;
+  if (tables && both) {
+    ProfScope ps(TG_A_TABLES, st);
+    AttnPads none;
+    none.n = 0;
+    CK(launch_k(attn_setup_kernel, (unsigned)ceil_div((int64_t)D.seq_len * 64, 256), 256, 0, st, D.seq_len, L.Sp, (double)D.rope_theta,
+                c.template p<float2>(L.cs_t), none, nullptr));
+  }
+  if (tables || both) {
     const int n_tab = L.n_tiles > L.groups + 1 ? L.n_tiles : L.groups + 1;
     { ProfScope ps(TG_A_TABLES, st);
     CK(launch_k(attn_tables_kernel, (unsigned)ceil_div(n_tab, 256), 256, 0, st, L.n_tiles, L.Sp / ROW_PAD,
@@ -228,7 +241,7 @@ static int a_project(const ACtx<T>& c, int side, const void* W, const float* bia
     if (c.fused()) {
       // bias, rotation and the head-major layout happen in the product's epilogue: no fp32 round trip
       p.epilogue = EPI_HEADS; p.C = heads;
-      p.hm_bias = bias; p.hm_cs = rotate ? c.template p<float2>(L.cs) : nullptr; p.hm_S = D.seq_len; p.hm_Sp = L.Sp;
+      p.hm_bias = bias; p.hm_cs = rotate ? c.template p<float2>(L.cs_t) : nullptr; p.hm_S = D.seq_len; p.hm_Sp = L.Sp;
       return a_gemm(c, p, TG_A_QKV);
     }
   }
@@ -469,7 +482,7 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
       { ProfScope ps(TG_A_FLASH, st);
       // the two launches also undo the rotation and write dq and dk|dv token-major in the operand type
       CKR(launch_flash_bwd(c.template p<bf16>(L.qh), c.template p<bf16>(L.kh), c.template p<bf16>(L.vh),
-                           c.template p<bf16>(L.doh), c.template p<float2>(L.lse_d), c.template p<float2>(L.cs), D.batch,
+                           c.template p<bf16>(L.doh), c.template p<float2>(L.lse_d), c.template p<float2>(L.cs_t), D.batch,
                            D.n_heads, D.n_kv_heads, D.seq_len, Sp, c.template p<bf16>(L.dq), d, c.template p<bf16>(L.dkv),
                            2 * (int64_t)dkv, dkv, c.status, st, cs.st));
       ++g_prof.launches;

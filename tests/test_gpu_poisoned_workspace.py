@@ -8,9 +8,11 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import revffn_attn_oracle as aorc
 from workloads import BlockConfig, make_streams, make_weights, to_bf16_values
+from workloads.generate import AttnConfig, make_attn_streams, make_attn_weights
 
-from helpers import dev, grad_buffers, make_block, max_block_rel_l2
+from helpers import dev, grad_buffers, make_block, max_block_rel_l2, rel_l2
 
 pytestmark = pytest.mark.gpu
 
@@ -57,3 +59,30 @@ def test_cuda_core_gradients_of_a_saved_tensor_core_evaluation(rv, d_expert):
     tensor = _step(rv, cfg, w, s, idx, 0)
     for n in clean:          # both back ends: bf16 operands, fp32 sums
         assert max_block_rel_l2(got[n].cpu().numpy()[None], tensor[n].cpu().numpy()[None]) < 2e-2, n
+
+
+@pytest.mark.parametrize("seq_len", [128, 200])
+@pytest.mark.parametrize("first_simt", [False, True], ids=["tensor_then_cuda", "cuda_then_tensor"])
+def test_attention_gradients_take_up_the_other_back_end(rv, first_simt, seq_len):
+    """inverse on one back end, backward with the key/value side it left on the other: each needs its own rotary table, and
+    the CUDA-core path the tables of its grouped products."""
+    cfg = AttnConfig("x", batch=2, seq_len=seq_len, d_model=512, n_heads=4, n_kv_heads=2, weight_dtype="bf16")
+    w, s = make_attn_weights(cfg, 2, std=0.05, bias_std=0.05), make_attn_streams(cfg, 2)
+    f32 = ("norm_gamma", "b_q", "b_k", "b_v")
+    dw = {n: torch.from_numpy(np.ascontiguousarray(v)).to("cuda", torch.float32 if n in f32 else torch.bfloat16) for n, v in w.items()}
+    br = rv.AttnBranch(batch=2, seq_len=seq_len, d_model=512, n_heads=4, n_kv_heads=2, weight_dtype=rv.BF16, weights=dw,
+                       norm_eps=cfg.norm_eps, rope_theta=cfg.rope_theta)
+    br.ws.fill_(0xFF)
+    oa = dict(S=seq_len, n_heads=4, n_kv_heads=2, eps=cfg.norm_eps, theta=cfg.rope_theta)
+    x1, x2, dy1 = dev(s["x1"]), dev(s["x2"]), dev(s["dy1"])
+    br.desc.flags = rv.FLAG_FORCE_SIMT if first_simt else 0
+    br.inverse(dev(aorc.forward(w, s["x1"], s["x2"], **oa).astype(np.float32)), x2, n_iter=1)
+    br.desc.flags = 0 if first_simt else rv.FLAG_FORCE_SIMT
+    grads = {n: torch.full(v.shape, float("nan"), dtype=torch.float32, device="cuda") for n, v in w.items()}
+    dx2 = torch.zeros_like(x2)
+    dx1 = br.backward(x1, x2, dy1, dx2, grads=grads, reuse_kv=True)
+    assert br.status() == 0
+    g1, g2, g = aorc.backward(w, s["x1"], s["x2"], s["dy1"], **oa)
+    assert rel_l2(dx1.cpu().numpy() - s["dy1"], g1 - s["dy1"]) < 2e-2 and rel_l2(dx2.cpu().numpy(), g2) < 2e-2
+    for n in w:
+        assert rel_l2(grads[n].cpu().numpy(), g[n]) < 2e-2, n
