@@ -71,6 +71,8 @@ typedef struct {
   const float* rowscale;
   const float* resid; int64_t ld_resid; float resid_sign;
   void* ab; int64_t ld_ab;         /* dswiglu: [M, 2N] bf16 a|b in, da|db out                  */
+  /* dswiglu, optional: [M, dg_ld] partial sums of <acc, H>.  Row tiles write 2 * ceil(N / 256) per row, token runs
+   * N / 32, the CUDA cores ceil(N / 64); fewer than the tcgen05 form needs: REVFFN_ERR_SHAPE */
   float* dg_part; int32_t dg_ld;
   /* grouping: 0 none, 1 rows grouped (group_off, tile_group, rows_total), 2 K grouped */
   int32_t group_mode, n_groups;
@@ -94,7 +96,9 @@ typedef struct {
   /* tests: 1 = load MN-major operands as 64 x 64 boxes of 2-D tensor maps, the form the library falls back to when a
    * leading dimension or column offset is not a multiple of 64 (0 = 3-D maps, 128 columns per load, where possible) */
   int32_t mn_boxes;
-  /* tests: columns per tile, 256, 128 or 64 (128 or 64 of each matrix of an N-concatenated pair); 0 = as planned */
+  /* tests: columns per tile, 256, 128 or 64 (128 or 64 of each matrix of an N-concatenated pair; at least 128 for a SwiGLU
+   * backward product, 256 with dg_part); 0 = as planned.  Others, and any width together with tok_chunks:
+   * REVFFN_ERR_UNSUPPORTED */
   int32_t tile_n;
 } revffn_dbg_gemm_args;
 int revffn_dbg_gemm(const revffn_dbg_gemm_args* args, int32_t* status_word_dev, void* cuda_stream);

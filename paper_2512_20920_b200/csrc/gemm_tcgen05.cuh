@@ -1783,7 +1783,8 @@ inline TcPlan tc_plan(const GemmProblem& p, int n_sms) {
 }
 
 // Partial sums of <dH, H> per row that a SwiGLU backward product writes: one per epilogue warp that holds columns of it.
-inline int tc_dg_parts(const GemmProblem& p) { return tc_plan(p, tc_state().n_sms).tr ? p.N / 32 : 2 * (int)ceil_div(p.N, 256); }
+inline int tc_dg_parts(const GemmProblem& p, bool tr) { return tr ? p.N / 32 : 2 * (int)ceil_div(p.N, 256); }
+inline int tc_dg_parts(const GemmProblem& p) { return tc_dg_parts(p, tc_plan(p, tc_state().n_sms).tr); }
 
 inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   TcState& s = tc_state();
@@ -1800,6 +1801,7 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
     q.tok_chunks = nullptr;
     return launch_gemm_tc(q, st);
   }
+  if (p.dg_part && p.dg_ld < tc_dg_parts(p, tr)) return REVFFN_ERR_SHAPE;
   P.tile_n = plan.tile_n;
   // what one load of B brings: this CTA's share of a tile's columns, at most 128 of them
   P.b_box = std::min(128, pair && p.concat != CONCAT_N ? P.tile_n / 2 : P.tile_n);

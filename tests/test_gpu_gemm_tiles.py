@@ -79,3 +79,20 @@ def test_swiglu_backward(rv, M, N, K):
     a, b = ab0[:, :N].float().requires_grad_(True), ab0[:, N:].float().requires_grad_(True)
     da, db = torch.autograd.grad((torch.nn.functional.silu(a) * b * dh).sum(), (a, b))
     _close(got, torch.cat([da, db], dim=1))
+
+
+@pytest.mark.parametrize("N,need", [(128, 2), (384, 4), (512, 4)])
+def test_too_few_columns_for_the_row_sums_are_rejected(rv, N, need):
+    """Two partial sums per row and 256 columns; nothing is launched for fewer, so the product's buffers stay as they are."""
+    import ctypes as C
+    from paper_2512_20920_b200.binding import DbgGemmArgs
+    A, B, ab, dg = _bf((8, 128), 1), _bf((128, N), 2), _bf((8, 2 * N), 3), _nan(8, need, dt=torch.float32)
+    before = ab.clone()
+    a = DbgGemmArgs(M=8, N=N, K=128, lda=128, ldb=N, b_mn_major=1, A=A.data_ptr(), B0=B.data_ptr(), epilogue=EPI["dswiglu"],
+                    ab=ab.data_ptr(), ld_ab=2 * N, dg_part=dg.data_ptr())
+    for ld, code in ((need - 1, -2), (0, -2), (need, 0)):
+        a.dg_ld = ld
+        assert rv.lib.revffn_dbg_gemm(C.byref(a), None, torch.cuda.current_stream().cuda_stream) == code
+        torch.cuda.synchronize()
+        assert torch.equal(ab, before) == (code != 0)
+    assert torch.isfinite(dg).all()
