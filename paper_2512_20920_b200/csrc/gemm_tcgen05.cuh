@@ -1789,6 +1789,7 @@ inline int tc_dg_parts(const GemmProblem& p) { return tc_dg_parts(p, tc_plan(p, 
 inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   TcState& s = tc_state();
   if (!s.ready) return REVFFN_ERR_CUDA;
+  if (p.epilogue > EPI_HEADS) return REVFFN_ERR_UNSUPPORTED;      // the update forms are chosen below
   if (p.M <= 0 || p.N <= 0) return REVFFN_OK;
   const int mma_n = 256;
   TcParams P;

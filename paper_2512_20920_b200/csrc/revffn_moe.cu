@@ -1644,19 +1644,19 @@ int revffn_prof_collect(float* ms, int32_t* count, int n_slots) {
 }
 
 // A forced tile width has to be one that the product's form has: row tiles of 256, 128 or 64 accumulator columns, half of
-// them for each matrix of a pair; a head of 128 columns, a SwiGLU backward's row sums (two per 256 columns) and its
-// epilogue do not fit narrower ones.  Token runs have no forced form.
+// them for each matrix of a pair; a SwiGLU backward's row sums (two per 256 columns) and its epilogue do not fit narrower
+// ones.  Token runs have no forced form.
 static bool dbg_tile_fits(const revffn_dbg_gemm_args& a) {
   if (a.tile_n == 0 || a.use_simt) return true;
   if ((a.tile_n != 64 && a.tile_n != 128 && a.tile_n != 256) || a.tok_chunks) return false;
   if (a.concat == CONCAT_N) return a.tile_n <= 128;
-  if (a.epilogue == EPI_DSWIGLU) return a.tile_n >= (a.dg_part ? 256 : 128);
-  return a.epilogue != EPI_HEADS || a.tile_n >= 128;
+  return a.epilogue != EPI_DSWIGLU || a.tile_n >= (a.dg_part ? 256 : 128);
 }
 
 int revffn_dbg_gemm(const revffn_dbg_gemm_args* a, int32_t* status_word_dev, void* cuda_stream) {
   if (!a) return REVFFN_ERR_NULL;
-  if (!dbg_tile_fits(*a)) return REVFFN_ERR_UNSUPPORTED;
+  // heads need a head layout and the update forms their weights: neither is part of these arguments
+  if (a->epilogue < EPI_STORE || a->epilogue > EPI_WGRAD || !dbg_tile_fits(*a)) return REVFFN_ERR_UNSUPPORTED;
   int r = check_device();
   if (r != REVFFN_OK) return r;
   GemmProblem p = blank_problem();

@@ -91,11 +91,19 @@ def test_null_and_misaligned_pointers_are_rejected_before_any_launch(rv):
 
 @pytest.mark.parametrize("kw", [dict(tile_n=32), dict(tile_n=512), dict(tile_n=-64), dict(tile_n=256, concat=1),
                                 dict(tile_n=128, tok_chunks=0x1000), dict(tile_n=64, epilogue=4),
-                                dict(tile_n=128, epilogue=4, dg_part=0x1000), dict(tile_n=64, epilogue=6)])
+                                dict(tile_n=128, epilogue=4, dg_part=0x1000)])
 def test_tile_widths_that_a_product_cannot_have_are_rejected(rv, kw):
     from paper_2512_20920_b200.binding import DbgGemmArgs
     a = DbgGemmArgs(M=256, N=256, K=256, lda=256, ldb=256, ldc=256, A=0x1000, B0=0x1000, B1=0x1000, C=0x1000, ab=0x1000, ld_ab=512,
                     dg_ld=64, **kw)
+    assert rv.lib.revffn_dbg_gemm(C.byref(a), None, None) == rv.ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("epilogue", [-1, 6, 7, 8, 9, 10])
+@pytest.mark.parametrize("simt", [0, 1])
+def test_epilogues_that_need_more_than_a_debug_product_has_are_rejected(rv, epilogue, simt):
+    from paper_2512_20920_b200.binding import DbgGemmArgs
+    a = DbgGemmArgs(M=256, N=256, K=256, lda=256, ldb=256, ldc=256, A=0x1000, B0=0x1000, C=0x1000, epilogue=epilogue, use_simt=simt)
     assert rv.lib.revffn_dbg_gemm(C.byref(a), None, None) == rv.ERR_UNSUPPORTED
 
 
