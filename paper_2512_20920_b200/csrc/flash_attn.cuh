@@ -274,7 +274,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
     const float cl = P.scale_log2e;
     bool ok = true;
     for (int j = 0; j < n_x; ++j) {
-      ok = __all_sync(0xffffffffu, mbar_wait(bar(B_SFULL + x), (uint32_t)j & 1u, abort_flag, P.status));
+      ok = mbar_wait_warp(bar(B_SFULL + x), (uint32_t)j & 1u, abort_flag, P.status);
       if (!ok) break;
       tc_fence_after();
       uint32_t pw[32], r2[32], r3[32];
@@ -345,7 +345,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(B_PFULL + x));
     }
-    if (n_x > 0 && ok) ok = __all_sync(0xffffffffu, mbar_wait(bar(B_OFULL + x), 0u, abort_flag, P.status));
+    if (n_x > 0 && ok) ok = mbar_wait_warp(bar(B_OFULL + x), 0u, abort_flag, P.status);
     if (n_x > 0 && ok) {
       tc_fence_after();
       // out through this tile's Q area (its products are complete), 64- and 128-byte row pieces per instruction
@@ -673,9 +673,9 @@ flash_bwd_dkv_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap
     for (int s = 0; s < n_steps; ++s) {
       const int b = s & 1;
       const uint32_t ph = (uint32_t)(s >> 1) & 1u;
-      if (!mbar_wait(bar(B_SDFULL + b), ph, abort_flag, P.status)) { ok = false; break; }
-      // this thread reads the stage's row statistics itself, so it observes the stage's barrier itself
-      if (!mbar_wait(bar(B_YFULL + s % NS), (uint32_t)(s / NS) & 1u, abort_flag, P.status)) { ok = false; break; }
+      if (!mbar_wait_warp(bar(B_SDFULL + b), ph, abort_flag, P.status)) { ok = false; break; }
+      // this thread reads the stage's row statistics itself, so it observes the stage's barrier itself (every lane does)
+      if (!mbar_wait_warp(bar(B_YFULL + s % NS), (uint32_t)(s / NS) & 1u, abort_flag, P.status)) { ok = false; break; }
       tc_fence_after();
       uint32_t rs[32], rd[32];
       tmem_ld32(lane_addr + (uint32_t)(b * 128 + 32 * hh), rs);
@@ -694,7 +694,7 @@ flash_bwd_dkv_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap
       if (mask) fb_tile<DKV, true>(rs, rd, ld_cols, own_ld, cl, scale, col0, own_pos, P.S, pp, pd);
       else fb_tile<DKV, false>(rs, rd, ld_cols, own_ld, cl, scale, col0, own_pos, P.S, pp, pd);
       // the operand tiles have one buffer: the previous step's accumulating products must have read them
-      if (!mbar_wait(bar(B_PDEMPTY), ((uint32_t)s & 1u) ^ 1u, abort_flag, P.status)) { ok = false; break; }
+      if (!mbar_wait_warp(bar(B_PDEMPTY), ((uint32_t)s & 1u) ^ 1u, abort_flag, P.status)) { ok = false; break; }
       uint8_t* prow = gen_base + FB_P_OFF + row * 128;
       uint8_t* drow = gen_base + FB_DS_OFF + row * 128;
 #pragma unroll
@@ -707,7 +707,7 @@ flash_bwd_dkv_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(B_PDFULL));
     }
-    if (ok && !mbar_wait(bar(B_ACCFULL), 0u, abort_flag, P.status)) ok = false;
+    if (ok) ok = mbar_wait_warp(bar(B_ACCFULL), 0u, abort_flag, P.status);
     if (ok) {
       tc_fence_after();
       // This thread takes columns [32 hh, +32) and their rotation partners [64 + 32 hh, +32) of its row.  The
@@ -916,7 +916,7 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
     bool ok = true;
     const bool edge = blk * FA_BLK + FA_BLK - 1 >= P.S;
     for (int s = 0; s < n_steps; ++s) {
-      if (!mbar_wait(bar(B_SDFULL), (uint32_t)s & 1u, abort_flag, P.status)) { ok = false; break; }
+      if (!mbar_wait_warp(bar(B_SDFULL), (uint32_t)s & 1u, abort_flag, P.status)) { ok = false; break; }
       __syncwarp();
       tc_fence_after();
       const bool mask = s == blk || edge;
@@ -939,7 +939,7 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
       if (mask) fb_tile<false, true>(rs, rd, nullptr, own_ld, cl, scale, col0 + 32, own_pos, P.S, pp, pb);
       else fb_tile<false, false>(rs, rd, nullptr, own_ld, cl, scale, col0 + 32, own_pos, P.S, pp, pb);
       // the operand tile has one buffer: the previous step's accumulating product must have read it
-      if (!mbar_wait(bar(B_PDEMPTY), ((uint32_t)s & 1u) ^ 1u, abort_flag, P.status)) { ok = false; break; }
+      if (!mbar_wait_warp(bar(B_PDEMPTY), ((uint32_t)s & 1u) ^ 1u, abort_flag, P.status)) { ok = false; break; }
       uint8_t* drow = gen_base + FQ_DS_OFF + hh * FA_TILE + row * 128;      // this thread's 64 keys are tile hh
 #pragma unroll
       for (int g = 0; g < 4; ++g) {
@@ -950,7 +950,7 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(B_PDFULL));
     }
-    if (ok && !mbar_wait(bar(B_ACCFULL), 0u, abort_flag, P.status)) ok = false;
+    if (ok) ok = mbar_wait_warp(bar(B_ACCFULL), 0u, abort_flag, P.status);
     if (ok) {
       tc_fence_after();
       // columns [32 hh, +32) and their rotation partners [64 + 32 hh, +32); every lane executes the warp-wide loads

@@ -141,7 +141,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
-// The same for a whole warp that stays converged (the result is the same in every lane).
+// The same for a whole warp that stays converged: the result is the same in every lane.  Each role that goes on with
+// warp-wide instructions (tensor-memory loads, shuffles, elect) waits like this: an abandoned wait ends each lane's spin at a
+// point of its own, and a lane that saw the barrier complete just then would go on without the others.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
                                                long long limit = TC_WAIT_CYCLES) {
   if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
@@ -1005,7 +1007,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           else upd_first<EPI == EPI_WADAM, false>(out, stg, lane, p.ldc);
         }
       }
-      if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
+      if (!mbar_wait_warp(tfull_bar(acc), acc_phase, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * MMA_N);
       // accumulator may be overwritten by the MMA warp

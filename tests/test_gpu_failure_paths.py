@@ -79,6 +79,46 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_survives(rv):
     assert rel_l2(out.float().cpu().numpy(), (A.float() @ B.float().T).cpu().numpy()) <= 1e-2
 
 
+@pytest.mark.parametrize("epilogue,kw", [(0, {}), (0, dict(out_f32=1)), (1, dict(concat=1)), (2, {}), (3, {}), (4, dict(b_mn_major=1)),
+                                         (5, dict(a_mn_major=1, b_mn_major=1))])
+def test_every_epilogue_leaves_a_starved_product_as_whole_warps(rv, epilogue, kw):
+    """The epilogue's lanes leave an abandoned wait at different times, and warp-wide instructions follow: bounds that run out
+    while the lanes spin, for each form of the epilogue, then the product itself, which finds the GPU as it should be."""
+    from paper_2512_20920_b200.binding import DbgGemmArgs
+    n = 256
+    g = torch.Generator("cuda").manual_seed(6)
+    A, B0, B1 = ((torch.randn(n, n, device="cuda", generator=g) * 0.2).to(torch.bfloat16) for _ in range(3))
+    ab = torch.randn(n, 2 * n, device="cuda", generator=g).to(torch.bfloat16)
+    ab0 = ab.clone()
+    f32 = epilogue in (3, 5) or "out_f32" in kw
+    out = torch.zeros(n, n, device="cuda", dtype=torch.float32 if f32 else torch.bfloat16)
+    scale, resid = torch.rand(n, device="cuda", generator=g), torch.randn(n, n, device="cuda", generator=g)
+    status = torch.zeros(64, dtype=torch.int32, device="cuda")
+    a = DbgGemmArgs(M=n, N=n, K=n, lda=n, ldb=n, ldc=n, A=A.data_ptr(), B0=B0.data_ptr(), B1=B1.data_ptr(), C=out.data_ptr(),
+                    rowscale=scale.data_ptr() if epilogue == 2 else None, resid=resid.data_ptr(), ld_resid=n, resid_sign=1.0,
+                    ab=ab.data_ptr(), ld_ab=2 * n, epilogue=epilogue, no_pair=1, starve_operands=1, **kw)
+    for wait in range(20_000, 60_000, 1_700):
+        status.zero_()
+        a.wait_cycles = wait
+        assert rv.lib.revffn_dbg_gemm(C.byref(a), status.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+        torch.cuda.synchronize()
+        assert int(status[0]) == rv.ERR_DEVICE_WAIT
+    assert float(out.float().abs().max()) == 0.0 and torch.equal(ab, ab0)
+    a.starve_operands, a.wait_cycles = 0, 0
+    status.zero_()
+    assert rv.lib.revffn_dbg_gemm(C.byref(a), status.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+    assert int(status[0]) == 0
+    x, w0, w1 = A.float(), B0.float(), B1.float()
+    acc = x.T @ w0 if "a_mn_major" in kw else x @ w0 if "b_mn_major" in kw else x @ w0.T
+    if epilogue == 4:
+        p, q = ab0[:, :n].float().requires_grad_(True), ab0[:, n:].float().requires_grad_(True)
+        got, want = ab, torch.cat(torch.autograd.grad((torch.nn.functional.silu(p) * q * acc).sum(), (p, q)), 1)
+    else:
+        got = out
+        want = {1: torch.nn.functional.silu(acc) * (x @ w1.T), 2: acc * scale[:, None], 3: resid + acc}.get(epilogue, acc)
+    assert rel_l2(got.float().cpu().numpy(), want.cpu().numpy()) <= 1e-2
+
+
 def test_expert_indices_out_of_range_are_reported_not_used(rv):
     cfg = _cfg()
     w, s = _weights(cfg, 1), make_streams(cfg, 1)
