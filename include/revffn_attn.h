@@ -49,8 +49,8 @@ extern "C" {
  *   weight_dtype REVFFN_BF16: h and d multiples of 128, head_dim 128 (TMA / tcgen05 tiles).
  * flags: REVFFN_FLAG_FORCE_SIMT; REVFFN_FLAG_REUSE_ACTIVATIONS on a backward call (below);
  *   REVFFN_FLAG_SINGLE_STREAM: as in revffn_moe.h, calls on the tcgen05 back end otherwise run the key/value side beside
- *   the query side and the weight gradients beside the input gradients on the library's second stream, with the same
- *   results; the caller's stream ends after everything of the call.
+ *   the query side and the weight gradients beside the input gradients on a second stream of the library's, with the
+ *   same results; the caller's stream ends after everything of the call.
  */
 typedef struct {
   int32_t batch, seq_len;       /* T = batch * seq_len tokens                              */

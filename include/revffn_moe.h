@@ -33,9 +33,9 @@
  *   - Work is enqueued on the caller's CUDA stream (cudaStream_t passed as
  *     void*), and the call is asynchronous on it: what the caller queues on that
  *     stream afterwards follows everything of the call.  Inside a call on the
- *     tcgen05 back end, launches that nothing later in the pass depends on run on a second stream that the library creates per device
- *     on its first call (with a ring of events that order it against the
- *     caller's stream); REVFFN_FLAG_SINGLE_STREAM keeps every launch on the
+ *     tcgen05 back end, launches that nothing later in the pass depends on run on
+ *     a second stream of the library's, ordered against the caller's by events;
+ *     REVFFN_FLAG_SINGLE_STREAM, which says more, keeps every launch on the
  *     caller's stream.  The results are the same bits either way.  The pipelined
  *     host step (REVFFN_FLAG_STEP_PIPELINED) owns one more stream, for uploads.
  *     Calls that share a workspace must be ordered on one stream, and calls on
@@ -150,10 +150,13 @@ enum { REVFFN_NORM_RMS = 0, REVFFN_NORM_NONE = 1 }; /* norm_kind                
 /* revffn_moe_step_host only: the pipelined form described there (two staging sets used in turn, results
  * complete when the copy stream completes).  Other entry points ignore it. */
 #define REVFFN_FLAG_STEP_PIPELINED 512u
-/* Keep every launch of the call on cuda_stream.  Without it, calls on the tcgen05 back end put launches that nothing later in the pass depends on (the shared expert beside the routed experts, the weight
- * gradients beside the input gradients) on a second stream that the library creates per device on first use,
- * ordered against cuda_stream by events; cuda_stream still ends after everything of the call, and the results
- * are the same bits either way. */
+/* Keep every launch of the call on cuda_stream.  Without it, calls on the tcgen05 back end put launches that nothing
+ * later in the pass depends on (the shared expert beside the routed experts, the weight gradients beside the input
+ * gradients) on a second stream, ordered against cuda_stream by events; cuda_stream still ends after everything of the call,
+ * and the results are the same bits either way.  The library makes its second streams on first use: one for each stream
+ * of the caller's, up to eight on a device (beyond that they are shared, which only costs time), and up to four more for
+ * captures.  A call under stream capture adds one of those to the capture until it ends, and runs on cuda_stream
+ * alone when all four are taken; calls on streams outside the capture are not affected. */
 #define REVFFN_FLAG_SINGLE_STREAM 1024u
 
 /*

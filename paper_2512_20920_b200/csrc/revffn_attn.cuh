@@ -122,13 +122,7 @@ struct ACtx {
   bool tc;
   bool fused() const { return std::is_same<T, bf16>::value && tc && L.hd == FA_HD; }      // attention core as tcgen05 kernels
   // what is queued on `to` from now on follows everything queued on `from` so far (no-op without the second stream)
-  int order(cudaStream_t from, cudaStream_t to) const {
-    if (!ov || from == to) return REVFFN_OK;
-    cudaError_t e;
-    cudaEvent_t x = ov->mark(from, &e);
-    if (e != cudaSuccess || cudaStreamWaitEvent(to, x, 0) != cudaSuccess) return REVFFN_ERR_CUDA;
-    return REVFFN_OK;
-  }
+  int order(cudaStream_t from, cudaStream_t to) const { return ov ? ov->order(from, to) : REVFFN_OK; }
   ACtx on_side() const { ACtx c = *this; if (ov) c.st = ov->side; return c; }
   template <typename U> U* p(const Buf& b) const { return reinterpret_cast<U*>(ws + b.off); }
 };
@@ -613,10 +607,9 @@ static int a_dispatch(APass pass, const revffn_attn_desc& D, const revffn_attn_w
   c.status = status ? status : c.template p<int>(L.status);
   c.clear = status == nullptr;
   if (c.tc) CKR(tc_prepare());
-  if (c.fused() && !g_prof.on && !(D.flags & REVFFN_FLAG_SINGLE_STREAM)) {
-    c.ov = overlap_state();
-    if (!c.ov) return REVFFN_ERR_CUDA;
-  }
+  SideStream side;
+  if (c.fused() && !g_prof.on && !(D.flags & REVFFN_FLAG_SINGLE_STREAM)) CKR(side.take(st));
+  c.ov = side.lane;
   if (L.T == 0) {
     if (c.clear) CK(launch_k(clear_status_kernel, 1, 1, 0, st, c.status));
     return REVFFN_OK;

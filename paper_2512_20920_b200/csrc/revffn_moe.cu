@@ -2,7 +2,6 @@
 // See include/revffn_moe.h for the contract of every entry point.
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -317,39 +316,100 @@ __global__ void clear_status_kernel(int* __restrict__ status) {
 // ---------------------------------------------------------------------------
 // Launch context
 // ---------------------------------------------------------------------------
-// A second stream per device for launches that do not depend on what the caller's stream is doing at that point
+// A second stream for launches that do not depend on what the caller's stream is doing at that point
 // (the shared expert beside the routed experts, the weight gradients beside the chain of input gradients).  The
 // matrix products are persistent kernels of one CTA per SM and equal tiles, so most of them end with a partly
 // empty last round of tiles; a kernel from the other stream starts on the SMs that fall idle there.  Ordering is by
 // events from a small ring (a wait refers to the record that preceded it, so an event can be recorded again while
-// an older wait is still pending).  Created on first use.
+// an older wait is still pending).
 struct Overlap {
   cudaStream_t side = nullptr;
-  cudaEvent_t ev[64];
-  std::atomic<unsigned> next{0};
+  cudaEvent_t ev[16];
+  unsigned next = 0;
   bool made = false;
-  cudaEvent_t mark(cudaStream_t s, cudaError_t* e) {       // an event that follows everything queued on s so far
-    cudaEvent_t x = ev[next.fetch_add(1) & 63u];
-    *e = cudaEventRecord(x, s);
-    return x;
+  std::mutex mu;
+  // held under the pool's lock
+  cudaStream_t user = nullptr;      // caller's stream that had it last
+  uint64_t used = 0;                // when
+  int busy = 0;                     // calls that are issuing on it
+  // what is queued on `to` from now on follows everything queued on `from` so far
+  int order(cudaStream_t from, cudaStream_t to) {
+    if (from == to) return REVFFN_OK;
+    std::lock_guard<std::mutex> lock(mu);      // nobody records the event again before the wait has taken it up
+    cudaEvent_t x = ev[next++ & 15u];
+    if (cudaEventRecord(x, from) != cudaSuccess || cudaStreamWaitEvent(to, x, 0) != cudaSuccess) return REVFFN_ERR_CUDA;
+    return REVFFN_OK;
+  }
+  int make() {
+    if (made) return REVFFN_OK;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;      // the first use may lie inside a capture
+    CK(cudaThreadExchangeStreamCaptureMode(&mode));
+    bool ok = cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking) == cudaSuccess;
+    for (auto& x : ev) ok = ok && cudaEventCreateWithFlags(&x, cudaEventDisableTiming) == cudaSuccess;
+    CK(cudaThreadExchangeStreamCaptureMode(&mode));
+    made = ok;
+    return ok ? REVFFN_OK : REVFFN_ERR_CUDA;
   }
 };
 
-static Overlap* overlap_state() {
-  static Overlap state[64];
-  static std::mutex mu;
-  std::lock_guard<std::mutex> lock(mu);
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-  Overlap& o = state[dev];
-  if (!o.made) {
-    for (auto& x : o.ev)
-      if (cudaEventCreateWithFlags(&x, cudaEventDisableTiming) != cudaSuccess) return nullptr;
-    if (cudaStreamCreateWithFlags(&o.side, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
-    o.made = true;
+// The second streams of a device, made when first wanted.  Each stream of a caller keeps the one that it had, so calls on
+// different streams do not queue behind each other until there are more than SIDE_STREAMS of them (then the one that
+// was used longest ago is shared; it only costs time).  A call under stream capture takes one of SIDE_CAPTURE others,
+// which belongs to that capture until it ends: nothing outside a capture ever waits on a stream inside it.  When
+// none is left, the call runs on the caller's stream alone, with the same results.
+constexpr int SIDE_STREAMS = 8, SIDE_CAPTURE = 4;
+class SideStream {
+ public:
+  Overlap* lane = nullptr;
+  int take(cudaStream_t st) {
+    static Pool pools[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return REVFFN_ERR_CUDA;
+    pool_ = &pools[dev];
+    unsigned long long id = 0, other = 0;
+    const cudaStreamCaptureStatus cap = capture(st, &id);
+    if (cap == cudaStreamCaptureStatusInvalidated) return REVFFN_OK;
+    std::lock_guard<std::mutex> lock(pool_->mu);
+    Overlap* pick = nullptr;
+    if (cap == cudaStreamCaptureStatusActive) {
+      for (Overlap& o : pool_->capture) {
+        if (!o.made) { if (!pick) pick = &o; continue; }
+        const cudaStreamCaptureStatus c = capture(o.side, &other);
+        if (c == cudaStreamCaptureStatusActive && other == id) { pick = &o; break; }
+        if (c == cudaStreamCaptureStatusNone && o.busy == 0 && !pick) pick = &o;
+      }
+      if (!pick) return REVFFN_OK;
+    } else {
+      pick = &pool_->plain[0];
+      for (Overlap& o : pool_->plain) {
+        if (o.made && o.user == st) { pick = &o; break; }
+        if (o.used < pick->used) pick = &o;
+      }
+      pick->user = st;
+      pick->used = ++pool_->clock;
+    }
+    if (pick->make() != REVFFN_OK) return REVFFN_ERR_CUDA;
+    ++pick->busy;
+    lane = pick;
+    return REVFFN_OK;
   }
-  return &o;
-}
+  ~SideStream() {
+    if (!lane) return;
+    std::lock_guard<std::mutex> lock(pool_->mu);
+    --lane->busy;
+  }
+
+ private:
+  struct Pool { std::mutex mu; uint64_t clock = 0; Overlap plain[SIDE_STREAMS], capture[SIDE_CAPTURE]; };
+  Pool* pool_ = nullptr;
+  // (the default stream cannot be asked while another blocking stream is captured: it is not captured itself then)
+  static cudaStreamCaptureStatus capture(cudaStream_t s, unsigned long long* id) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamGetCaptureInfo(s, &c, id) == cudaSuccess) return c;
+    cudaGetLastError();
+    return cudaStreamCaptureStatusNone;
+  }
+};
 
 template <typename T>
 struct Ctx {
@@ -361,13 +421,7 @@ struct Ctx {
   int* status;             // device status word: the workspace's own, or that of the block call this one is part of
   Overlap* ov = nullptr;   // non-null: the second stream is in use for this call
   // what is queued on `to` from now on follows everything queued on `from` so far (no-op without the second stream)
-  int order(cudaStream_t from, cudaStream_t to) const {
-    if (!ov || from == to) return REVFFN_OK;
-    cudaError_t e;
-    cudaEvent_t x = ov->mark(from, &e);
-    if (e != cudaSuccess || cudaStreamWaitEvent(to, x, 0) != cudaSuccess) return REVFFN_ERR_CUDA;
-    return REVFFN_OK;
-  }
+  int order(cudaStream_t from, cudaStream_t to) const { return ov ? ov->order(from, to) : REVFFN_OK; }
   cudaStream_t side() const { return ov ? ov->side : st; }
   bool tc;   // tcgen05 back end for the matrix products
   template <typename U> U* p(const Buf& b) const { return reinterpret_cast<U*>(ws + b.off); }
@@ -1013,10 +1067,9 @@ static int dispatch(Pass pass, const revffn_moe_desc& D, const revffn_moe_weight
   c.tc = std::is_same<T, bf16>::value && !(D.flags & REVFFN_FLAG_FORCE_SIMT);
   // second stream: every call on the tcgen05 back end (at 512 tokens, where the launches are short, the step still
   // gains 13 %), never while the per-launch profiler is on (its events bracket launches on one stream)
-  if (c.tc && !g_prof.on && !(D.flags & REVFFN_FLAG_SINGLE_STREAM)) {
-    c.ov = overlap_state();
-    if (!c.ov) return REVFFN_ERR_CUDA;
-  }
+  SideStream side;
+  if (c.tc && !g_prof.on && !(D.flags & REVFFN_FLAG_SINGLE_STREAM)) CKR(side.take(st));
+  c.ov = side.lane;
   if (c.tc) CKR(tc_prepare());
   c.status = status ? status : c.template p<int>(L.status);
   if (!status && !(D.flags & REVFFN_FLAG_KEEP_STATUS)) CK(launch_k(clear_status_kernel, 1, 1, 0, st, c.status));
