@@ -1902,11 +1902,14 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
     }
     if (p.split_m > 0 && (p.epilogue != EPI_WGRAD || p.M != 2 * p.split_m || p.split_m % TC_BM != 0)) return REVFFN_ERR_SHAPE;
     if (p.epilogue == EPI_WGRAD && p.upd_w) {
-      // fused update: the weights (and master copies) are read and rewritten 8 / 16 bytes at a time
+      // fused update: master copies and moments are read and rewritten 16 bytes at a time, and so are bf16 weights without a
+      // master copy (the row-wise form asks for them by cp.async)
+      const bool bare = !p.upd_m || (p.split_m > 0 && !p.upd_m2);
       if ((reinterpret_cast<uintptr_t>(p.upd_w) & 15u) || (reinterpret_cast<uintptr_t>(p.upd_w2) & 15u) ||
           (reinterpret_cast<uintptr_t>(p.upd_m) & 15u) || (reinterpret_cast<uintptr_t>(p.upd_m2) & 15u) ||
           (reinterpret_cast<uintptr_t>(p.upd_mom) & 15u) || (reinterpret_cast<uintptr_t>(p.upd_mom2) & 15u) ||
-          (reinterpret_cast<uintptr_t>(p.upd_var) & 15u) || (reinterpret_cast<uintptr_t>(p.upd_var2) & 15u) || p.ldc % 4 != 0)
+          (reinterpret_cast<uintptr_t>(p.upd_var) & 15u) || (reinterpret_cast<uintptr_t>(p.upd_var2) & 15u) ||
+          p.ldc % (bare ? 8 : 4) != 0)
         return REVFFN_ERR_ALIGN;
       if (p.split_m > 0 && !p.upd_w2) return REVFFN_ERR_NULL;
       if (p.upd.kind == 1 && (!p.upd_mom || !p.upd_var || (p.split_m > 0 && (!p.upd_mom2 || !p.upd_var2)))) return REVFFN_ERR_NULL;
