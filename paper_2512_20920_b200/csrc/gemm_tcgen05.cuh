@@ -240,17 +240,10 @@ __device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                ::"r"(bar), "h"((uint16_t)3) : "memory");
 }
-__device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
-}
 
 // One product with the descriptors given as (low, high) words: the high words never change inside a kernel, and
-// the low words move by small additions, so the issuing thread carries 32-bit values only.
-// The same for e4m3 operands (kind::f8f6f4: 32 one-byte elements of K per instruction, the same 32 bytes).
+// the low words move by small additions, so the issuing thread carries 32-bit values only.  Here for e4m3 operands
+// (kind::f8f6f4: 32 one-byte elements of K per instruction, the same 32 bytes as 16 bf16 ones).
 template <bool PAIR>
 __device__ __forceinline__ void tc_mma_lohi_f8(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
                                                uint32_t idesc, uint32_t acc) {
@@ -355,11 +348,6 @@ __device__ __forceinline__ void store32_bf16(bf16* dst, const float* f) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) o[i] = pack8(f + 8 * i);
 }
-__device__ __forceinline__ void load32_bf16(const bf16* src, float* f) {
-  const uint4* s = reinterpret_cast<const uint4*>(src);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) unpack8(s[i], f + 8 * i);
-}
 
 // Output staging.  A warp stages a 32-row x 32-column bf16 block, one row per lane, in the layout
 // the store's tensor map expects: rows of 64 bytes under the 64-byte swizzle.  `buf` is aligned to
@@ -387,13 +375,6 @@ __device__ __forceinline__ void blk_stage_to_global(const uint8_t* buf, int lane
 
 // Logistic function from one ex2.approx and one rcp.approx (relative error about 2^-21, far inside what the
 // bf16 results around it can show).
-__device__ __forceinline__ float sigmoid_approx(float x) {
-  float e, r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x * -1.4426950408889634f));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + e));
-  return r;
-}
-
 __device__ __forceinline__ float2 sigmoid_approx2(float2 x) {
   const float2 t = __fmul2_rn(x, make_float2(-1.4426950408889634f, -1.4426950408889634f));
   float e0, e1, r0, r1;
