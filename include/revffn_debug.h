@@ -79,9 +79,12 @@ typedef struct {
   const int32_t *group_off, *tile_group, *rows_total;
   int64_t b_group_stride, c_group_stride;
   int32_t a_col0, b_col0;
-  /* rows grouped: optional table of (expert, first row, rows, 0) runs of real rows, rows a multiple of
+  /* rows grouped: optional table of (expert, first row, rows, padding) runs of real rows, rows a multiple of
    * 32 and at most 256, int32 x 4 each, 16-byte aligned; their number at rows_total[1].  With it the
-   * tcgen05 back end works store / gate-scale products with the rows on the MMA N side. */
+   * tcgen05 back end works bf16 store, gate-scale, SwiGLU and SwiGLU backward products with the rows on the MMA N
+   * side where they have enough tiles.  padding: rows after the run that a SwiGLU product writes as zeros, to the
+   * next multiple of 64 in an expert's last run and 0 in the others (rows + padding at most 256); a K-grouped
+   * product over the rows reads up to there. */
   const void* tok_chunks;
   int32_t no_pair;                 /* tcgen05 back end: one CTA per tile even where CTA pairs apply */
   /* Failure-path test (tcgen05 back end, one CTA per tile only).  wait_cycles > 0 replaces the bound on

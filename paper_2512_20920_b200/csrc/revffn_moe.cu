@@ -1275,7 +1275,7 @@ int revffn_moe_ws_lookup(const revffn_moe_desc* desc, const char* name, size_t* 
   struct { const char* n; const Buf* b; } tab[] = {
       {"status", &L.status}, {"rows_total", &L.rows_total}, {"w_rc", &L.w_rc}, {"n", &L.n}, {"r", &L.r},
       {"idx", &L.idx}, {"gates", &L.gates}, {"sgate", &L.sgate}, {"expert_cnt", &L.expert_cnt},
-      {"expert_off", &L.expert_off}, {"tile_group", &L.tile_group}, {"tok_row", &L.tok_row},
+      {"expert_off", &L.expert_off}, {"tile_group", &L.tile_group}, {"tok_chunks", &L.tok_chunks}, {"tok_row", &L.tok_row},
       {"row_tok", &L.row_tok}, {"row_gate", &L.row_gate}, {"u", &L.u}, {"up", &L.up}, {"hmid", &L.hmid},
       {"o", &L.o}, {"hs", &L.hs}, {"s", &L.s}, {"z", &L.z}, {"ab", &L.ab}, {"abs", &L.abs}, {"gb", &L.gb},
       {"dz", &L.dz}, {"ds", &L.ds}, {"dl", &L.dl}, {"dop", &L.dop}, {"dg_part", &L.dg_part},

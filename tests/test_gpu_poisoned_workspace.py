@@ -61,6 +61,34 @@ def test_cuda_core_gradients_of_a_saved_tensor_core_evaluation(rv, d_expert):
         assert max_block_rel_l2(got[n].cpu().numpy()[None], tensor[n].cpu().numpy()[None]) < 2e-2, n
 
 
+@pytest.mark.parametrize("d_expert", [128, 4096])
+def test_a_step_reads_nothing_that_it_has_not_written(rv, d_expert):
+    cfg, w, s, idx = _problem(d_expert)
+    clean, got = (_step(rv, cfg, w, s, idx, fill) for fill in (0, 0xFF))
+    for n in clean:
+        assert torch.equal(clean[n], got[n]), n
+    blk, y1, x2 = make_block(cfg, w), dev(s["y1"]), dev(s["x2"])
+    y2 = []
+    for fill in (0, 0xFF):
+        blk.ws.fill_(fill)
+        y2.append(blk.forward(y1, x2))
+        assert blk.status() == 0
+    assert torch.equal(*y2)
+
+
+@pytest.mark.parametrize("d_expert", [128, 2048])
+def test_e4m3_experts_read_nothing_that_the_call_has_not_written(rv, d_expert):
+    cfg, w, s, idx = _problem(d_expert)
+    blk = make_block(cfg, w, flags=rv.FLAG_FP8_EXPERTS)
+    blk.quantize_experts()
+    y1, y2, sets, x2 = dev(s["y1"]), dev(s["x2"]), dev(idx), []
+    for fill in (0, 0xFF):
+        blk.ws.fill_(fill)
+        x2.append(blk.inverse(y1, y2, topk_idx_in=sets))
+        assert blk.status() == 0
+    assert torch.equal(*x2) and torch.isfinite(x2[0]).all()
+
+
 @pytest.mark.parametrize("seq_len", [128, 200])
 @pytest.mark.parametrize("first_simt", [False, True], ids=["tensor_then_cuda", "cuda_then_tensor"])
 def test_attention_gradients_take_up_the_other_back_end(rv, first_simt, seq_len):

@@ -67,6 +67,17 @@ def test_routing_tables(rv, tokens, d, E, k):
     row_tok = np.full(off[E], -1)
     row_tok[tok_row] = np.arange(flat.size) // k
     assert (blk.buffer("row_tok", torch.int32)[: off[E]].cpu().numpy() == row_tok).all()
+    row_gate = np.zeros(off[E], np.float32)
+    row_gate[tok_row] = gates.reshape(-1)
+    assert (blk.buffer("row_gate", torch.float32)[: off[E]].cpu().numpy() == row_gate).all()
+    # token runs: an expert's rows to a multiple of 32, at most 256 a run; the last run names the rows from there to the
+    # next multiple of 64, which products write as zeros
+    runs = []
+    for e in range(E):
+        n = (cnt[e] + 31) // 32 * 32
+        runs += [[e, off[e] + r, min(256, n - r), (cnt[e] + 63) // 64 * 64 - n if r + 256 >= n else 0] for r in range(0, n, 256)]
+    got = blk.buffer("tok_chunks", torch.int32)[: 4 * len(runs)].view(-1, 4).cpu().numpy()
+    assert (got == np.array(runs)).all()
 
 
 def test_logits_do_not_depend_on_the_batch(rv):
