@@ -352,7 +352,7 @@ inline cudaError_t launch_du_reduce(const T* dUp, const int32_t* tok_row, const 
 // gradient in separate passes, 33 us together.
 struct NormBwdRows { const float* dn; const float* y; const float* r; const float* base; float* out; };
 constexpr int NORM_BWD_MAX_H = 1024;
-constexpr int NORM_BWD_MAX_BLOCKS = 444;
+constexpr int NORM_BWD_MAX_BLOCKS = 3 * 148;      // three blocks per SM of a B200; a constant because the scratch is planned without a device
 inline int norm_bwd_blocks(int64_t rows) { return (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(rows, 8), NORM_BWD_MAX_BLOCKS)); }
 
 __global__ void __launch_bounds__(256)
