@@ -71,8 +71,8 @@ __device__ __forceinline__ void set_status(int* status, int code) {
 //                kernel calls it, in every thread, before its first access to global memory and before any early return:
 //                that also makes "the kernel before me has completed" imply "so have all before that one".
 //   pdl_trigger  lets the next launch on the stream be set up (once every block has called it or has exited).
-// What it saves is the 1.5-4 us between two dependent launches; a small stack of blocks is 530 of them (four d = 512 blocks, 384 tokens:
-// 3788 -> 2908 us a training step; attention branch, 7 x 613 positions: 1337 -> 1252).
+// What it saves is the 1.5-4 us between two dependent launches (a training step of four d = 512 blocks, 384 tokens, was some
+// 530 launches then, 94 a block now: 3788 -> 2908 us; attention branch, 7 x 613 positions: 1337 -> 1252).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // Short kernels release the next launch at once; the matrix products and attention kernels do it when a block's last

@@ -1704,8 +1704,8 @@ inline int tc_launch(const TcParams& P, const CUtensorMap& ma, const CUtensorMap
 // How a product is cut: CTA pairs or single CTAs, columns per tile, and whether it runs transposed.
 struct TcPlan { bool tr, pair; int tile_n; };
 
-// Pair mode is open wherever a 256-row tile cannot straddle two experts, transposed pair mode to expert-grouped plain
-// stores.  (With 256 columns a ragged 128-wide last tile splits into 64-column halves, which only the [K, N] storage
+// Pair mode is open wherever a 256-row tile cannot straddle two experts, transposed pair mode to expert-grouped bf16
+// stores, gate-scaled ones, SwiGLU and SwiGLU backward.  (With 256 columns a ragged 128-wide last tile splits into 64-column halves, which only the [K, N] storage
 // of B can load.)  A product whose wide tiles do not fill the GPU once is latency: it takes the narrower tile with the
 // shortest reckoned time (main loop plus fill and epilogue), if that is a fifth shorter.  The constants are clocks measured
 // on the kernel: a K step is bound by its tensor work (2 clk per column; the pair's instructions add about 90) or by the
@@ -1795,7 +1795,8 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   P.bk = f8 ? 2 * TC_BK : TC_BK;
   P.k_blocks = (int)ceil_div(p.K, P.bk);
   if (f8) {
-    // e4m3 operands: K-major on both sides, the SwiGLU pair (one CTA per tile) or the transposed store
+    // e4m3 operands: K-major on both sides, the SwiGLU pair (transposed, or one CTA per row tile where that leaves SMs
+    // idle) or the transposed store
     if (p.a_mn_major || p.b_mn_major || p.concat == CONCAT_K || !p.a_scale || !p.b_scale0 ||
         (p.concat == CONCAT_N && !p.b_scale1) || p.lda % 16 != 0 || p.ldb % 16 != 0 || p.K % 16 != 0)
       return REVFFN_ERR_UNSUPPORTED;

@@ -2,8 +2,8 @@
 
 A forward block holds two tiles of 128 query positions and walks the key blocks that they need: sequence lengths on
 both sides of one, two, three and four tiles (an odd number of tiles leaves the last block one), grouped key/value
-heads; and weights large enough that row maxima grow by more than 2^8 along the keys, which the softmax's running
-reference has to follow.  Tolerance: the path's stated 2e-2 (bf16 operands, P rounded to bf16, fp32 sums).  The scores
+heads; and row maxima that grow along the keys past what the softmax's reference may stay behind (a sum of 64 weights of
+2^20, a single weight of 2^14).  Tolerance: the path's stated 2e-2 (bf16 operands, P rounded to bf16, fp32 sums).  The scores
 have a standard deviation of (16 std)^2 sqrt(128) = 18.5 at std 0.08; q and k rounded to bf16 (2^-9 / sqrt(3) relative
 each) move a score by 18.5 * 2^-9 * sqrt(2/3) = 0.03 and so each unsaturated weight by 3 %, which the sum over keys
 brings below 2e-2; at std 0.12 it would be 6.6 %, too much for that tolerance whatever the kernel."""
