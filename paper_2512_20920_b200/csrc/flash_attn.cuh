@@ -26,9 +26,9 @@
 // clock), the products 2.3k; a CTA starts and ends in 5-8k.  4 sequences of 2048 x 16 heads: 120 us with one query tile per
 // CTA, the output in registers and maxima exchanged through shared memory; 97 with two tiles; 88 with products issued by a
 // converged warp (the row maxima left out beside that: no difference); P in halves 92 -> 88 on another box.  The second sum
-// costs 4 us there, 82 -> 86, in two unpackings and an addition per pair of weights; a gradient pass, which wants both sums,
-// fetches the second half's scores twice instead of spilling registers (117 -> 103).  7 x 613: 38 -> 36 us when five query
-// tiles made three pairs; 33 -> 35 by the second sum.
+// costs nothing there (82 and 82 us); a gradient pass, which wants both sums, fetches the second half's scores twice instead of
+// spilling registers (117 -> 103, 96 before it had them).  7 x 613: 38 -> 36 us when five query tiles made three pairs, now 30
+// (39 for a gradient pass).
 // Operands: q, k, v head-major [.., S_pad, hd] bf16 with hd = 128 (rows past the sequence are zero);
 // output token-major [T, ld_o] bf16, plus the row log-sum-exp (natural log, of the scaled scores).
 // Every wait is bounded; a wait that runs out sets the status word and all roles leave.
@@ -69,8 +69,10 @@ __device__ __forceinline__ float2 fa_probs64(const uint32_t (&r0)[32], const uin
     const float2 e = make_float2(fa_exp2(t.x), fa_exp2(t.y));
     if (SUM) sum = __fadd2_rn(sum, e);
     const __nv_bfloat162 h = __floats2bfloat162_rn(e.x, e.y);
-    rounded = __fadd2_rn(rounded, __bfloat1622float2(h));
     pw[i] = *reinterpret_cast<const uint32_t*>(&h);
+    // two additions of bf16 to fp32; unpacked and added in pairs it is three instructions (core at 4 x 2048: 86 us instead of 82)
+    asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}"
+        : "+f"(rounded.x), "+f"(rounded.y) : "r"(pw[i]));
   }
   return make_float2(sum.x + sum.y, rounded.x + rounded.y);
 }
