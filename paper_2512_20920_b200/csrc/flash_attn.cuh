@@ -101,13 +101,14 @@ __device__ __forceinline__ void tc_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint
 struct FlashParams {
   int S, Sp, n_heads, rep;        // rep = query heads per key/value head
   bf16* o; int64_t ld_o;          // [T, ld_o]
-  float* lse;                     // GRAD: [B * n_heads * Sp]
-  float* o32;                     // GRAD: [B * n_heads * Sp, 128], the output before rounding, head-major
+  const bf16* d_o;                // GRAD: gradient of the output, head-major [B * n_heads * Sp, 128]
+  float* lse_d;                   // GRAD: statistics of the rows for the gradient kernels, see FlashBwdParams
   float scale_log2e, scale;
   int* status;
 };
 
-// GRAD: for a gradient pass, which also wants the row log-sum-exp and the output before rounding.
+// GRAD: for a gradient pass, which also wants of each row the log-sum-exp and D = <dO, O>.  O is taken before its rounding to
+// bf16: D stands for sum_j P_j dP_j, and with a peaked row dP - D cancels, so an error in D would show in dS.
 template <bool GRAD>
 __global__ void __launch_bounds__(FA_THREADS, 1)
 flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -354,6 +355,7 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
       const int s_pos0 = (2 * qp + x) * FA_BLK + q * 32, s_pos = s_pos0 + lane;
       const int rows_ok = min(32, P.S - s_pos0);
       const float inv = 1.f / l.y;
+      float2 dot = make_float2(0.f, 0.f);      // GRAD: <dO, O> of even and odd columns
       const int seq = bh / P.n_heads, head = bh % P.n_heads;
       uint8_t* stg = gen_base + FA_Q_OFF + x * 2 * FA_TILE + q * 8192;
       bf16* dst = P.o + ((int64_t)seq * P.S + s_pos0) * P.ld_o + (int64_t)head * FA_HD;
@@ -366,26 +368,27 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
 #pragma unroll
         for (int i = 0; i < 32; ++i) f[i] = __uint_as_float(o[i]) * inv;
         stage32_bf16(stg, lane, f);
-        if (GRAD) {
+        if (GRAD && lane < rows_ok) {
+          const uint4* g4 = reinterpret_cast<const uint4*>(P.d_o + ((int64_t)bh * P.Sp + s_pos) * FA_HD + c);
 #pragma unroll
-          for (int g = 0; g < 8; ++g)
-            *reinterpret_cast<float4*>(stg + 4096 + lane * 128 + ((g ^ (lane & 7)) << 4)) =
-                make_float4(f[4 * g], f[4 * g + 1], f[4 * g + 2], f[4 * g + 3]);
-        }
-        __syncwarp();
-        blk_stage_to_global(stg, lane, dst + c, P.ld_o, rows_ok);
-        if (GRAD) {
-          float* d32 = P.o32 + ((int64_t)bh * P.Sp + s_pos0) * FA_HD + c;
+          for (int g = 0; g < 4; ++g) {
+            float y[8];
+            unpack8(g4[g], y);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int r = 4 * i + (lane >> 3);
-            const float4 v = *reinterpret_cast<const float4*>(stg + 4096 + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
-            if (r < rows_ok) *reinterpret_cast<float4*>(d32 + (int64_t)r * FA_HD + (lane & 7) * 4) = v;
+            for (int i = 0; i < 8; i += 2)
+              dot = __ffma2_rn(make_float2(f[8 * g + i], f[8 * g + i + 1]), make_float2(y[i], y[i + 1]), dot);
           }
         }
         __syncwarp();
+        blk_stage_to_global(stg, lane, dst + c, P.ld_o, rows_ok);
+        __syncwarp();
       }
-      if (GRAD && lane < rows_ok) P.lse[(int64_t)bh * P.Sp + s_pos] = m * P.scale + logf(l.x);
+      if (GRAD) {      // rows past the end of the sequence: weights of zero
+        const int64_t at = (int64_t)bh * P.Sp + s_pos;
+        float* ld = P.lse_d + 4 * (at >> 1) + (at & 1);
+        ld[0] = lane < rows_ok ? -(m * P.scale + logf(l.x)) * 1.4426950408889634f : -INFINITY;
+        ld[2] = lane < rows_ok ? -(dot.x + dot.y) * P.scale : 0.f;
+      }
     }
   }
 
@@ -408,10 +411,10 @@ flash_fwd_kernel(const FlashParams P, const __grid_constant__ CUtensorMap map_q,
   }
 }
 
-// q: [B * n_heads * Sp, 128], k, v: [B * n_kv_heads * Sp, 128] bf16 head-major; o: [B * S, ld_o] bf16.  lse and o32 are
-// written when o32 is given.
+// q: [B * n_heads * Sp, 128], k, v: [B * n_kv_heads * Sp, 128] bf16 head-major; o: [B * S, ld_o] bf16.  lse_d is written when
+// d_o is given.
 inline int launch_flash_fwd(const bf16* q, const bf16* k, const bf16* v, int batch, int n_heads, int n_kv_heads, int S, int Sp,
-                            bf16* o, int64_t ld_o, float* lse, float* o32, int* status, cudaStream_t st) {
+                            bf16* o, int64_t ld_o, const bf16* d_o, float* lse_d, int* status, cudaStream_t st) {
   TcState& s = tc_state();
   if (!s.ready) return REVFFN_ERR_CUDA;
   if (batch <= 0) return REVFFN_OK;
@@ -433,48 +436,43 @@ inline int launch_flash_fwd(const bf16* q, const bf16* k, const bf16* v, int bat
   if (r) return r;
   FlashParams P;
   P.S = S; P.Sp = Sp; P.n_heads = n_heads; P.rep = n_heads / n_kv_heads;
-  P.o = o; P.ld_o = ld_o; P.lse = lse; P.o32 = o32;
+  P.o = o; P.ld_o = ld_o; P.d_o = d_o; P.lse_d = lse_d;
   P.scale = 1.f / sqrtf((float)FA_HD);
   P.scale_log2e = P.scale * 1.4426950408889634f;
   P.status = status;
   const int grid = batch * n_heads * ((Sp / FA_BLK + 1) / 2);
-  launch_k(o32 ? flash_fwd_kernel<true> : flash_fwd_kernel<false>, grid, FA_THREADS, FA_SMEM_BYTES, st, P, mq, mk, mv);
+  launch_k(d_o ? flash_fwd_kernel<true> : flash_fwd_kernel<false>, grid, FA_THREADS, FA_SMEM_BYTES, st, P, mq, mk, mv);
   return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 
 // ---------------------------------------------------------------------------
-// ---------------------------------------------------------------------------
 // Backward of the attention core, also without a score matrix in HBM.  P is rebuilt from the row
 // log-sum-exp the forward kernel stored:  P = exp(scale * S - lse),  dS = scale * P * (dP - D) with
 // D = <dO_row, O_row>.  Two kernels, neither uses atomics:
-//   flash_bwd_dkv_kernel  a CTA owns 128 keys of one key/value head and walks the 64-row query tiles at or
+//   flash_bwd_dkv_kernel  an item is 128 keys of one key/value head, which walk the 128-row query tiles at or
 //                         below them (of every query head of the group):  dV += P^T dO,  dK += dS^T Q
-//   flash_bwd_dq_kernel   a CTA owns 128 query rows of one head and walks the 128-key tiles up to its diagonal:
+//   flash_bwd_dq_kernel   an item is 128 query rows of one head, which walk the 128-key tiles up to their diagonal:
 //                         dQ += dS K
-// In both the "own" side is the MMA M side and the walked tile the N side.  dK/dV, per step:
-//   S' = K_j Q_t^T,  dP' = V_j dO_t^T   (128 x 64, K = hd)
-// into TMEM (double-buffered), eight warps (two threads per key row, 32 query columns each) turn them into P' and
-// dS' as bf16 K-major operand tiles in shared memory, and the accumulators (fresh TMEM columns, summed over
-// all steps by the tensor core itself) take  dV += P' dO_t  and  dK += dS' Q_t,  where the same shared-memory
-// bytes of a walked tile that served as a K-major operand are read again as an MN-major one.
+// In both the item's own side is the MMA M side and the walked tile the N side of S' and dP'.  All four or three products
+// of a step are 128 x 128 x 128.  Eight warps (two threads per own row, 64 columns each) turn S' into P' and dP' into dS'
+// in two phases, so that the tensor pipe always has the other half of a step to work on; P' and dS' go back to tensor memory
+// over the columns that they came from, from where the accumulating products take them as their A operand, and the walked
+// tile's shared-memory bytes are read a second time as their MN-major B operand.  One in-order queue of products makes every
+// "over the columns" safe: what overwrites a region is issued behind what reads it.
+// Persistent blocks: items in descending order of their steps, dealt out to the blocks forwards and backwards in turn; the
+// steps of all items of a block are one stream: the loads and the first products of the next item run under the end of this
+// one, and four warps of their own write the output beside it.
 // No cross-thread reduction is needed: the row statistics come from memory.
+// What bounds them, per 128 x 128 block: dK/dV 2.7k clk in the middle of an item, the tensor pipe, whose S' and dP' read both
+// operands out of shared memory (256 KB a step at 128 bytes a clock, arriving tiles included); dQ 2.2k, the softmax warps'
+// exponentials (1.15k) and dS' (0.55k) and the products between them.  The first steps of an item take twice that, under the output
+// of the item before.  4 sequences of 2048 x 16 heads: 64-wide query tiles, P' and dS' through shared memory and a block per item took
+// 5.8k and 4.9k, 180 and 150 us; now 245 together, and 29 less without a launch for the row dots (7 x 613, 4 key/value heads: 121 -> 81).
+// A quarter or a third of the exponentials by a polynomial on the FMA pipe: no difference.
 // ---------------------------------------------------------------------------
-// Shared memory of the dK/dV kernel: [K_j, V_j 64 KB | 3 stages of walked tiles 96 KB | P' tile 16 KB | dS' tile
-// 16 KB | barriers | row statistics of the stages].  A stage: [Q_t 2 x 8 KB | dO_t 2 x 8 KB].  The walked tiles
-// come from L2 with a latency of more than one step, hence the ring of three.
-constexpr int FB_X_OFF = 0;
-constexpr int FB_STAGE = 2 * FA_TILE;
-constexpr int FB_NS = 3;
-constexpr int FB_Y_OFF = 4 * FA_TILE;
-constexpr int FB_P_OFF = FB_Y_OFF + FB_NS * FB_STAGE;
-constexpr int FB_DS_OFF = FB_P_OFF + FA_TILE;
-constexpr int FB_BAR_OFF = FB_DS_OFF + FA_TILE;
-constexpr int FB_LD_OFF = FB_BAR_OFF + 256;        // (lse * log2 e, D * scale) of a stage's 64 query rows, 512 B per stage
-constexpr int FB_SMEM_BYTES = FB_LD_OFF + 2048 + 1024;
-
 struct FlashBwdParams {
   int S, Sp, n_heads, rep;
-  const float2* lse_d;            // per query row (head-major index): (lse * log2 e, D * scale)
+  const float4* lse_d;            // a pair of query rows (head-major index / 2): -lse * log2 e of both, then -D * scale of both
   const bf16* x0; const bf16* x1; // dQ kernel: its owned operands (q, d_o head-major), read by the CTA's threads themselves
   // Outputs, token-major bf16 [T, ld_out]: a row's head lands at column col + head * 128.  out0: dV (dK/dV kernel, as
   // it is); out1: dK or dQ, with the rotation of the forward pass undone (its transpose), pairs (i, i + 64).
@@ -482,6 +480,7 @@ struct FlashBwdParams {
   int64_t ld_out0, ld_out1;
   int col0, col1;
   int heads_own;                  // heads per sequence on the owned side (key/value heads for dK/dV, query heads for dQ)
+  int items;
   const float2* cs;               // [64, S] (cos, sin): the lanes' positions are neighbours
   float scale_log2e, scale;
   int* status;
@@ -492,81 +491,177 @@ __device__ __forceinline__ void bulk_load_1d(uint32_t dst, const void* src, uint
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(dst), "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar) : "memory");
 }
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
+}
 
-// This thread's 32 elements of a step: P' = exp2(s * cl - lse2), dS' = P' * (dP * scale - D * scale), packed to bf16.
-// The row statistics belong to the query: the column's (DKV, read from shared memory) or this thread's own row's.
-// MASK: the tile touches the causal diagonal or the end of the sequence and every element is tested.
-template <bool DKV, bool MASK>
-__device__ __forceinline__ void fb_tile(const uint32_t (&rs)[32], const uint32_t (&rd)[32], const float4* __restrict__ ld_cols,
-                                        float2 own_ld, float cl, float scale, int col0, int own_pos, int S, uint4 (&pp)[4],
-                                        uint4 (&pd)[4]) {
+// Item of a block's round r: forwards in even rounds, backwards in odd ones.
+__device__ __forceinline__ int fb_item(int r) {
+  return r * (int)gridDim.x + ((r & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
+}
+
+// The causal diagonal's tile: registers of columns whose query comes before their key.  edge: the thread's own position relative
+// to the first of the 32 columns.  (DKV: own row = key, column = query; else the roles swap.)  A pass of its own over the registers
+// and not a second form of the arithmetic, which would run once an item.
+template <bool DKV>
+__device__ __forceinline__ void fb_mask(uint32_t (&x)[32], int edge, uint32_t value) {
 #pragma unroll
-  for (int g = 0; g < 4; ++g) {
-    float pv[8], dv[8];
+  for (int i = 0; i < 32; ++i)
+    if (DKV ? i < edge : i > edge) x[i] = value;
+}
+// 32 scores of this thread's row -> weights p = exp2(s * cl - lse2) in their place, and packed to bf16.  The row statistics
+// belong to the query: the column's (DKV, two columns to an entry of ld) or this thread's own row's; those past the end of
+// the sequence have weights of zero.
+template <bool DKV>
+__device__ __forceinline__ void fb_probs(uint32_t (&s)[32], const float4* ld, float own_nl, float cl, uint32_t (&pw)[16]) {
+  const float2 c2 = make_float2(cl, cl);
 #pragma unroll
-    for (int i = 0; i < 8; i += 2) {
-      float4 ld = make_float4(own_ld.x, own_ld.y, own_ld.x, own_ld.y);
-      if (DKV) ld = ld_cols[(8 * g + i) >> 1];          // two columns' (lse2, D * scale)
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int c = 8 * g + i + e;
-        const float l2 = e ? ld.z : ld.x, dsc = e ? ld.w : ld.y;
-        float p = fa_exp2(__uint_as_float(rs[c]) * cl - l2);
-        float ds = p * fmaf(__uint_as_float(rd[c]), scale, -dsc);
-        if (MASK) {
-          // DKV: own row = key, column = query (needs query >= key, query inside the sequence); else the roles swap
-          const bool valid = DKV ? (col0 + c >= own_pos && col0 + c < S) : (col0 + c <= own_pos && own_pos < S);
-          if (!valid) { p = 0.f; ds = 0.f; }
-        }
-        pv[i + e] = p;
-        dv[i + e] = ds;
-      }
+  for (int i = 0; i < 16; ++i) {
+    float2 nl = make_float2(own_nl, own_nl);
+    if (DKV) nl = *reinterpret_cast<const float2*>(ld + i);
+    const float2 t = __ffma2_rn(make_float2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), c2, nl);
+    const float2 e = make_float2(fa_exp2(t.x), fa_exp2(t.y));
+    s[2 * i] = __float_as_uint(e.x);
+    s[2 * i + 1] = __float_as_uint(e.y);
+    if (DKV) {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(e.x, e.y);
+      pw[i] = *reinterpret_cast<const uint32_t*>(&h);
     }
-    if (DKV) pp[g] = pack8(pv);
-    pd[g] = pack8(dv);
+  }
+}
+// dS' = P' * (dP * scale - D * scale) of 32 columns, packed to bf16.
+template <bool DKV>
+__device__ __forceinline__ void fb_dscores(const uint32_t (&p)[32], const uint32_t (&rd)[32], const float4* ld, float own_nd, float scale,
+                                           uint32_t (&dw)[16]) {
+  const float2 s2 = make_float2(scale, scale);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    float2 nd = make_float2(own_nd, own_nd);
+    if (DKV) nd = *(reinterpret_cast<const float2*>(ld + i) + 1);
+    const float2 x = __ffma2_rn(make_float2(__uint_as_float(rd[2 * i]), __uint_as_float(rd[2 * i + 1])), s2, nd);
+    const float2 d = __fmul2_rn(make_float2(__uint_as_float(p[2 * i]), __uint_as_float(p[2 * i + 1])), x);
+    const __nv_bfloat162 h = __floats2bfloat162_rn(d.x, d.y);
+    dw[i] = *reinterpret_cast<const uint32_t*>(&h);
   }
 }
 
-__global__ void __launch_bounds__(FA_THREADS, 1)
-flash_bwd_dkv_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap map_x0, const __grid_constant__ CUtensorMap map_x1,
-                 const __grid_constant__ CUtensorMap map_y0, const __grid_constant__ CUtensorMap map_y1) {
-  extern __shared__ uint8_t fa_smem_raw[];
-  const uint32_t raw = smem_u32(fa_smem_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  uint8_t* gen_base = fa_smem_raw + (base - raw);
+// Four neighbouring lanes hold four 16-byte pieces each: piece k of lane j changes place with piece j of lane k.  A warp whose
+// lanes are rows then reads or writes rows of 64 contiguous bytes, eight per instruction; 16-byte pieces of 32 rows
+// take an instruction four times as long, and everything else that goes through the same unit (the softmax warps'
+// statistics) waits behind it (dK/dV at 4 x 2048, a step on average: 3.85k clk -> 3.64k).
+__device__ __forceinline__ void quad_transpose(uint4 (&v)[4], int lane) {
+  auto trade = [&](uint4& a, uint4& b, bool hi, int mask) {      // the low lane gives b for the high lane's a
+    const uint4 s = hi ? a : b;
+    uint4 r;
+    r.x = __shfl_xor_sync(0xffffffffu, s.x, mask); r.y = __shfl_xor_sync(0xffffffffu, s.y, mask);
+    r.z = __shfl_xor_sync(0xffffffffu, s.z, mask); r.w = __shfl_xor_sync(0xffffffffu, s.w, mask);
+    if (hi) a = r; else b = r;
+  };
+  trade(v[0], v[1], lane & 1, 1); trade(v[2], v[3], lane & 1, 1);
+  trade(v[0], v[2], lane & 2, 2); trade(v[1], v[3], lane & 2, 2);
+}
+
+// A warp's 32 rows x 128 columns of an accumulator to the token-major output, the rotation undone when cs is given
+// (columns 0..31 turn with 64..95, 32..63 with 96..127; cs: at this lane's position).  dst: the warp's first row, rows: how
+// many of its rows exist.  `drained` is called when the last columns are in registers.
+template <typename Drained>
+__device__ __forceinline__ void fb_output(uint32_t acc, const float2* cs, int64_t cs_step, int lane, int rows, bf16* dst, int64_t ld, Drained drained) {
+  dst += (int64_t)(lane & ~3) * ld + (lane & 3) * 8;
+#pragma unroll 1
+  for (int c = 0; c < 64; c += 32) {
+    uint32_t rl[32], rh[32];
+    tmem_ld32(acc + (uint32_t)c, rl);
+    tmem_ld32(acc + (uint32_t)(64 + c), rh);
+    tmem_ld_wait();
+    if (c == 32) drained();
+    if (cs && lane < rows) {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const float2 t = cs[(int64_t)(c + i) * cs_step];
+        const float a0 = __uint_as_float(rl[i]), b0 = __uint_as_float(rh[i]);
+        rl[i] = __float_as_uint(a0 * t.x + b0 * t.y);
+        rh[i] = __float_as_uint(b0 * t.x - a0 * t.y);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+      uint4 v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = pack8(reinterpret_cast<const float*>(w ? rh : rl) + 8 * k);
+      quad_transpose(v, lane);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if ((lane & ~3) + k < rows) *reinterpret_cast<uint4*>(dst + (int64_t)k * ld + 64 * w + c) = v[k];
+    }
+    __syncwarp();
+  }
+}
+
+constexpr int FB_THREADS = 512;
+// Registers of the roles' warpgroups: loads and products | P', dS' | P', dS' | output.  Their sum is at most the 4 x 128
+// that the block is launched with.
+constexpr int FB_REGS_ISSUE = 72, FB_REGS_SOFTMAX = 160, FB_REGS_OUT = 112;
+static_assert(FB_REGS_ISSUE + 2 * FB_REGS_SOFTMAX + FB_REGS_OUT <= 4 * 128, "register file");
+template <int N> __device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+
+// Shared memory of the dK/dV kernel: [K_j, V_j 64 KB | 3 query tiles 96 KB | 2 dO tiles 64 KB | their row statistics | barriers].
+// A query tile is in use from its S' to its dK, more than a step, a dO tile from its dP' to its dV.
+constexpr int FB_QS = 3, FB_OS = 2;
+constexpr int FB_TILE = 2 * FA_TILE;              // 128 rows x 128 columns
+constexpr int FB_X_OFF = 0;
+constexpr int FB_Q_OFF = 2 * FB_TILE;
+constexpr int FB_O_OFF = FB_Q_OFF + FB_QS * FB_TILE;
+constexpr int FB_LD_OFF = FB_O_OFF + FB_OS * FB_TILE;
+constexpr int FB_BAR_OFF = FB_LD_OFF + FB_OS * 1024;
+constexpr int FB_SMEM_BYTES = FB_BAR_OFF + 256;
+
+__global__ void __launch_bounds__(FB_THREADS, 1)
+flash_bwd_dkv_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                     const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o) {
+  extern __shared__ __align__(1024) uint8_t fb_smem[];
+  const uint32_t base = smem_u32(fb_smem);
+  if (base & 1023u) {                              // the whole of the block's shared memory is in use: no room to align by hand
+    pdl_wait();
+    set_status(P.status, REVFFN_ERR_CUDA);
+    return;
+  }
   const uint32_t bars = base + FB_BAR_OFF;
   auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
-  constexpr int NS = FB_NS;
-  constexpr int Y_OFF = FB_Y_OFF;
-  constexpr bool DKV = true;      // the element routine is shared with the dQ kernel and takes the role as a parameter
-  enum { B_XFULL = 0, B_YFULL = 1, B_YEMPTY = 1 + FB_NS, B_SDFULL = 1 + 2 * FB_NS, B_SDEMPTY = B_SDFULL + 2,
-         B_PDFULL = B_SDEMPTY + 2, B_PDEMPTY = B_PDFULL + 1, B_ACCFULL = B_PDEMPTY + 1, B_COUNT = B_ACCFULL + 1 };
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen_base + FB_BAR_OFF + 8 * B_COUNT);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(gen_base + FB_BAR_OFF + 8 * B_COUNT + 8);
-  int* issued = reinterpret_cast<int*>(gen_base + FB_BAR_OFF + 8 * B_COUNT + 16);   // [1 + NS]: x, y stages -> phase + 1
+  enum { B_KFULL = 0, B_VFULL, B_KEMPTY, B_VEMPTY, B_QFULL, B_QEMPTY = B_QFULL + FB_QS, B_OFULL = B_QEMPTY + FB_QS, B_OEMPTY = B_OFULL + FB_OS,
+         B_SFULL = B_OEMPTY + FB_OS, B_PHALF, B_PFULL, B_DPFULL, B_DSFULL, B_DVFULL, B_DKFULL, B_DVEMPTY, B_DKEMPTY, B_DRAIN, B_COUNT };
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fb_smem + FB_BAR_OFF + 8 * B_COUNT);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  int* issued = reinterpret_cast<int*>(tmem_slot + 2);      // [2 + FB_QS + FB_OS]: k, v, query stages, dO stages -> phase + 1
+  static_assert(8 * B_COUNT + 4 * (2 + 2 + FB_QS + FB_OS) <= 256, "barrier block");
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int n_blk = P.Sp / FA_BLK;                  // 128-row blocks per head
-  const int n_t64 = P.Sp / 64;                      // 64-row tiles per head
-  // heavy work first: low key blocks see the most query tiles
-  const int per = (int)gridDim.x / n_blk;
-  const int blk = (int)blockIdx.x / per;            // own 128-key block within the head
-  const int grp = (int)blockIdx.x % per;            // sequence * n_kv_heads + kv head
-  const int own_row0 = grp * P.Sp + blk * FA_BLK;
-  const int t_begin = 2 * blk;
-  const int n_inner = n_t64 - 2 * blk;
-  const int n_steps = P.rep * n_inner;              // every query head of the group in turn
-  const int y_base = grp * P.rep * P.Sp;            // first row of the group's first query head
-  auto y_row_of = [&](int s) -> int { return y_base + (s / n_inner) * P.Sp + 64 * (t_begin + s % n_inner); };
+  const int per = P.items / n_blk;                  // (sequence, key/value head) pairs
+  // items with low key blocks come first: they see the most query tiles
+  struct Item { int blk, grp, steps; };
+  auto item_of = [&](int r) -> Item {
+    const int it = fb_item(r);
+    Item x;
+    x.blk = it / per; x.grp = it - x.blk * per;
+    x.steps = it < P.items ? P.rep * (n_blk - x.blk) : 0;      // every query head of the group in turn
+    return x;
+  };
 
   if (threadIdx.x == 0) {
-    mbar_init(bar(B_XFULL), 1);
-    mbar_init(bar(B_ACCFULL), 1);
-    mbar_init(bar(B_PDFULL), 8);
-    mbar_init(bar(B_PDEMPTY), 1);
-    for (int s = 0; s < NS; ++s) { mbar_init(bar(B_YFULL + s), 1); mbar_init(bar(B_YEMPTY + s), 1); }
-    for (int s = 0; s < 2; ++s) { mbar_init(bar(B_SDFULL + s), 1); mbar_init(bar(B_SDEMPTY + s), 8); }
-    for (int i = 0; i < 1 + NS; ++i) issued[i] = 0;
+    mbar_init(bar(B_KFULL), 1); mbar_init(bar(B_VFULL), 1); mbar_init(bar(B_KEMPTY), 1); mbar_init(bar(B_VEMPTY), 1);
+    for (int s = 0; s < FB_QS; ++s) { mbar_init(bar(B_QFULL + s), 1); mbar_init(bar(B_QEMPTY + s), 1); }
+    for (int s = 0; s < FB_OS; ++s) { mbar_init(bar(B_OFULL + s), 1); mbar_init(bar(B_OEMPTY + s), 1 + 8); }
+    mbar_init(bar(B_SFULL), 1); mbar_init(bar(B_PHALF), 8); mbar_init(bar(B_PFULL), 8);
+    mbar_init(bar(B_DPFULL), 1); mbar_init(bar(B_DSFULL), 8);
+    mbar_init(bar(B_DVFULL), 1); mbar_init(bar(B_DKFULL), 1); mbar_init(bar(B_DVEMPTY), 4); mbar_init(bar(B_DKEMPTY), 4);
+    mbar_init(bar(B_DRAIN), 1);
+    for (int i = 0; i < 2 + FB_QS + FB_OS; ++i) issued[i] = 0;
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -581,268 +676,84 @@ flash_bwd_dkv_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  // TMEM columns: step buffer b: S' at 128 b, dP' at 128 b + 64; acc0 at 256, acc1 at 384
-  const uint32_t idesc_sd = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(FA_BLK >> 4) << 24);
-  const uint32_t idesc_acc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(FA_HD >> 3) << 17) |
-                             ((uint32_t)(FA_BLK >> 4) << 24);
-
-  if (warp == 0) {
-    // ------------------------------------------------------------------ producer
-    if (lane == 0) {
-      mbar_expect_tx(bar(B_XFULL), 4 * FA_TILE);
-      issued[0] = 1;
-      for (int kb = 0; kb < 2; ++kb) {
-        tma_load_2d(base + FB_X_OFF + kb * FA_TILE, &map_x0, 64 * kb, own_row0, bar(B_XFULL));
-        tma_load_2d(base + FB_X_OFF + (2 + kb) * FA_TILE, &map_x1, 64 * kb, own_row0, bar(B_XFULL));
-      }
-      for (int s = 0; s < n_steps; ++s) {
-        const int st = s % NS;
-        const uint32_t ph = (uint32_t)(s / NS) & 1u;
-        if (!mbar_wait(bar(B_YEMPTY + st), ph ^ 1u, abort_flag, P.status)) break;
-        mbar_expect_tx(bar(B_YFULL + st), FB_STAGE + 512);
-        issued[1 + st] = (int)ph + 1;
-        const int yr = y_row_of(s);
-        bulk_load_1d(base + FB_LD_OFF + st * 512, P.lse_d + yr, 512, bar(B_YFULL + st));
-        const uint32_t ys = base + Y_OFF + st * FB_STAGE;
-        for (int kb = 0; kb < 2; ++kb) {
-          tma_load_2d(ys + kb * 8192, &map_y0, 64 * kb, yr, bar(B_YFULL + st));
-          tma_load_2d(ys + FA_TILE + kb * 8192, &map_y1, 64 * kb, yr, bar(B_YFULL + st));
-        }
-      }
-      pdl_trigger();
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer
-    const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0), sb = __shfl_sync(0xffffffffu, base, 0);
-    auto wait = [&](int i, uint32_t parity) -> bool {
-      const bool got = mbar_wait_warp(bar(i), parity, abort_flag, P.status);
-      tc_fence_after();
-      return got;
-    };
-    bool ok = wait(B_XFULL, 0u);
-    auto issue_sd = [&](int s) -> bool {
-      const int b = s & 1, st = s % NS;
-      const uint32_t ph = (uint32_t)(s >> 1) & 1u;
-      if (!wait(B_YFULL + st, (uint32_t)(s / NS) & 1u)) return false;
-      if (!wait(B_SDEMPTY + b, ph ^ 1u)) return false;
-      const uint64_t a_desc = make_smem_desc(sb + FB_X_OFF, 16, 1024);
-      const uint64_t b_desc = make_smem_desc(sb + Y_OFF + st * FB_STAGE, 16, 1024);
-      if (elect_one()) {
-#pragma unroll
-        for (int w = 0; w < 2; ++w) {            // w = 0: S' = X0 Y0^T, w = 1: dP' = X1 Y1^T
-#pragma unroll
-          for (int k = 0; k < 8; ++k)            // 64-column tiles of 16 KB (X) and 8 KB (Y), 16 columns an instruction
-            tc_mma(tb + (uint32_t)(b * 128 + w * 64), a_desc + (uint64_t)((2 * w + (k >> 2)) * (FA_TILE >> 4) + 2 * (k & 3)),
-                   b_desc + (uint64_t)((2 * w + (k >> 2)) * (8192 >> 4) + 2 * (k & 3)), idesc_sd, k != 0 ? 1u : 0u);
-        }
-        tc_commit(bar(B_SDFULL + b));
-      }
-      __syncwarp();
-      return true;
-    };
-    if (ok) ok = issue_sd(0);
-    for (int s = 0; ok && s < n_steps; ++s) {
-      if (s + 1 < n_steps && !issue_sd(s + 1)) { ok = false; break; }
-      const int st = s % NS;
-      if (!(ok = wait(B_PDFULL, (uint32_t)s & 1u))) break;
-      // the walked tiles again, now as [64 rows (K), 128 columns (N)] operands: the two 64-column halves are 8 KB apart
-      const uint64_t a_desc = make_smem_desc(sb + FB_P_OFF, 16, 1024);
-      const uint64_t b_desc = make_smem_desc(sb + Y_OFF + st * FB_STAGE, 8192, 1024);
-      if (elect_one()) {
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-          tc_mma(tb + 256u, a_desc + (uint64_t)(2 * ks), b_desc + (uint64_t)((FA_TILE >> 4) + 128 * ks), idesc_acc, (s | ks) != 0 ? 1u : 0u);
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-          tc_mma(tb + 384u, a_desc + (uint64_t)(((FB_DS_OFF - FB_P_OFF) >> 4) + 2 * ks), b_desc + (uint64_t)(128 * ks), idesc_acc,
-                 (s | ks) != 0 ? 1u : 0u);
-        tc_commit(bar(B_YEMPTY + st));
-        tc_commit(bar(B_PDEMPTY));
-        if (s + 1 == n_steps) tc_commit(bar(B_ACCFULL));
-      }
-      __syncwarp();
-    }
-  } else {
-    // ------------------------------------------------------------------ P' / dS' (warps 2..9)
-    const int q = warp & 3;                      // TMEM lane quadrant this warp may access
-    const int hh = (warp - 2) >> 2;              // which 32 of the step's 64 columns
-    const int row = q * 32 + lane;               // own row within the block
-    const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
-    const float cl = P.scale_log2e, scale = P.scale;
-    const int own_pos = blk * FA_BLK + row;      // position in the sequence of this thread's own row
-    const float2 own_ld = make_float2(0.f, 0.f);      // unused by the key-row role
-    bool ok = true;
-    for (int s = 0; s < n_steps; ++s) {
-      const int b = s & 1;
-      const uint32_t ph = (uint32_t)(s >> 1) & 1u;
-      if (!mbar_wait_warp(bar(B_SDFULL + b), ph, abort_flag, P.status)) { ok = false; break; }
-      // this thread reads the stage's row statistics itself, so it observes the stage's barrier itself (every lane does)
-      if (!mbar_wait_warp(bar(B_YFULL + s % NS), (uint32_t)(s / NS) & 1u, abort_flag, P.status)) { ok = false; break; }
-      tc_fence_after();
-      uint32_t rs[32], rd[32];
-      tmem_ld32(lane_addr + (uint32_t)(b * 128 + 32 * hh), rs);
-      tmem_ld32(lane_addr + (uint32_t)(b * 128 + 64 + 32 * hh), rd);
-      tmem_ld_wait();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(B_SDEMPTY + b));
-      const int t = t_begin + s % n_inner;
-      const int col0 = 64 * t + 32 * hh;         // position in the sequence of this thread's first column
-      // tiles that touch the diagonal or the end of the sequence need the element-wise test
-      const bool mask = t < 2 * blk + 2 || 64 * t + 63 >= P.S;
-      // the step's row statistics came with the walked tiles
-      const float4* ld_cols = reinterpret_cast<const float4*>(gen_base + FB_LD_OFF + (s % NS) * 512) + 16 * hh;
-      uint4 pp[4], pd[4];
-      if (mask) fb_tile<DKV, true>(rs, rd, ld_cols, own_ld, cl, scale, col0, own_pos, P.S, pp, pd);
-      else fb_tile<DKV, false>(rs, rd, ld_cols, own_ld, cl, scale, col0, own_pos, P.S, pp, pd);
-      // the operand tiles have one buffer: the previous step's accumulating products must have read them
-      if (!mbar_wait_warp(bar(B_PDEMPTY), ((uint32_t)s & 1u) ^ 1u, abort_flag, P.status)) { ok = false; break; }
-      uint8_t* prow = gen_base + FB_P_OFF + row * 128;
-      uint8_t* drow = gen_base + FB_DS_OFF + row * 128;
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        const int piece = ((4 * hh + g) ^ (row & 7)) << 4;
-        *reinterpret_cast<uint4*>(prow + piece) = pp[g];
-        *reinterpret_cast<uint4*>(drow + piece) = pd[g];
-      }
-      fence_async_smem();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(B_PDFULL));
-    }
-    if (ok) ok = mbar_wait_warp(bar(B_ACCFULL), 0u, abort_flag, P.status);
-    if (ok) {
-      tc_fence_after();
-      // This thread takes columns [32 hh, +32) and their rotation partners [64 + 32 hh, +32) of its row.  The
-      // tensor-memory loads are warp-wide instructions: every lane executes them, rows past the sequence only
-      // skip the stores.
-      const bool row_ok = own_pos < P.S;
-      const int seq = grp / P.heads_own, head = grp % P.heads_own;
-      const int64_t tok = (int64_t)seq * P.S + (row_ok ? own_pos : 0);
-      {
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {          // a = 0: dV as it is, a = 1: dK with the rotation undone
-          uint32_t rl[32], rh[32];
-          __syncwarp();               // lanes that skipped the previous output rejoin before the warp-wide loads
-          tmem_ld32(lane_addr + (uint32_t)(256 + 128 * a + 32 * hh), rl);
-          tmem_ld32(lane_addr + (uint32_t)(256 + 128 * a + 64 + 32 * hh), rh);
-          tmem_ld_wait();
-          if (!row_ok) continue;
-          float y0[32], y1[32];
-#pragma unroll
-          for (int i = 0; i < 32; ++i) { y0[i] = __uint_as_float(rl[i]); y1[i] = __uint_as_float(rh[i]); }
-          if (a == 1) {
-            const float2* cs2 = P.cs + (int64_t)(32 * hh) * P.S + own_pos;
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              const float2 cs = cs2[(int64_t)i * P.S];
-              const float a0 = y0[i], b0 = y1[i];
-              y0[i] = a0 * cs.x + b0 * cs.y;
-              y1[i] = b0 * cs.x - a0 * cs.y;
-            }
-          }
-          bf16* dst = (a == 0 ? P.out0 + tok * P.ld_out0 + P.col0 : P.out1 + tok * P.ld_out1 + P.col1) + head * FA_HD + 32 * hh;
-          store32_bf16(dst, y0);
-          store32_bf16(dst + 64, y1);
-        }
-      }
-    }
-  }
-
-  // ------------------------------------------------------------------ teardown
-  tc_fence_before();
-  __syncthreads();
-  if (*abort_flag && threadIdx.x == 0) {
-    for (int i = 0; i < 1 + NS; ++i) {      // slot 0: the owned operands, slot 1 + st: stage st of the walked tiles
-      if (issued[i] == 0) continue;
-      long long t0 = clock64();
-      while (!mbar_try_wait(bar(i == 0 ? B_XFULL : B_YFULL + i - 1), (uint32_t)(issued[i] - 1)) && clock64() - t0 < TC_WAIT_CYCLES) {}
-    }
-  }
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
-  }
-}
-
-// ---------------------------------------------------------------------------
-// dQ with 128-key walked tiles.  The 128 x 64 x 16 instructions of the kernel above run at 55 clk against 32 at
-// full rate; the dQ launch has the tensor memory for the 128-wide shape: its owned operands (Q_i, dO_i) sit in
-// tensor memory as A operands (128 columns), S' and dP' take 128 columns each (one buffer: the softmax warps free
-// it once the scores are in registers) and dQ the last 128.  Shared memory: three 64 KB stages of [K_t | V_t] and
-// the dS' operand tile.
-// ---------------------------------------------------------------------------
-constexpr int FQ_NS = 3;
-constexpr int FQ_STAGE = 4 * FA_TILE;
-constexpr int FQ_DS_OFF = FQ_NS * FQ_STAGE;
-constexpr int FQ_BAR_OFF = FQ_DS_OFF + 2 * FA_TILE;
-constexpr int FQ_SMEM_BYTES = FQ_BAR_OFF + 256 + 1024;
-
-__global__ void __launch_bounds__(FA_THREADS, 1)
-flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v) {
-  extern __shared__ uint8_t fa_smem_raw[];
-  const uint32_t raw = smem_u32(fa_smem_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  uint8_t* gen_base = fa_smem_raw + (base - raw);
-  const uint32_t bars = base + FQ_BAR_OFF;
-  auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
-  enum { B_XFULL = 0, B_YFULL = 1, B_YEMPTY = 1 + FQ_NS, B_SDFULL = 1 + 2 * FQ_NS, B_SDEMPTY, B_PDFULL, B_PDEMPTY, B_ACCFULL, B_COUNT };
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen_base + FQ_BAR_OFF + 8 * B_COUNT);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(gen_base + FQ_BAR_OFF + 8 * B_COUNT + 8);
-  int* issued = reinterpret_cast<int*>(gen_base + FQ_BAR_OFF + 8 * B_COUNT + 16);   // [FQ_NS]: stage -> phase + 1
-
-  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-  const int n_blk = P.Sp / FA_BLK;
-  const int per = (int)gridDim.x / n_blk;
-  const int blk = n_blk - 1 - (int)blockIdx.x / per;     // heavy work first: high query blocks see the most key tiles
-  const int grp = (int)blockIdx.x % per;                 // sequence * n_heads + head
-  const int own_row0 = grp * P.Sp + blk * FA_BLK;
-  const int n_steps = blk + 1;                           // key tiles 0 .. the diagonal one
-  const int kv_row0 = (grp / P.rep) * P.Sp;
-
-  if (threadIdx.x == 0) {
-    mbar_init(bar(B_XFULL), 8);
-    mbar_init(bar(B_SDFULL), 1); mbar_init(bar(B_SDEMPTY), 8);
-    mbar_init(bar(B_PDFULL), 8); mbar_init(bar(B_PDEMPTY), 1);
-    mbar_init(bar(B_ACCFULL), 1);
-    for (int s = 0; s < FQ_NS; ++s) { mbar_init(bar(B_YFULL + s), 1); mbar_init(bar(B_YEMPTY + s), 1); issued[s] = 0; }
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                 ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  pdl_wait();
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-  // TMEM columns: S' 0..127, dP' 128..255, Q_i 256..319, dO_i 320..383 (packed pairs), dQ 384..511
+  // TMEM columns: S' 0..127, dP' 128..255, dV 256..383, dK 384..511.  P' and dS' (bf16 pairs): 32 columns at the start of each
+  // half of S' and dP', so that a warp overwrites only what it has read itself.
+  // fp32 accumulate, bf16 operands, M = N = 128; the accumulating products' B is stored [row, hd] (N contiguous)
   const uint32_t idesc_sd = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(FA_BLK >> 3) << 17) | ((uint32_t)(FA_BLK >> 4) << 24);
   const uint32_t idesc_acc = idesc_sd | (1u << 16);
+  const int role = warp >> 2;                       // warpgroup: loads and products, softmax, softmax, output
+  auto arrive = [&](int i) {
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar(i));
+  };
 
-  if (warp == 0) {
+  if (role == 0) {
+    regs_dec<FB_REGS_ISSUE>();
+    if (warp == 0) {
     // ------------------------------------------------------------------ producer
     if (lane == 0) {
-      for (int s = 0; s < n_steps; ++s) {
-        const int st = s % FQ_NS;
-        const uint32_t ph = (uint32_t)(s / FQ_NS) & 1u;
-        if (!mbar_wait(bar(B_YEMPTY + st), ph ^ 1u, abort_flag, P.status)) break;
-        mbar_expect_tx(bar(B_YFULL + st), FQ_STAGE);
-        issued[st] = (int)ph + 1;
-        const int yr = kv_row0 + s * FA_BLK;
-        const uint32_t ys = base + st * FQ_STAGE;
-        for (int kb = 0; kb < 2; ++kb) {
-          tma_load_2d(ys + kb * FA_TILE, &map_k, 64 * kb, yr, bar(B_YFULL + st));
-          tma_load_2d(ys + (2 + kb) * FA_TILE, &map_v, 64 * kb, yr, bar(B_YFULL + st));
+      bool ok = true;
+      int nq = 0, no = 0;                  // query and dO tiles loaded so far
+      auto load_q = [&](int yr) {
+        const int st = nq % FB_QS;
+        const uint32_t ph = (uint32_t)(nq / FB_QS) & 1u;
+        ok = mbar_wait(bar(B_QEMPTY + st), ph ^ 1u, abort_flag, P.status);
+        if (!ok) return;
+        mbar_expect_tx(bar(B_QFULL + st), FB_TILE);
+        issued[2 + st] = (int)ph + 1;
+        for (int kb = 0; kb < 2; ++kb)
+          tma_load_2d(base + FB_Q_OFF + st * FB_TILE + kb * FA_TILE, &map_q, 64 * kb, yr, bar(B_QFULL + st));
+        ++nq;
+      };
+      auto load_o = [&](int yr) {
+        const int st = no % FB_OS;
+        const uint32_t ph = (uint32_t)(no / FB_OS) & 1u;
+        ok = mbar_wait(bar(B_OEMPTY + st), ph ^ 1u, abort_flag, P.status);
+        if (!ok) return;
+        mbar_expect_tx(bar(B_OFULL + st), FB_TILE + 1024);
+        issued[2 + FB_QS + st] = (int)ph + 1;
+        bulk_load_1d(base + FB_LD_OFF + st * 1024, P.lse_d + yr / 2, 1024, bar(B_OFULL + st));
+        for (int kb = 0; kb < 2; ++kb)
+          tma_load_2d(base + FB_O_OFF + st * FB_TILE + kb * FA_TILE, &map_o, 64 * kb, yr, bar(B_OFULL + st));
+        ++no;
+      };
+      // K_j and V_j of item r, once the last product of the item before has read its own
+      auto load_k = [&](int r, const Item& x) {
+        ok = mbar_wait(bar(B_KEMPTY), ((uint32_t)r & 1u) ^ 1u, abort_flag, P.status);
+        if (!ok) return;
+        mbar_expect_tx(bar(B_KFULL), FB_TILE);
+        issued[0] = (r & 1) + 1;
+        for (int kb = 0; kb < 2; ++kb)
+          tma_load_2d(base + FB_X_OFF + kb * FA_TILE, &map_k, 64 * kb, x.grp * P.Sp + x.blk * FA_BLK, bar(B_KFULL));
+      };
+      auto load_v = [&](int r, const Item& x) {
+        ok = mbar_wait(bar(B_VEMPTY), ((uint32_t)r & 1u) ^ 1u, abort_flag, P.status);
+        if (!ok) return;
+        mbar_expect_tx(bar(B_VFULL), FB_TILE);
+        issued[1] = (r & 1) + 1;
+        for (int kb = 0; kb < 2; ++kb)
+          tma_load_2d(base + FB_X_OFF + FB_TILE + kb * FA_TILE, &map_v, 64 * kb, x.grp * P.Sp + x.blk * FA_BLK, bar(B_VFULL));
+      };
+      // in the order in which places fall free: dO of step g, then the query tile of step g + 1
+      Item x = item_of(0);
+      if (x.steps > 0) load_k(0, x);
+      if (ok && x.steps > 0) load_q(x.grp * P.rep * P.Sp + x.blk * FA_BLK);
+      for (int r = 0; ok && x.steps > 0; ++r) {
+        load_v(r, x);
+        int head = x.grp * P.rep, t = x.blk;      // a head's rows at and below the keys; then the group's next head
+        for (int s = 0; ok && s < x.steps; ++s) {
+          load_o(head * P.Sp + t * FA_BLK);
+          if (++t == n_blk) { t = x.blk; ++head; }
+          if (ok && s + 1 < x.steps) load_q(head * P.Sp + t * FA_BLK);
         }
+        x = item_of(r + 1);
+        if (ok && x.steps > 0) load_k(r + 1, x);
+        if (ok && x.steps > 0) load_q(x.grp * P.rep * P.Sp + x.blk * FA_BLK);
       }
       pdl_trigger();
     }
-  } else if (warp == 1) {
+    } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0), sb = __shfl_sync(0xffffffffu, base, 0);
     auto wait = [&](int i, uint32_t parity) -> bool {
@@ -850,134 +761,163 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
       tc_fence_after();
       return got;
     };
-    bool ok = wait(B_XFULL, 0u);
-    auto issue_sd = [&](int s) -> bool {
-      const int st = s % FQ_NS;
-      if (!wait(B_YFULL + st, (uint32_t)(s / FQ_NS) & 1u)) return false;
-      if (!wait(B_SDEMPTY, ((uint32_t)s & 1u) ^ 1u)) return false;
-      const uint64_t b_desc = make_smem_desc(sb + st * FQ_STAGE, 16, 1024);
-      if (elect_one()) {
-#pragma unroll
-        for (int w = 0; w < 2; ++w) {            // w = 0: S' = Q_i K_t^T, w = 1: dP' = dO_i V_t^T
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-            tc_mma_ta(tb + (uint32_t)(128 * w), tb + (uint32_t)(256 + 64 * w + 8 * k),
-                      b_desc + (uint64_t)((2 * w + (k >> 2)) * (FA_TILE >> 4) + 2 * (k & 3)), idesc_sd, k != 0 ? 1u : 0u);
-        }
-        tc_commit(bar(B_SDFULL));
-      }
-      __syncwarp();
-      return true;
-    };
-    if (ok) ok = issue_sd(0);
-    for (int s = 0; ok && s < n_steps; ++s) {
-      if (s + 1 < n_steps && !issue_sd(s + 1)) { ok = false; break; }
-      const int st = s % FQ_NS;
-      if (!(ok = wait(B_PDFULL, (uint32_t)s & 1u))) break;
-      // dQ += dS' K_t: K_t's two 64-column tiles read as one [128 keys, 128 columns] operand, halves 16 KB apart
-      const uint64_t a_desc = make_smem_desc(sb + FQ_DS_OFF, 16, 1024);
-      const uint64_t b_desc = make_smem_desc(sb + st * FQ_STAGE, 2 * 8192, 1024);
+    // S' = K_j Q_t^T (w = 0), dP' = V_j dO_t^T (w = 1); both operands in 64-column tiles of 16 KB, 16 columns an instruction
+    auto issue_sd = [&](int w, uint32_t y_off, int done, int free) {
+      const uint64_t a_desc = make_smem_desc(sb + FB_X_OFF + w * FB_TILE, 16, 1024), b_desc = make_smem_desc(sb + y_off, 16, 1024);
       if (elect_one()) {
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          tc_mma(tb + 384u, a_desc + (uint64_t)((k >> 2) * (FA_TILE >> 4) + 2 * (k & 3)), b_desc + (uint64_t)(128 * k), idesc_acc,
-                 (s | k) != 0 ? 1u : 0u);
-        tc_commit(bar(B_YEMPTY + st));
-        tc_commit(bar(B_PDEMPTY));
-        if (s + 1 == n_steps) tc_commit(bar(B_ACCFULL));
+          tc_mma(tb + (uint32_t)(128 * w), a_desc + (uint64_t)((k >> 2) * (FA_TILE >> 4) + 2 * (k & 3)),
+                 b_desc + (uint64_t)((k >> 2) * (FA_TILE >> 4) + 2 * (k & 3)), idesc_sd, k != 0 ? 1u : 0u);
+        tc_commit(bar(done));
+        if (free >= 0) tc_commit(bar(free));      // the item's last product with K_j or V_j
       }
       __syncwarp();
+    };
+    // the walked tile again, as a [128 rows (K), 128 columns (N)] operand: two 64-column halves 16 KB apart; 16 rows (8 packed
+    // columns of the A operand) an instruction, the second 64 rows from the second half of the score columns.  k0 = 0, 2: the
+    // first or second 32 rows of each half.
+    auto issue_acc = [&](int w, uint32_t y_off, int k0, bool first) {
+      const uint64_t b_desc = make_smem_desc(sb + y_off, FA_TILE, 1024);
+      if (elect_one()) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int k = (i & 1) + k0 + 4 * (i >> 1);
+          tc_mma_ta(tb + (uint32_t)(256 + 128 * w), tb + (uint32_t)(128 * w + 64 * (k >> 2) + 8 * (k & 3)), b_desc + (uint64_t)(128 * k),
+                    idesc_acc, first && i == 0 ? 0u : 1u);
+        }
+      }
+      __syncwarp();
+    };
+    auto commit = [&](int i) {
+      if (elect_one()) tc_commit(bar(i));
+      __syncwarp();
+    };
+    auto s_prime = [&](int g, bool last) -> bool {      // S' of step g; last: of its item
+      if (!wait(B_QFULL + g % FB_QS, (uint32_t)(g / FB_QS) & 1u)) return false;
+      issue_sd(0, (uint32_t)(FB_Q_OFF + g % FB_QS * FB_TILE), B_SFULL, last ? B_KEMPTY : -1);
+      return true;
+    };
+    auto dp_prime = [&](int g, bool last) -> bool {
+      if (!wait(B_OFULL + g % FB_OS, (uint32_t)(g / FB_OS) & 1u)) return false;
+      issue_sd(1, (uint32_t)(FB_O_OFF + g % FB_OS * FB_TILE), B_DPFULL, last ? B_VEMPTY : -1);
+      return true;
+    };
+    int g = 0;                             // steps so far, of all items
+    int steps = item_of(0).steps;
+    bool ok = wait(B_KFULL, 0u) && s_prime(0, steps == 1) && wait(B_VFULL, 0u) && dp_prime(0, steps == 1);
+    for (int r = 0; ok && steps > 0; ++r) {
+      const int next_steps = item_of(r + 1).steps;
+      const uint32_t item_ph = (uint32_t)r & 1u;
+      for (int s = 0; s < steps; ++s, ++g) {
+        const uint32_t ph = (uint32_t)g & 1u;
+        const bool last = s + 1 == steps, more = !last || next_steps > 0;
+        const bool ends = last ? next_steps == 1 : s + 2 == steps;      // step g + 1 is the last of its item
+        const uint32_t q_off = (uint32_t)(FB_Q_OFF + g % FB_QS * FB_TILE), o_off = (uint32_t)(FB_O_OFF + g % FB_OS * FB_TILE);
+        if (!(ok = wait(B_PHALF, ph) && (s > 0 || r == 0 || wait(B_DVEMPTY, item_ph ^ 1u)))) break;
+        issue_acc(0, o_off, 0, s == 0);
+        if (!(ok = wait(B_PFULL, ph))) break;
+        issue_acc(0, o_off, 2, false);
+        commit(B_OEMPTY + g % FB_OS);
+        if (last) commit(B_DVFULL);
+        if (more && !(ok = (!last || wait(B_KFULL, item_ph ^ 1u)) && s_prime(g + 1, ends))) break;
+        if (!(ok = wait(B_DSFULL, ph) && (s > 0 || r == 0 || wait(B_DKEMPTY, item_ph ^ 1u)))) break;
+        issue_acc(1, q_off, 0, s == 0);
+        issue_acc(1, q_off, 2, false);
+        commit(B_QEMPTY + g % FB_QS);
+        if (last) commit(B_DKFULL);
+        if (more && !(ok = (!last || wait(B_VFULL, item_ph ^ 1u)) && dp_prime(g + 1, ends))) break;
+      }
+      steps = next_steps;
+    }
+    if (!ok) {
+      // an abandoned wait: products issued so far must have finished before the teardown frees what they use
+      commit(B_DRAIN);
+      const long long t0 = clock64();
+      while (!mbar_try_wait(bar(B_DRAIN), 0u) && clock64() - t0 < TC_WAIT_CYCLES) {}
+    }
+    __syncwarp();
+    }
+  } else if (role < 3) {
+    // ------------------------------------------------------------------ P' / dS' (warps 4..11)
+    regs_inc<FB_REGS_SOFTMAX>();
+    const int q = warp & 3;                      // TMEM lane quadrant this warp may access
+    const int hh = role - 1;                     // which 64 of the step's 128 columns
+    const int row = q * 32 + lane;               // own row within the block
+    const uint32_t s_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(64 * hh), d_addr = s_addr + 128u;
+    const float cl = P.scale_log2e, scale = P.scale;
+    bool ok = true;
+    int g = 0;
+    for (int r = 0; ok; ++r) {
+      const Item x = item_of(r);
+      if (x.steps == 0) break;
+      const int edge = row - 64 * hh;            // in the diagonal tile
+      int t = x.blk;
+      for (int s = 0; s < x.steps; ++s, ++g) {
+        const uint32_t ph = (uint32_t)g & 1u;
+        const bool mask = t == x.blk;            // the diagonal tile
+        // the tile's row statistics came with its dO
+        const float4* ld = reinterpret_cast<const float4*>(fb_smem + FB_LD_OFF + (g % FB_OS) * 1024) + 32 * hh;
+        uint32_t p0[32], p1[32], w[16];
+        if (!mbar_wait_warp(bar(B_OFULL + g % FB_OS), (uint32_t)(g / FB_OS) & 1u, abort_flag, P.status)) { ok = false; break; }
+        if (!mbar_wait_warp(bar(B_SFULL), ph, abort_flag, P.status)) { ok = false; break; }
+        tc_fence_after();
+        tmem_ld32(s_addr, p0);
+        tmem_ld32(s_addr + 32, p1);
+        tmem_ld_wait();
+        if (mask) { fb_mask<true>(p0, edge, 0xff800000u); fb_mask<true>(p1, edge - 32, 0xff800000u); }
+        __syncwarp();
+        fb_probs<true>(p0, ld, 0.f, cl, w);
+        tmem_st16(s_addr, w);
+        tmem_st_wait();
+        arrive(B_PHALF);
+        fb_probs<true>(p1, ld + 16, 0.f, cl, w);
+        tmem_st16(s_addr + 16, w);
+        tmem_st_wait();
+        arrive(B_PFULL);
+        if (!mbar_wait_warp(bar(B_DPFULL), ph, abort_flag, P.status)) { ok = false; break; }
+        tc_fence_after();
+        uint32_t rd[32], w1[16];
+        tmem_ld32(d_addr, rd);
+        tmem_ld_wait();
+        if (mask) fb_mask<true>(rd, edge, 0u);      // (their weights are zero, their products may be anything)
+        __syncwarp();
+        fb_dscores<true>(p0, rd, ld, 0.f, scale, w);
+        tmem_ld32(d_addr + 32, rd);
+        tmem_ld_wait();
+        if (mask) fb_mask<true>(rd, edge - 32, 0u);
+        __syncwarp();
+        tmem_st16(d_addr, w);
+        fb_dscores<true>(p1, rd, ld + 16, 0.f, scale, w1);
+        tmem_st16(d_addr + 16, w1);
+        tmem_st_wait();
+        arrive(B_DSFULL);
+        if (lane == 0) mbar_arrive(bar(B_OEMPTY + g % FB_OS));      // the statistics have been read
+        if (++t == n_blk) t = x.blk;
+      }
     }
   } else {
-    // ------------------------------------------------------------------ dS' (warps 2..9)
+    // ------------------------------------------------------------------ output (warps 12..15), beside the next item's steps
+    regs_dec<FB_REGS_OUT>();
     const int q = warp & 3;
-    const int hh = (warp - 2) >> 2;              // which 64 of the tile's 128 keys
-    const int row = q * 32 + lane;
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
-    const float cl = P.scale_log2e, scale = P.scale;
-    const int own_pos = blk * FA_BLK + row;
-    float2 own_ld = make_float2(0.f, 0.f);
-    if (own_pos < P.S) own_ld = P.lse_d[own_row0 + row];
-    __syncwarp();
-    // the owned operands into tensor memory: this thread's 64 columns of its row of Q_i and of dO_i
-#pragma unroll
-    for (int w = 0; w < 2; ++w) {
-      const uint4* src = reinterpret_cast<const uint4*>((w ? P.x1 : P.x0) + (int64_t)(own_row0 + row) * FA_HD + 64 * hh);
-      uint32_t xw[32];
-#pragma unroll
-      for (int g = 0; g < 8; ++g) {
-        const uint4 v = __ldg(src + g);
-        xw[4 * g] = v.x; xw[4 * g + 1] = v.y; xw[4 * g + 2] = v.z; xw[4 * g + 3] = v.w;
+    for (int r = 0;; ++r) {
+      const Item x = item_of(r);
+      if (x.steps == 0) break;
+      const int pos0 = x.blk * FA_BLK + q * 32, rows = min(32, P.S - pos0);
+      const int seq = x.grp / P.heads_own, head = x.grp % P.heads_own;
+      const int64_t tok = (int64_t)seq * P.S + pos0;
+      const uint32_t ph = (uint32_t)r & 1u;
+      bool ok = true;
+#pragma unroll 1
+      for (int a = 0; a < 2; ++a) {          // a = 0: dV as it is, a = 1: dK with the rotation undone
+        if (!(ok = mbar_wait_warp(bar(B_DVFULL + a), ph, abort_flag, P.status))) break;
+        tc_fence_after();
+        const int64_t ld = a ? P.ld_out1 : P.ld_out0;
+        fb_output(lane_addr + (uint32_t)(256 + 128 * a), a ? P.cs + pos0 + lane : nullptr, P.S, lane, rows,
+                  (a ? P.out1 + P.col1 : P.out0 + P.col0) + tok * ld + head * FA_HD, ld, [&]() { arrive(B_DVEMPTY + a); });
       }
-      tmem_st32(lane_addr + (uint32_t)(256 + 64 * w + 32 * hh), xw);
-    }
-    tmem_st_wait();
-    tc_fence_before();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(bar(B_XFULL));
-    bool ok = true;
-    const bool edge = blk * FA_BLK + FA_BLK - 1 >= P.S;
-    for (int s = 0; s < n_steps; ++s) {
-      if (!mbar_wait_warp(bar(B_SDFULL), (uint32_t)s & 1u, abort_flag, P.status)) { ok = false; break; }
-      __syncwarp();
-      tc_fence_after();
-      const bool mask = s == blk || edge;
-      const int col0 = FA_BLK * s + 64 * hh;     // position in the sequence of this thread's first key
-      uint32_t rs[32], rd[32];
-      uint4 pp[4], pa[4], pb[4];
-      tmem_ld32(lane_addr + (uint32_t)(64 * hh), rs);
-      tmem_ld32(lane_addr + (uint32_t)(128 + 64 * hh), rd);
-      tmem_ld_wait();
-      if (mask) fb_tile<false, true>(rs, rd, nullptr, own_ld, cl, scale, col0, own_pos, P.S, pp, pa);
-      else fb_tile<false, false>(rs, rd, nullptr, own_ld, cl, scale, col0, own_pos, P.S, pp, pa);
-      __syncwarp();
-      tmem_ld32(lane_addr + (uint32_t)(64 * hh + 32), rs);
-      tmem_ld32(lane_addr + (uint32_t)(128 + 64 * hh + 32), rd);
-      tmem_ld_wait();
-      // every score of the step is in registers: the buffer may take the next tile's
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(B_SDEMPTY));
-      if (mask) fb_tile<false, true>(rs, rd, nullptr, own_ld, cl, scale, col0 + 32, own_pos, P.S, pp, pb);
-      else fb_tile<false, false>(rs, rd, nullptr, own_ld, cl, scale, col0 + 32, own_pos, P.S, pp, pb);
-      // the operand tile has one buffer: the previous step's accumulating product must have read it
-      if (!mbar_wait_warp(bar(B_PDEMPTY), ((uint32_t)s & 1u) ^ 1u, abort_flag, P.status)) { ok = false; break; }
-      uint8_t* drow = gen_base + FQ_DS_OFF + hh * FA_TILE + row * 128;      // this thread's 64 keys are tile hh
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        *reinterpret_cast<uint4*>(drow + ((g ^ (row & 7)) << 4)) = pa[g];
-        *reinterpret_cast<uint4*>(drow + (((4 + g) ^ (row & 7)) << 4)) = pb[g];
-      }
-      fence_async_smem();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(B_PDFULL));
-    }
-    if (ok) ok = mbar_wait_warp(bar(B_ACCFULL), 0u, abort_flag, P.status);
-    if (ok) {
-      tc_fence_after();
-      // columns [32 hh, +32) and their rotation partners [64 + 32 hh, +32); every lane executes the warp-wide loads
-      const bool row_ok = own_pos < P.S;
-      const int seq = grp / P.heads_own, head = grp % P.heads_own;
-      const int64_t tok = (int64_t)seq * P.S + (row_ok ? own_pos : 0);
-      uint32_t rl[32], rh[32];
-      __syncwarp();
-      tmem_ld32(lane_addr + (uint32_t)(384 + 32 * hh), rl);
-      tmem_ld32(lane_addr + (uint32_t)(384 + 64 + 32 * hh), rh);
-      tmem_ld_wait();
-      if (row_ok) {
-        float y0[32], y1[32];
-        const float2* cs2 = P.cs + (int64_t)(32 * hh) * P.S + own_pos;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const float2 cs = cs2[(int64_t)i * P.S];
-          const float a0 = __uint_as_float(rl[i]), b0 = __uint_as_float(rh[i]);
-          y0[i] = a0 * cs.x + b0 * cs.y;
-          y1[i] = b0 * cs.x - a0 * cs.y;
-        }
-        bf16* dst = P.out1 + tok * P.ld_out1 + P.col1 + head * FA_HD + 32 * hh;
-        store32_bf16(dst, y0);
-        store32_bf16(dst + 64, y1);
-      }
+      if (!ok) break;
     }
   }
 
@@ -985,10 +925,12 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
   tc_fence_before();
   __syncthreads();
   if (*abort_flag && threadIdx.x == 0) {
-    for (int i = 0; i < FQ_NS; ++i) {
+    // loads already issued into this CTA's shared memory must land before the CTA exits
+    for (int i = 0; i < 2 + FB_QS + FB_OS; ++i) {
       if (issued[i] == 0) continue;
-      long long t0 = clock64();
-      while (!mbar_try_wait(bar(B_YFULL + i), (uint32_t)(issued[i] - 1)) && clock64() - t0 < TC_WAIT_CYCLES) {}
+      const int b = i < 2 ? B_KFULL + i : (i < 2 + FB_QS ? B_QFULL + i - 2 : B_OFULL + i - 2 - FB_QS);
+      const long long t0 = clock64();
+      while (!mbar_try_wait(bar(b), (uint32_t)(issued[i] - 1)) && clock64() - t0 < TC_WAIT_CYCLES) {}
     }
   }
   __syncthreads();
@@ -998,27 +940,308 @@ flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap 
   }
 }
 
-// (lse * log2 e, scale * <dO_row, O_row>) per query row; one warp per head-major row.  O is taken before its rounding to
-// bf16: D stands for sum_j P_j dP_j, and with a peaked row dP - D cancels, so an error in D would show in dS.
-__global__ void attn_rowdot_kernel(const float* __restrict__ o32, const bf16* __restrict__ d_o, const float* __restrict__ lse,
-                                   int S, int Sp, int64_t rows, float scale, float2* __restrict__ lse_d) {
-  pdl_sync();
-  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (row >= rows || (int)(row % Sp) >= S) return;
-  const float4 a = *reinterpret_cast<const float4*>(o32 + row * FA_HD + 4 * lane);
-  const uint2 b = *reinterpret_cast<const uint2*>(d_o + row * FA_HD + 4 * lane);
-  const __nv_bfloat162* bh = reinterpret_cast<const __nv_bfloat162*>(&b);
-  const float2 y0 = __bfloat1622float2(bh[0]), y1 = __bfloat1622float2(bh[1]);
-  float dot = a.x * y0.x + a.y * y0.y + a.z * y1.x + a.w * y1.y;
-  dot = warp_sum(dot);
-  if (lane == 0) lse_d[row] = make_float2(lse[row] * 1.4426950408889634f, dot * scale);
+// ---------------------------------------------------------------------------
+// dQ: the owned operands (Q_i, dO_i) sit in tensor memory as A operands (128 columns), S' and dP' take 128 columns each and
+// dQ the last 128.  The score columns are free once they are in registers, so S' of the next step runs under this
+// step's exponentials.  Shared memory: rings of key and value tiles; a key tile is in use from its S' to its dQ, a value
+// tile for one product.  The output warps also bring the next item's owned operands.
+// ---------------------------------------------------------------------------
+constexpr int FQ_KS = 4, FQ_VS = 3;
+constexpr int FQ_V_OFF = FQ_KS * FB_TILE;
+constexpr int FQ_BAR_OFF = FQ_V_OFF + FQ_VS * FB_TILE;
+constexpr int FQ_SMEM_BYTES = FQ_BAR_OFF + 256;
+
+__global__ void __launch_bounds__(FB_THREADS, 1)
+flash_bwd_dq_kernel(const FlashBwdParams P, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v) {
+  extern __shared__ __align__(1024) uint8_t fb_smem[];
+  const uint32_t base = smem_u32(fb_smem);
+  if (base & 1023u) {
+    pdl_wait();
+    set_status(P.status, REVFFN_ERR_CUDA);
+    return;
+  }
+  const uint32_t bars = base + FQ_BAR_OFF;
+  auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
+  // X: the item's own operands, Q_i (0) and dO_i (1): in place, and no product reads them any more
+  enum { B_XFULL = 0, B_XEMPTY = 2, B_KFULL = 4, B_KEMPTY = B_KFULL + FQ_KS, B_VFULL = B_KEMPTY + FQ_KS, B_VEMPTY = B_VFULL + FQ_VS,
+         B_SFULL = B_VEMPTY + FQ_VS, B_SEMPTY, B_DPFULL, B_DSHALF, B_DSFULL, B_ACCFULL, B_ACCEMPTY, B_DRAIN, B_COUNT };
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fb_smem + FQ_BAR_OFF + 8 * B_COUNT);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  int* issued = reinterpret_cast<int*>(tmem_slot + 2);      // [FQ_KS + FQ_VS]: stage -> phase + 1
+  static_assert(8 * B_COUNT + 4 * (2 + FQ_KS + FQ_VS) <= 256, "barrier block");
+
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const int n_blk = P.Sp / FA_BLK;
+  const int per = P.items / n_blk;                       // (sequence, head) pairs
+  // items with high query blocks come first: they see the most key tiles
+  struct Item { int blk, grp, steps; };
+  auto item_of = [&](int r) -> Item {
+    const int it = fb_item(r);
+    Item x;
+    x.blk = n_blk - 1 - it / per; x.grp = it % per;
+    x.steps = it < P.items ? x.blk + 1 : 0;              // key tiles 0 .. the diagonal one
+    return x;
+  };
+
+  if (threadIdx.x == 0) {
+    for (int w = 0; w < 2; ++w) { mbar_init(bar(B_XFULL + w), 4); mbar_init(bar(B_XEMPTY + w), 1); }
+    for (int s = 0; s < FQ_KS; ++s) { mbar_init(bar(B_KFULL + s), 1); mbar_init(bar(B_KEMPTY + s), 1); }
+    for (int s = 0; s < FQ_VS; ++s) { mbar_init(bar(B_VFULL + s), 1); mbar_init(bar(B_VEMPTY + s), 1); }
+    mbar_init(bar(B_SFULL), 1); mbar_init(bar(B_SEMPTY), 8);
+    mbar_init(bar(B_DPFULL), 1); mbar_init(bar(B_DSHALF), 8); mbar_init(bar(B_DSFULL), 8);
+    mbar_init(bar(B_ACCFULL), 1); mbar_init(bar(B_ACCEMPTY), 4); mbar_init(bar(B_DRAIN), 1);
+    for (int i = 0; i < FQ_KS + FQ_VS; ++i) issued[i] = 0;
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  pdl_wait();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  // TMEM columns: S' 0..127, dP' 128..255 (dS' as bf16 pairs at the start of each half of it), Q_i 256..319, dO_i 320..383
+  // (packed pairs), dQ 384..511
+  const uint32_t idesc_sd = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(FA_BLK >> 3) << 17) | ((uint32_t)(FA_BLK >> 4) << 24);
+  const uint32_t idesc_acc = idesc_sd | (1u << 16);
+  const int role = warp >> 2;
+  auto arrive = [&](int i) {
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar(i));
+  };
+
+  if (role == 0) {
+    regs_dec<FB_REGS_ISSUE>();
+    if (warp == 0) {
+    // ------------------------------------------------------------------ producer
+    if (lane == 0) {
+      bool ok = true;
+      int g = 0;
+      for (int r = 0; ok; ++r) {
+        const Item x = item_of(r);
+        if (x.steps == 0) break;
+        const int kv_row0 = (x.grp / P.rep) * P.Sp;
+        for (int s = 0; s < x.steps; ++s, ++g) {
+          const int yr = kv_row0 + s * FA_BLK, sk = g % FQ_KS, sv = g % FQ_VS;
+          const uint32_t phk = (uint32_t)(g / FQ_KS) & 1u, phv = (uint32_t)(g / FQ_VS) & 1u;
+          if (!(ok = mbar_wait(bar(B_KEMPTY + sk), phk ^ 1u, abort_flag, P.status))) break;
+          mbar_expect_tx(bar(B_KFULL + sk), FB_TILE);
+          issued[sk] = (int)phk + 1;
+          for (int kb = 0; kb < 2; ++kb) tma_load_2d(base + sk * FB_TILE + kb * FA_TILE, &map_k, 64 * kb, yr, bar(B_KFULL + sk));
+          if (!(ok = mbar_wait(bar(B_VEMPTY + sv), phv ^ 1u, abort_flag, P.status))) break;
+          mbar_expect_tx(bar(B_VFULL + sv), FB_TILE);
+          issued[FQ_KS + sv] = (int)phv + 1;
+          for (int kb = 0; kb < 2; ++kb) tma_load_2d(base + FQ_V_OFF + sv * FB_TILE + kb * FA_TILE, &map_v, 64 * kb, yr, bar(B_VFULL + sv));
+        }
+      }
+      pdl_trigger();
+    }
+    } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer
+    const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0), sb = __shfl_sync(0xffffffffu, base, 0);
+    auto wait = [&](int i, uint32_t parity) -> bool {
+      const bool got = mbar_wait_warp(bar(i), parity, abort_flag, P.status);
+      tc_fence_after();
+      return got;
+    };
+    // S' = Q_i K_t^T (w = 0), dP' = dO_i V_t^T (w = 1) of step g; last: of its item
+    auto issue_sd = [&](int w, int g, bool last) {
+      const uint64_t b_desc = make_smem_desc(sb + (w ? FQ_V_OFF + g % FQ_VS * FB_TILE : g % FQ_KS * FB_TILE), 16, 1024);
+      if (elect_one()) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          tc_mma_ta(tb + (uint32_t)(128 * w), tb + (uint32_t)(256 + 64 * w + 8 * k),
+                    b_desc + (uint64_t)((k >> 2) * (FA_TILE >> 4) + 2 * (k & 3)), idesc_sd, k != 0 ? 1u : 0u);
+        tc_commit(bar(w ? B_DPFULL : B_SFULL));
+        if (w) tc_commit(bar(B_VEMPTY + g % FQ_VS));
+        if (last) tc_commit(bar(B_XEMPTY + w));
+      }
+      __syncwarp();
+    };
+    auto wait_k = [&](int s) { return wait(B_KFULL + s % FQ_KS, (uint32_t)(s / FQ_KS) & 1u); };
+    auto wait_v = [&](int s) { return wait(B_VFULL + s % FQ_VS, (uint32_t)(s / FQ_VS) & 1u); };
+    int g = 0;                             // steps so far, of all items
+    int steps = item_of(0).steps;
+    bool ok = wait(B_XFULL, 0u) && wait_k(0);
+    if (ok) issue_sd(0, 0, steps == 1);
+    ok = ok && wait(B_XFULL + 1, 0u) && wait_v(0);
+    if (ok) issue_sd(1, 0, steps == 1);
+    for (int r = 0; ok && steps > 0; ++r) {
+      const int next_steps = item_of(r + 1).steps;
+      const uint32_t item_ph = (uint32_t)r & 1u;
+      for (int s = 0; s < steps; ++s, ++g) {
+        const uint32_t ph = (uint32_t)g & 1u;
+        const bool last = s + 1 == steps, more = !last || next_steps > 0;
+        const bool ends = last ? next_steps == 1 : s + 2 == steps;      // step g + 1 is the last of its item
+        if (more) {
+          if (!(ok = (!last || wait(B_XFULL, item_ph ^ 1u)) && wait_k(g + 1) && wait(B_SEMPTY, ph))) break;
+          issue_sd(0, g + 1, ends);
+        }
+        // dQ += dS' K_t, as the halves of dS' become readable: K_t's two 64-column tiles read as one [128 keys, 128 columns]
+        // operand, halves 16 KB apart
+        const uint64_t b_desc = make_smem_desc(sb + g % FQ_KS * FB_TILE, FA_TILE, 1024);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (ok) ok = wait(h ? B_DSFULL : B_DSHALF, ph) && (h > 0 || s > 0 || r == 0 || wait(B_ACCEMPTY, item_ph ^ 1u));
+          if (ok && elect_one()) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int k = (i & 1) + 2 * h + 4 * (i >> 1);
+              tc_mma_ta(tb + 384u, tb + (uint32_t)(128 + 64 * (k >> 2) + 8 * (k & 3)), b_desc + (uint64_t)(128 * k), idesc_acc, (s | h | i) != 0 ? 1u : 0u);
+            }
+            if (h) tc_commit(bar(B_KEMPTY + g % FQ_KS));
+            if (h && last) tc_commit(bar(B_ACCFULL));
+          }
+          __syncwarp();
+        }
+        if (!ok) break;
+        if (more) {
+          if (!(ok = (!last || wait(B_XFULL + 1, item_ph ^ 1u)) && wait_v(g + 1))) break;
+          issue_sd(1, g + 1, ends);
+        }
+      }
+      steps = next_steps;
+    }
+    if (!ok) {
+      // an abandoned wait: products issued so far must have finished before the teardown frees what they use
+      if (elect_one()) tc_commit(bar(B_DRAIN));
+      __syncwarp();
+      const long long t0 = clock64();
+      while (!mbar_try_wait(bar(B_DRAIN), 0u) && clock64() - t0 < TC_WAIT_CYCLES) {}
+    }
+    __syncwarp();
+    }
+  } else if (role < 3) {
+    // ------------------------------------------------------------------ dS' (warps 4..11)
+    regs_inc<FB_REGS_SOFTMAX>();
+    const int q = warp & 3;
+    const int hh = role - 1;                     // which 64 of the tile's 128 keys
+    const int row = q * 32 + lane;
+    const uint32_t s_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(64 * hh), d_addr = s_addr + 128u;
+    const float cl = P.scale_log2e, scale = P.scale;
+    bool ok = true;
+    int g = 0;
+    for (int r = 0; ok; ++r) {
+      const Item x = item_of(r);
+      if (x.steps == 0) break;
+      const int64_t at = (int64_t)x.grp * P.Sp + x.blk * FA_BLK + row;
+      const float* const stats = reinterpret_cast<const float*>(P.lse_d + (at >> 1)) + (at & 1);
+      const float nl = stats[0], nd = stats[2];
+      const int edge = row - 64 * hh;            // in the diagonal tile
+      for (int s = 0; s < x.steps; ++s, ++g) {
+        const uint32_t ph = (uint32_t)g & 1u;
+        const bool mask = s == x.blk;
+        uint32_t p0[32], p1[32], w[16], w1[16], rd[32];
+        if (!mbar_wait_warp(bar(B_SFULL), ph, abort_flag, P.status)) { ok = false; break; }
+        tc_fence_after();
+        tmem_ld32(s_addr, p0);
+        tmem_ld32(s_addr + 32, p1);
+        tmem_ld_wait();
+        arrive(B_SEMPTY);
+        if (mask) { fb_mask<false>(p0, edge, 0xff800000u); fb_mask<false>(p1, edge - 32, 0xff800000u); }
+        __syncwarp();
+        fb_probs<false>(p0, nullptr, nl, cl, w);
+        fb_probs<false>(p1, nullptr, nl, cl, w);
+        if (!mbar_wait_warp(bar(B_DPFULL), ph, abort_flag, P.status)) { ok = false; break; }
+        tc_fence_after();
+        tmem_ld32(d_addr, rd);
+        tmem_ld_wait();
+        if (mask) fb_mask<false>(rd, edge, 0u);
+        __syncwarp();
+        fb_dscores<false>(p0, rd, nullptr, nd, scale, w);
+        tmem_ld32(d_addr + 32, rd);
+        tmem_ld_wait();
+        if (mask) fb_mask<false>(rd, edge - 32, 0u);
+        __syncwarp();
+        tmem_st16(d_addr, w);
+        tmem_st_wait();
+        arrive(B_DSHALF);
+        fb_dscores<false>(p1, rd, nullptr, nd, scale, w1);
+        tmem_st16(d_addr + 16, w1);
+        tmem_st_wait();
+        arrive(B_DSFULL);
+      }
+    }
+  } else {
+    // ------------------------------------------------------------------ owned operands and output (warps 12..15)
+    regs_dec<FB_REGS_OUT>();
+    const int q = warp & 3;
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+    // this thread's row of Q_i (w = 0) or dO_i (w = 1) of item x into tensor memory, once the item before is done with it
+    auto own = [&](int w, int r, const Item& x) -> bool {
+      // eight rows of 64 bytes an instruction, then four pieces of one row to each lane
+      const uint4* src = reinterpret_cast<const uint4*>((w ? P.x1 : P.x0) + (int64_t)(x.grp * P.Sp + x.blk * FA_BLK + q * 32 + (lane & ~3)) * FA_HD) + (lane & 3);
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        uint4 v[2][4];
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) v[c][k] = __ldg(src + k * (FA_HD / 8) + 8 * half + 4 * c);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) quad_transpose(v[c], lane);
+        if (half == 0) {
+          if (!mbar_wait_warp(bar(B_XEMPTY + w), ((uint32_t)r & 1u) ^ 1u, abort_flag, P.status)) return false;
+          tc_fence_after();
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          uint32_t x16[16];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) { x16[4 * k] = v[c][k].x; x16[4 * k + 1] = v[c][k].y; x16[4 * k + 2] = v[c][k].z; x16[4 * k + 3] = v[c][k].w; }
+          tmem_st16(lane_addr + (uint32_t)(256 + 64 * w + 32 * half + 16 * c), x16);
+        }
+      }
+      tmem_st_wait();
+      arrive(B_XFULL + w);
+      return true;
+    };
+    Item x = {0, 0, 0};
+    bool ok = true;
+    for (int r = -1; ok; ++r) {
+      const Item nx = item_of(r + 1);
+#pragma unroll 1
+      for (int w = 0; ok && w < 2 && nx.steps > 0; ++w) ok = own(w, r + 1, nx);
+      if (!ok) break;
+      if (r < 0) { x = nx; if (x.steps == 0) break; continue; }
+      const int pos0 = x.blk * FA_BLK + q * 32, rows = min(32, P.S - pos0);
+      const int seq = x.grp / P.heads_own, head = x.grp % P.heads_own;
+      const int64_t tok = (int64_t)seq * P.S + pos0;
+      if (!(ok = mbar_wait_warp(bar(B_ACCFULL), (uint32_t)r & 1u, abort_flag, P.status))) break;
+      tc_fence_after();
+      fb_output(lane_addr + 384u, P.cs + pos0 + lane, P.S, lane, rows, P.out1 + tok * P.ld_out1 + P.col1 + head * FA_HD, P.ld_out1, [&]() { arrive(B_ACCEMPTY); });
+      x = nx;
+      if (x.steps == 0) break;
+    }
+  }
+
+  // ------------------------------------------------------------------ teardown
+  tc_fence_before();
+  __syncthreads();
+  if (*abort_flag && threadIdx.x == 0) {
+    for (int i = 0; i < FQ_KS + FQ_VS; ++i) {
+      if (issued[i] == 0) continue;
+      const long long t0 = clock64();
+      while (!mbar_try_wait(bar(i < FQ_KS ? B_KFULL + i : B_VFULL + i - FQ_KS), (uint32_t)(issued[i] - 1)) && clock64() - t0 < TC_WAIT_CYCLES) {}
+    }
+  }
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+  }
 }
 
 // q, d_o: [B * n_heads * Sp, 128]; k, v: [B * n_kv_heads * Sp, 128] bf16 head-major (rows past the sequence zero).
 // Outputs token-major bf16, rotation undone: dq [T, ld_dq]; dk at column 0 and dv at column dv_col of dkv [T, ld_dkv].
 // The two launches depend on nothing of each other: st_dkv and st_dq may be different streams.
-inline int launch_flash_bwd(const bf16* q, const bf16* k, const bf16* v, const bf16* d_o, const float2* lse_d, const float2* cs,
+inline int launch_flash_bwd(const bf16* q, const bf16* k, const bf16* v, const bf16* d_o, const float* lse_d, const float2* cs,
                             int batch, int n_heads, int n_kv_heads, int S, int Sp, bf16* dq, int64_t ld_dq, bf16* dkv,
                             int64_t ld_dkv, int dv_col, int* status, cudaStream_t st_dkv, cudaStream_t st_dq) {
   TcState& s = tc_state();
@@ -1034,16 +1257,16 @@ inline int launch_flash_bwd(const bf16* q, const bf16* k, const bf16* v, const b
     attr_set[dev] = true;
   }
   const uint64_t q_rows = (uint64_t)batch * n_heads * Sp, kv_rows = (uint64_t)batch * n_kv_heads * Sp;
-  CUtensorMap k128, v128, q64, do64;
+  CUtensorMap k128, v128, q128, do128;
   int r = 0;
   if (!r) r = tc_make_map(&k128, k, FA_HD, kv_rows, FA_HD, 64, 128);
   if (!r) r = tc_make_map(&v128, v, FA_HD, kv_rows, FA_HD, 64, 128);
-  if (!r) r = tc_make_map(&q64, q, FA_HD, q_rows, FA_HD, 64, 64);
-  if (!r) r = tc_make_map(&do64, d_o, FA_HD, q_rows, FA_HD, 64, 64);
+  if (!r) r = tc_make_map(&q128, q, FA_HD, q_rows, FA_HD, 64, 128);
+  if (!r) r = tc_make_map(&do128, d_o, FA_HD, q_rows, FA_HD, 64, 128);
   if (r) return r;
   FlashBwdParams P;
   P.S = S; P.Sp = Sp; P.n_heads = n_heads; P.rep = n_heads / n_kv_heads;
-  P.lse_d = lse_d;
+  P.lse_d = reinterpret_cast<const float4*>(lse_d);
   P.scale = 1.f / sqrtf((float)FA_HD);
   P.scale_log2e = P.scale * 1.4426950408889634f;
   P.status = status;
@@ -1052,13 +1275,15 @@ inline int launch_flash_bwd(const bf16* q, const bf16* k, const bf16* v, const b
   P.out1 = dkv; P.ld_out1 = ld_dkv; P.col1 = 0;
   P.heads_own = n_kv_heads;
   P.x0 = nullptr; P.x1 = nullptr;
-  launch_k(flash_bwd_dkv_kernel, batch * n_kv_heads * (Sp / FA_BLK), FA_THREADS, FB_SMEM_BYTES, st_dkv, P, k128, v128, q64, do64);
+  P.items = batch * n_kv_heads * (Sp / FA_BLK);
+  launch_k(flash_bwd_dkv_kernel, std::min(P.items, s.n_sms), FB_THREADS, FB_SMEM_BYTES, st_dkv, P, k128, v128, q128, do128);
   if (cudaGetLastError() != cudaSuccess) return REVFFN_ERR_CUDA;
   P.out0 = nullptr; P.ld_out0 = 0; P.col0 = 0;
   P.out1 = dq; P.ld_out1 = ld_dq; P.col1 = 0;
   P.heads_own = n_heads;
   P.x0 = q; P.x1 = d_o;
-  launch_k(flash_bwd_dq_kernel, batch * n_heads * (Sp / FA_BLK), FA_THREADS, FQ_SMEM_BYTES, st_dq, P, k128, v128);
+  P.items = batch * n_heads * (Sp / FA_BLK);
+  launch_k(flash_bwd_dq_kernel, std::min(P.items, s.n_sms), FB_THREADS, FQ_SMEM_BYTES, st_dq, P, k128, v128);
   return cudaGetLastError() == cudaSuccess ? REVFFN_OK : REVFFN_ERR_CUDA;
 }
 

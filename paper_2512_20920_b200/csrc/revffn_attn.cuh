@@ -15,7 +15,7 @@
 namespace revffn {
 
 struct AttnLayout {
-  Buf status, rows_total, tile_group, group_off, cs, cs_t, n12, r12, u12, raw, qh, kh, vh, lse, sc, p, oh, o, a;
+  Buf status, rows_total, tile_group, group_off, cs, cs_t, n12, r12, u12, raw, qh, kh, vh, sc, p, oh, o, a;
   size_t fwd_bytes = 0;
   Buf dyb, da, dob, doh, ds, dqh, dkh, dvh, dq, dkv, du12, dn12, part, npart, lse_d;
   size_t bwd_bytes = 0;
@@ -52,7 +52,6 @@ static AttnLayout plan_attn(const revffn_attn_desc& D) {
   take(L.qh, (size_t)L.rows * hd * ts);
   take(L.kh, (size_t)L.kv_rows * hd * ts);
   take(L.vh, (size_t)L.kv_rows * hd * ts);
-  take(L.lse, (size_t)L.rows * 4);
   take(L.sc, (size_t)L.rows * Sp * 4);
   take(L.p, (size_t)L.rows * Sp * ts);
   take(L.oh, (size_t)L.rows * hd * ts);
@@ -262,7 +261,7 @@ static GemmProblem a_grouped_rows(const ACtx<T>& c) {
 // O (token-major) from the head-major q, k, v.  need_p: the backward pass reads P afterwards, so the score
 // matrix is materialised; otherwise the tcgen05 back end runs the attention core as one kernel.
 template <typename T>
-static int a_core(const ACtx<T>& c, bool need_p, bool keep_o32 = false) {
+static int a_core(const ACtx<T>& c, bool need_p, bool grad = false) {
   const revffn_attn_desc& D = c.D;
   const AttnLayout& L = c.L;
   if constexpr (std::is_same<T, bf16>::value) {
@@ -270,7 +269,7 @@ static int a_core(const ACtx<T>& c, bool need_p, bool keep_o32 = false) {
       ProfScope ps(TG_A_FLASH, c.st);
       return launch_flash_fwd(c.template p<bf16>(L.qh), c.template p<bf16>(L.kh), c.template p<bf16>(L.vh), D.batch,
                               D.n_heads, D.n_kv_heads, D.seq_len, L.Sp, c.template p<bf16>(L.o), D.d_model,
-                              c.template p<float>(L.lse), keep_o32 ? c.template p<float>(L.sc) : nullptr,
+                              grad ? c.template p<bf16>(L.doh) : nullptr, grad ? c.template p<float>(L.lse_d) : nullptr,
                               c.status, c.st);
     }
   }
@@ -461,22 +460,17 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
   }
   if (!reuse_kv) CKR(a_kv_side(c, x2));
   CKR(a_query(c, x1));
-  CKR(a_core(c, !fused, fused));        // fused: the score buffer holds the unrounded output instead
-  CKR(c.order(cs.st, st));
+  CKR(c.order(cs.st, st));              // the fused core reads dO: it leaves the rows' statistics for the two kernels below
+  CKR(a_core(c, !fused, fused));
 
   // attention core backward
   if (fused) {
     if constexpr (std::is_same<T, bf16>::value) {
-      { ProfScope ps(TG_A_SOFTMAX, st);
-      CK(launch_k(attn_rowdot_kernel, (unsigned)ceil_div(L.rows * 32, 256), 256, 0, st, c.template p<float>(L.sc),
-                  c.template p<bf16>(L.doh), c.template p<float>(L.lse), D.seq_len, Sp, L.rows, 1.f / sqrtf((float)hd),
-                  c.template p<float2>(L.lse_d)));
-      }
       CKR(c.order(st, cs.st));
       { ProfScope ps(TG_A_FLASH, st);
       // the two launches also undo the rotation and write dq and dk|dv token-major in the operand type
       CKR(launch_flash_bwd(c.template p<bf16>(L.qh), c.template p<bf16>(L.kh), c.template p<bf16>(L.vh),
-                           c.template p<bf16>(L.doh), c.template p<float2>(L.lse_d), c.template p<float2>(L.cs_t), D.batch,
+                           c.template p<bf16>(L.doh), c.template p<float>(L.lse_d), c.template p<float2>(L.cs_t), D.batch,
                            D.n_heads, D.n_kv_heads, D.seq_len, Sp, c.template p<bf16>(L.dq), d, c.template p<bf16>(L.dkv),
                            2 * (int64_t)dkv, dkv, c.status, st, cs.st));
       ++g_prof.launches;
