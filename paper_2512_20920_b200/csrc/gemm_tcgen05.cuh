@@ -700,8 +700,10 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
             }
           }
           if (lb) {
-            const bool second = p.concat == CONCAT_K && kb >= k_half;
+            bool second = p.concat == CONCAT_K && kb >= k_half;
             const int kbp = second ? kb - k_half : kb;
+            int b_row = t.n0 + nhalf * crank;
+            if (EPI == EPI_HEADS && p.hm_split && t.n0 >= p.hm_split) { second = true; b_row -= p.hm_split; }
             if (!p.b_mn_major) {
               // this CTA's half of the accumulator columns: gate rows (rank 0) or up rows (rank 1) of a
               // SwiGLU pair, else rows n0 + nhalf rank .. of B
@@ -710,9 +712,9 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
                 if (crank == 0) tma_load_2d_pair(sb, &map_b0, kbp * TC_BK, t.n0, fbc);
                 else tma_load_2d_pair(sb, &map_b1, kbp * TC_BK, t.n0, fbc);
               } else if (second) {
-                tma_load_2d_pair(sb, &map_b1, kbp * TC_BK, t.n0 + nhalf * crank, fbc);
+                tma_load_2d_pair(sb, &map_b1, kbp * TC_BK, b_row, fbc);
               } else {
-                tma_load_2d_pair(sb, &map_b0, kbp * TC_BK, t.n0 + nhalf * crank, fbc);
+                tma_load_2d_pair(sb, &map_b0, kbp * TC_BK, b_row, fbc);
               }
             } else {
               const int krow = t.krow0 + kbp * TC_BK;
@@ -761,6 +763,8 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           if (!p.b_mn_major) {
             // rows of the flattened [groups * N, K] weight tensor
             int row0 = (p.group_mode == GROUP_M ? t.group * p.N : 0) + t.n0;
+            bool second = p.concat == CONCAT_K && kb >= k_half;
+            if (EPI == EPI_HEADS && p.hm_split && t.n0 >= p.hm_split) { second = true; row0 -= p.hm_split; }
             if (p.concat == CONCAT_N) {
               tma_load_2d(sb, &map_b0, kb_b * P.bk, row0, fb);
               tma_load_2d(sb + P.tile_n * 128, &map_b1, kb_b * P.bk, row0, fb);
@@ -1315,23 +1319,25 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
         // 64-byte pieces of the row's place in the head-major tensor.
         uint32_t r1[32];
         const int seq = m_ok ? m / p.hm_S : 0, pos = m_ok ? m % p.hm_S : 0;
-        const int n_heads = p.N / 128;
+        const bool other = p.hm_split && t.n0 >= p.hm_split;      // the second matrix
+        const int n_heads = (!p.hm_split ? p.N : (other ? p.N - p.hm_split : p.hm_split)) / 128;
+        const float* const bias = other ? p.hm_bias1 : p.hm_bias;
         const int64_t row_at = ((int64_t)seq * n_heads * p.hm_Sp + pos) * 128;      // this lane's row, head 0
 #pragma unroll 1
         for (int c = half * 32; c < t.ncols; c += 128) {
           if (!slab_ok) continue;      // warp-uniform
-          const int n = t.n0 + c;      // first column of the lower half-range; n + 64 is its partner
+          const int n = t.n0 + c - (other ? p.hm_split : 0);      // first column of the lower half-range; n + 64 is its partner
           tmem_ld32(taddr + c, r0);
           tmem_ld32(taddr + c + 64, r1);
           tmem_ld_wait();
           const int head = n / 128, i0 = n % 128;            // i0 is 0 or 32
-          bf16* dst = reinterpret_cast<bf16*>(p.C) + (int64_t)head * p.hm_Sp * 128 + i0;
+          bf16* dst = reinterpret_cast<bf16*>(other ? p.C1 : p.C) + (int64_t)head * p.hm_Sp * 128 + i0;
           float y0[32], y1[32];
 #pragma unroll
           for (int i = 0; i < 32; ++i) { y0[i] = __uint_as_float(r0[i]); y1[i] = __uint_as_float(r1[i]); }
-          if (p.hm_bias) {
-            const float4* b0 = reinterpret_cast<const float4*>(p.hm_bias + n);        // the same for every lane
-            const float4* b1 = reinterpret_cast<const float4*>(p.hm_bias + n + 64);
+          if (bias) {
+            const float4* b0 = reinterpret_cast<const float4*>(bias + n);        // the same for every lane
+            const float4* b1 = reinterpret_cast<const float4*>(bias + n + 64);
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
               const float4 u = b0[i], v = b1[i];
@@ -1339,7 +1345,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
               y1[4 * i] += v.x; y1[4 * i + 1] += v.y; y1[4 * i + 2] += v.z; y1[4 * i + 3] += v.w;
             }
           }
-          if (p.hm_cs) {
+          if (p.hm_cs && !other) {
             // the table is [pair, position]: the lanes' positions are neighbours
             const float2* cs2 = p.hm_cs + (int64_t)i0 * p.hm_S + pos;
 #pragma unroll
@@ -1810,7 +1816,7 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   // is 4-5 % faster and no product is slower (the one-thread form stays selectable for such measurements).
   P.split_loads = p.dbg_split_loads != 2;
   if (p.dbg_starve && !p.no_pair) return REVFFN_ERR_UNSUPPORTED;      // the starved-wait test runs one CTA per tile
-  if (p.N % 128 != 0) return REVFFN_ERR_SHAPE;
+  if (p.N % 128 != 0 || (p.hm_split && p.epilogue != EPI_HEADS)) return REVFFN_ERR_SHAPE;
   // K need not be a multiple of the 64-wide K step: the tensor maps end at K, so the rest of the last
   // step is loaded as zeros (K-major rows must still start on 16-byte boundaries: lda, ldb)
   if (p.concat == CONCAT_K && (P.k_blocks & 1)) return REVFFN_ERR_SHAPE;
@@ -1838,10 +1844,10 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
     }
     // B
     if (!p.b_mn_major) {
-      uint64_t rows = (p.group_mode == GROUP_M) ? (uint64_t)groups * p.N : (uint64_t)p.N;
-      int r = tc_make_map(&mb0, p.B0, (uint64_t)k_half, rows, (uint64_t)p.ldb, f8 ? 128 : 64, tr ? 128 : P.b_box, f8);
+      const uint64_t rows = (p.group_mode == GROUP_M) ? (uint64_t)groups * p.N : (uint64_t)p.N;
+      int r = tc_make_map(&mb0, p.B0, (uint64_t)k_half, p.hm_split ? p.hm_split : rows, (uint64_t)p.ldb, f8 ? 128 : 64, tr ? 128 : P.b_box, f8);
       if (r) return r;
-      r = tc_make_map(&mb1, p.B1 ? p.B1 : p.B0, (uint64_t)k_half, rows, (uint64_t)p.ldb, f8 ? 128 : 64, tr ? 128 : P.b_box, f8);
+      r = tc_make_map(&mb1, p.B1 ? p.B1 : p.B0, (uint64_t)k_half, rows - p.hm_split, (uint64_t)p.ldb, f8 ? 128 : 64, tr ? 128 : P.b_box, f8);
       if (r) return r;
     } else {
       uint64_t rows = (p.group_mode == GROUP_M) ? (uint64_t)groups * k_half : (uint64_t)p.K;
@@ -1868,6 +1874,9 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   if (p.epilogue == EPI_HEADS) {
     // plain stores into the head-major tensor, no output map
     if (p.group_mode != 0 || p.N % 128 != 0 || p.hm_S <= 0 || p.hm_Sp < p.hm_S || (reinterpret_cast<uintptr_t>(p.C) & 15u))
+      return REVFFN_ERR_SHAPE;
+    if (p.hm_split && (p.hm_split < 0 || p.hm_split >= p.N || p.hm_split % 256 != 0 || p.b_mn_major || p.concat != CONCAT_NONE || !p.B1 ||
+                       !p.C1 || (reinterpret_cast<uintptr_t>(p.C1) & 15u)))
       return REVFFN_ERR_SHAPE;
   } else if (p.epilogue == EPI_DSWIGLU) {
     // a|b are read and rewritten in place with plain 16-byte accesses, no tensor map
