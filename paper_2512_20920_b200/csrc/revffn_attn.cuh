@@ -427,8 +427,10 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
   cudaStream_t st = c.st;
   const ACtx<T> cs = c.on_side();
 
+  // out2: second output of a product whose M is two stacked gradients.  Gradients of few tiles are split over K as in the MoE
+  // branch; the partial sums take the score matrix's place, which the fused core does not write, where they fit in it.
   auto wgrad = [&](const ACtx<T>& on, float* out, int M, int N, const void* A, int64_t lda, int a_col0, const void* B, int64_t ldb,
-                   int K) -> int {
+                   int K, float* out2 = nullptr) -> int {
     GemmProblem p = blank_problem();
     p.M = M; p.N = N; p.K = K;
     p.a_mn_major = 1; p.b_mn_major = 1;
@@ -436,7 +438,20 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
     p.B0 = B; p.ldb = ldb;
     p.epilogue = EPI_WGRAD; p.accumulate = acc;
     p.C = out; p.ldc = N;
-    return a_gemm(on, p, TG_A_WGRAD);
+    if (out2) { p.C2 = out2; p.split_m = M / 2; }
+    int n_split = 1;
+    if constexpr (std::is_same<T, bf16>::value) {
+      if (on.fused()) n_split = wgrad_splits(M, N, K, L.sc.bytes);
+    }
+    if (n_split <= 1) return a_gemm(on, p, TG_A_WGRAD);
+    const int64_t count = (int64_t)M * N;
+    p.group_mode = GROUP_K; p.n_groups = n_split;
+    p.C = on.template p<float>(L.sc); p.C2 = nullptr; p.split_m = 0; p.c_group_stride = count; p.accumulate = 0;
+    CKR(a_gemm(on, p, TG_A_WGRAD));
+    ProfScope ps(TG_A_WGRAD, on.st);
+    CK(launch_k(splitk_reduce_kernel<T>, (unsigned)ceil_div(count, 4 * 256), 256, 0, on.st, on.template p<float>(L.sc), n_split, count, out,
+                out2, out2 ? count / 2 : count, acc, nullptr, nullptr, UpdRule{}, nullptr, nullptr));
+    return REVFFN_OK;
   };
   auto dgrad = [&](const ACtx<T>& on, int tag, int M, int N, int K, const void* A, int64_t lda, const void* W, int64_t ldw, void* C,
                    bool f32) -> int {
@@ -568,8 +583,13 @@ static int a_backward(const ACtx<T>& c, const float* x1, const float* x2, const 
   }
   if (G.w_o) CKR(wgrad(cs, G.w_o, d, d, c.template p<T>(L.da), d, 0, c.template p<T>(L.o), d, Tn));
   if (G.w_q) CKR(wgrad(cs, G.w_q, d, d, c.template p<T>(L.dq), d, 0, u1, d, Tn));
-  if (G.w_k) CKR(wgrad(cs, G.w_k, dkv, d, c.template p<T>(L.dkv), 2 * (int64_t)dkv, 0, u2, d, Tn));
-  if (G.w_v) CKR(wgrad(cs, G.w_v, dkv, d, c.template p<T>(L.dkv), 2 * (int64_t)dkv, dkv, u2, d, Tn));
+  // dk | dv is one buffer and both gradients read u2: one product where both are wanted (on the CUDA cores it has one output)
+  if (G.w_k && G.w_v && c.tc) {
+    CKR(wgrad(cs, G.w_k, 2 * dkv, d, c.template p<T>(L.dkv), 2 * (int64_t)dkv, 0, u2, d, Tn, G.w_v));
+  } else {
+    if (G.w_k) CKR(wgrad(cs, G.w_k, dkv, d, c.template p<T>(L.dkv), 2 * (int64_t)dkv, 0, u2, d, Tn));
+    if (G.w_v) CKR(wgrad(cs, G.w_v, dkv, d, c.template p<T>(L.dkv), 2 * (int64_t)dkv, dkv, u2, d, Tn));
+  }
   {
     ColSegs<T> s;
     int n = 0, cols = 0;

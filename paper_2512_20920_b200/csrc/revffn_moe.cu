@@ -453,6 +453,16 @@ static GemmProblem blank_problem() {
   return p;
 }
 
+// A dense weight gradient with few output tiles (the adapters': 32 tiles of 256 x 256) leaves most of the GPU
+// idle while every tile walks all K tokens.  Split K over the tokens into as many slices as fill the GPU, write
+// the partial results to a scratch of `room` bytes and add them in a second, fixed-order pass, which also does what the
+// epilogue would have done (store, accumulate or the fused update).
+static int wgrad_splits(int M, int N, int K, size_t room) {
+  const int64_t tiles = ceil_div(M, 2 * TC_BM) * ceil_div(N, 256);
+  const int n = (int)std::min<int64_t>(SPLIT_K_MAX, tc_state().n_sms / 2 / (tiles > 0 ? tiles : 1));
+  return (size_t)n * M * N * 4 > room || K < 64 * 8 * n || (M * (int64_t)N) % 4 != 0 || M % TC_BM != 0 ? 1 : n;
+}
+
 // ---------------------------------------------------------------------------
 // F = MLP(Norm(Y1)) up to z (the input of P_down).  save_ab keeps the SwiGLU
 // pre-activations for the backward pass.
@@ -817,18 +827,9 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
       p.group_off = c.template p<int32_t>(L.expert_off);
       p.group_cnt = c.template p<int32_t>(L.expert_cnt);
     }
-    // A dense weight gradient with few output tiles (the adapters': 32 tiles of 256 x 256) leaves most of the GPU
-    // idle while every tile walks all T tokens.  Split K over the tokens into as many slices as fill the GPU, write
-    // the partial results to the workspace and add them in a second, fixed-order pass, which also does what the
-    // epilogue would have done (store, accumulate or the fused update).
     int n_split = 1;
     if constexpr (std::is_same<T, bf16>::value) {
-      if (c.tc && !grouped && !p.split_m) {
-        const int64_t tiles = ceil_div(M, 2 * TC_BM) * ceil_div(N, 256);
-        const int pairs = tc_state().n_sms / 2;
-        n_split = (int)std::min<int64_t>(SPLIT_K_MAX, pairs / (tiles > 0 ? tiles : 1));
-        if ((size_t)n_split * M * N * 4 > L.ksplit.bytes || Tn < 64 * 8 * n_split || (M * (int64_t)N) % 4 != 0 || M % TC_BM != 0) n_split = 1;
-      }
+      if (c.tc && !grouped && !p.split_m) n_split = wgrad_splits(M, N, Tn, L.ksplit.bytes);
     }
     if (n_split <= 1) return run_gemm(cw, p, tag);
     p.group_mode = GROUP_K; p.n_groups = n_split; p.group_off = nullptr;
@@ -839,7 +840,7 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
       ProfScope ps(tag, cw.st);
       const int64_t count = (int64_t)M * N;
       launch_k(splitk_reduce_kernel<T>, (unsigned)ceil_div(count, 4 * 256), 256, 0, cw.st, 
-          c.template p<float>(L.ksplit), n_split, count, out, acc, upd ? reinterpret_cast<T*>(const_cast<void*>(W)) : nullptr,
+          c.template p<float>(L.ksplit), n_split, count, out, nullptr, count, acc, upd ? reinterpret_cast<T*>(const_cast<void*>(W)) : nullptr,
           upd ? master : nullptr, upd ? sgd->rule : UpdRule{}, upd ? sgd->mom[wi] : nullptr, upd ? sgd->var[wi] : nullptr);
     }
     CK(cudaGetLastError());

@@ -1,5 +1,6 @@
 """Gradients of the attention branch where its kernels and products are cut: more items than blocks (a block then walks several,
-the next one's first products under this one's output), keys and values as one product or as two.  Against the oracle at the path's stated 2e-2."""
+the next one's first products under this one's output), keys and values as one product or as two,
+weight gradients split over K.  Against the oracle at the path's stated 2e-2."""
 import numpy as np
 import pytest
 import torch
@@ -19,6 +20,7 @@ F32 = ("norm_gamma", "b_q", "b_k", "b_v")
     (5, 1000, 512, 4, 4),        # 160 of each, of 1 to 8 steps
     (2, 150, 384, 3, 3),         # three key/value heads: two products
     (2, 150, 256, 2, 2),         # two: one product of one tile per matrix
+    (3, 700, 512, 4, 2),         # 2100 tokens: gradients in four slices of K, keys' and values' in one product
 ])
 def test_gradients(batch, seq_len, d_model, n_heads, n_kv_heads):
     import paper_2512_20920_b200 as rv
