@@ -1,10 +1,10 @@
 // tcgen05 / TMEM / TMA back end for every bf16 matrix product on the path.
 //
-// One persistent, warp-specialised kernel (1 CTA per SM, 352 threads):
+// One warp-specialised kernel (1 CTA per SM, 384 threads; a CTA works tiles until there are none, see warp 11):
 //   warps 0, 10 TMA producers: cp.async.bulk.tensor loads (128-byte swizzle) of
 //               A and B tiles into a ring of shared-memory stages, completion on
-//               mbarriers (no multicast LOADS anywhere: every CTA fetches its own operands; the only
-//               cluster-wide instruction is the pair mode's tcgen05.commit, a barrier arrive).  Warp 0
+//               mbarriers (no multicast LOADS anywhere: every CTA fetches its own operands; cluster-wide
+//               are only the pair mode's tcgen05.commit, a barrier arrive, and the answer of warp 11's request).  Warp 0
 //               announces a stage's bytes and loads the first operand's share, warp 10 loads the second
 //               operand's: one warp cannot issue a stage's loads as fast as the tensor core consumes them.
 //   warp 1      MMA issuer: owns the TMEM allocation (two accumulators, so the
@@ -20,6 +20,9 @@
 //               (64-byte swizzle), fp32 blocks are transposed there and written with plain
 //               16-byte stores, four 128-byte rows per instruction.  Global writes are whole
 //               lines whatever the row stride.
+//   warp 11     tiles: describes the CTA's (pair's) next tile to the other warps and asks the hardware for the tile after it
+//               (cluster launch control: the grid has a CTA or pair per tile, and a running one takes over the
+//               place of one that has not been launched yet).
 // Tile = 128 rows x 256 columns (the last column tile of a row may be 128 wide: N only has
 // to be a multiple of 128), K step 64 (one 128-byte swizzle atom of bf16).  Products that would leave SMs idle with
 // it take tiles of 128 or 64 columns, as tc_plan() reckons.
@@ -58,8 +61,10 @@ namespace revffn {
 
 constexpr int TC_BM = 128;
 constexpr int TC_BK = 64;
-constexpr int TC_THREADS = 352;      // warp 0, 10: operand loads; warp 1: products; warps 2..9: epilogue
+constexpr int TC_THREADS = 384;      // warp 0, 10: operand loads; warp 1: products; warps 2..9: epilogue; warp 11: tiles
 constexpr int TC_LOAD_WARP_B = 10;   // the second load warp
+constexpr int TC_TILE_WARP = 11;     // hands out the tiles
+constexpr int TC_TILE_SLOTS = 4;     // tiles described ahead: the loads are up to two tiles ahead of the epilogue
 constexpr int TC_EPI_WARPS = 8;
 constexpr int TR_SMALL = 64;            // transposed: halves of a token chunk up to here come in 32-row boxes (experts of 4 rows: 66.7 -> 64.3 us)
 constexpr int TC_A_BYTES = TC_BM * TC_BK * 2;            // 16 KB
@@ -78,7 +83,7 @@ template <int MMA_N, int EPI, bool PAIR> struct TcCfg {
   // every stage is a multiple of 1024 bytes, so the staging area is aligned too
   static constexpr int EPI_OFF = STAGES * STAGE_BYTES;
   static constexpr int BAR_OFF = EPI_OFF + TC_EPI_WARPS * EPI_WARP_BYTES;
-  static constexpr int SMEM_BYTES = BAR_OFF + 1024 /*align*/ + 512 /*barriers*/;
+  static constexpr int SMEM_BYTES = BAR_OFF + 1024 /*align*/ + 768 /*barriers, tile descriptions*/;
 };
 
 struct TcParams {
@@ -485,76 +490,39 @@ __device__ __forceinline__ void upd_half(const UpdRule& rule, const SlabOut& o, 
   }
 }
 
-// Tile coordinates shared by the three roles.
-struct TcTile {
+// A tile as its roles see it: 32 bytes, described by the tile warp.
+struct alignas(16) TcTile {
   int m0, n0, group, k_blocks, krow0;
   int ncols;      // accumulator columns in use: the tile's, or 128 in the last column tile of an odd multiple of 128
   int pad;        // tr: rows of zero padding after the chunk's, to the next multiple of 64 (an expert's last chunk only)
+  int valid;      // 0: no tile, the last one is done
 };
 
-// A role's walk over the tiles w0, w0 + stride, ...: the tile's index split into its parts, and the table entries that the
-// rest of its description comes from.  step() moves on by additions and asks for the next tile's entries; tc_tile() looks
-// at them when the role begins that tile, the loads are then long done.  Divided and looked up when needed, each of the
-// three roles spent 1200-2000 clk per tile on this, the tensor core idle for most of it (experts' gate | up weight
-// gradient, one K step per tile: 285 -> 269 us).
-struct TcWalk {
-  int tm, tn, group;                 // row tile (tr: token chunk), column tile (tr: feature tile), group
-  int left;                          // tiles of this role that are left, this one included
-  int dm, dn, dg, tiles_m, tiles_n;  // what a step adds; how far the parts count
-  int4 e;
-  __device__ __forceinline__ void ask(const GemmProblem& p, bool tr) {
-    if (left <= 0) return;
-    if (tr) e = p.tok_chunks[tm];
-    else if (p.group_mode == GROUP_M) e.x = p.tile_group[tm];
-    else if (p.group_mode == GROUP_K && p.group_off) {
-      e.x = p.group_off[group];
-      e.y = p.group_off[group + 1];
-      e.z = p.group_cnt ? p.group_cnt[group] : 0x7fffff00;
-    }
-  }
-  // tiles_m_dev: 128-row tiles as counted on the device (row tiles or token chunks of the grouped forms)
-  __device__ __forceinline__ void begin(const TcParams& P, int w0, int stride, int tiles_m_dev, int pair_rank) {
-    const GemmProblem& p = P.p;
-    tiles_n = P.tr ? P.tiles_f : P.tiles_n;
-    tiles_m = P.tr ? p.rows_total[1] : (pair_rank >= 0 ? (tiles_m_dev + 1) / 2 : tiles_m_dev);
-    const int per = tiles_m * tiles_n, total = per * (p.group_mode == GROUP_K ? p.n_groups : 1);
-    e = make_int4(0, 0, 0, 0);
-    left = w0 < total ? (total - w0 + stride - 1) / stride : 0;
-    tm = tn = group = dm = dn = dg = 0;
-    if (left == 0) return;
-    group = w0 / per; tm = (w0 - group * per) / tiles_n; tn = w0 - group * per - tm * tiles_n;
-    dg = stride / per; dm = (stride - dg * per) / tiles_n; dn = stride - dg * per - dm * tiles_n;
-    ask(p, P.tr);
-  }
-  __device__ __forceinline__ void step(const TcParams& P) {
-    --left;
-    tn += dn; tm += dm; group += dg;
-    if (tn >= tiles_n) { tn -= tiles_n; ++tm; }
-    if (tm >= tiles_m) { tm -= tiles_m; ++group; }
-    ask(P.p, P.tr);
-  }
-};
-
-// pair_rank < 0: one CTA per 128-row tile.  pair_rank 0 / 1: a tile is 256 rows worked by two CTAs,
-// this CTA takes rows 128 * pair_rank .. + 127 of it (rows past M are loaded as zeros and never stored).
-__device__ __forceinline__ TcTile tc_tile(const TcParams& P, const TcWalk& a, int pair_rank = -1) {
+// Tile `idx` (of tiles_m row tiles or token chunks x tiles_n column or feature tiles a group).  pair_rank < 0: one CTA per
+// 128-row tile.  pair_rank 0 / 1: a tile is 256 rows worked by two CTAs, this CTA takes rows 128 * pair_rank .. + 127 of it
+// (rows past M are loaded as zeros and never stored).
+__device__ __forceinline__ TcTile tc_tile(const TcParams& P, int idx, int tiles_m, int tiles_n, int pair_rank) {
   TcTile t;
   const GemmProblem& p = P.p;
+  const int row = idx / tiles_n, tn = idx - row * tiles_n, group = row / tiles_m, tm = row - group * tiles_m;
+  t.valid = 1;
   t.krow0 = 0;
   t.pad = 0;
   t.k_blocks = P.k_blocks;
   if (P.tr) {
     // m0 = first token row, ncols = token rows (the MMA N), n0 = first feature of this CTA's 128
-    t.group = a.e.x; t.m0 = a.e.y; t.ncols = a.e.z;
-    t.n0 = (a.tn * 2 + pair_rank) * (p.concat == CONCAT_N ? TC_BM / 2 : TC_BM);
-    t.pad = a.e.w;
+    const int4 e = p.tok_chunks[tm];
+    t.group = e.x; t.m0 = e.y; t.ncols = e.z;
+    t.n0 = (tn * 2 + pair_rank) * (p.concat == CONCAT_N ? TC_BM / 2 : TC_BM);
+    t.pad = e.w;
     return t;
   }
-  t.group = a.group;
+  t.group = group;
   if (p.group_mode == GROUP_K) {
     if (p.group_off) {
-      t.krow0 = a.e.x;
-      t.k_blocks = min((a.e.y - a.e.x) / TC_BK, (a.e.z + TC_BK - 1) / TC_BK);   // skip all-zero K blocks
+      const int r0 = p.group_off[group], r1 = p.group_off[group + 1], cnt = p.group_cnt ? p.group_cnt[group] : 0x7fffff00;
+      t.krow0 = r0;
+      t.k_blocks = min((r1 - r0) / TC_BK, (cnt + TC_BK - 1) / TC_BK);   // skip all-zero K blocks
     } else {
       // equal slices of a dense K (split-K): rows past K in the last K step load as zeros
       const int slice = (int)split_k_rows(p.K, p.n_groups);
@@ -563,11 +531,36 @@ __device__ __forceinline__ TcTile tc_tile(const TcParams& P, const TcWalk& a, in
       t.k_blocks = (k1 - k0 + TC_BK - 1) / TC_BK;
     }
   }
-  t.m0 = (pair_rank >= 0) ? a.tm * 2 * TC_BM + pair_rank * TC_BM : a.tm * TC_BM;
-  t.n0 = a.tn * P.tile_n;
+  t.m0 = (pair_rank >= 0) ? tm * 2 * TC_BM + pair_rank * TC_BM : tm * TC_BM;
+  t.n0 = tn * P.tile_n;
   t.ncols = (p.concat == CONCAT_N) ? 2 * P.tile_n : min(P.tile_n, p.N - t.n0);
-  if (p.group_mode == GROUP_M) t.group = a.e.x;
+  if (p.group_mode == GROUP_M) t.group = p.tile_group[tm];
   return t;
+}
+
+// Cluster launch control.  Asks the hardware for a cluster of this grid that has not been launched yet; the answer (16 bytes)
+// arrives on the barrier, in both CTAs of a pair.
+template <bool PAIR>
+__device__ __forceinline__ void clc_ask(uint32_t answer, uint32_t bar) {
+  if constexpr (PAIR)
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.multicast::cluster::all.b128 [%0], [%1];"
+                 ::"r"(answer), "r"(bar) : "memory");
+  else
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+                 ::"r"(answer), "r"(bar) : "memory");
+}
+// blockIdx.x of the first CTA of the cluster that the answer grants, or -1 when none was left.
+__device__ __forceinline__ int clc_granted(uint32_t answer) {
+  int x;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 a;\n\t.reg .b64 lo, hi;\n\t"
+      "ld.shared.v2.b64 {lo, hi}, [%1];\n\t"
+      "mov.b128 a, {lo, hi};\n\t"
+      "mov.s32 %0, -1;\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, a;\n\t}"
+      : "=r"(x) : "r"(answer) : "memory");
+  return x;
 }
 
 // ---------------------------------------------------------------------------
@@ -597,17 +590,26 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int* issued = reinterpret_cast<int*>(tmem_slot + 2);   // [STAGES] parity+1 of the last load issued per stage
   int* issued_b = issued + Cfg::STAGES;                  // the same for the second load warp: nonzero once it has issued
+  // tiles: their descriptions, a barrier each for "described" and "read by all roles"; "the loads have begun a tile", the answer
+  // of the hardware and "both CTAs have read the answer"
+  auto dfull_bar = [&](int i) { return bars + 336u + 8u * i; };
+  auto dempty_bar = [&](int i) { return bars + 336u + 8u * (TC_TILE_SLOTS + i); };
+  const uint32_t begun_bar = bars + 400u, answer_bar = bars + 408u, heard_bar = bars + 416u, answer = bars + 432u;
+  TcTile* const tiles = reinterpret_cast<TcTile*>(gen_base + Cfg::BAR_OFF + 448);
+  static_assert(TC_TILE_SLOTS == 4 && sizeof(TcTile) == 32, "barrier block");
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int crank = PAIR ? (int)cluster_ctarank() : 0;     // rank in the pair; rank 0 issues the MMAs
   const int prank = PAIR ? crank : -1;
-  const int w0 = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;       // first tile and tile stride of this CTA / pair
-  const int wstride = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < Cfg::STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); issued[s] = 0; issued_b[s] = 0; }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), PAIR ? 2 * TC_EPI_WARPS : TC_EPI_WARPS); }
     mbar_init(drain_bar, 1);
+    // readers of a description: the load warps that load, the products' warp where it runs, the epilogue warps
+    const int readers = (P.split_loads ? 2 : 1) + (crank == 0 ? 1 : 0) + TC_EPI_WARPS;
+    for (int i = 0; i < TC_TILE_SLOTS; ++i) { mbar_init(dfull_bar(i), 1); mbar_init(dempty_bar(i), readers); }
+    mbar_init(begun_bar, 1); mbar_init(answer_bar, 1); mbar_init(heard_bar, PAIR ? 2 : 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -630,8 +632,20 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  int tiles_m_dev = P.tiles_m;
+  int tiles_m_dev = P.tiles_m;      // 128-row tiles as counted on the device
   if (p.group_mode == GROUP_M) tiles_m_dev = min(P.tiles_m, *p.rows_total / TC_BM);
+
+  // The next tile of this role, all lanes together.  0: there is none; -1: the wait was abandoned.
+  int slot = 0;
+  uint32_t slot_phase = 0;
+  auto next_tile = [&](TcTile& t) -> int {
+    if (!mbar_wait_warp(dfull_bar(slot), slot_phase, abort_flag, p.status, P.wait_cycles)) return -1;
+    t = tiles[slot];
+    __syncwarp();
+    if (lane == 0) mbar_arrive(dempty_bar(slot));
+    if (++slot == TC_TILE_SLOTS) { slot = 0; slot_phase ^= 1u; }
+    return t.valid;
+  };
 
   if (warp == 0 || warp == TC_LOAD_WARP_B) {
     // ------------------------------------------------------------------ operand loads
@@ -652,8 +666,6 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      TcWalk walk;
-      walk.begin(P, w0, wstride, tiles_m_dev, prank);
       // this warp's loads of K step kb of tile t, by one elected lane
       auto issue = [&](const TcTile& t, int kb, int k_half) {
         const uint32_t sa = base + stage * Cfg::STAGE_BYTES;
@@ -798,9 +810,9 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           }
         }
       };
-      while (ok && walk.left > 0) {
-        const TcTile t = tc_tile(P, walk, prank);
-        walk.step(P);
+      TcTile t;
+      while (ok && next_tile(t) > 0) {
+        if (la && crank == 0 && lane == 0) mbar_arrive(begun_bar);
         const int k_half = t.k_blocks / 2;
         for (int kb = 0; kb < t.k_blocks; ++kb) {
           if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
@@ -835,11 +847,10 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       const uint32_t b_step = n_mn ? (2048u >> 4) : (32u >> 4);
       constexpr uint32_t SB16 = (uint32_t)Cfg::STAGE_BYTES >> 4;  // the whole ring stays below 256 KB: no carry out of the field
       uint32_t a_lo = a_lo0, b_lo = b_lo0, fbar = full_bar(0), ebar = empty_bar(0);
-      TcWalk walk;
-      walk.begin(P, w0, wstride, tiles_m_dev, prank);
-      for (; ok && walk.left > 0; ++it) {
-        const TcTile t = tc_tile(P, walk, prank);
-        walk.step(P);
+      TcTile t;
+      for (; ok; ++it) {
+        const int got = next_tile(t);
+        if (got <= 0) { ok = got == 0; break; }
         const int acc = it & 1;
         const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
         if (!mbar_wait_warp(tempty_bar(acc), acc_phase ^ 1u, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
@@ -884,6 +895,73 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
         while (!mbar_try_wait(drain_bar, 0u) && clock64() - t0 < P.wait_cycles) {}
       }
     }
+  } else if (warp == TC_TILE_WARP) {
+    // ------------------------------------------------------------------ tiles
+    // The grid has a CTA (pair) per tile, of which as many run as there is room for; a running one takes on the tile of
+    // another that has not been launched yet whenever its loads begin a tile.  So it does not matter when an SM becomes free:
+    // with tiles dealt out in advance, CTAs whose SM another stream's kernel held kept everybody waiting at the end, and the
+    // SMs that had finished earlier idled.  Both sides in turn: forward of 64 tokens 263 -> 249 us, steps at 512, 2741, 8192, 16384
+    // (Zipf) and 32768 tokens 1334 -> 1291, 2225 -> 2177, 5012 -> 4923, 9406 -> 9001, 18079 -> 17236, with fused Adam 7501 -> 7312, four
+    // d = 512 blocks 1476 -> 1421, three whole blocks 21815 -> 21161; attention alone, whose streams rarely meet, 2170 -> 2163.
+    // A tile's description costs this warp two divisions and a table look-up, one tile ahead of the loads.
+    const int tiles_n = P.tr ? P.tiles_f : P.tiles_n;
+    const int tiles_m = P.tr ? p.rows_total[1] : (PAIR ? (tiles_m_dev + 1) / 2 : tiles_m_dev);
+    const int total = tiles_m * tiles_n * (p.group_mode == GROUP_K ? p.n_groups : 1);
+    // A table of shorter runs than the launcher reckons with has more tiles than the grid: those follow at this distance.
+    const int granted = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
+    int idx = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+    uint32_t begun_phase = 0, answer_phase = 0, heard_phase = 0;
+    bool ok = true;
+    auto describe = [&](const TcTile& t) -> bool {
+      if (!mbar_wait_warp(dempty_bar(slot), slot_phase ^ 1u, abort_flag, p.status, P.wait_cycles)) return false;
+      if (lane == 0) {
+        tiles[slot] = t;
+        mbar_arrive(dfull_bar(slot));
+      }
+      __syncwarp();
+      if (++slot == TC_TILE_SLOTS) { slot = 0; slot_phase ^= 1u; }
+      return true;
+    };
+    while (true) {
+      // (a grid planned by a bound on the tiles has some that do not exist)
+      for (; ok && idx < total; idx += granted) {
+        ok = describe(tc_tile(P, idx, tiles_m, tiles_n, prank));
+        if (ok && crank == 0) {
+          ok = mbar_wait_warp(begun_bar, begun_phase, abort_flag, p.status, P.wait_cycles);
+          begun_phase ^= 1u;
+        }
+      }
+      if (!ok) break;
+      if (lane == 0) mbar_expect_tx(answer_bar, 16);
+      if (crank == 0) {
+        if (!(ok = mbar_wait_warp(heard_bar, heard_phase ^ 1u, abort_flag, p.status, P.wait_cycles))) break;
+        heard_phase ^= 1u;
+        if (elect_one()) clc_ask<PAIR>(answer, answer_bar);
+        __syncwarp();
+      }
+      if (!(ok = mbar_wait_warp(answer_bar, answer_phase, abort_flag, p.status, P.wait_cycles))) break;
+      answer_phase ^= 1u;
+      idx = clc_granted(answer);
+      if (PAIR) idx >>= 1;            // -1 stays
+      // read before the hardware writes the next one
+      asm volatile("fence.proxy.async;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) {
+        if constexpr (PAIR) mbar_arrive_cluster(mapa_u32(heard_bar, 0));
+        else mbar_arrive(heard_bar);
+      }
+      if (idx < 0) {
+        const TcTile none = {};
+        describe(none);
+        break;
+      }
+    }
+    if (!ok) {
+      // an answer that is still on its way must not land in shared memory that this CTA no longer has
+      const long long t0 = clock64();
+      while (!mbar_try_wait(answer_bar, answer_phase) && clock64() - t0 < 4000000LL) {}
+      __syncwarp();
+    }
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..9)
     const int q = warp & 3;                      // TMEM lane quadrant this warp may access
@@ -925,11 +1003,9 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
     };
     SlabOut next_out;      // Adam, row-wise: the next tile's slab, whose first units this tile has asked for (primed)
     bool primed = false;
-    TcWalk walk;
-    walk.begin(P, w0, wstride, tiles_m_dev, prank);
-    for (; ok && walk.left > 0; ++it) {
-      const TcTile t = tc_tile(P, walk, prank);
-      walk.step(P);
+    TcTile t;
+    for (; ok; ++it) {
+      if (next_tile(t) <= 0) break;
       const int acc = it & 1;
       const uint32_t acc_phase = (uint32_t)(it >> 1) & 1u;
       const int m = t.m0 + row_in_tile;
@@ -1234,11 +1310,12 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
               const bool last = cb * 128 + 128 >= t.ncols;
               if (last) release();      // the tile's last columns are out of tensor memory
               if (last) {
-                primed = EPI == EPI_WADAM && walk.left > 0;
+                // (the next tile, where it is described already: the loads are ahead of this warp)
+                primed = EPI == EPI_WADAM && __all_sync(0xffffffffu, mbar_try_wait(dfull_bar(slot), slot_phase));
                 if (primed) {
-                  const TcTile tn = tc_tile(P, walk, prank);
+                  const TcTile tn = tiles[slot];
                   next_out = slab_of(tn);
-                  primed = next_out.rows > 0;
+                  primed = tn.valid && next_out.rows > 0;
                 }
               }
               if (out.m) upd_half<EPI == EPI_WADAM, true>(p.upd, out, next_out, stg, lane, p.ldc, cb, last, primed);
@@ -1929,20 +2006,20 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   P.tiles_f = (int)ceil_div(p.N, p.concat == CONCAT_N ? 128 : 256);
   P.tr_swap = tr && p.concat == CONCAT_N && reinterpret_cast<uintptr_t>(p.B1) < reinterpret_cast<uintptr_t>(p.B0);
   if (tr && p.concat == CONCAT_N) mb0 = m_gu;
+  // a CTA or a CTA pair per tile
   int64_t total = (int64_t)P.tiles_m * P.tiles_n * (p.group_mode == GROUP_K ? groups : 1);
-  int grid = (int)(total < s.n_sms ? total : s.n_sms);
   if (tr) {
-    // the number of token chunks is only known on the device: a full persistent grid
-    grid = s.n_sms;
+    // the number of token chunks is only known on the device: runs of 256 of each expert's rows, which are padded to 128
+    total = (p.M + 128 * (int64_t)groups) / 256 * P.tiles_f;
     P.idesc = (1u << 4) | fmt | ((uint32_t)(p.b_mn_major ? 1 : 0) << 15) |
               ((uint32_t)(p.a_mn_major ? 1 : 0) << 16) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(2 * TC_BM >> 4) << 24);
   } else if (pair) {
     total = (int64_t)((P.tiles_m + 1) / 2) * P.tiles_n * (p.group_mode == GROUP_K ? groups : 1);
-    const int64_t pairs = total < s.n_sms / 2 ? total : s.n_sms / 2;
-    grid = (int)(2 * pairs);
     P.idesc = (P.idesc & ~(0x1Fu << 24)) | ((uint32_t)(2 * TC_BM >> 4) << 24);   // M = 256 across the pair
   }
-  if (grid <= 0) return REVFFN_OK;
+  if (total <= 0) return REVFFN_OK;
+  if (total > (1 << 30)) return REVFFN_ERR_SHAPE;
+  const int grid = (int)(pair ? 2 * total : total);
 
 #define TC_CASE(N_, E_) \
   if (mma_n == N_ && epi == E_) return tc_launch<N_, E_>(P, ma, mb0, mb1, mc, mc1, grid, pair, st);

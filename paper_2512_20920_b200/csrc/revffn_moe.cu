@@ -318,7 +318,7 @@ __global__ void clear_status_kernel(int* __restrict__ status) {
 // ---------------------------------------------------------------------------
 // A second stream for launches that do not depend on what the caller's stream is doing at that point
 // (the shared expert beside the routed experts, the weight gradients beside the chain of input gradients).  The
-// matrix products are persistent kernels of one CTA per SM and equal tiles, so most of them end with a partly
+// matrix products hold one CTA per SM and work equal tiles, so most of them end with a partly
 // empty last round of tiles; a kernel from the other stream starts on the SMs that fall idle there.  Ordering is by
 // events from a small ring (a wait refers to the record that preceded it, so an event can be recorded again while
 // an older wait is still pending).
@@ -495,9 +495,9 @@ static int run_branch(const Ctx<T>& c, const float* y1, const int32_t* idx_in, i
     return run_gemm(c, p, TG_PUP);
   };
   // The logits and P_up can run at the same time, but once the logits' blocks fill the GPU they only get in each
-  // other's way: a product CTA needs a whole SM and its tiles are dealt out in advance, so SMs that the router
-  // gives up late hold up the whole product.  At 8192 tokens, in the inverse pass: beside each other 104-148 us for
-  // P_up, maps ready after 150 us; one after the other 42 us and after 128 us.  The line is two router blocks per SM.
+  // other's way: a product CTA needs a whole SM, and the router's blocks get the SMs only as the product's fall free.  At 8192
+  // tokens, in the inverse pass: beside each other 104-148 us for P_up, maps ready after 150 us; one after the other 42 us and
+  // after 128 us.  The line is two router blocks per SM.
   const bool router_fills = ceil_div(Tn, RT_TOK) * ROUTE_CLUSTER > 2 * tc_state().n_sms, pup_first = rt != st && router_fills;
 
   // Router: fold through P_up, logits, top-k, gates -- or everything from a routing record.  The router reads y1

@@ -18,7 +18,7 @@ F32 = ("norm_gamma", "b_q", "b_k", "b_v")
 @pytest.mark.parametrize("batch,seq_len,d_model,n_heads,n_kv_heads", [
     (45, 130, 512, 4, 2),        # 360 items of dQ, 180 of dK/dV
     (5, 1000, 512, 4, 4),        # 160 of each, of 1 to 8 steps
-    (2, 150, 384, 3, 3),         # three key/value heads: two products
+    (2, 150, 768, 6, 3),         # three key/value heads: two products
     (2, 150, 256, 2, 2),         # two: one product of one tile per matrix
     (3, 700, 512, 4, 2),         # 2100 tokens: gradients in four slices of K, keys' and values' in one product
 ])
