@@ -179,15 +179,20 @@ inline cudaError_t launch_fold_router(const T* w_router, const T* w_sgate, const
 
 // ---------------------------------------------------------------------------
 // The same fold on the fp64 tensor-core path, K split across blocks.
-//   fold_router_mma_kernel: block (x: 64 columns i, y: 64 rows e, z: slice of rows j) computes the slice's
-//     part[z][e][i] = sum_{j in slice z} W_r'[e, j] * W_up[j, i] with mma.sync m8n8k4 (warp = 16 rows x
-//     32 columns as 2 x 4 fragments).
+//   fold_router_mma_kernel: block (x: 32 columns i, y: 32 rows e, z: slice of rows j) computes the slice's
+//     part[z][e][i] = sum_{j in slice z} W_r'[e, j] * W_up[j, i] with mma.sync m8n8k4 (two warps of 32 rows x
+//     16 columns as 4 x 2 fragments).
 //   fold_router_reduce_kernel: W_rc[e][i] = sum_z part[z][e][i], z ascending (fixed order).
+// Bound by the fp64 pipe (64 multiply-adds a clock and SM: 7 us for 61 x 2048 x 1024) and the first loads.  The blocks are small so
+// that an SM holds several at once, which load together, and none ends with a half-empty round: 1024 of them at this size,
+// 6.9 per SM.  (256 blocks of 64 x 64, 1.7 per SM: the pipe of most SMs worked
+// for two.  Forward of 64 tokens 253 -> 250 us, four d = 512 blocks 1438 -> 1418.)
 // Needs FOLD_SLICES * (E+1) * h doubles of scratch, which the workspace has; the entry point that may
 // not use a workspace keeps the FMA kernel above.
 // ---------------------------------------------------------------------------
 constexpr int FOLD_SLICES = 16;        // upper bound on the K slices
 constexpr int FM_J_BYTES = 256;        // a slice is this many bytes of a W_r' row: 128 rows j in bf16, 64 in fp32
+constexpr int FM_E = 32, FM_I = 32, FM_THREADS = 64;
 template <typename T> __host__ __device__ constexpr int fold_slice_rows() { return FM_J_BYTES / (int)sizeof(T); }
 constexpr int FM_PAD = 8;              // elements of padding per staged row (keeps rows 16-byte aligned)
 
@@ -196,67 +201,65 @@ __device__ __forceinline__ void fold_dmma(double& d0, double& d1, double a, doub
                : "+d"(d0), "+d"(d1) : "d"(a), "d"(b));
 }
 
-// The block's whole operand slices are fetched with 16-byte loads that are all in flight together
-// (one memory round trip), kept in shared memory in their storage type, and widened to fp64 as the
-// fragments are read.
+// The block's whole operand slices come in by cp.async, all in flight together (one memory round trip), stay in shared memory in
+// their storage type, and are widened to fp64 as the fragments are read.
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(FM_THREADS)
 fold_router_mma_kernel(const T* __restrict__ w_router, const T* __restrict__ w_sgate, const T* __restrict__ w_up,
                        int E, int d, int h, double* __restrict__ part) {
   pdl_sync();
   constexpr int PER16 = 16 / (int)sizeof(T);
   constexpr int FM_J = fold_slice_rows<T>();
-  constexpr int LDA = FM_J + FM_PAD, LDB = 64 + FM_PAD;
-  __shared__ __align__(16) T as[64 * LDA];       // W_r' slice  [e][j]
+  constexpr int LDA = FM_J + FM_PAD, LDB = FM_I + FM_PAD;
+  __shared__ __align__(16) T as[FM_E * LDA];     // W_r' slice  [e][j]
   __shared__ __align__(16) T bs[FM_J * LDB];     // W_up slice  [j][i]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int i0 = blockIdx.x * 64, e0 = blockIdx.y * 64, jb = blockIdx.z * FM_J;
+  const int i0 = blockIdx.x * FM_I, e0 = blockIdx.y * FM_E, jb = blockIdx.z * FM_J;
   const int EP = E + 1;
-  const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
   // d and h are multiples of 8, so a 16-byte piece never straddles the end of a row
-  for (int piece = tid; piece < 64 * (FM_J / PER16); piece += 256) {
-    const int ee = piece / (FM_J / PER16), jj = (piece % (FM_J / PER16)) * PER16;
+#pragma unroll
+  for (int q = 0; q < FM_E * (FM_J / PER16) / FM_THREADS; ++q) {
+    const int piece = tid + q * FM_THREADS, ee = piece / (FM_J / PER16), jj = (piece % (FM_J / PER16)) * PER16;
     const int e = e0 + ee, j = jb + jj;
     const T* src = (e < E) ? (w_router + (int64_t)e * d) : (e == E ? w_sgate : nullptr);
-    *reinterpret_cast<uint4*>(&as[ee * LDA + jj]) =
-        (src != nullptr && j < d) ? *reinterpret_cast<const uint4*>(src + j) : zero4;
+    const bool ok = src != nullptr && j < d;
+    cp_async16(&as[ee * LDA + jj], ok ? src + j : w_router, ok);
   }
-  for (int piece = tid; piece < FM_J * (64 / PER16); piece += 256) {
-    const int jj = piece / (64 / PER16), ii = (piece % (64 / PER16)) * PER16;
-    const int j = jb + jj, i = i0 + ii;
-    *reinterpret_cast<uint4*>(&bs[jj * LDB + ii]) =
-        (j < d && i < h) ? *reinterpret_cast<const uint4*>(w_up + (int64_t)j * h + i) : zero4;
+#pragma unroll
+  for (int q = 0; q < FM_J * (FM_I / PER16) / FM_THREADS; ++q) {
+    const int piece = tid + q * FM_THREADS, jj = piece / (FM_I / PER16), ii = (piece % (FM_I / PER16)) * PER16;
+    const bool ok = jb + jj < d && i0 + ii < h;
+    cp_async16(&bs[jj * LDB + ii], ok ? w_up + (int64_t)(jb + jj) * h + i0 + ii : w_up, ok);
   }
+  cp_async_commit();
+  cp_async_wait<0>();
   __syncthreads();
-  const int wm = warp >> 1, wn = warp & 1, fr = lane >> 2, fc = lane & 3;
-  double acc[2][4][2];
+  const int fr = lane >> 2, fc = lane & 3;
+  double acc[4][2][2];
 #pragma unroll
-  for (int a = 0; a < 2; ++a)
+  for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) { acc[a][b][0] = 0.0; acc[a][b][1] = 0.0; }
+    for (int b = 0; b < 2; ++b) { acc[a][b][0] = 0.0; acc[a][b][1] = 0.0; }
 #pragma unroll 4
   for (int kk = 0; kk < FM_J; kk += 4) {
-    double af[2], bf[4];
+    double af[4], bf[2];
 #pragma unroll
-    for (int a = 0; a < 2; ++a) af[a] = (double)to_f32(as[(wm * 16 + a * 8 + fr) * LDA + kk + fc]);
+    for (int a = 0; a < 4; ++a) af[a] = (double)to_f32(as[(a * 8 + fr) * LDA + kk + fc]);
 #pragma unroll
-    for (int b = 0; b < 4; ++b) bf[b] = (double)to_f32(bs[(kk + fc) * LDB + wn * 32 + b * 8 + fr]);
+    for (int b = 0; b < 2; ++b) bf[b] = (double)to_f32(bs[(kk + fc) * LDB + warp * 16 + b * 8 + fr]);
 #pragma unroll
-    for (int a = 0; a < 2; ++a)
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int b = 0; b < 4; ++b) fold_dmma(acc[a][b][0], acc[a][b][1], af[a], bf[b]);
+      for (int b = 0; b < 2; ++b) fold_dmma(acc[a][b][0], acc[a][b][1], af[a], bf[b]);
   }
   double* out = part + (int64_t)blockIdx.z * EP * h;
 #pragma unroll
-  for (int a = 0; a < 2; ++a)
+  for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const int e = e0 + wm * 16 + a * 8 + fr;
-        const int i = i0 + wn * 32 + b * 8 + 2 * fc + c;
-        if (e < EP && i < h) out[(int64_t)e * h + i] = acc[a][b][c];
-      }
+    for (int b = 0; b < 2; ++b) {
+      const int e = e0 + a * 8 + fr, i = i0 + warp * 16 + b * 8 + 2 * fc;
+      if (e < EP && i < h) *reinterpret_cast<double2*>(out + (int64_t)e * h + i) = make_double2(acc[a][b][0], acc[a][b][1]);      // h is even
+    }
 }
 
 __global__ void fold_router_reduce_kernel(const double* __restrict__ part, int n_slices, int64_t n,
@@ -275,8 +278,8 @@ inline cudaError_t launch_fold_router_mma(const T* w_router, const T* w_sgate, c
                                           double* part, double* w_rc, cudaStream_t st) {
   const int n_slices = (int)ceil_div(d, fold_slice_rows<T>());
   if (n_slices > FOLD_SLICES) return cudaErrorInvalidValue;
-  dim3 grid((unsigned)ceil_div(h, 64), (unsigned)ceil_div(E + 1, 64), (unsigned)n_slices);
-  launch_k(fold_router_mma_kernel<T>, grid, 256, 0, st, w_router, w_sgate, w_up, E, d, h, part);
+  dim3 grid((unsigned)ceil_div(h, FM_I), (unsigned)ceil_div(E + 1, FM_E), (unsigned)n_slices);
+  launch_k(fold_router_mma_kernel<T>, grid, FM_THREADS, 0, st, w_router, w_sgate, w_up, E, d, h, part);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int64_t n = (int64_t)(E + 1) * h;
