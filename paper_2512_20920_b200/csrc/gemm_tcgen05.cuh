@@ -417,7 +417,8 @@ __device__ __forceinline__ uint2 pack4(const float4& v) {
 // offset: with two epilogue warps per scheduler an instruction costs its latency, and the first form of this loop
 // (kind and ring depth looked up at run time) took 950 clk per unit before any memory traffic.  Adam's last
 // units of a tile ask for the first ones of the next, so that reads go on while its accumulator is staged (experts'
-// gate | up at 1024 tokens, 9.0 GB: 2088 -> 1965 us; the SGD step, 1.4 GB, got slower by it, 309 -> 362).
+// gate | up at 1024 tokens, 9.0 GB: 2088 -> 1965 us, now 1469, 6.1 TB/s, where a bare read-modify-write kernel of this shape
+// reaches 6.3; the SGD step, 1.4 GB, got slower by it, 309 -> 362).
 template <bool ADAM, bool MASTER> struct UpdRing {
   static constexpr int W = MASTER ? 1024 : 512;                    // bytes of weights in a unit
   static constexpr int UNIT = W + (ADAM ? 2048 : 0);
