@@ -707,13 +707,13 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
             const int b_cols = (p.b_mn_major && P.mn3d) ? P.b_box : nhalf;
             if (crank == 0) mbar_expect_tx(full_bar(stage), 2 * (TC_A_BYTES + b_cols * TC_BK * 2));
             if (!p.a_mn_major) {
-              tma_load_2d_pair(sa, &map_a, kb * TC_BK, t.m0, fbc);
+              tma_load_2d_pair(sa, &map_a, t.krow0 + kb * TC_BK, t.m0, fbc);
             } else {
               tma_load_mn128_pair(P.mn3d, sa, &map_a, p.a_col0 + t.m0, t.krow0 + kb * TC_BK, fbc);
             }
           }
           if (lb) {
-            bool second = p.concat == CONCAT_K && kb >= k_half;
+            bool second = p.concat == CONCAT_K && t.krow0 / TC_BK + kb >= k_half;
             const int kbp = second ? kb - k_half : kb;
             int b_row = t.n0 + nhalf * crank;
             if (EPI == EPI_HEADS && p.hm_split && t.n0 >= p.hm_split) { second = true; b_row -= p.hm_split; }
@@ -725,9 +725,9 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
                 if (crank == 0) tma_load_2d_pair(sb, &map_b0, kbp * TC_BK, t.n0, fbc);
                 else tma_load_2d_pair(sb, &map_b1, kbp * TC_BK, t.n0, fbc);
               } else if (second) {
-                tma_load_2d_pair(sb, &map_b1, kbp * TC_BK, b_row, fbc);
+                tma_load_2d_pair(sb, &map_b1, t.krow0 + kbp * TC_BK, b_row, fbc);
               } else {
-                tma_load_2d_pair(sb, &map_b0, kbp * TC_BK, b_row, fbc);
+                tma_load_2d_pair(sb, &map_b0, t.krow0 + kbp * TC_BK, b_row, fbc);
               }
             } else {
               const int krow = t.krow0 + kbp * TC_BK;
@@ -738,7 +738,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           return;
         }
         const uint32_t fb = full_bar(stage);
-        const bool second = p.concat == CONCAT_K && kb >= k_half;
+        const bool second = p.concat == CONCAT_K && t.krow0 / TC_BK + kb >= k_half;
         const int kb_b = second ? kb - k_half : kb;
         // An MN-major B tile is four 64 x 64 boxes against one or two loads for A: with two load threads the
         // first takes B's last boxes too (3 + 2 loads, or 3 + 3 when A is MN-major as well).
@@ -748,7 +748,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           issued[stage] = (int)phase + 1;
           // A tile
           if (!p.a_mn_major) {
-            tma_load_2d(sa, &map_a, kb * P.bk, t.m0, fb);
+            tma_load_2d(sa, &map_a, t.krow0 + kb * P.bk, t.m0, fb);
           } else {
             tma_load_mn128(P.mn3d, sa, &map_a, p.a_col0 + t.m0, t.krow0 + kb * TC_BK, fb);
           }
@@ -776,7 +776,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
           if (!p.b_mn_major) {
             // rows of the flattened [groups * N, K] weight tensor
             int row0 = (p.group_mode == GROUP_M ? t.group * p.N : 0) + t.n0;
-            bool second = p.concat == CONCAT_K && kb >= k_half;
+            bool second = p.concat == CONCAT_K && t.krow0 / TC_BK + kb >= k_half;
             if (EPI == EPI_HEADS && p.hm_split && t.n0 >= p.hm_split) { second = true; row0 -= p.hm_split; }
             if (p.concat == CONCAT_N) {
               tma_load_2d(sb, &map_b0, kb_b * P.bk, row0, fb);
@@ -785,8 +785,8 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
 #pragma unroll
               for (int j = 0; j < MMA_N / 128; ++j) {
                 if (128 * j >= t.ncols) continue;
-                if (second) tma_load_2d(sb + j * 16384, &map_b1, kb_b * P.bk, row0 + 128 * j, fb);
-                else tma_load_2d(sb + j * 16384, &map_b0, kb_b * P.bk, row0 + 128 * j, fb);
+                if (second) tma_load_2d(sb + j * 16384, &map_b1, t.krow0 + kb_b * P.bk, row0 + 128 * j, fb);
+                else tma_load_2d(sb + j * 16384, &map_b0, t.krow0 + kb_b * P.bk, row0 + 128 * j, fb);
               }
             }
           } else {
@@ -814,7 +814,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       TcTile t;
       while (ok && next_tile(t) > 0) {
         if (la && crank == 0 && lane == 0) mbar_arrive(begun_bar);
-        const int k_half = t.k_blocks / 2;
+        const int k_half = P.k_blocks / 2;
         for (int kb = 0; kb < t.k_blocks; ++kb) {
           if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status, P.wait_cycles)) { ok = false; break; }
           if (elect_one()) issue(t, kb, k_half);
@@ -1966,7 +1966,8 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
     if (p.group_mode == GROUP_K) {
       // group g's block must start g * M rows further down one 2D tensor (g * split_m rows with two outputs)
       const int64_t m_out = p.split_m > 0 ? p.split_m : p.M;
-      if (p.M % TC_BM != 0 || p.c_group_stride != m_out * p.ldc) return REVFFN_ERR_SHAPE;
+      // (a product split over K whose rows are rows of A may end inside a tile)
+      if ((p.M % TC_BM != 0 && (p.a_mn_major || p.upd_w)) || p.c_group_stride != m_out * p.ldc) return REVFFN_ERR_SHAPE;
       rows = (uint64_t)groups * p.M;
     }
     if (p.split_m > 0 && (p.epilogue != EPI_WGRAD || p.M != 2 * p.split_m || p.split_m % TC_BM != 0)) return REVFFN_ERR_SHAPE;
@@ -2026,8 +2027,8 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
   if (mma_n == N_ && epi == E_) return tc_launch<N_, E_>(P, ma, mb0, mb1, mc, mc1, grid, pair, st);
   // A fused update of a grouped product runs in its own form while the K range of a group is short (rows of K on average):
   // beyond, the operand ring that the form gives up is worth more than its reads and writes.  Per 256 x 256 tile: a K step costs
-  // about 1400 clk with two stages, 1000 with three and 600 with six, the row-wise epilogue 46 k (Adam) or 9 k (SGD),
-  // the block-wise one 57 k or 17 k.
+  // about 1400 clk with two stages, 1000 with three and 600 with six, the row-wise epilogue 39 k (Adam) or 9 k (SGD),
+  // the block-wise one 65 k or 17 k.  (Adam, experts' gate | up: 1491 against 2481 us at 8192 tokens, 1784 against 2594 at 16384.)
   const int64_t k_group = p.K / groups;
   const int epi = p.epilogue != EPI_WGRAD ? p.epilogue
                   : p.upd_w && p.group_off && k_group <= (p.upd.kind ? 2560 : 1152) ? (p.upd.kind ? EPI_WADAM : EPI_WSGD)

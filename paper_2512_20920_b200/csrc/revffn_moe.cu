@@ -463,6 +463,15 @@ static int wgrad_splits(int M, int N, int K, size_t room) {
   return (size_t)n * M * N * 4 > room || K < 64 * 8 * n || (M * (int64_t)N) % 4 != 0 || M % TC_BM != 0 ? 1 : n;
 }
 
+// The same for a stored product with a long K (M x N outputs, K in two halves): slices of at least 1024, so that the second launch
+// and the fp32 partial sums cost less than the steps saved.
+static int store_splits(int M, int N, int K, size_t room) {
+  const int64_t tiles = ceil_div(M, 2 * TC_BM) * ceil_div(N, 256);
+  int n = SPLIT_K_MAX;
+  while (n > 1 && (tiles * n > tc_state().n_sms / 2 || K < 1024 * n || K % (64 * n) != 0 || (size_t)n * M * N * 4 > room)) n /= 2;
+  return n;
+}
+
 // ---------------------------------------------------------------------------
 // F = MLP(Norm(Y1)) up to z (the input of P_down).  save_ab keeps the SwiGLU
 // pre-activations for the backward pass.
@@ -892,7 +901,22 @@ static int run_backward(const Ctx<T>& c, const float* y1, const float* dy2, floa
       p.A = c.template p<T>(L.abs); p.lda = 2 * (int64_t)Is;
       p.B0 = c.W.ws_gate; p.B1 = c.W.ws_up; p.ldb = d; p.b_mn_major = 1; p.concat = CONCAT_K;
       p.epilogue = EPI_STORE; p.C = c.template p<T>(L.dush); p.ldc = d;
+      // K = 2 I_s is long: at 512 tokens 64 tiles walk 176 K steps each, 62 us on less than half of the GPU (in four slices the
+      // step took 1301 us instead of 1318).  The partial sums take the place of the routed experts' input gradients, which come
+      // later on this stream.
+      const int n_split = c.tc ? store_splits(Tn, d, 2 * Is, L.dup.bytes) : 1;
+      if (n_split > 1) {
+        p.group_mode = GROUP_K; p.n_groups = n_split;
+        p.epilogue = EPI_WGRAD; p.C = c.template p<float>(L.dup); p.c_group_stride = (int64_t)Tn * d;
+      }
       CKR(run_gemm(c, p, TG_SH_DU));
+      if constexpr (std::is_same<T, bf16>::value) {
+        if (n_split > 1) {
+          ProfScope ps(TG_SH_DU, st);
+          CK(launch_k(splitk_store_kernel, (unsigned)ceil_div((int64_t)Tn * d, 8 * 256), 256, 0, st, c.template p<float>(L.dup), n_split,
+                      (int64_t)Tn * d, c.template p<bf16>(L.dush)));
+        }
+      }
     }
     {
       // as for the routed experts below: da|db is one buffer and both gradients read u, so when both are wanted in
