@@ -2,11 +2,12 @@
 // See include/revffn_attn.h for the contract of every entry point.  Included at the end of
 // revffn_moe.cu: it uses that file's launch accounting, error macros and GEMM back ends.
 //
-// Attention core: forward and inverse run it as one tcgen05 kernel (flash_attn.cuh) that never
-// writes the score matrix.  The backward pass, and the CUDA-core cross-check path, materialise it:
-// scores = Q K^T as one grouped product over all heads (fp32), a row kernel turns it into the
-// causal softmax P (operand type), O = P V is a second grouped product; then dP = dO V^T, the row
-// kernel for dS, dV = P^T dO and dK = dS^T Q as grouped weight-gradient-style products, dQ = dS K.
+// Attention core: with bf16 weights and heads of 128 both directions run as fused tcgen05 kernels
+// (flash_attn.cuh) that never write the score matrix.  The CUDA-core cross-check path, fp32 weights
+// and heads of another width materialise it: scores = Q K^T as one grouped product over all heads
+// (fp32), a row kernel turns it into the causal softmax P (operand type), O = P V is a second grouped
+// product; then dP = dO V^T, the row kernel for dS, dV = P^T dO and dK = dS^T Q as grouped
+// weight-gradient-style products, dQ = dS K.
 #pragma once
 
 #include "../../include/revffn_attn.h"
