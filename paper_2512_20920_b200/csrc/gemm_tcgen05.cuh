@@ -29,7 +29,7 @@
 // Both operands may be K-major or MN-major; MN-major tiles are fetched 128 columns x 64 K rows at a time through a
 // 3-D view of the matrix (64 x 64 boxes of a 2-D map as the fallback) and described to the tensor core with
 // leading/stride offsets.
-// Every wait is bounded; on expiry the kernel sets the status word and leaves.
+// Every wait is bounded; on expiry the kernel sets the status word, drops the tiles that have not begun and leaves.
 //
 // Pair mode (template flag PAIR; dense and K-grouped problems whose N is a multiple of 256, or of 128
 // when B is stored [K, N]):
@@ -912,7 +912,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
     const int granted = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
     int idx = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
     uint32_t begun_phase = 0, answer_phase = 0, heard_phase = 0;
-    bool ok = true;
+    bool ok = true, armed = false, asked = false;      // armed, asked: the answer's bytes are announced; the hardware has been asked
     auto describe = [&](const TcTile& t) -> bool {
       if (!mbar_wait_warp(dempty_bar(slot), slot_phase ^ 1u, abort_flag, p.status, P.wait_cycles)) return false;
       if (lane == 0) {
@@ -934,14 +934,17 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       }
       if (!ok) break;
       if (lane == 0) mbar_expect_tx(answer_bar, 16);
+      armed = true;
       if (crank == 0) {
         if (!(ok = mbar_wait_warp(heard_bar, heard_phase ^ 1u, abort_flag, p.status, P.wait_cycles))) break;
         heard_phase ^= 1u;
         if (elect_one()) clc_ask<PAIR>(answer, answer_bar);
         __syncwarp();
+        asked = true;
       }
       if (!(ok = mbar_wait_warp(answer_bar, answer_phase, abort_flag, p.status, P.wait_cycles))) break;
       answer_phase ^= 1u;
+      armed = asked = false;
       idx = clc_granted(answer);
       if (PAIR) idx >>= 1;            // -1 stays
       // read before the hardware writes the next one
@@ -958,9 +961,32 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
       }
     }
     if (!ok) {
-      // an answer that is still on its way must not land in shared memory that this CTA no longer has
-      const long long t0 = clock64();
-      while (!mbar_try_wait(answer_bar, answer_phase) && clock64() - t0 < 4000000LL) {}
+      // A wait was abandoned.  An answer that is still on its way must not land in shared memory that this CTA no longer has;
+      // and the CTAs that have not been launched yet must not be, each to wait for its own bound: this one takes what is left of the
+      // grid and drops it (in a pair the even CTA, into its own shared memory alone: its partner has stopped listening, or will).
+      auto settle = [&]() -> bool {
+        const long long t0 = clock64();
+        while (!__all_sync(0xffffffffu, mbar_try_wait(answer_bar, answer_phase)))
+          if (__any_sync(0xffffffffu, clock64() - t0 > 4000000LL)) return false;
+        answer_phase ^= 1u;
+        return true;
+      };
+      if (crank != 0) {
+        if (armed) settle();
+      } else {
+        for (int left = granted; left >= 0; --left) {      // (nothing may be asked after the answer that nothing is left)
+          if (!asked) {
+            if (!armed && lane == 0) mbar_expect_tx(answer_bar, 16);
+            __syncwarp();
+            if (elect_one()) clc_ask<false>(answer, answer_bar);
+            __syncwarp();
+          }
+          if (!settle() || clc_granted(answer) < 0) break;
+          armed = asked = false;
+          asm volatile("fence.proxy.async;" ::: "memory");
+          __syncwarp();
+        }
+      }
       __syncwarp();
     }
   } else {

@@ -119,6 +119,44 @@ def test_every_epilogue_leaves_a_starved_product_as_whole_warps(rv, epilogue, kw
     assert rel_l2(got.float().cpu().numpy(), want.cpu().numpy()) <= 1e-2
 
 
+@pytest.mark.parametrize("M,N,tile_n", [(8192, 8192, 64), (12800, 12800, 256)])
+def test_an_abandoned_wait_ends_a_launch_of_many_rounds(rv, M, N, tile_n):
+    """8192 and 5000 tiles on some 148 SMs, none of which ever gets its operands: a CTA that gives up has to take the tiles that have
+    not been launched yet with it, or every round of the grid waits for its own bound.  The bound is 2 M clocks (about
+    a millisecond); a launch may take a few of them and the time that the launch queue needs to hand out its tiles (about a
+    microsecond each to one CTA, shared by all), not 34 or 55 of them."""
+    from paper_2512_20920_b200.binding import DbgGemmArgs
+    K, wait = 64, 2_000_000
+    g = torch.Generator("cuda").manual_seed(7)
+    A, B = ((torch.randn(n, K, device="cuda", generator=g) * 0.3).to(torch.bfloat16) for n in (M, N))
+    out = torch.zeros(M, N, device="cuda", dtype=torch.bfloat16)
+    status = torch.zeros(64, dtype=torch.int32, device="cuda")
+    a = DbgGemmArgs(M=M, N=N, K=K, lda=K, ldb=K, ldc=N, A=A.data_ptr(), B0=B.data_ptr(), C=out.data_ptr(), resid_sign=1.0, no_pair=1,
+                    tile_n=tile_n)
+
+    def run():
+        t = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        status.zero_()
+        t[0].record()
+        assert rv.lib.revffn_dbg_gemm(C.byref(a), status.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+        t[1].record()
+        torch.cuda.synchronize()
+        return int(status[0]), t[0].elapsed_time(t[1])
+
+    def right():
+        return all(rel_l2(out[r].float().cpu().numpy(), (A[r].float() @ B.float().T).cpu().numpy()) <= 4e-3
+                   for r in (slice(0, 300), slice(M - 300, M)))
+    assert run()[0] == 0 and right()
+    out.zero_()
+    a.starve_operands, a.wait_cycles = 1, wait
+    code, ms = run()
+    assert code == rv.ERR_DEVICE_WAIT
+    assert float(out.float().abs().max()) == 0.0
+    assert ms < 20.0, ms
+    a.starve_operands, a.wait_cycles = 0, 0
+    assert run()[0] == 0 and right()
+
+
 def test_expert_indices_out_of_range_are_reported_not_used(rv):
     cfg = _cfg()
     w, s = _weights(cfg, 1), make_streams(cfg, 1)
