@@ -34,3 +34,51 @@ def test_partial_sums(M, N, K, slices, halves, mn, simt):
         k = slice(s * step, min(K, (s + 1) * step))
         want = A[:, k].float() @ W[k].float()
         assert float((out[s] - want).norm()) <= 1e-5 * float(want.norm())
+
+
+@pytest.mark.parametrize("tokens,d_shared,E,launches", [
+    (1, 2048, 6, 2),         # four slices of 1024
+    (100, 2048, 6, 2),       # the last block of the sums' kernel has a part of its rows
+    (256, 2048, 16, 2),      # whole blocks
+    (333, 1024, 8, 2),       # two slices, two row tiles
+    (333, 512, 8, 1),        # K = 1024: none
+    (2000, 2048, 6, 1),      # the partial sums do not fit: none
+])
+def test_shared_experts_input_gradient_in_slices(tokens, d_shared, E, launches):
+    """The shared expert's input gradient split over K, through the gradient pass, against the oracle and the CUDA cores (which do not
+    split) at the path's stated 2e-2."""
+    import paper_2512_20920_b200 as rv
+    from oracle import revffn_oracle as orc
+    from workloads import BlockConfig, make_streams, make_weights, to_bf16_values
+    from helpers import dev, grad_buffers, make_block, rel_l2
+    cfg = BlockConfig("d", tokens=tokens, d_model=256, n_experts=E, top_k=2, d_expert=128, d_shared=d_shared, weight_dtype="bf16")
+    w, s = make_weights(cfg, 3), make_streams(cfg, 3)
+    for n in w:
+        if n != "norm_gamma":
+            w[n] = to_bf16_values(w[n] * (4.0 if not n.startswith("ws_") else 2.0))
+    y1, x2, dy2 = dev(s["y1"]), dev(s["x2"]), dev(s["dy2"])
+    idx = torch.empty(tokens, 2, dtype=torch.int32, device="cuda")
+    make_block(cfg, w).forward(y1, x2, topk_idx_out=idx)
+
+    def run(flags):
+        blk = make_block(cfg, w, flags=flags)
+        dy1, g = torch.zeros_like(y1), grad_buffers(cfg, w)
+        blk.backward(y1, dy2, dy1, g, topk_idx_in=idx)
+        assert blk.status() == 0
+        return dy1, g
+    rv.revffn_prof_enable(True)
+    try:
+        dy1, g = run(0)
+        slots = rv.revffn_prof_collect()
+    finally:
+        rv.revffn_prof_enable(False)
+    assert slots["bwd/gemm_shared_du"][1] == launches, slots
+    ref = orc.backward(w, s["y1"], s["dy2"], 2, cfg.norm_eps, route_override=idx.cpu().numpy())
+    dy1_c, g_c = run(rv.FLAG_FORCE_SIMT)
+    for other, g_other in ((ref["dy1"], {n: ref[n] for n in g}), (dy1_c.cpu().numpy(), {n: t.cpu().numpy() for n, t in g_c.items()})):
+        assert rel_l2(dy1.cpu().numpy(), other) < 2e-2
+        for n in ("w_up", "norm_gamma"):      # what the input gradient reaches
+            assert rel_l2(g[n].cpu().numpy(), g_other[n]) < 2e-2, n
+    # the same without timing, where the gradients run on a second stream
+    dy1_s, g_s = run(0)
+    assert torch.equal(dy1, dy1_s) and all(torch.equal(g[n], g_s[n]) for n in g)
