@@ -45,7 +45,7 @@ def _make(acfg: AttnConfig, mcfg: BlockConfig, layers: int, std: float, iters: i
     return st, host, cfg, dev_a, dev_m
 
 
-def _run(acfg, mcfg, layers, std, tol, iters=1, flags=0, moe_scale=6.0):
+def _run(acfg, mcfg, layers, std, tol, iters=1, flags=0, moe_scale=6.0, near_tie=1e-4):
     st, host, cfg, dev_a, dev_m = _make(acfg, mcfg, layers, std, iters, flags, moe_scale)
     s = make_attn_streams(acfg, 5)
     T, k = acfg.tokens, mcfg.top_k
@@ -62,7 +62,7 @@ def _run(acfg, mcfg, layers, std, tol, iters=1, flags=0, moe_scale=6.0):
     for l in range(layers):
         margin = moe.topk_margin(infos[l]["logits"], k)
         same = (np.sort(ov[l], 1) == np.sort(moe.topk_indices(infos[l]["logits"], k), 1)).all(1)
-        assert (same | (margin < 1e-4)).all(), f"layer {l}: selection differs outside a near-tie"
+        assert (same | (margin < near_tie)).all(), f"layer {l}: selection differs outside a near-tie"
     assert rel_l2(a.cpu().numpy() - X1, Y1 - X1) < tol and rel_l2(b.cpu().numpy() - X2, Y2 - X2) < tol
 
     # reversible back-propagation from the oracle's outputs (same starting point on both sides)
@@ -115,6 +115,15 @@ def test_two_bf16_blocks_against_the_oracle(simt):
     mcfg = BlockConfig("m", tokens=384, d_model=256, n_experts=8, top_k=2, d_expert=128, d_shared=128, weight_dtype="bf16")
     # bf16 intermediates through four branches in a row: the path's 2e-2 per branch compounds
     _run(acfg, mcfg, 2, 0.05, 3e-2, flags=rv.FLAG_FORCE_SIMT if simt else 0, moe_scale=3.0)
+
+
+def test_three_bf16_blocks_of_full_width_against_the_oracle():
+    """The benchmark's widths with few experts and tokens: what one layer rounds differently is rounded again by every layer below, and
+    here all of it is held against 64 bits.  (The router reads a stream that carries the rounding of the attention branch
+    before it, 4e-3 of logits of order one, hence the wider near-tie.)"""
+    acfg = AttnConfig("a", batch=2, seq_len=256, d_model=2048, n_heads=16, n_kv_heads=4, weight_dtype="bf16")
+    mcfg = BlockConfig("m", tokens=512, d_model=2048, n_experts=4, top_k=2, d_expert=1408, d_shared=5632, weight_dtype="bf16")
+    _run(acfg, mcfg, 3, 0.02, 3e-2, moe_scale=1.0, near_tie=2e-2)
 
 
 def test_mismatched_descriptors_are_rejected():
