@@ -183,3 +183,66 @@ def test_reversible_stack_sweep_as_one_adam_step(rv):
             step = masters[n].cpu().numpy().astype(np.float64) - w_old[n]
             assert rel_l2(step, new[n] - ws_host[l][n]) <= 2 * TOL_BF16, (l, n, rel_l2(step, new[n] - ws_host[l][n]))
             assert torch.equal(weights[l][n], masters[n].to(torch.bfloat16)), (l, n)
+
+
+# a gradient of zero, so that the stored moments alone decide: m = beta1 m0, v = beta2 v0, exactly
+@pytest.mark.parametrize("names", [("w_gate", "w_downx"), ("w_up", "ws_down")], ids=["experts", "dense"])
+@pytest.mark.parametrize("simt", [False, True], ids=["tcgen05", "cuda_cores"])
+def test_second_moments_at_the_ends_of_their_range(rv, simt, names):
+    """Second moments of zero, subnormal, near the largest fp32 value, infinite and not a number.  The root of an infinite moment is
+    infinite and the step zero, as IEEE division has it; one that is not a number counts as zero, and so does a negative one.  All steps are
+    compared with fp64 at 2^-20: root and quotient by the hardware's approximations (2^-23 and 2 ulp) and three roundings (2^-24 each)
+    come to 2^-20.9.  2100 tokens: the adapter's update is that of the sums of its slices, the others' that of the product itself."""
+    cfg = BlockConfig("U", tokens=2100, d_model=256, n_experts=4, top_k=2, d_expert=128, d_shared=256, weight_dtype="bf16")
+    w, s = _weights(cfg, 35), make_streams(cfg, 35)
+    blk = make_block(cfg, w, flags=rv.FLAG_FORCE_SIMT if simt else 0)
+    y1 = dev(s["y1"])
+    inf, nan = float("inf"), float("nan")
+    vals = torch.tensor([0.0, 1.5e-45, 3e-42, 1e-39, 1.2e-38, 1e-30, 1e-12, 1.0, 1e20, 1e37, 3.4e38, inf, nan, -1.0], device="cuda")
+    eps, step, lr = 1e-20, 1000000, 1.0      # both bias corrections are 1 here
+    mom, var, masters, v0 = {}, {}, {}, {}
+    for n in names:
+        count = blk.weights[n].numel()
+        v0[n] = vals[torch.arange(count, device="cuda") % len(vals)].reshape(blk.weights[n].shape)
+        # first moments of the size of the root: steps of order one
+        root = torch.sqrt(torch.nan_to_num(v0[n].double().clamp(min=0), nan=0.0, posinf=1e38)) + eps
+        mom[n] = (root * (0.5 + torch.rand(root.shape, device="cuda", generator=torch.Generator("cuda").manual_seed(4)))).float().clamp(min=1e-30)
+        var[n], masters[n] = v0[n].clone(), torch.zeros_like(v0[n])
+    m0 = {n: t.clone() for n, t in mom.items()}
+    adam = rv.make_adam(lr, step, names, mom, var, masters, beta1=B1, beta2=B2, eps=eps)
+    blk.backward(y1, torch.zeros_like(y1), torch.zeros_like(y1), {}, sgd=adam)
+    assert blk.status() == 0
+    for n in names:
+        v = var[n].double()
+        assert torch.equal(torch.isnan(v), torch.isnan(v0[n]))
+        fin = torch.isfinite(v)
+        assert torch.allclose(v[fin], B2 * v0[n].double()[fin], rtol=2e-7, atol=2e-45)
+        assert torch.allclose(mom[n].double(), B1 * m0[n].double(), rtol=2e-7, atol=0)
+        root = torch.sqrt(torch.where(torch.isnan(v), torch.zeros_like(v), v).clamp(min=0))
+        want = -lr * mom[n].double() / (root + eps)
+        got = masters[n].double()
+        assert torch.isfinite(got).all() and (got[torch.isinf(v)] == 0).all()
+        assert torch.allclose(got, want, rtol=2.0 ** -20, atol=0), n
+
+
+def test_steps_against_64_bits(rv):
+    """The step of 400 k elements with second moments over eighty binary orders, from where eps decides to where it is lost.  A root
+    rounded correctly (2^-24), its sum with eps (2^-24) and a quotient by the hardware's reciprocal leave an rms error of 5.04e-8
+    (eight seeds: 5.03 .. 5.05) and 2^-22 at most; a root of the hardware's own precision leaves 5.37e-8."""
+    cfg = BlockConfig("U", tokens=200, d_model=256, n_experts=4, top_k=2, d_expert=128, d_shared=256, weight_dtype="bf16")
+    w, s = _weights(cfg, 36), make_streams(cfg, 36)
+    names = ("w_gate", "w_upx", "w_downx")
+    blk = make_block(cfg, w)
+    y1 = dev(s["y1"])
+    gen = torch.Generator("cuda").manual_seed(6)
+    eps, mom, var, masters = float(torch.tensor(1e-8)), {}, {}, {}      # (as fp32 holds it)
+    for n in names:
+        shape = blk.weights[n].shape
+        var[n] = torch.exp2(torch.rand(shape, device="cuda", generator=gen) * 81 - 66)
+        mom[n] = (var[n].sqrt() + eps) * (0.1 + 2 * torch.rand(shape, device="cuda", generator=gen))
+        masters[n] = torch.zeros(shape, device="cuda")
+    adam = rv.make_adam(1.0, 1000000, names, mom, var, masters, beta1=B1, beta2=B2, eps=eps)      # bias corrections of 1
+    blk.backward(y1, torch.zeros_like(y1), torch.zeros_like(y1), {}, sgd=adam)
+    assert blk.status() == 0
+    err = torch.cat([(-masters[n].double() * (var[n].double().sqrt() + eps) / mom[n].double() - 1).flatten() for n in names])
+    assert float(err.abs().max()) <= 2.0 ** -22 and float(err.square().mean().sqrt()) <= 5.2e-8
