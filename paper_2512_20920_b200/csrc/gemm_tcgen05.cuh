@@ -410,6 +410,14 @@ __device__ __forceinline__ uint2 pack4(const float4& v) {
   __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
   return make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
 }
+__device__ __forceinline__ float4 adam_step4(const UpdRule& r, const float4& w, const float4& g, float4& mom, float4& var) {
+  float2 m[2] = {make_float2(mom.x, mom.y), make_float2(mom.z, mom.w)}, v[2] = {make_float2(var.x, var.y), make_float2(var.z, var.w)};
+  const float2 lo = adam_step2(r, make_float2(w.x, w.y), make_float2(g.x, g.y), m[0], v[0]);
+  const float2 hi = adam_step2(r, make_float2(w.z, w.w), make_float2(g.z, g.w), m[1], v[1]);
+  mom = make_float4(m[0].x, m[0].y, m[1].x, m[1].y);
+  var = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+  return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
 
 // Fused update of a grouped product's tile (EPI_WADAM, EPI_WSGD): a warp's 16 rows x 128 columns, eight units of two rows.  Weights (the
 // fp32 master copy, or the bf16 weights themselves) and Adam's moments of a unit come by cp.async into a ring of UpdRing
@@ -476,10 +484,7 @@ __device__ __forceinline__ void upd_half(const UpdRule& rule, const SlabOut& o, 
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       if (ADAM) {
-        w[i].x = upd_step(rule, w[i].x, g[i].x, &mo[i].x, &va[i].x);
-        w[i].y = upd_step(rule, w[i].y, g[i].y, &mo[i].y, &va[i].y);
-        w[i].z = upd_step(rule, w[i].z, g[i].z, &mo[i].z, &va[i].z);
-        w[i].w = upd_step(rule, w[i].w, g[i].w, &mo[i].w, &va[i].w);
+        w[i] = adam_step4(rule, w[i], g[i], mo[i], va[i]);
         *reinterpret_cast<float4*>(o.mom + at + i * ldc) = mo[i];
         *reinterpret_cast<float4*>(o.var + at + i * ldc) = va[i];
       } else {
@@ -1369,10 +1374,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
                   if (!row_ok(h4 + i)) continue;
                   const float4 v = staged(h4 + i);
                   const int64_t at = out.at0 + c + (h4 + i) * out.ld4;
-                  w4[i].x = upd_step(p.upd, w4[i].x, v.x, &mo[i].x, &va[i].x);
-                  w4[i].y = upd_step(p.upd, w4[i].y, v.y, &mo[i].y, &va[i].y);
-                  w4[i].z = upd_step(p.upd, w4[i].z, v.z, &mo[i].z, &va[i].z);
-                  w4[i].w = upd_step(p.upd, w4[i].w, v.w, &mo[i].w, &va[i].w);
+                  w4[i] = adam_step4(p.upd, w4[i], v, mo[i], va[i]);
                   *reinterpret_cast<float4*>(out.mom + at) = mo[i];
                   *reinterpret_cast<float4*>(out.var + at) = va[i];
                   if (out.m) *reinterpret_cast<float4*>(out.m + at) = w4[i];
