@@ -1374,7 +1374,10 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
                   if (!row_ok(h4 + i)) continue;
                   const float4 v = staged(h4 + i);
                   const int64_t at = out.at0 + c + (h4 + i) * out.ld4;
-                  w4[i] = adam_step4(p.upd, w4[i], v, mo[i], va[i]);
+                  w4[i].x = upd_step(p.upd, w4[i].x, v.x, &mo[i].x, &va[i].x);
+                  w4[i].y = upd_step(p.upd, w4[i].y, v.y, &mo[i].y, &va[i].y);
+                  w4[i].z = upd_step(p.upd, w4[i].z, v.z, &mo[i].z, &va[i].z);
+                  w4[i].w = upd_step(p.upd, w4[i].w, v.w, &mo[i].w, &va[i].w);
                   *reinterpret_cast<float4*>(out.mom + at) = mo[i];
                   *reinterpret_cast<float4*>(out.var + at) = va[i];
                   if (out.m) *reinterpret_cast<float4*>(out.m + at) = w4[i];
