@@ -2056,13 +2056,14 @@ inline int launch_gemm_tc(const GemmProblem& p, cudaStream_t st) {
 
 #define TC_CASE(N_, E_) \
   if (mma_n == N_ && epi == E_) return tc_launch<N_, E_>(P, ma, mb0, mb1, mc, mc1, grid, pair, st);
-  // A fused update of a grouped product runs in its own form while the K range of a group is short (rows of K on average):
-  // beyond, the operand ring that the form gives up is worth more than its reads and writes.  Per 256 x 256 tile: a K step costs
-  // about 1400 clk with two stages, 1000 with three and 600 with six, the row-wise epilogue 39 k (Adam) or 9 k (SGD),
-  // the block-wise one 65 k or 17 k.  (Adam, experts' gate | up: 1491 against 2481 us at 8192 tokens, 1784 against 2594 at 16384.)
+  // A fused update of a grouped product runs in its own form while the K range of a group is short (rows of K on average): that form
+  // writes whole rows but has two stages (Adam) or three (SGD) where the other has six, so beyond some length the operand ring is worth
+  // more than the reads and writes.  The experts' two updates together, medians of three in turn, us, own form | the other:
+  // Adam at 1764 rows 3328 | 3838, 2037 3841 | 4048, 2105 3974 | 4169, 2173 4003 | 3992, 2310 4282 | 3933, 2446 4524 | 4222;
+  // SGD at 1081 1050 | 1318, 1218 1142 | 1301, 1354 1261 | 1301, 1491 1430 | 1353, 1627 1551 | 1381.
   const int64_t k_group = p.K / groups;
   const int epi = p.epilogue != EPI_WGRAD ? p.epilogue
-                  : p.upd_w && p.group_off && k_group <= (p.upd.kind ? 2560 : 1152) ? (p.upd.kind ? EPI_WADAM : EPI_WSGD)
+                  : p.upd_w && p.group_off && k_group <= (p.upd.kind ? 2176 : 1408) ? (p.upd.kind ? EPI_WADAM : EPI_WSGD)
                   : p.upd_w || p.accumulate ? EPI_WRMW : EPI_WGRAD;
   TC_CASE(256, EPI_STORE) TC_CASE(256, EPI_SWIGLU) TC_CASE(256, EPI_ROWSCALE) TC_CASE(256, EPI_COUPLE)
   TC_CASE(256, EPI_DSWIGLU) TC_CASE(256, EPI_WGRAD) TC_CASE(256, EPI_WADAM) TC_CASE(256, EPI_WSGD) TC_CASE(256, EPI_WRMW)

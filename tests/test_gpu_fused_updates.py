@@ -16,8 +16,8 @@ def rv():
     return rv
 
 
-# (tokens, experts, top_k): short K with empty experts; a K range past the row-wise form's bound for both rules
-@pytest.mark.parametrize("tokens,E,k", [(5, 6, 1), (300, 5, 2), (3000, 2, 2)])
+# (tokens, experts, top_k): short K with empty experts; a K range next to the row-wise form's bound for SGD and for Adam; past both
+@pytest.mark.parametrize("tokens,E,k", [(5, 6, 1), (300, 5, 2), (1250, 2, 2), (2000, 2, 2), (3000, 2, 2)])
 @pytest.mark.parametrize("master", [False, True])
 def test_update_equals_the_update_of_the_written_gradient(rv, tokens, E, k, master):
     cfg = BlockConfig("U", tokens=tokens, d_model=256, n_experts=E, top_k=k, d_expert=384, d_shared=0, weight_dtype="bf16")
