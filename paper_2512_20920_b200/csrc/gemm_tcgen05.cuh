@@ -347,12 +347,6 @@ __device__ __forceinline__ void unpack8(uint4 u, float* f) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) { float2 t = __bfloat1622float2(h[i]); f[2 * i] = t.x; f[2 * i + 1] = t.y; }
 }
-// store 32 floats as 32 bf16 (64 contiguous bytes)
-__device__ __forceinline__ void store32_bf16(bf16* dst, const float* f) {
-  uint4* o = reinterpret_cast<uint4*>(dst);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) o[i] = pack8(f + 8 * i);
-}
 
 // Output staging.  A warp stages a 32-row x 32-column bf16 block, one row per lane, in the layout
 // the store's tensor map expects: rows of 64 bytes under the 64-byte swizzle.  `buf` is aligned to
