@@ -900,9 +900,11 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
     // The grid has a CTA (pair) per tile, of which as many run as there is room for; a running one takes on the tile of
     // another that has not been launched yet whenever its loads begin a tile.  So it does not matter when an SM becomes free:
     // with tiles dealt out in advance, CTAs whose SM another stream's kernel held kept everybody waiting at the end, and the
-    // SMs that had finished earlier idled.  Both sides in turn: forward of 64 tokens 263 -> 249 us, steps at 512, 2741, 8192, 16384
-    // (Zipf) and 32768 tokens 1334 -> 1291, 2225 -> 2177, 5012 -> 4923, 9406 -> 9001, 18079 -> 17236, with fused Adam 7501 -> 7312, four
-    // d = 512 blocks 1476 -> 1421, three whole blocks 21815 -> 21161; attention alone, whose streams rarely meet, 2170 -> 2163.
+    // SMs that had finished earlier idled.  Both sides in turn, us, with what two runs of one side differ by in brackets: steps at 512,
+    // 8192, 16384 (Zipf) and 32768 tokens 1331 -> 1286 (0.0 %), 4955 -> 4844 (0.8), 8999 -> 8836 (0.5), 17304 -> 16926 (0.6), four d = 512
+    // blocks 1510 -> 1454 (0.2), attention alone, whose streams rarely meet, 2152 -> 2142 (0.0), three whole blocks 21267 -> 21074 (0.7: no
+    // difference shown); on other boxes forward of 64 tokens 263 -> 249, the step at 2741 2225 -> 2177, with fused Adam at 8192 7501 -> 7312.
+    // Where runs differ by 3-5 %, at the power cap, the steps from 8192 tokens on show nothing of it.
     // A tile's description costs this warp two divisions and a table look-up, one tile ahead of the loads.
     const int tiles_n = P.tr ? P.tiles_f : P.tiles_n;
     const int tiles_m = P.tr ? p.rows_total[1] : (PAIR ? (tiles_m_dev + 1) / 2 : tiles_m_dev);
