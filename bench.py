@@ -38,10 +38,10 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # (dram__bytes_read.sum + dram__bytes_write.sum; profiles/tensor_pipe_gemms_C1.md).
 # Keyed by pass/kernel; anything else, or any other workload, reports null.
 NCU_TRAFFIC_BYTES = {
-    "fwd/gemm_expert_gate_up_swiglu": 968_200_000, "inv/gemm_expert_gate_up_swiglu": 1_175_700_000,
-    "fwd/gemm_shared_gate_up_swiglu": 184_800_000, "inv/gemm_shared_gate_up_swiglu": 437_500_000,
-    "bwd/wgrad_expert_gate_up": 1_660_100_000, "bwd/wgrad_expert_down": 876_400_000,
-    "bwd/gemm_expert_du": 1_220_700_000, "bwd/wgrad_shared_gate_up": 425_400_000,
+    "fwd/gemm_expert_gate_up_swiglu": 920_800_000, "inv/gemm_expert_gate_up_swiglu": 1_097_900_000,
+    "fwd/gemm_shared_gate_up_swiglu": 179_000_000, "inv/gemm_shared_gate_up_swiglu": 440_400_000,
+    "bwd/wgrad_expert_gate_up": 1_659_800_000, "bwd/wgrad_expert_down": 869_900_000,
+    "bwd/gemm_expert_du": 1_011_500_000, "bwd/wgrad_shared_gate_up": 417_200_000,
 }
 
 
