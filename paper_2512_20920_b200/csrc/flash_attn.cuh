@@ -25,7 +25,7 @@
 // quarter k lies under the softmax, barriers); the exponentials alone are 2.0k (two warps per scheduler on a unit of four a
 // clock), the products 2.3k; a CTA starts and ends in 5-8k.  4 sequences of 2048 x 16 heads: 120 us with one query tile per
 // CTA, the output in registers and maxima exchanged through shared memory; 97 with two tiles; 88 with products issued by a
-// converged warp (the row maxima left out beside that: no difference); P in halves 92 -> 88 on another box.  The second sum
+// converged warp (the row maxima left out beside that: no difference); P in halves 92 -> 88 on another GPU.  The second sum
 // costs nothing there (82 and 82 us); a gradient pass, which wants both sums, fetches the second half's scores twice instead of
 // spilling registers (117 -> 103, 96 before it had them).  7 x 613: 38 -> 36 us when five query tiles made three pairs, now 30
 // (39 for a gradient pass).

@@ -903,7 +903,7 @@ gemm_tc_kernel(const __grid_constant__ TcParams P, const __grid_constant__ CUten
     // SMs that had finished earlier idled.  Both sides in turn, us, with what two runs of one side differ by in brackets: steps at 512,
     // 8192, 16384 (Zipf) and 32768 tokens 1331 -> 1286 (0.0 %), 4955 -> 4844 (0.8), 8999 -> 8836 (0.5), 17304 -> 16926 (0.6), four d = 512
     // blocks 1510 -> 1454 (0.2), attention alone, whose streams rarely meet, 2152 -> 2142 (0.0), three whole blocks 21267 -> 21074 (0.7: no
-    // difference shown); on other boxes forward of 64 tokens 263 -> 249, the step at 2741 2225 -> 2177, with fused Adam at 8192 7501 -> 7312.
+    // difference shown); on other GPUs forward of 64 tokens 263 -> 249, the step at 2741 2225 -> 2177, with fused Adam at 8192 7501 -> 7312.
     // Where runs differ by 3-5 %, at the power cap, the steps from 8192 tokens on show nothing of it.
     // A tile's description costs this warp two divisions and a table look-up, one tile ahead of the loads.
     const int tiles_n = P.tr ? P.tiles_f : P.tiles_n;
